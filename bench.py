@@ -305,7 +305,6 @@ def kernel_work(w, n_sel, selected=True):
         "select_count_kernel": (w.N * (8 + 4 * 4), None),
         "select_group_kernel": (w.N * 6 * 4, None),
         "select_sample_kernel": (w.N * 4 * 4, None),
-        "gather_kernel": (2 * 3 * kept * row, None),
         "attn_fwd_kernel": (3 * kept * row + kept * row + kept * w.H * 4, 4.0 * w.B * w.H * n_sel * n_sel * w.D),
         "bwd_prep_kernel": (2 * kept * row + kept * row + kept * w.H * 64 * 4, None),
         "attn_bwd_kernel": (5 * kept * row + kept * w.H * 4 + grads, 10.0 * w.B * w.H * n_sel * n_sel * w.D),
@@ -427,7 +426,7 @@ def traffic_targets(torch, vd, inputs, dist_util, device, rank, peaks, barrier, 
             "n862_attn_fwd_us": off["attn_fwd_ms"] * 1e3, "n862_attn_bwd_us": off["attn_bwd_ms"] * 1e3,
             "n862_attn_tflops": off["attn_tflops"], "n862_attn_frac_of_bf16_peak": off["attn_frac_of_bf16_peak"],
             "n862_attn_target_frac": 0.5,
-            "hash": pick("hash_kernel"), "select": pick("select_small_kernel"), "gather": pick("gather_kernel"),
+            "hash": pick("hash_kernel"), "select": pick("select_small_kernel"),
             "hbm_target_frac": 0.6,
             "note": "per-kernel durations by CUDA events around every launch; fractions use algorithmic bytes / flops and the measured peaks"}
 

@@ -219,7 +219,7 @@ int vardrop_gather_rows(const float* x, const int32_t* sel_idx, const int32_t* n
  * o           [B, N, H, D] bf16 out; rows 0..n_sel[s(b)]-1 of instance b hold O', the rest is untouched.
  * lse         [B, H, N] float32 out; entries 0..n_sel[s(b)]-1 valid.
  * ws          scratch of vardrop_attn_workspace_bytes.  After the call it holds what the backward pass of the same
- *             step needs (staged Q', K', V' where the library stages them, a cleared dQ' accumulator):
+ *             step needs (a cleared dQ' accumulator, counters):
  *             vardrop_attn_bwd must be given the same, unmodified workspace, once per forward call.
  * ---------------------------------------------------------------------------------------------- */
 typedef struct {

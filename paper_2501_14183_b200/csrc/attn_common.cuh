@@ -9,12 +9,12 @@
 namespace vardrop {
 
 constexpr int kTile = 128;          // tokens per query tile and per key tile
-constexpr int kDP = 64;             // head dimension the kernels run at (D = 32 is zero-padded to it)
+constexpr int kDP = 64;             // elements per tile row (heads of 32 leave the upper half zero)
 constexpr int kRowBytes = kDP * 2;  // one (token, head) row of bf16: 128 bytes = one swizzle row
 constexpr int kTileBytes = kTile * kRowBytes;   // 16 KiB
 
 struct AttnWs {
-    size_t qg, kg, vg, dog;   // staged [B, Ncap, H, 64] bf16 copies (gathered and/or padded)
+    size_t staged[4];         // [B, Ncap, H, D] bf16 copies of the kept rows of Q, K, V and of dO (selections of many tiles)
     size_t delta;             // [B, H, Ncap] fp32
     size_t dq_acc;            // [B, Ncap, H, 64] fp32
     size_t tile_done;         // [B, H] int32: key tiles of (b, h) whose backward work is complete
@@ -25,25 +25,19 @@ struct AttnWs {
 inline AttnWs attn_layout(const vardrop_attn_cfg& c) {
     AttnWs w;
     w.Ncap = (c.N + kTile - 1) / kTile * kTile;
-    const size_t staged = static_cast<size_t>(c.B) * w.Ncap * c.H * kRowBytes;
     size_t o = kWsHeaderBytes;
-    w.qg = o; o += align_up(staged, 1024);
-    w.kg = o; o += align_up(staged, 1024);
-    w.vg = o; o += align_up(staged, 1024);
-    w.dog = o; o += align_up(staged, 1024);
+    for (size_t& s : w.staged) { s = o; o += align_up(static_cast<size_t>(c.B) * w.Ncap * c.H * kRowBytes, 1024); }
     w.delta = o; o += align_up(sizeof(float) * c.B * c.H * w.Ncap, 1024);
-    w.dq_acc = o; o += align_up(staged * 2, 1024);
+    w.dq_acc = o; o += align_up(static_cast<size_t>(c.B) * w.Ncap * c.H * kDP * sizeof(float), 1024);
     w.tile_done = o; o += align_up(sizeof(int32_t) * c.B * c.H, 1024);
     w.total = o;
     return w;
 }
 
-// Tensor map over a [B, tokens, H, 64] bf16 tensor: box = one (b, h) tile of 128 tokens x 64 elements,
-// 128-byte swizzle, out-of-range rows read as zero.  `tokens` is the extent the copy engine may touch,
-// `token_stride` the allocated tokens per instance.
-// Tensor map over the same memory seen as [rows, 64] bf16 (rows = B * tokens * H) for row gathers: box = one row,
-// 128-byte swizzle, rows outside the tensor read as zero.
-int make_row_map(CUtensorMap* map, const void* base, long long rows, long long row_stride_elems);
+// Tensor map over a [B, tokens, H, D] bf16 tensor with the given element strides: box = one (b, h) tile of 128 tokens x 64
+// elements, 128-byte swizzle.  What lies outside the tensor reads as zero: tokens past the end, and the upper half of a 64-element
+// row of a tensor with D = 32.
+int make_tile_map(CUtensorMap* map, const void* base, int D, int B, int tokens, int H, long long sB, long long sN, long long sH);
 
 // Tensor map over the fp32 dQ' accumulator [B, Ncap, H, 64]: box = 128 tokens x 32 floats (one 128-byte swizzled row
 // per token) of one head, the unit of the backward kernel's bulk reduce-add.
@@ -52,15 +46,9 @@ int make_acc_map(CUtensorMap* map, const void* base, int B, int Ncap, int H);
 // Number of SMs of the current device (cached per thread and device).
 int sm_count();
 
-int make_tile_map(CUtensorMap* map, const void* base, int B, int tokens, int H, long long sB, long long sN, long long sH);
-
-// Element strides of q, k, v as the kernels see them.  The row view (one 64-element row per (instance, token, head), rows a
-// constant distance apart) exists when sN and sB are multiples of sH: row(b, n, h) = b row_b + n row_n + h.
+// Element strides of q, k, v (the head dimension is contiguous).
 struct QkvLayout {
-    long long sB, sN, sH;       // element strides
-    bool row_linear;            // the row view exists
-    long long rows_total;       // rows of that view (one past the last is the zero row of the gathers)
-    long long row_b, row_n;
+    long long sB, sN, sH;
 };
 inline QkvLayout qkv_layout(const vardrop_attn_cfg& c) {
     QkvLayout L;
@@ -68,10 +56,6 @@ inline QkvLayout qkv_layout(const vardrop_attn_cfg& c) {
     L.sH = dflt ? c.D : c.sH;
     L.sN = dflt ? static_cast<long long>(c.H) * c.D : c.sN;
     L.sB = dflt ? static_cast<long long>(c.N) * c.H * c.D : c.sB;
-    L.row_linear = L.sN % L.sH == 0 && L.sB % L.sH == 0;
-    L.row_n = L.row_linear ? L.sN / L.sH : 0;
-    L.row_b = L.row_linear ? L.sB / L.sH : 0;
-    L.rows_total = L.row_linear ? (c.B - 1) * L.row_b + (c.N - 1) * L.row_n + c.H : 0;
     return L;
 }
 
@@ -80,79 +64,102 @@ __device__ __forceinline__ unsigned char* align_tiles(unsigned char* p) {
     return reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~static_cast<uintptr_t>(1023));
 }
 
-// How a 128-token operand tile reaches shared memory.
-//   tiled    one 4-D box of the [B, tokens, H, 64] tensor (tokens tok0 .. tok0 + 127 of head h, instance b)
-//   gathered 32 row gathers of 4 rows each from the [rows, 64] view: slot j of the tile is variate idx[tok0 + j]
-//            (idx = NULL: the slot itself) while tok0 + j < n_valid, and a row past the end (zeros) otherwise.
-// Called by all 32 lanes of one warp; `lane0_expect` bytes are announced on the barrier by lane 0 first.
-struct TileSource {
-    const int32_t* idx;    // gather indices of the instance's selection (NULL: identity)
-    int gathered;          // 0: tiled box, 1: row gathers
-    int tokens;            // tokens per instance in the gathered tensor
-    int rows_total;        // rows of the [rows, 64] view; row(b, n, h) = b row_b + n row_n + h
-    int row_b, row_n;
+// ---- how a 128-token operand tile reaches shared memory ------------------------------------------------------------
+// Without a selection: one box of the caller's tensor by the copy engine.  With one: 16-byte asynchronous copies of the kept
+// variates' rows straight from the caller's tensor, any strides (row j of the tile is variate idx[tok0 + j], zeros from n_valid
+// on).  (Row gathers by the copy engine, four rows an instruction, take 18 ns each, 0.6 us a tile: the many-tile forward of 1423 kept
+// tokens ran 134 us with them against 97 with copies.)
+__device__ __forceinline__ void cp_async16(uint32_t dst_smem, const void* src, uint32_t src_bytes) {      // src_bytes 16, or 0: zeros
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst_smem), "l"(src), "r"(src_bytes) : "memory");
+}
+// This thread arrives on `bar` once all its copies so far have landed (the barrier's count includes the arrival).  The tensor core
+// reads through the async proxy: the waiter puts a proxy fence between its wait and the product.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// Two warps share a tile, 64 rows each; `part` is this warp's place.  Eight lanes copy a row, lane group g = lane / 8 the sixteen rows
+// from 64 part + 16 g on, whose sources every lane holds (no exchange between lanes: the copies share their issue queue with the
+// exponentials of the softmax warps).
+struct RowPicks {
+    int n[16];                      // source rows, -1: none
 };
-// Rows of the [rows, 64] view that the four slots tok0 + 4 lane .. + 3 of a gathered tile name (a row past the end for
-// slots at or past n_valid).  `picks` are the four entries idx[tok0 + 4 lane ..] (see tile_picks), fetched ahead of
-// time so that several tiles over the same slots share one fetch.
-__device__ __forceinline__ int4 tile_picks(const TileSource& src, int tok0) {
-    const int lane = threadIdx.x & 31;
-    const int slot = tok0 + 4 * lane;
-    if (!src.gathered || !src.idx) return make_int4(slot, slot + 1, slot + 2, slot + 3);
-    int4 p;
-    p.x = slot + 0 < src.tokens ? src.idx[slot + 0] : -1;
-    p.y = slot + 1 < src.tokens ? src.idx[slot + 1] : -1;
-    p.z = slot + 2 < src.tokens ? src.idx[slot + 2] : -1;
-    p.w = slot + 3 < src.tokens ? src.idx[slot + 3] : -1;
+__device__ __forceinline__ RowPicks tile_picks(const int32_t* idx, int tok0, int n_valid, int part) {
+    RowPicks p;
+    const int slot = tok0 + part * 64 + ((threadIdx.x & 31) >> 3) * 16;
+    if (slot + 16 <= n_valid && (reinterpret_cast<uintptr_t>(idx + slot) & 15) == 0) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int4 v = __ldg(reinterpret_cast<const int4*>(idx + slot) + e);
+            p.n[4 * e] = v.x; p.n[4 * e + 1] = v.y; p.n[4 * e + 2] = v.z; p.n[4 * e + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) p.n[e] = slot + e < n_valid ? __ldg(idx + slot + e) : -1;
+    }
     return p;
 }
-__device__ __forceinline__ void load_tile_picked(unsigned char* dst, const CUtensorMap* map, uint64_t* bar, const TileSource& src, int4 picks,
-                                                 int tok0, int n_valid, int h, int b, int H) {
-    const int lane = threadIdx.x & 31;
-    if (!src.gathered) {
-        if (lane == 0) tma_load_4d(dst, map, bar, 0, h, tok0, b);
-        return;
-    }
-    const int slot = tok0 + 4 * lane;
-    const int n[4] = {picks.x, picks.y, picks.z, picks.w};
-    int rows[4];
+// The picked rows of one tensor to a tile, or of two tensors (with kTwo) to two tiles in a row.
+template <bool kTwo>
+__device__ __forceinline__ void copy_tile_rows(unsigned char* tile, const __nv_bfloat16* base, const __nv_bfloat16* base2, long long sN, const RowPicks& picks, int D, int part) {
+    const int lane = threadIdx.x & 31, chunk = lane & 7;
+    const uint32_t live = chunk * 8 < D ? 16u : 0u;             // heads of 32: the upper half of the row is zeros
+    const int c0 = live ? chunk * 8 : 0;
+    const uint32_t dst = smem_u32(tile) + (part * 64 + (lane >> 3) * 16) * kRowBytes;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) rows[e] = (slot + e < n_valid && n[e] >= 0) ? b * src.row_b + n[e] * src.row_n + h : src.rows_total;
-    tma_gather4(dst + lane * 4 * kRowBytes, map, bar, 0, rows[0], rows[1], rows[2], rows[3]);
+    for (int it = 0; it < 16; ++it) {
+        const long long off = static_cast<long long>(max(picks.n[it], 0)) * sN + c0;
+        const uint32_t to = dst + it * kRowBytes + (static_cast<uint32_t>(chunk ^ (it & 7)) << 4), bytes = picks.n[it] >= 0 ? live : 0u;
+        cp_async16(to, base + off, bytes);
+        if (kTwo) cp_async16(to + kTileBytes, base2 + off, bytes);
+    }
 }
-__device__ __forceinline__ void load_tile(unsigned char* dst, const CUtensorMap* map, uint64_t* bar, const TileSource& src, int tok0, int n_valid,
-                                          int h, int b, int H) {
-    load_tile_picked(dst, map, bar, src, tile_picks(src, tok0), tok0, n_valid, h, b, H);
+// One warp's share of a tile when the whole CTA loads: 32 rows from tok0 on.  (Two loader warps need some 500 cycles a tile, bound by
+// the latency of their address chains; a dozen warps bring the first tiles of a CTA in together.)
+__device__ __forceinline__ void copy_32_rows(unsigned char* rows, const __nv_bfloat16* base, long long sN, const int32_t* idx, int tok0, int n_valid, int D) {
+    const int lane = threadIdx.x & 31, chunk = lane & 7, slot = tok0 + lane;
+    const int pick = slot < n_valid ? (idx ? __ldg(idx + slot) : slot) : -1;
+    const uint32_t live = chunk * 8 < D ? 16u : 0u;
+    const __nv_bfloat16* src = base + (live ? chunk * 8 : 0);
+    const uint32_t dst = smem_u32(rows) + (lane >> 3) * kRowBytes + (static_cast<uint32_t>(chunk ^ (lane >> 3)) << 4);
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int n = __shfl_sync(0xffffffffu, pick, 4 * it + (lane >> 3));
+        cp_async16((dst ^ ((it & 1) * 64u)) + it * 4 * kRowBytes, src + static_cast<long long>(max(n, 0)) * sN, n >= 0 ? live : 0u);
+    }
+}
+// Quotient of 0 <= a by 1 <= d in a few instructions (an integer division is some forty dependent ones); the correction loops run
+// more than once only for quotients beyond 2^22.
+__device__ __forceinline__ int small_div(int a, int d) {
+    int q = static_cast<int>(__fdividef(static_cast<float>(a), static_cast<float>(d)));
+    int r = a - q * d;
+#pragma unroll 1
+    while (r < 0) { r += d; --q; }
+#pragma unroll 1
+    while (r >= d) { r -= d; ++q; }
+    return q;
 }
 
-// Three ways for the operand tiles to reach shared memory:
-//   direct   4-D boxes of the caller's tensors                       (no selection, D = 64)
-//   gathered row gathers of the kept variates from the caller's tensors   (selection, D = 64, N <= kGatherMaxN: the kept set
-//            is at most a few tiles, so re-gathering rows per tile pair costs less than a staging pass)
-//   staged   4-D boxes of compacted copies in the workspace, written by the gather kernel   (D = 32, which is also
-//            zero-padded to 64 there; or a selection at large N, where every tile is re-read many times and
-//            contiguous, L2-resident tiles pay for the extra pass)
-constexpr int kGatherMaxN = 512;
+// Whether the backward may meet many key tiles per head and instance, and so takes its row statistics and the dQ' accumulator from a
+// launch of its own: the kept count is only known on the device, so the host goes by the largest it can be.  A selection keeps a
+// fraction of the variates (a tenth to a third in the paper's settings); up to kManyTilesN variates that is a handful of tiles.
+constexpr int kManyTilesN = 2048;
+inline bool attn_many_tiles(const vardrop_attn_cfg& c, const int32_t* sel_idx) { return sel_idx ? c.N > kManyTilesN : c.N > 2 * kTile; }
+
+// Whether the forward pass clears the dQ' accumulator, under its own work: for a selection (only training passes one), and where no
+// prep launch follows; without a selection the forward pass may be inference, and the prep launch does it.
+inline bool attn_fwd_clears(const vardrop_attn_cfg& c, const int32_t* sel_idx) { return sel_idx != nullptr || !attn_many_tiles(c, sel_idx); }
+
 // Number of selection rows: one shared by the batch, or one per instance.
 inline int attn_sel_rows(const vardrop_attn_cfg& c) { return c.S > 1 ? c.S : 1; }
 
-// Largest kept count over the selection rows (device, whole CTA; `scratch` is one int of shared memory).
-__device__ __forceinline__ int max_kept(const int32_t* n_sel, int S, int N, int* scratch) {
+// Kept count that sizes the work: of the one selection, the largest of several (each warp looks on its own), or N.
+__device__ __forceinline__ int largest_kept(const int32_t* n_sel, int S, int N) {
     if (!n_sel) return N;
-    if (threadIdx.x == 0) *scratch = 0;
-    __syncthreads();
+    if (S <= 1) return __ldg(n_sel);
     int m = 0;
-    for (int s = threadIdx.x; s < S; s += blockDim.x) m = max(m, n_sel[s]);
-    if (m > 0) atomicMax(scratch, m);
-    __syncthreads();
-    return *scratch;
+#pragma unroll 1
+    for (int s = threadIdx.x & 31; s < S; s += 32) m = max(m, __ldg(n_sel + s));
+    return __reduce_max_sync(0xffffffffu, m);
 }
-
-// (row gathers also need the row view of the caller's strides and row indices that fit 31 bits; other layouts are staged)
-inline bool attn_uses_gather(const vardrop_attn_cfg& c, const int32_t* sel_idx) {
-    const QkvLayout L = qkv_layout(c);
-    return c.D == kDP && sel_idx != nullptr && c.N <= kGatherMaxN && L.row_linear && L.rows_total < (1ll << 31);
-}
-inline bool attn_uses_staging(const vardrop_attn_cfg& c, const int32_t* sel_idx) { return c.D != kDP || (sel_idx != nullptr && !attn_uses_gather(c, sel_idx)); }
 
 }  // namespace vardrop

@@ -85,6 +85,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// One look at a phase, without the suspension that try_wait allows itself.
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 // Bounded wait: polls until the phase completes or about two seconds of wall time have passed, then reports
 // failure instead of spinning forever.
 __device__ __forceinline__ uint64_t global_ns() {
@@ -93,30 +105,30 @@ __device__ __forceinline__ uint64_t global_ns() {
     return t;
 }
 constexpr uint64_t kWaitLimitNs = 2000000000ull;      // every wait of the library gives up after about two seconds
+// (The poll loops stay rolled: unrolled they made a kernel with a dozen waits 120 to 200 KB of code, and what runs once an item then
+// spends its time on instruction fetch.)
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
-    for (int it = 0; it < 64; ++it)
-        if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = global_ns();
+    uint32_t polls = 0;
+#pragma unroll 1
     for (;;) {
-        for (int it = 0; it < 256; ++it)
-            if (mbar_try_wait(bar, parity)) return true;
-        if (global_ns() - t0 > limit_ns) return false;
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((++polls & 63u) == 0 && global_ns() - t0 > limit_ns) return false;
     }
 }
-// The same for warps off the critical path: a failed poll is followed by a short sleep, so that a waiting warp leaves the
-// issue slots of its scheduler to the warps that work (a spinning warp issues a poll loop's instructions back to back).
-#ifndef VD_SLEEP_NS
-#define VD_SLEEP_NS 32
-#endif
+// The same for warps that wait long or are off the critical path: after a few polls every further one is followed by a short sleep,
+// so that a waiting warp leaves the issue slots of its scheduler to the warps that work (a spinning warp issues a poll loop's
+// instructions back to back).
 __device__ __forceinline__ bool mbar_wait_relaxed(uint64_t* bar, uint32_t parity) {
     if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = global_ns();
+    uint32_t polls = 0;
+#pragma unroll 1
     for (;;) {
-        for (int it = 0; it < 64; ++it) {
-            if (mbar_try_wait(bar, parity)) return true;
-            if (VD_SLEEP_NS > 0) __nanosleep(VD_SLEEP_NS);
-        }
-        if (global_ns() - t0 > kWaitLimitNs) return false;
+        if (mbar_try_wait(bar, parity)) return true;
+        if (++polls > 4) __nanosleep(20);
+        if ((polls & 63u) == 0 && global_ns() - t0 > kWaitLimitNs) return false;
     }
 }
 
