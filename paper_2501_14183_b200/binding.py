@@ -1,4 +1,4 @@
-"""ctypes binding of libvardrop.so: argument marshalling only.
+"""Binding of libvardrop.so: argument marshalling only (the calls of a step by the extension module `_marshal`, the rest by ctypes).
 
 Every function has the name and the argument order of its C entry point in ``include/vardrop.h``; tensors are
 ``torch.Tensor`` objects on the CUDA device (PyTorch is used for device memory and streams only), the stream is
@@ -14,6 +14,7 @@ import torch
 
 _LIB_PATH = Path(__file__).resolve().parent / "libvardrop.so"
 _lib = None
+_marshal = None
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_NONFINITE = range(7)
 SCOPE_BATCH_MEAN, SCOPE_PER_INSTANCE = 0, 1
@@ -96,6 +97,15 @@ def load() -> C.CDLL:
     return _lib
 
 
+def _load_marshal():
+    """The extension module that reads pointers off the tensors and calls the library (built next to it; a missing one is an error)."""
+    global _marshal
+    load()
+    from . import _marshal as module
+    _marshal = module
+    return module
+
+
 def _ptr(t):
     return None if t is None else t.data_ptr()        # a plain int converts to void* without a ctypes object per argument
 
@@ -130,37 +140,29 @@ def vardrop_attn_workspace_bytes(cfg: AttnCfg) -> int:
 
 
 def vardrop_hash(x, cfg: HashCfg, keys, freqs, amp_dbg, ws) -> None:
-    _check(load().vardrop_hash(_ptr(x), C.byref(cfg), _ptr(keys), _ptr(freqs), _ptr(amp_dbg), _ptr(ws),
-                               ws.numel() * ws.element_size(), _stream()), "vardrop_hash")
+    _check((_marshal or _load_marshal()).hash(x, cfg, keys, freqs, amp_dbg, ws), "vardrop_hash")
 
 
 def vardrop_select(keys, cfg: SelectCfg, group_id, group_offsets, members, n_groups, sel_idx, n_sel, inv_idx, ws) -> None:
-    _check(load().vardrop_select(_ptr(keys), C.byref(cfg), _ptr(group_id), _ptr(group_offsets), _ptr(members), _ptr(n_groups),
-                                 _ptr(sel_idx), _ptr(n_sel), _ptr(inv_idx), _ptr(ws), ws.numel() * ws.element_size(),
-                                 _stream()), "vardrop_select")
+    _check((_marshal or _load_marshal()).select(keys, cfg, group_id, group_offsets, members, n_groups, sel_idx, n_sel, inv_idx, ws), "vardrop_select")
 
 
 def vardrop_select_static(keys, cfg: SelectCfg, group_id, group_offsets, members, n_groups, sel_idx, n_sel, inv_idx) -> None:
     """vardrop_select for callers that cannot allocate: no workspace argument, the scratch is a fixed array inside the
     library (S * N <= 16384).  Calls whose GPU work overlaps share that array and race."""
-    _check(load().vardrop_select_static(_ptr(keys), C.byref(cfg), _ptr(group_id), _ptr(group_offsets), _ptr(members),
-                                        _ptr(n_groups), _ptr(sel_idx), _ptr(n_sel), _ptr(inv_idx), _stream()),
-           "vardrop_select_static")
+    _check((_marshal or _load_marshal()).select_static(keys, cfg, group_id, group_offsets, members, n_groups, sel_idx, n_sel, inv_idx), "vardrop_select_static")
 
 
 def vardrop_gather_rows(x, sel_idx, n_sel, cfg: GatherCfg, x_sel) -> None:
-    _check(load().vardrop_gather_rows(_ptr(x), _ptr(sel_idx), _ptr(n_sel), C.byref(cfg), _ptr(x_sel), _stream()), "vardrop_gather_rows")
+    _check((_marshal or _load_marshal()).gather_rows(x, sel_idx, n_sel, cfg, x_sel), "vardrop_gather_rows")
 
 
 def vardrop_attn_fwd(q, k, v, sel_idx, n_sel, cfg: AttnCfg, o, lse, ws) -> None:
-    _check(load().vardrop_attn_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(sel_idx), _ptr(n_sel), C.byref(cfg), _ptr(o), _ptr(lse),
-                                   _ptr(ws), ws.numel() * ws.element_size(), _stream()), "vardrop_attn_fwd")
+    _check((_marshal or _load_marshal()).attn_fwd(q, k, v, sel_idx, n_sel, cfg, o, lse, ws), "vardrop_attn_fwd")
 
 
 def vardrop_attn_bwd(q, k, v, o, lse, d_o, sel_idx, n_sel, inv_idx, cfg: AttnCfg, dq, dk, dv, ws) -> None:
-    _check(load().vardrop_attn_bwd(_ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(d_o), _ptr(sel_idx), _ptr(n_sel),
-                                   _ptr(inv_idx), C.byref(cfg), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(ws),
-                                   ws.numel() * ws.element_size(), _stream()), "vardrop_attn_bwd")
+    _check((_marshal or _load_marshal()).attn_bwd(q, k, v, o, lse, d_o, sel_idx, n_sel, inv_idx, cfg, dq, dk, dv, ws), "vardrop_attn_bwd")
 
 
 def vardrop_pearson_workspace_bytes(cfg: PearsonCfg) -> int:
@@ -168,8 +170,7 @@ def vardrop_pearson_workspace_bytes(cfg: PearsonCfg) -> int:
 
 
 def vardrop_pearson_max(x, cfg: PearsonCfg, max_rho, n_above, ws) -> None:
-    _check(load().vardrop_pearson_max(_ptr(x), C.byref(cfg), _ptr(max_rho), _ptr(n_above), _ptr(ws), ws.numel() * ws.element_size(),
-                                      _stream()), "vardrop_pearson_max")
+    _check((_marshal or _load_marshal()).pearson_max(x, cfg, max_rho, n_above, ws), "vardrop_pearson_max")
 
 
 def vardrop_launch_count() -> int:

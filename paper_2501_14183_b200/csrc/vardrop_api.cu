@@ -1,5 +1,6 @@
 // C ABI of the library: argument checks, workspace carving, status text.  All arithmetic lives in the
 // kernel translation units; nothing here allocates device memory or synchronises.
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -42,19 +43,19 @@ static int check_ws(const void* ws, size_t have, size_t need) {
 // ---- launch counter and optional per-kernel event timer ---------------------------------------------------
 namespace {
 std::mutex g_prof_mutex;
-bool g_prof_on = false;
-long long g_launches = 0;
+std::atomic<bool> g_prof_on{false};                                        // read on every launch, so without the lock
+std::atomic<long long> g_launches{0};
 std::vector<std::pair<cudaEvent_t, cudaEvent_t>> g_prof_events[K_COUNT];   // pairs recorded since the timer was armed
 std::vector<std::pair<cudaEvent_t, cudaEvent_t>> g_prof_free;              // pairs ready for reuse
-const char* const g_kernel_names[K_COUNT] = {"hash_kernel", "select_small_kernel", "select_count_kernel", "select_group_kernel", "select_sample_kernel", 
+const char* const g_kernel_names[K_COUNT] = {"hash_kernel", "select_small_kernel", "select_count_kernel", "select_group_kernel", "select_sample_kernel",
                                              "attn_fwd_kernel", "bwd_prep_kernel", "attn_bwd_kernel", "bwd_convert_kernel", "pearson_normalize_kernel",
                                              "pearson_max_kernel", "gather_rows_kernel"};
 }  // namespace
 
 LaunchScope::LaunchScope(int id, cudaStream_t stream) : id_(id), stream_(stream), stop_(nullptr) {
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (!g_prof_on.load(std::memory_order_relaxed)) return;
     std::lock_guard<std::mutex> lock(g_prof_mutex);
-    ++g_launches;
-    if (!g_prof_on) return;
     std::pair<cudaEvent_t, cudaEvent_t> ev;
     if (!g_prof_free.empty()) {
         ev = g_prof_free.back();
@@ -128,8 +129,7 @@ int vardrop_probe_bounded_wait(void* ws, size_t ws_bytes, unsigned int limit_us,
 }
 
 long long vardrop_launch_count(void) {
-    std::lock_guard<std::mutex> lock(g_prof_mutex);
-    return g_launches;
+    return g_launches.load(std::memory_order_relaxed);
 }
 
 int vardrop_profile_kernels(void) { return K_COUNT; }
