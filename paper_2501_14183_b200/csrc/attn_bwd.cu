@@ -110,7 +110,7 @@ struct BwdParams {
     __nv_bfloat16* dv;
     const int32_t* sel_idx; // [S, N]; NULL: identity
     const int32_t* inv_idx; // [S, N]; NULL: identity (nothing dropped)
-    int32_t* tile_done;     // [B, H] key tiles finished per (instance, head); zeroed by the forward pass
+    int32_t* tile_done;     // few tiles: [B, H] items whose part of dQ' has landed; zeroed by the forward pass
     const int32_t* n_sel;   // [S]; NULL: N
     int* status;
     long long sB, sN, sH;   // element strides of q, k, v
@@ -119,21 +119,15 @@ struct BwdParams {
 };
 
 constexpr int kBwdGroup = 256;
-// Few key tiles: the first warpgroup issues and loads, two worker groups follow, one of which also takes dQ out of tensor memory.  Many: a
-// second warpgroup of its own takes dQ out (8192 variates: 3500 us against 3790 without it; one or two tiles: 23 us against 19).
-// Register split (setmaxnreg works on whole warpgroups), within what the block was launched with: few, 640 x 96 = 128 x 64 + 512 x 104;
-// many, 768 x 80 = 256 x 48 + 512 x 96.
-template <bool kMany>
-struct BwdShape {
-    static constexpr int kFirst = kMany ? 8 : 4;                   // first worker warp
-    static constexpr int kThreads = kFirst * 32 + 2 * kBwdGroup;
-    static constexpr int kSmallRegs = kMany ? 48 : 64, kBigRegs = kMany ? 96 : 104;
-};
+constexpr int kBwdThreads = 256 + 2 * kBwdGroup;
+// Register split (setmaxnreg works on whole warpgroups): launched with 768 x 80 = 61440 registers; the first two warpgroups keep 56 a
+// thread, the teams take 88: 256 x 56 + 512 x 88 = 59392.
+constexpr int kBwdSmallRegs = 56;
+constexpr int kBwdBigRegs = 88;
 constexpr uint32_t kBwdTmemCols = 512;
-constexpr int kSlots = 3;              // ring of query-tile operands (Q tile, dO tile)
-constexpr int kBwdHeader = 6144;       // barriers, item list, row statistics
-constexpr int kBwdSmemBytes = kBwdHeader + 2 * kTileBytes /*K, V*/ + 2 * kSlots * kTileBytes /*Q, dO ring*/ + 2 * kTileBytes /*dS^T*/ +
-                              2 * kTileBytes /*dQ tile, fp32, two 32-column halves*/;
+constexpr int kBwdHeader = 3072;       // barriers, item list, row statistics
+constexpr int kBwdSmemBytes = kBwdHeader + 4 * kTileBytes /*K, V of two key tiles*/ + 4 * kTileBytes /*two slots of Q, dO*/ +
+                              4 * kTileBytes /*dS^T of two key tiles*/ + 2 * kTileBytes /*dQ tile, fp32, two 32-column halves*/;
 
 // The arithmetic between the products, as instructions that keep their order: left to itself the compiler puts the consumers of a pair
 // of exponentials right behind it and a warp runs at the latency of the special-function unit instead of its rate.
@@ -162,6 +156,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     uint32_t d;
     asm volatile("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
     return d;
+}
+
+// A pair of floats from shared memory, issued here.  Read by all lanes alike, 8 bytes take 0.6 cycles of the shared-memory pipe, 16 bytes 2.1.
+__device__ __forceinline__ uint64_t lds_pair(uint32_t addr) {
+    uint64_t v;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr));
+    return v;
 }
 
 // every lane of the warp waits; the result is the same in all of them
@@ -196,33 +197,43 @@ __device__ __forceinline__ bool drain_sync_and(bool ok) {     // the same among 
 }
 __device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, 256;" ::"r"(id) : "memory"); }
 
-// Zero rows of dq, dk, dv for every dropped variate, by warps off the critical path.  The rows of all instances are dealt out in rounds
-// of 32 per warp: `part` of `parts` warps of the grid looks rows (part + round parts) 32 .. + 31 up in inv_idx, one a lane, and
-// writes the dropped ones, 512 bytes a store instruction.
-__device__ __forceinline__ int zero_row_rounds(const BwdParams& P, int parts) { return P.inv_idx ? (P.B * P.N + parts * 32 - 1) / (parts * 32) : 0; }
-__device__ __forceinline__ void zero_rows_round(const BwdParams& P, int part, int parts, int round) {
+// Zero rows of dq, dk, dv for every dropped variate, by whichever warps of the CTA have nothing else to do: they take the CTA's rows eight at
+// a time from a shared counter, look them up in inv_idx, and write one dropped row a call, 512 bytes a store instruction.  One row at a time,
+// between other work: written in one go by every CTA at once they fill the memory's queues, and row loads behind them took 10000 cycles (200
+// of 862 kept).
+struct ZeroRows {
+    int* taken;                         // groups of eight rows taken so far, by all warps of the CTA
+    int base;
+    unsigned mask;                      // dropped rows of the current group still to write
+};
+__device__ __forceinline__ bool write_zero_row(const BwdParams& P, ZeroRows& z) {      // false: none left
     const int lane = threadIdx.x & 31;
+    if (!P.inv_idx) return false;
+#pragma unroll 1
+    while (z.mask == 0) {
+        int g = 0;
+        if (lane == 0) g = atomicAdd(z.taken, 1);
+        z.base = (blockIdx.x + __shfl_sync(0xffffffffu, g, 0) * gridDim.x) * 8;
+        if (z.base >= P.B * P.N) return false;
+        const int r = z.base + lane;
+        bool dropped = false;
+        if (lane < 8 && r < P.B * P.N) {
+            const int b = small_div(r, P.N), n = r - b * P.N;
+            dropped = __ldg(P.inv_idx + static_cast<size_t>(P.S > 1 ? b : 0) * P.N + n) < 0;
+        }
+        z.mask = __ballot_sync(0xffffffffu, dropped);
+    }
     const int chunks_row = P.H * (P.D / 8);                    // 16-byte chunks per (instance, variate) row
-    const int base = (part + round * parts) * 32;
-    const int r = base + lane;
-    bool dropped = false;
-    if (r < P.B * P.N) {
-        const int b = small_div(r, P.N), n = r - b * P.N;
-        dropped = __ldg(P.inv_idx + static_cast<size_t>(P.S > 1 ? b : 0) * P.N + n) < 0;
-    }
-    unsigned mask = __ballot_sync(0xffffffffu, dropped);
-    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-    uint4* dq4 = reinterpret_cast<uint4*>(P.dq);
-    uint4* dk4 = reinterpret_cast<uint4*>(P.dk);
-    uint4* dv4 = reinterpret_cast<uint4*>(P.dv);
+    const size_t row0 = static_cast<size_t>(z.base + __ffs(z.mask) - 1) * chunks_row;
+    z.mask &= z.mask - 1;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
-    while (mask) {
-        const int l = __ffs(mask) - 1;
-        mask &= mask - 1;
-        const size_t row0 = static_cast<size_t>(base + l) * chunks_row;
-#pragma unroll 1
-        for (int c = lane; c < chunks_row; c += 32) { dq4[row0 + c] = z; dk4[row0 + c] = z; dv4[row0 + c] = z; }
+    for (int c = lane; c < chunks_row; c += 32) {
+        reinterpret_cast<uint4*>(P.dq)[row0 + c] = zero;
+        reinterpret_cast<uint4*>(P.dk)[row0 + c] = zero;
+        reinterpret_cast<uint4*>(P.dv)[row0 + c] = zero;
     }
+    return true;
 }
 
 // This thread's 32 columns (half `half`) of its row of a 64-column accumulator, scaled and rounded, to a bf16 staging tile.
@@ -249,6 +260,48 @@ __device__ __forceinline__ void store_rows(const unsigned char* tile, __nv_bfloa
         if (n[x] >= 0) *reinterpret_cast<uint4*>(out + static_cast<size_t>(n[x]) * P.H * P.D) = *reinterpret_cast<const uint4*>(from + x * 32 * kRowBytes);
 }
 
+// P^T = exp2(S^T scale - lse) of a thread's 32 queries, in place, and as bf16: batches of eight (exponents of g, exponentials of g - 1,
+// rounding of g - 2) keep the special-function unit at its rate.
+__device__ __forceinline__ void exp_step(float (&s)[32], uint32_t (&pk)[16], const uint64_t (&l)[16], uint64_t scale2) {
+#pragma unroll
+    for (int g = 0; g < 6; ++g) {
+        if (g < 4) {
+#pragma unroll
+            for (int e = 8 * g; e < 8 * g + 8; e += 2) halves_of(fma_pair(pair_of(s[e], s[e + 1]), scale2, l[e >> 1]), s[e], s[e + 1]);
+        }
+        if (g >= 1 && g < 5) {
+#pragma unroll
+            for (int e = 8 * g - 8; e < 8 * g; ++e) s[e] = fast_exp2(s[e]);
+        }
+        if (g >= 2) {
+#pragma unroll
+            for (int e = 8 * g - 16; e < 8 * g - 8; e += 2) pk[e >> 1] = pack_bf16(s[e], s[e + 1]);
+        }
+    }
+}
+// dS^T = P^T o (dP^T - Delta) as bf16; Delta of eight queries is in registers, the next eight on their way.
+__device__ __forceinline__ void ds_step(const float (&s)[32], float (&d)[32], uint32_t (&pk)[16], uint64_t (&dl)[2][4], uint32_t dlt) {
+    const uint64_t minus1 = pair_of(-1.f, -1.f);
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        if (g < 3) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dl[(g + 1) & 1][e] = lds_pair(dlt + 32 * g + 32 + 8 * e);
+        }
+#pragma unroll
+        for (int e = 8 * g; e < 8 * g + 8; e += 2) {
+            halves_of(mul_pair(pair_of(s[e], s[e + 1]), fma_pair(dl[g & 1][(e >> 1) & 3], minus1, pair_of(d[e], d[e + 1]))), d[e], d[e + 1]);
+            pk[e >> 1] = pack_bf16(d[e], d[e + 1]);
+        }
+    }
+}
+// Four 16-byte chunks (32 queries) of a row of a 64-query panel.
+__device__ __forceinline__ void store_panel(unsigned char* panel, int row, int half, const uint32_t (&pk)[16]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<uint4*>(panel + row * kRowBytes + (((half * 4 + q) ^ (row & 7)) << 4)) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+}
+
 // ---------------------------------------------------------------------------------------------------------
 // single: a kept set of one tile
 // ---------------------------------------------------------------------------------------------------------
@@ -268,7 +321,7 @@ __device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigne
     const int warp = gt >> 5, row = gt & (kTile - 1), half = gt >> 7, id = team + 1;
     const uint32_t tm = tm0 + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     const uint64_t d_q = umma_desc_sw128(smem_u32(sQ), 16, 1024), m_q = umma_desc_sw128(smem_u32(sQ), kTileBytes, 1024);
-    const uint64_t scale2 = pair_of(P.scale_log2, P.scale_log2), minus1 = pair_of(-1.f, -1.f);
+    const uint64_t scale2 = pair_of(P.scale_log2, P.scale_log2);
     if (half == 0) s_none[row] = -INFINITY;
     uint32_t t = 0;
 #pragma unroll 1
@@ -334,7 +387,7 @@ __device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigne
         group_sync(id);
         ok = mbar_wait(bar, t & 1);
         tc_fence_after();
-        // P^T = exp2(S^T scale - lse) and dS^T = P^T o (dP^T - Delta), 32 queries at a time
+        // P^T and dS^T, 32 queries at a time (a thread's half of the tile is one panel)
         const float* lse = row < n ? s_lse : s_none;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
@@ -342,41 +395,19 @@ __device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigne
             if (q0 >= n) break;
             float s[32], d[32];
             uint32_t pk[16];
+            uint64_t l[16], dl[2][4];
             tmem_ld32(tm + q0, s);
-            tmem_ld32(tm + 128 + q0, d);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) l[e] = lds_pair(smem_u32(lse + q0) + 8 * e);
             tmem_ld_wait();
-#pragma unroll
-            for (int g = 0; g < 6; ++g) {                // batches of eight: exponents of g, exponentials of g - 1, the rest of g - 2
-                if (g < 4) {
-#pragma unroll
-                    for (int i = 8 * g; i < 8 * g + 8; i += 4) {
-                        const float4 l4 = *reinterpret_cast<const float4*>(lse + q0 + i);
-                        halves_of(fma_pair(pair_of(s[i], s[i + 1]), scale2, pair_of(l4.x, l4.y)), s[i], s[i + 1]);
-                        halves_of(fma_pair(pair_of(s[i + 2], s[i + 3]), scale2, pair_of(l4.z, l4.w)), s[i + 2], s[i + 3]);
-                    }
-                }
-                if (g >= 1 && g < 5) {
-#pragma unroll
-                    for (int i = 8 * g - 8; i < 8 * g; ++i) s[i] = fast_exp2(s[i]);
-                }
-                if (g >= 2) {
-#pragma unroll
-                    for (int i = 8 * g - 16; i < 8 * g - 8; i += 4) {
-                        const float4 d4 = *reinterpret_cast<const float4*>(s_delta + q0 + i);
-                        const uint64_t p01 = pair_of(s[i], s[i + 1]), p23 = pair_of(s[i + 2], s[i + 3]);
-                        halves_of(mul_pair(p01, fma_pair(pair_of(d4.x, d4.y), minus1, pair_of(d[i], d[i + 1]))), d[i], d[i + 1]);
-                        halves_of(mul_pair(p23, fma_pair(pair_of(d4.z, d4.w), minus1, pair_of(d[i + 2], d[i + 3]))), d[i + 2], d[i + 3]);
-                        pk[i >> 1] = pack_bf16(s[i], s[i + 1]);
-                        pk[(i >> 1) + 1] = pack_bf16(s[i + 2], s[i + 3]);
-                    }
-                }
-            }
+            exp_step(s, pk, l, scale2);
+            tmem_ld32(tm + 128 + q0, d);
             tmem_st16(tm + half * 64 + c * 16, pk);
-            unsigned char* to = sdS + half * kTileBytes + row * kRowBytes;
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                *reinterpret_cast<uint4*>(to + (((c * 4 + q) ^ (row & 7)) << 4)) =
-                    make_uint4(pack_bf16(d[8 * q], d[8 * q + 1]), pack_bf16(d[8 * q + 2], d[8 * q + 3]), pack_bf16(d[8 * q + 4], d[8 * q + 5]), pack_bf16(d[8 * q + 6], d[8 * q + 7]));
+            for (int e = 0; e < 4; ++e) dl[0][e] = lds_pair(smem_u32(s_delta + q0) + 8 * e);
+            tmem_ld_wait();
+            ds_step(s, d, pk, dl, smem_u32(s_delta + q0));
+            store_panel(sdS + half * kTileBytes, row, c, pk);
         }
         tmem_st_wait();
         fence_proxy_async_smem();
@@ -422,61 +453,58 @@ __device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigne
 // ---------------------------------------------------------------------------------------------------------
 // the kernel
 // ---------------------------------------------------------------------------------------------------------
-// Pipeline: the query loop of a key tile is two phases on 256 threads each, phase A of query tile i + 1 beside phase B of tile i (warp
-// numbers of the few-tile form; in the many-tile form four warps that take dQ out come between the loaders and the phases).
-//   warps 0, 1   issue the products (all lanes run the issue code, an elected lane executes a group of products): S^T and dV, the chain
-//                through P^T, and dP^T, dK and dQ, the chain through dS^T
-//   warps 2, 3   load K, V and a ring of (Q, dO) tiles with their row statistics; warp 3 decodes the items, warp 2 writes the zero rows
-//   warps 4-11   phase A: P^T = exp2(S^T scale - lse), bf16, to tensor memory (the A operand of dV += P^T dO)
-//   warps 12-19  phase B: dS^T = P^T o (dP^T - Delta) to shared memory (dK += dS^T Q, and dQ = dS K through the transposed view); dQ of the
-//                tile before out of tensor memory for the bulk reduce-add; dV and dK of a finished key tile
-// A phase frees what it has copied to registers at once: S^T and dP^T of the next tile are produced under the arithmetic of this one, and
-// dS^T stays in registers until dK and dQ of the tile before have read the shared-memory tile.  (dS^T handed to dK through dP^T's own
-// columns, as an earlier form did, makes phase B wait for dK and the next dP^T: 3900 cycles a tile pair.)
-// What bounds it: shared-memory bandwidth and the hand-offs around it (a tile pair reads and writes some 270 KB of shared memory, 2200
-// cycles, where its products need 1280) with many tiles; the chain of latencies with few.  Measured, B = 32, H = 8, D = 64: 119 kept 19 us
-// (27 before), 200 kept 76 us without prep and convert launches (57 + 11 + 11); all of 862 215 us (229); all of 8192, B = 8, 3590 us (3640);
-// 1423 kept of 8192, B = 8, 174 us.
-// Tensor memory: S^T [0,128) dP^T [128,256) dV [256,320) dK [320,384) dQ [384,448) P^T [448,512).
+// Pipeline: a work item is two neighbouring 128-key tiles of a (head, instance), one to a team of 256 threads, over all its query tiles in
+// steps of 64 queries.  The two key tiles share the operands of a query tile, and dQ of a query tile leaves tensor memory once for both.
+//   warps 0, 1    issue the products of team 0, 1 (all lanes run the issue code, an elected lane executes a group of products)
+//   warps 2, 3    load a two-slot ring of (Q, dO) tiles with their row statistics, and K, V where boxes bring them; warp 3 decodes the items
+//   warps 4-7     dQ of a query tile: issue it once both teams have handed over their dS^T, take it out of tensor memory, add it to the
+//                 accumulator (or write it, with two key tiles or fewer); Delta and the zero rows (few tiles)
+//   warps 8-15    team 0, warps 16-23  team 1: two threads a key row, 32 queries each.  A step: S^T to registers, P^T = exp2(S^T scale - lse)
+//                 to tensor memory (the A operand of dV += P^T dO), dP^T to registers, dS^T = P^T o (dP^T - Delta) to shared memory (dK +=
+//                 dS^T Q, and dQ = dS K through the transposed view); dV and dK of a finished key tile
+// S^T and dP^T of a team share 64 columns: each is produced under the arithmetic on the other, and no product waits for P^T or dS^T to be
+// read but by a whole step.  A warp arrives with one lane (256 arrivals on one barrier serialise).
+// Tensor memory of team w, from 224 w: S^T / dP^T 64 | P^T 32 | dV 64 | dK 64; dQ from 448.
+constexpr uint32_t kTeamCols = 224, kColP = 64, kColDv = 96, kColDk = 160, kColDq = 448;
+constexpr int kTeamWarps = 8;
+
 template <bool kMany>
-__global__ void __launch_bounds__(BwdShape<kMany>::kThreads, 1) attn_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                                                                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
-                                                                   const __grid_constant__ CUtensorMap map_acc, const BwdParams P) {
-    constexpr int kFirst = BwdShape<kMany>::kFirst;
+__global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                                                                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
+                                                                  const __grid_constant__ CUtensorMap map_acc, const BwdParams P) {
     extern __shared__ unsigned char smem_dyn[];
     // Set-up first (shared-memory carve-up, barriers, tensor memory): it touches nothing another kernel produces, so it runs
     // while the previous kernel of the stream is still finishing.
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_dyn);
-    uint64_t* bar_kv_full = bars + 0;
-    uint64_t* bar_kv_free = bars + 1;               // every product of the item is done (both issue warps)
-    uint64_t* bar_q_full = bars + 2;                // [kSlots]
-    uint64_t* bar_q_free = bar_q_full + kSlots;     // [kSlots] every product reading the slot is done (both issue warps)
-    uint64_t* bar_s = bar_q_free + kSlots;          // S^T of a query tile complete
-    uint64_t* bar_sfree = bar_s + 1;                // phase A holds S^T in registers (256)
-    uint64_t* bar_p = bar_s + 2;                    // P^T in tensor memory (256)
-    uint64_t* bar_pfree = bar_s + 3;                // phase B holds P^T in registers (256) and dV has read it (1)
-    uint64_t* bar_dp = bar_s + 4;                   // dP^T of a query tile complete
-    uint64_t* bar_dpfree = bar_s + 5;               // phase B holds dP^T in registers (256)
-    uint64_t* bar_ds = bar_s + 6;                   // dS^T in shared memory (256)
-    uint64_t* bar_dsfree = bar_s + 7;               // many: dK and dQ have read dS^T
-    uint64_t* bar_g = bar_s + 8;                    // dQ of a query tile complete (few: and dK before it, dS^T has been read)
-    uint64_t* bar_dqfree = bar_s + 9;               // dQ has left tensor memory (128 or 256)
-    uint64_t* bar_acc = bar_s + 10;                 // dV, dK of the item final (both issue warps)
-    uint64_t* bar_accfree = bar_s + 11;             // phase B holds them in registers (256)
-    uint64_t* bar_first = bar_s + 13;               // the first item's row copies have landed (512)
-    uint64_t* bar_item = bar_s + 14;                // [8] entry of the item list is written
-    uint64_t* bar_team = bar_item + 8;              // [2][2] single: scores, gradients
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_team + 4);
+    uint64_t* bar_kv_full = bars;                   // [2] K, V of team w
+    uint64_t* bar_kv_free = bars + 2;               // every product of the item is done (both issue warps and the dQ warps)
+    uint64_t* bar_q_full = bars + 3;                // [2] slot holds a query tile
+    uint64_t* bar_q_free = bars + 5;                // [2] every product reading the slot is done (both issue warps)
+    uint64_t* bar_x = bars + 7;                     // [2] S^T, then dP^T of a step complete
+    uint64_t* bar_xfree = bars + 9;                 // [2] S^T is in registers, then dP^T (and P^T in tensor memory)
+    uint64_t* bar_ds = bars + 13;                   // [2] dS^T in shared memory
+    uint64_t* bar_dk = bars + 15;                   // [2] dV and dK of a step done
+    uint64_t* bar_tile = bars + 17;                 // [2] dS^T of the whole query tile in shared memory
+    uint64_t* bar_accfree = bars + 19;              // [2] dV, dK of a key tile in registers
+    uint64_t* bar_delta = bars + 21;                // [2] few: Delta of the slot's rows
+    uint64_t* bar_g = bars + 23;                    // dQ of a query tile complete
+    uint64_t* bar_first = bars + 24;                // the first query tile's row copies have landed (128)
+    uint64_t* bar_item = bars + 25;                 // [8] entry of the item list is written
+    uint64_t* bar_team = bars + 33;                 // [2][2] single: scores, gradients
+    uint64_t* bar_conv = bars + 37;                 // few: whether this item was the last of its dQ' is known
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
     int* s_flag = reinterpret_cast<int*>(tmem_slot + 1);
+    ZeroRows zeros{s_flag + 1, 0, 0u};
     struct alignas(16) Item { int jt, h, b, n_sel; };               // n_sel < 0 ends the list
-    Item* s_item = reinterpret_cast<Item*>(smem_dyn + 384);         // [8]
-    float* s_lse = reinterpret_cast<float*>(smem_dyn + 512);        // [kSlots][128] minus the lse of the query tile in the slot, log2 domain
-    float* s_delta = s_lse + kSlots * kTile;                        // [kSlots][128] its Delta
-    static_assert(2 * kSlots <= 8, "the single teams keep eight arrays of 128 there");
-    unsigned char* sK = align_tiles(reinterpret_cast<unsigned char*>(s_lse + 8 * kTile));
-    unsigned char* sQ = sK + 2 * kTileBytes;            // kSlots slots of (Q tile, dO tile)
-    unsigned char* sdSt = sQ + 2 * kSlots * kTileBytes; // dS^T : rows = keys, columns = queries (two 64-query panels); dV, dK staging at the end of an item
-    unsigned char* sDQ = sdSt + 2 * kTileBytes;         // dQ_i as fp32: panel `half` = head dimensions 32 half .. 32 half + 31, 128-byte swizzled rows
+    Item* s_item = reinterpret_cast<Item*>(smem_dyn + 320);         // [8]
+    float* s_lse = reinterpret_cast<float*>(smem_dyn + 512);        // [2][128] minus the lse of the slot's rows, log2 domain
+    float* s_delta = s_lse + 2 * kTile;                             // [2][128] their Delta
+    float* s_none = s_delta + 2 * kTile;                            // [128] minus the lse for key rows that do not exist: -inf throughout
+    static_assert(512 + 5 * kTile * sizeof(float) <= kBwdHeader, "header too small");
+    unsigned char* sKV = align_tiles(smem_dyn + kBwdHeader);        // K, V of team 0, K, V of team 1
+    unsigned char* sQ = sKV + 4 * kTileBytes;           // two slots of (Q tile, dO tile)
+    unsigned char* sdS = sQ + 4 * kTileBytes;           // dS^T of team 0, 1: rows = keys, two 64-query panels; dV, dK staging at the end of an item
+    unsigned char* sDQ = sdS + 4 * kTileBytes;          // dQ as fp32: two 32-column panels of 128-byte swizzled rows
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (sDQ + 2 * kTileBytes > smem_dyn + kBwdSmemBytes) {
         chain_wait();
@@ -489,26 +517,22 @@ __global__ void __launch_bounds__(BwdShape<kMany>::kThreads, 1) attn_bwd_kernel(
         tmem_relinquish();
     }
     if (tid == 0) {
-        // a box: one announcing arrival; row copies: one of every loader lane, and one of each loader for the row statistics
-        mbar_init(bar_kv_full, boxes ? 1 : 64);
-        mbar_init(bar_kv_free, 2);
-        for (int st = 0; st < kSlots; ++st) {
-            mbar_init(bar_q_full + st, boxes ? 1 : 66);
-            mbar_init(bar_q_free + st, 2);
+        for (int w = 0; w < 2; ++w) {
+            mbar_init(bar_kv_full + w, boxes ? 1 : kBwdGroup);      // a box: one announcing arrival; row copies: every thread of the team
+            mbar_init(bar_q_full + w, boxes ? 1 : 66);              // row copies: every loader lane, and one of each loader for the statistics
+            mbar_init(bar_q_free + w, 2);
+            mbar_init(bar_x + w, 1);
+            mbar_init(bar_xfree + w, kTeamWarps);
+            mbar_init(bar_ds + w, kTeamWarps);
+            mbar_init(bar_dk + w, 1);
+            mbar_init(bar_tile + w, kTeamWarps);
+            mbar_init(bar_accfree + w, kTeamWarps);
+            mbar_init(bar_delta + w, 4);
         }
-        mbar_init(bar_s, 1);
-        mbar_init(bar_sfree, kBwdGroup);
-        mbar_init(bar_p, kBwdGroup);
-        mbar_init(bar_pfree, kBwdGroup + 1);
-        mbar_init(bar_dp, 1);
-        mbar_init(bar_dpfree, kBwdGroup);
-        mbar_init(bar_ds, kBwdGroup);
+        mbar_init(bar_kv_free, 3);
         mbar_init(bar_g, 1);
-        mbar_init(bar_dsfree, 1);
-        mbar_init(bar_dqfree, kMany ? kTile : kBwdGroup);
-        mbar_init(bar_acc, 2);
-        mbar_init(bar_accfree, kBwdGroup);
-        mbar_init(bar_first, 2 * kBwdGroup);
+        mbar_init(bar_conv, 1);
+        mbar_init(bar_first, 128);
         for (int i = 0; i < 8; ++i) mbar_init(bar_item + i, 1);
         for (int i = 0; i < 4; ++i) mbar_init(bar_team + i, 1);
         mbar_fence_init();
@@ -520,20 +544,25 @@ __global__ void __launch_bounds__(BwdShape<kMany>::kThreads, 1) attn_bwd_kernel(
         }
         tma_prefetch_desc(&map_acc);
     }
+    if (tid < kTile) s_none[tid] = -INFINITY;
+    if (tid == 0) *zeros.taken = 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     bool ok = true;
-    int kept = 0, n_t = 0, n_items = 0;
+    int kept = 0, n_t = 0, per_item = 1, n_slots = 0, n_items = 0;
     auto begin = [&]() {
         chain_wait();
         chain_release();
         kept = largest_kept(P.n_sel, P.S, P.N);
         n_t = (kept + kTile - 1) / kTile;                      // tiles of the longest selection
-        n_items = n_t * P.H * P.B;                             // pipeline: (key tile, head, instance); short instances skip tiles
+        // Key tiles of an item: two, except that where every key tile can have a CTA of its own it gets one (1000 of 2000 kept, B = 1, H = 8:
+        // 64 tiles).  Two tiles are always one item, whose dQ is complete in place: the forward pass does not clear the accumulator then.
+        per_item = n_t == 2 || n_t * P.H * P.B > static_cast<int>(gridDim.x) ? 2 : 1;
+        n_slots = (n_t + per_item - 1) / per_item;
+        n_items = n_slots * P.H * P.B;                         // pipeline: (key tiles, head, instance); short instances skip some
     };
-
     auto item_at = [&](uint32_t i) {
         Item it;
         ok &= warp_wait_relaxed(bar_item + (i & 7), (i >> 3) & 1);
@@ -541,100 +570,107 @@ __global__ void __launch_bounds__(BwdShape<kMany>::kThreads, 1) attn_bwd_kernel(
         it.jt = x.x; it.h = x.y; it.b = x.z; it.n_sel = ok ? x.w : -1;
         return it;
     };
+    auto warp_arrive = [&](uint64_t* bar) {                    // all lanes are done
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
+    };
+    // first token of team w's key tile (n_sel: it has none)
+    auto key0_of = [&](const Item& it, int w) { return w < per_item ? (it.jt + w) * kTile : it.n_sel; };
+    // steps of query tile x: the second one only if it holds a query
+    auto steps_of = [&](const Item& it, int x) { return it.n_sel - x * kTile > 64 ? 2 : 1; };
 
-    if (warp < kFirst) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(BwdShape<kMany>::kSmallRegs));
+    if (warp < 8) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kBwdSmallRegs));
     begin();
     // One backward pass per forward pass: the forward kernel left a mark (and cleared this workspace's counters); a backward pass that
     // does not find it (a second backward for the same forward, or two forwards sharing the workspace before their backwards) would
     // add into stale state, so it reports the call instead of returning wrong gradients.
     if (blockIdx.x == 0 && tid == 0 && atomicExch(P.status + kWsPairingWord, 0) != 1) set_status(P.status, VARDROP_ERR_INVALID_ARG);
     if (!kMany && n_t <= 1) {
-        const int parts = 4 * gridDim.x, rounds = zero_row_rounds(P, parts);
+        if (warp < 2)                                    // (four warps at it hold the teams' loads up: 20 us against 18.8 at 119 of 321 kept)
 #pragma unroll 1
-        for (int round = 0; round < rounds; ++round) zero_rows_round(P, blockIdx.x * 4 + warp, parts, round);
+            while (write_zero_row(P, zeros)) {}
     } else if (warp < 2) {
         // ------------------------------------------------------------ issue ---------------------------------------------
-        const uint32_t idesc_kk = umma_idesc_bf16(128, 128, 0, 0);         // K-major x K-major, N = 128
+        const int w = warp;
+        const uint32_t idesc_kk = umma_idesc_bf16(128, 64, 0, 0);          // K-major x K-major, 64 queries
         const uint32_t idesc_kmn = umma_idesc_bf16(128, P.D, 0, 1);        // A K-major, B MN-major
-        const uint32_t idesc_mnmn = umma_idesc_bf16(128, P.D, 1, 1);       // A MN-major, B MN-major
-        const uint64_t d_k = umma_desc_sw128(smem_u32(sK), 16, 1024), m_k = umma_desc_sw128(smem_u32(sK), kTileBytes, 1024);
-        constexpr uint32_t kQOff = 2 * kTileBytes, kDsOff = (2 + 2 * kSlots) * kTileBytes;
-        uint32_t t = 0;                                  // query tiles so far
+        const uint64_t d_k = umma_desc_sw128(smem_u32(sKV), 16, 1024), m_k = umma_desc_sw128(smem_u32(sKV), kTileBytes, 1024);
+        constexpr uint32_t kQOff = 4 * kTileBytes, kDsOff = 8 * kTileBytes;
+        const uint32_t tm = tmem + w * kTeamCols;
+        uint32_t t = 0, u = 0, ai = 0;                   // query tiles, steps of this team, items of this team so far
 #pragma unroll 1
         for (uint32_t i = 0; ok; ++i) {
             const Item it = item_at(i);
             if (it.n_sel < 0) break;
             const int n_q = (it.n_sel + kTile - 1) / kTile;
-            ok &= warp_wait_relaxed(bar_kv_full, i & 1);
+            if (i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
+            if (key0_of(it, w) >= it.n_sel) {            // no key tile for this team: pass the slots on
+#pragma unroll 1
+                for (int x = 0; x < n_q && ok; ++x, ++t) {
+                    ok &= warp_wait_relaxed(bar_q_full + (t & 1), (t >> 1) & 1);
+                    warp_arrive(bar_q_free + (t & 1));
+                }
+                warp_arrive(bar_kv_free);
+                continue;
+            }
+            ok &= warp_wait_relaxed(bar_kv_full + w, ai & 1);
             auto wait_slot = [&](uint32_t tt) {
-                ok &= warp_wait_relaxed(bar_q_full + tt % kSlots, (tt / kSlots) & 1);
+                ok &= warp_wait_relaxed(bar_q_full + (tt & 1), (tt >> 1) & 1);
                 if (!boxes) fence_proxy_async_smem();    // rows written by asynchronous copies are read by the tensor core
                 tc_fence_after();
             };
-            auto scores = [&](uint32_t tt) {             // S^T = K Q^T (warp 0) or dP^T = V dO^T (warp 1) of query tile tt
-                wait_slot(tt);
-                const uint32_t q_off = kQOff + (tt % kSlots) * 2 * kTileBytes;
+            auto scores = [&](uint32_t tt, int hs, uint32_t which) {     // S^T = K Q^T (which 0) or dP^T = V dO^T (1) of 64 queries
                 if (elect_one()) {
-                    const uint64_t a = umma_desc_advance(d_k, warp * kTileBytes), bd = umma_desc_advance(d_k, q_off + warp * kTileBytes);
-                    const uint32_t d = tmem + warp * 128;
-                    tc_mma_bf16(d, a, bd, idesc_kk, 0u);
-                    tc_mma_bf16(d, umma_desc_advance(a, 32), umma_desc_advance(bd, 32), idesc_kk, 1u);
+                    const uint64_t a = umma_desc_advance(d_k, (2 * w + which) * kTileBytes);
+                    const uint64_t bd = umma_desc_advance(d_k, kQOff + (2 * (tt & 1) + which) * kTileBytes + hs * 64 * kRowBytes);
+                    tc_mma_bf16(tm, a, bd, idesc_kk, 0u);
+                    tc_mma_bf16(tm, umma_desc_advance(a, 32), umma_desc_advance(bd, 32), idesc_kk, 1u);
                     if (P.D > 32) {
-                        tc_mma_bf16(d, umma_desc_advance(a, 64), umma_desc_advance(bd, 64), idesc_kk, 1u);
-                        tc_mma_bf16(d, umma_desc_advance(a, 96), umma_desc_advance(bd, 96), idesc_kk, 1u);
+                        tc_mma_bf16(tm, umma_desc_advance(a, 64), umma_desc_advance(bd, 64), idesc_kk, 1u);
+                        tc_mma_bf16(tm, umma_desc_advance(a, 96), umma_desc_advance(bd, 96), idesc_kk, 1u);
                     }
-                    tc_commit(warp == 0 ? bar_s : bar_dp);
+                    tc_commit(bar_x + w);
                 }
                 __syncwarp();
             };
-            scores(t);
+            wait_slot(t);
+            scores(t, 0, 0);
 #pragma unroll 1
             for (int x = 0; x < n_q && ok; ++x, ++t) {
-                const uint32_t slot = t % kSlots, q_off = kQOff + slot * 2 * kTileBytes, acc = x > 0 ? 1u : 0u;
-                if (x + 1 < n_q) {           // the next tile's scores, as soon as this one's are in registers
-                    ok &= warp_wait_relaxed(warp == 0 ? bar_sfree : bar_dpfree, t & 1);
-                    scores(t + 1);
-                }
-                if (warp == 0) {
-                    ok &= warp_wait_relaxed(bar_p, t & 1);
-                    if (x == 0 && i > 0) ok &= warp_wait_relaxed(bar_accfree, (i - 1) & 1);     // dV, dK of the previous item are out
+                const int nh = steps_of(it, x);
+                const uint32_t q_off = kQOff + 2 * (t & 1) * kTileBytes;
+#pragma unroll 1
+                for (int hs = 0; hs < nh && ok; ++hs, ++u) {
+                    const uint32_t acc = x + hs > 0 ? 1u : 0u;
+                    ok &= warp_wait(bar_xfree + w, 0);
                     tc_fence_after();
-                    if (elect_one()) {                   // dV += P^T dO over the 128 queries
-                        const uint64_t bd = umma_desc_advance(m_k, q_off + kTileBytes);
+                    scores(t, hs, 1);
+                    if (hs + 1 == nh && x + 1 < n_q) wait_slot(t + 1);
+                    ok &= warp_wait(bar_xfree + w, 1);
+                    if (acc == 0 && ai > 0) ok &= warp_wait(bar_accfree + w, (ai - 1) & 1);      // dV, dK of the previous item are out
+                    tc_fence_after();
+                    if (elect_one()) {                   // dV += P^T dO
+                        const uint64_t bd = umma_desc_advance(m_k, q_off + kTileBytes + hs * 64 * kRowBytes);
 #pragma unroll
-                        for (int ks = 0; ks < 8; ++ks) tc_mma_bf16_ta(tmem + 256, tmem + 448 + ks * 8, umma_desc_advance(bd, ks * 2048), idesc_kmn, ks > 0 ? 1u : acc);
-                        tc_commit(bar_pfree);
-                        tc_commit(bar_q_free + slot);
+                        for (int ks = 0; ks < 4; ++ks) tc_mma_bf16_ta(tm + kColDv, tm + kColP + ks * 8, umma_desc_advance(bd, ks * 2048), idesc_kmn, ks > 0 ? 1u : acc);
                     }
-                } else {
-                    ok &= warp_wait_relaxed(bar_ds, t & 1);
-                    tc_fence_after();
-                    const uint64_t ad = umma_desc_advance(d_k, kDsOff), bd = umma_desc_advance(m_k, q_off), am = umma_desc_advance(m_k, kDsOff);
-                    auto issue_dk = [&]() {              // dK += dS^T Q (phase B has seen P^T of this tile: dV's wait for bar_accfree precedes)
-#pragma unroll
-                        for (int ks = 0; ks < 8; ++ks)
-                            tc_mma_bf16(tmem + 320, umma_desc_advance(ad, (ks >> 2) * kTileBytes + (ks & 3) * 32), umma_desc_advance(bd, ks * 2048), idesc_kmn, ks > 0 ? 1u : acc);
-                        tc_commit(bar_q_free + slot);
-                    };
-                    if (!kMany && elect_one()) issue_dk();
                     __syncwarp();
-                    if (t > 0) ok &= warp_wait_relaxed(bar_dqfree, (t - 1) & 1);      // the previous dQ has left tensor memory
+                    if (hs + 1 < nh) scores(t, 1, 0);
+                    else if (x + 1 < n_q) scores(t + 1, 0, 0);
+                    ok &= warp_wait(bar_ds + w, u & 1);
                     tc_fence_after();
-                    if (elect_one()) {                   // dQ = dS K over the 128 keys, dS the transposed view of the tile
+                    if (elect_one()) {                   // dK += dS^T Q
+                        const uint64_t ad = umma_desc_advance(d_k, kDsOff + (2 * w + hs) * kTileBytes), bd = umma_desc_advance(m_k, q_off + hs * 64 * kRowBytes);
 #pragma unroll
-                        for (int ks = 0; ks < 8; ++ks)
-                            tc_mma_bf16(tmem + 384, umma_desc_advance(am, ks * 2048), umma_desc_advance(m_k, ks * 2048), idesc_mnmn, ks > 0);
-                        tc_commit(bar_g);
-                        if (kMany) {                     // many: dQ first, it leaves tensor memory under dK
-                            issue_dk();
-                            tc_commit(bar_dsfree);
-                        }
+                        for (int ks = 0; ks < 4; ++ks) tc_mma_bf16(tm + kColDk, umma_desc_advance(ad, ks * 32), umma_desc_advance(bd, ks * 2048), idesc_kmn, ks > 0 ? 1u : acc);
+                        tc_commit(bar_dk + w);
+                        if (hs + 1 == nh) tc_commit(bar_q_free + (t & 1));
                     }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
-            tc_commit_w(bar_acc);
+            ++ai;
             tc_commit_w(bar_kv_free);
         }
     } else if (warp < 4) {
@@ -645,8 +681,8 @@ __global__ void __launch_bounds__(BwdShape<kMany>::kThreads, 1) attn_bwd_kernel(
             Item it{0, 0, 0, -1};
 #pragma unroll 1
             for (; it.n_sel < 0 && k < n_items; k += gridDim.x) {
-                const int hb = small_div(k, n_t);
-                it.jt = k - hb * n_t;
+                const int hb = small_div(k, n_slots);
+                it.jt = (k - hb * n_slots) * per_item;
                 it.b = small_div(hb, P.H);
                 it.h = hb - it.b * P.H;
                 const int n = P.S > 1 ? P.n_sel[it.b] : kept;
@@ -658,98 +694,94 @@ __global__ void __launch_bounds__(BwdShape<kMany>::kThreads, 1) attn_bwd_kernel(
             }
             __syncwarp();
         };
-        uint32_t t = 0;
-        int z_round = 0;
-        const int z_rounds = part == 1 ? zero_row_rounds(P, gridDim.x) : 0;
-        if (kMany)                                       // nothing else to do for this warp
+        if (kMany && part == 1) {                        // boxes are one warp's work: the other writes the zero rows
 #pragma unroll 1
-            for (; z_round < z_rounds; ++z_round) zero_rows_round(P, blockIdx.x, gridDim.x, z_round);
-        const int z_slice = (z_rounds + n_t - 1) / n_t;  // rounds behind every query tile: done within the first item's
+            while (write_zero_row(P, zeros)) {}
+        }
+        uint32_t t = 0;
         if (part == 0) publish(0);
 #pragma unroll 1
-        for (uint32_t i = 0; ok; ++i) {
+        for (uint32_t i = 0; ok && !(boxes && part == 1); ++i) {
             if (part == 0) publish(i + 1);
             const Item it = item_at(i);
             if (it.n_sel < 0) break;
             const int n_q = (it.n_sel + kTile - 1) / kTile;
-            int x = 0;
             // Row statistics of a query tile travel with it: asked for ahead of the wait for the slot, four rows a lane.
             const float* lse_row = P.lse + (static_cast<size_t>(it.b) * P.H + it.h) * P.N;
-            const float* delta_row = P.delta ? P.delta + (static_cast<size_t>(it.b) * P.H + it.h) * P.Ncap : nullptr;
-            const bool has_lse = part == 0, has_delta = delta_row && (boxes || part == 1);
+            const float* delta_row = kMany ? P.delta + (static_cast<size_t>(it.b) * P.H + it.h) * P.Ncap : nullptr;
             float st_lse[4], st_delta[4];
             auto stats_load = [&](int tile) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int r = tile * kTile + e * 32 + lane;
-                    st_lse[e] = has_lse && r < it.n_sel ? __ldg(lse_row + r) : INFINITY;
-                    st_delta[e] = has_delta && r < it.n_sel ? __ldg(delta_row + r) : 0.f;
+                    st_lse[e] = part == 0 && r < it.n_sel ? __ldg(lse_row + r) : INFINITY;
+                    if (kMany) st_delta[e] = r < it.n_sel ? __ldg(delta_row + r) : 0.f;
                 }
             };
             auto stats_store = [&](uint32_t slot) {      // minus the lse in the log2 domain: -inf switches a missing query off
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    if (has_lse) s_lse[slot * kTile + e * 32 + lane] = st_lse[e] * -1.4426950408889634f;
-                    if (has_delta) s_delta[slot * kTile + e * 32 + lane] = st_delta[e];
+                    if (part == 0) s_lse[slot * kTile + e * 32 + lane] = st_lse[e] * -1.4426950408889634f;
+                    if (kMany) s_delta[slot * kTile + e * 32 + lane] = st_delta[e];
                 }
                 __syncwarp();
             };
             if (boxes) {
-                if (part == 0) {
-                    ok = warp_wait_relaxed(bar_kv_free, (i & 1) ^ 1);
+#pragma unroll 1
+                for (int x = 0; x < n_q; ++x, ++t) {
+                    const uint32_t slot = t & 1;
+                    stats_load(x);
+                    ok = warp_wait_relaxed(bar_q_free + slot, ((t >> 1) & 1) ^ 1);
                     if (!ok) break;
+                    stats_store(slot);
                     if (lane == 0) {
-                        mbar_expect_tx(bar_kv_full, 2 * kTileBytes);
-                        tma_load_4d(sK, &map_k, bar_kv_full, 0, it.h, it.jt * kTile, it.b);
-                        tma_load_4d(sK + kTileBytes, &map_v, bar_kv_full, 0, it.h, it.jt * kTile, it.b);
+                        mbar_expect_tx(bar_q_full + slot, 2 * kTileBytes);
+                        tma_load_4d(sQ + slot * 2 * kTileBytes, &map_q, bar_q_full + slot, 0, it.h, x * kTile, it.b);
+                        tma_load_4d(sQ + slot * 2 * kTileBytes + kTileBytes, &map_do, bar_q_full + slot, 0, it.h, x * kTile, it.b);
                     }
                     __syncwarp();
-#pragma unroll 1
-                    for (; x < n_q; ++x, ++t) {
-                        const uint32_t slot = t % kSlots;
-                        stats_load(x);
-                        ok = warp_wait_relaxed(bar_q_free + slot, ((t / kSlots) & 1) ^ 1);
+                    if (x == 0) {                        // the first query tile comes in under the item before; K and V replace that one's
+                        ok = warp_wait_relaxed(bar_kv_free, (i & 1) ^ 1);
                         if (!ok) break;
-                        stats_store(slot);
                         if (lane == 0) {
-                            mbar_expect_tx(bar_q_full + slot, 2 * kTileBytes);
-                            tma_load_4d(sQ + slot * 2 * kTileBytes, &map_q, bar_q_full + slot, 0, it.h, x * kTile, it.b);
-                            tma_load_4d(sQ + slot * 2 * kTileBytes + kTileBytes, &map_do, bar_q_full + slot, 0, it.h, x * kTile, it.b);
+#pragma unroll 1
+                            for (int w = 0; w < 2; ++w) {
+                                const int tok0 = key0_of(it, w);
+                                if (tok0 >= it.n_sel) break;
+                                mbar_expect_tx(bar_kv_full + w, 2 * kTileBytes);
+                                tma_load_4d(sKV + 2 * w * kTileBytes, &map_k, bar_kv_full + w, 0, it.h, tok0, it.b);
+                                tma_load_4d(sKV + (2 * w + 1) * kTileBytes, &map_v, bar_kv_full + w, 0, it.h, tok0, it.b);
+                            }
                         }
                         __syncwarp();
                     }
                 }
             } else {
                 const int32_t* idx = P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N;
-                const long long base = it.b * P.sB + it.h * P.sH;
+                const __nv_bfloat16* q_base = P.q + it.b * P.sB + it.h * P.sH;
                 const __nv_bfloat16* d_o = P.d_o + (static_cast<size_t>(it.b) * P.N * P.H + it.h) * P.D;
-                if (i == 0) {                            // brought in by the other warps: pass it on
+                int x = 0;
+                if (i == 0) {                            // brought in by the dQ warps: pass it on
                     stats_load(0);
                     stats_store(0);
                     if (lane == 0) mbar_arrive(bar_q_full);
                     ok = warp_wait(bar_first, 0);
                     if (!ok) break;
-                    mbar_arrive(bar_kv_full);
                     mbar_arrive(bar_q_full);
                     x = 1;
                     t = 1;
-                } else {
-                    ok = warp_wait_relaxed(bar_kv_free, (i & 1) ^ 1);
-                    if (!ok) break;
-                    copy_tile_rows<true>(sK, P.k + base, P.v + base, P.sN, tile_picks(idx, it.jt * kTile, it.n_sel, part), P.D, part);
-                    cp_async_arrive(bar_kv_full);
                 }
 #pragma unroll 1
                 for (; x < n_q; ++x, ++t) {
-                    const uint32_t slot = t % kSlots;
+                    const uint32_t slot = t & 1;
                     RowPicks picks = tile_picks(idx, x * kTile, it.n_sel, part);
                     stats_load(x);
-                    ok = warp_wait_relaxed(bar_q_free + slot, ((t / kSlots) & 1) ^ 1);
+                    ok = warp_wait_relaxed(bar_q_free + slot, ((t >> 1) & 1) ^ 1);
                     if (!ok) break;
                     stats_store(slot);
                     if (lane == 0) mbar_arrive(bar_q_full + slot);
                     unsigned char* to = sQ + slot * 2 * kTileBytes;
-                    const __nv_bfloat16* from = P.q + base;
+                    const __nv_bfloat16* from = q_base;
                     long long step = P.sN;
 #pragma unroll 1
                     for (int e = 0; e < 2; ++e) {        // Q rows, then dO rows (compact and contiguous)
@@ -764,308 +796,276 @@ __global__ void __launch_bounds__(BwdShape<kMany>::kThreads, 1) attn_bwd_kernel(
                         }
                     }
                     cp_async_arrive(bar_q_full + slot);
-#pragma unroll 1
-                    for (int z = 0; z < z_slice && z_round < z_rounds; ++z, ++z_round) zero_rows_round(P, blockIdx.x, gridDim.x, z_round);
                 }
             }
         }
-#pragma unroll 1
-        for (; z_round < z_rounds; ++z_round) zero_rows_round(P, blockIdx.x, gridDim.x, z_round);
         asm volatile("cp.async.wait_all;" ::: "memory");
-    } else if (kMany) {
-        // ------------------------------------------------------------ dQ out of tensor memory ---------------------------
+    } else {
+        // ------------------------------------------------------------ dQ ------------------------------------------------
         const int row = tid & (kTile - 1);
-        const uint32_t tm = tmem + 384 + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const uint32_t tm = tmem + kColDq + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const bool owner = row == 0;                     // the one thread that owns the bulk reductions
-        uint32_t t = 0;
+        const uint32_t idesc_mnmn = umma_idesc_bf16(128, P.D, 1, 1);       // A MN-major, B MN-major
+        const uint64_t m_k = umma_desc_sw128(smem_u32(sKV), kTileBytes, 1024);
+        bool zeros_left = !kMany;
+        uint32_t t = 0, t1 = 0;                          // query tiles so far, and those with a second key tile
 #pragma unroll 1
         for (uint32_t i = 0; ok; ++i) {
             const Item it = item_at(i);
             if (it.n_sel < 0) break;
             const int n_q = (it.n_sel + kTile - 1) / kTile;
+            const bool two = key0_of(it, 1) < it.n_sel;
+            const bool direct = !kMany && n_q <= per_item;      // dQ is complete here
+            const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
+            const int c8 = row & 7, r8 = row >> 3;
+            const size_t compact = (static_cast<size_t>(it.b) * P.N * P.H + it.h) * P.D;
+            if (!boxes && i == 0) {                      // the first query tile's rows, 32 a warp
+                copy_32_rows(sQ + (warp & 3) * 32 * kRowBytes, P.q + it.b * P.sB + it.h * P.sH, P.sN, sel, (warp & 3) * 32, it.n_sel, P.D);
+                copy_32_rows(sQ + kTileBytes + (warp & 3) * 32 * kRowBytes, P.d_o + compact, static_cast<long long>(P.H) * P.D, nullptr, (warp & 3) * 32, it.n_sel, P.D);
+                cp_async_arrive(bar_first);
+            }
+            // Delta of a query tile: eight threads a row of O (from memory) and dO (from the slot)
+            auto delta_of = [&](int x, uint32_t tt) {
+                const __nv_bfloat16* from = P.o + compact + c8 * 8;
+                const unsigned char* sdO = sQ + (2 * (tt & 1) + 1) * kTileBytes;
+                float* dlt = s_delta + (tt & 1) * kTile;
+                uint4 o[8];                              // asked for together, ahead of the wait for the slot
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int r = x * kTile + r8 + 16 * e;
+                    o[e] = r < it.n_sel && c8 * 8 < P.D ? __ldg(reinterpret_cast<const uint4*>(from + static_cast<size_t>(r) * P.H * P.D)) : make_uint4(0u, 0u, 0u, 0u);
+                }
+                ok &= warp_wait_relaxed(bar_q_full + (tt & 1), (tt >> 1) & 1);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int r = r8 + 16 * e;
+                    const float part = sum8(dot8(o[e], *reinterpret_cast<const uint4*>(sdO + r * kRowBytes + ((c8 ^ (r & 7)) << 4))));
+                    if (c8 == 0) dlt[r] = part;
+                }
+                warp_arrive(bar_delta + (tt & 1));
+            };
+            if (!kMany) delta_of(0, t);
 #pragma unroll 1
             for (int x = 0; x < n_q; ++x, ++t) {
+                if (!kMany && x + 1 < n_q) delta_of(x + 1, t + 1);
+                while (zeros_left && warp != 4 && !__all_sync(0xffffffffu, mbar_test(bar_tile, t & 1))) {       // nothing else to do
+                    zeros_left = write_zero_row(P, zeros);
+                    __nanosleep(100);
+                }
+                ok &= warp_wait_relaxed(bar_tile, t & 1);
+                if (two) ok &= warp_wait_relaxed(bar_tile + 1, t1 & 1);
+                t1 += two ? 1 : 0;
                 if (owner) bulk_wait_group_read0();      // the previous reduction has read the staging tile
-                ok &= warp_wait_relaxed(bar_g, t & 1);
-                ok = drain_sync_and(ok);
+                ok = drain_sync_and(ok);                 // and every thread has read the previous dQ
                 if (!ok) break;
+                if (warp == 4) {
+                    fence_proxy_async_smem();
+                    tc_fence_after();
+                    if (elect_one()) {                   // dQ = dS K over the keys of both tiles, dS the transposed view of dS^T
+#pragma unroll 1
+                        for (int w = 0; w < (two ? 2 : 1); ++w) {
+                            const uint64_t am = umma_desc_advance(m_k, (8 + 2 * w) * kTileBytes), bm = umma_desc_advance(m_k, 2 * w * kTileBytes);
+#pragma unroll
+                            for (int ks = 0; ks < 8; ++ks)
+                                tc_mma_bf16(tmem + kColDq, umma_desc_advance(am, ks * 2048), umma_desc_advance(bm, ks * 2048), idesc_mnmn, w + ks > 0 ? 1u : 0u);
+                        }
+                        tc_commit(bar_g);
+                    }
+                    __syncwarp();
+                }
+                int nout[8];                             // where this thread's rows go: looked up under the product
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int j = x * kTile + r8 + 16 * e;
+                    nout[e] = direct && j < it.n_sel ? (sel ? __ldg(sel + j) : j) : -1;
+                }
+                ok &= warp_wait_relaxed(bar_g, t & 1);
+                if (warp == 4 && x + 1 == n_q && lane == 0) mbar_arrive(bar_kv_free);
                 tc_fence_after();
 #pragma unroll 1
                 for (int c = 0; c < P.D; c += 32) {
                     float v[32];
                     tmem_ld32(tm + c, v);
                     tmem_ld_wait();
-                    if (c + 32 >= P.D) {
-                        tc_fence_before();
-                        mbar_arrive(bar_dqfree);         // dQ is in registers: the next one may be produced
-                    }
-                    unsigned char* to = sDQ + (c >> 5) * kTileBytes + row * kRowBytes;      // fp32, 32-column panels of 128-byte swizzled rows
+                    if (!direct) {                       // fp32, 32-column panels of 128-byte swizzled rows
+                        unsigned char* to = sDQ + (c >> 5) * kTileBytes + row * kRowBytes;
 #pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        *reinterpret_cast<float4*>(to + (e ^ (row & 7)) * 16) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+                        for (int e = 0; e < 8; ++e)
+                            *reinterpret_cast<float4*>(to + (e ^ (row & 7)) * 16) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+                    } else {
+                        unsigned char* to = sDQ + row * kRowBytes;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            *reinterpret_cast<uint4*>(to + (((c >> 3) + e) ^ (row & 7)) * 16) =
+                                make_uint4(pack2(v[8 * e] * P.scale, v[8 * e + 1] * P.scale), pack2(v[8 * e + 2] * P.scale, v[8 * e + 3] * P.scale),
+                                           pack2(v[8 * e + 4] * P.scale, v[8 * e + 5] * P.scale), pack2(v[8 * e + 6] * P.scale, v[8 * e + 7] * P.scale));
+                    }
                 }
+                tc_fence_before();
                 fence_proxy_async_smem();
-                drain_sync_and(true);                    // the staging tile is complete
-                if (owner) {
-                    tma_reduce_add_4d(&map_acc, sDQ, 0, it.h, x * kTile, it.b);
-                    if (P.D > 32) tma_reduce_add_4d(&map_acc, sDQ + kTileBytes, 32, it.h, x * kTile, it.b);
-                    bulk_commit_group();
+                ok = drain_sync_and(ok);                 // the staging tile is complete
+                if (!direct) {
+                    if (owner) {
+                        tma_reduce_add_4d(&map_acc, sDQ, 0, it.h, x * kTile, it.b);
+                        if (P.D > 32) tma_reduce_add_4d(&map_acc, sDQ + kTileBytes, 32, it.h, x * kTile, it.b);
+                        bulk_commit_group();
+                    }
+                } else if (c8 * 8 < P.D) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int r = r8 + 16 * e;
+                        if (nout[e] >= 0)
+                            *reinterpret_cast<uint4*>(P.dq + ((static_cast<size_t>(it.b) * P.N + nout[e]) * P.H + it.h) * P.D + c8 * 8) =
+                                *reinterpret_cast<const uint4*>(sDQ + r * kRowBytes + ((c8 ^ (r & 7)) << 4));
+                    }
                 }
+            }
+            if (!ok) break;
+            if (!kMany && !direct && owner) {            // dQ' of this (instance, head) is complete once all its items are: the teams of the last convert it
+                bulk_wait_group0();                      // this item's reductions have landed
+                __threadfence();
+                *s_flag = atomicAdd(P.tile_done + it.b * P.H + it.h, 1) == (n_q - 1) / per_item;
+                mbar_arrive(bar_conv);
             }
         }
         if (owner) bulk_wait_group0();                   // the last dQ reductions have landed
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
     } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(BwdShape<kMany>::kBigRegs));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kBwdBigRegs));
     begin();
+    const int w = (warp - 8) >> 3, gt = tid & (kBwdGroup - 1);
     if (!kMany && n_t <= 1) {
-        const int team = (warp - 4) >> 3;
-        bwd_single(P, kept, sK, s_lse, bar_team + 2 * team, tmem + team * 256, team, (tid - 128) & (kBwdGroup - 1), ok);
+        bwd_single(P, kept, sKV, reinterpret_cast<float*>(sDQ), bar_team + 2 * w, tmem + w * 256, w, gt, ok);
     } else {
-        // ------------------------------------------------------------ workers -------------------------------------------
-        const int gt = (tid - kFirst * 32) & (kBwdGroup - 1), row = gt & (kTile - 1), half = gt >> 7;
-        const uint32_t tm = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        const int c8 = gt & 7, r8 = gt >> 3;
-        if (!boxes) {                                    // the first item's K, V, Q, dO rows: one 32-row group a warp
-            const Item it = item_at(0);
-            if (it.n_sel >= 0) {
-                const int x = (warp - kFirst) >> 2, g = (warp & 3) * 32;
-                const bool own = x < 3;
-                const __nv_bfloat16* from = own ? (x == 0 ? P.k : x == 1 ? P.v : P.q) + it.b * P.sB + it.h * P.sH : P.d_o + (static_cast<size_t>(it.b) * P.N * P.H + it.h) * P.D;
-                copy_32_rows(sK + x * kTileBytes + g * kRowBytes, from, own ? P.sN : static_cast<long long>(P.H) * P.D,
-                             own ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr, (x < 2 ? it.jt * kTile : 0) + g, it.n_sel, P.D);
-                cp_async_arrive(bar_first);
-            }
-        }
-        uint32_t t = 0;
-        if (warp < kFirst + 8) {
-            // -------------------------------------------------------- phase A: P^T ---------------------------------------
-            const uint64_t scale2 = pair_of(P.scale_log2, P.scale_log2);
+        // ------------------------------------------------------------ teams ---------------------------------------------
+        const int row = gt & (kTile - 1), half = gt >> 7, id = w + 1;
+        const uint32_t tm = tmem + w * kTeamCols + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const int r8 = gt >> 3;
+        unsigned char* panels = sdS + 2 * w * kTileBytes;
+        const uint64_t scale2 = pair_of(P.scale_log2, P.scale_log2);
+        uint32_t t = 0, u = 0, n_conv = 0;               // query tiles, steps of this team, items with an accumulated dQ' so far
 #pragma unroll 1
-            for (uint32_t i = 0; ok; ++i) {
-                const Item it = item_at(i);
-                if (it.n_sel < 0) break;
-                const int n_q = (it.n_sel + kTile - 1) / kTile;
-                const bool key_valid = it.jt * kTile + row < it.n_sel;
+        for (uint32_t i = 0; ok; ++i) {
+            const Item it = item_at(i);
+            if (it.n_sel < 0) break;
+            const int n_q = (it.n_sel + kTile - 1) / kTile, key0 = key0_of(it, w);
+            if (!boxes && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
+            // dQ' of an (instance, head) of more than two tiles: both teams of the CTA that brought its last part
+            auto convert_dq = [&]() {
+                if (kMany || n_q <= per_item) return;
+                ok &= warp_wait_relaxed(bar_conv, n_conv & 1);
+                ++n_conv;
+                const int c8 = gt & 7;
+                if (!*s_flag || c8 * 8 >= P.D) return;
+                __threadfence();
+                const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
+                const float4* acc = reinterpret_cast<const float4*>(P.dq_acc + (static_cast<size_t>(it.b) * P.Ncap * P.H + it.h) * kDP) + c8 * 2;
+                __nv_bfloat16* out = P.dq + (static_cast<size_t>(it.b) * P.N * P.H + it.h) * P.D + c8 * 8;
 #pragma unroll 1
-                for (int x = 0; x < n_q; ++x, ++t) {
-                    const bool have = mbar_test(bar_q_full + t % kSlots, (t / kSlots) & 1);     // the row statistics, with the tile
-                    ok &= warp_wait(bar_s, t & 1);
-                    if (!__all_sync(0xffffffffu, have)) ok &= warp_wait(bar_q_full + t % kSlots, (t / kSlots) & 1);
-                    tc_fence_after();
-                    float s[64];
-                    tmem_ld32(tm + half * 64, s);
-                    tmem_ld32(tm + half * 64 + 32, s + 32);
-                    tmem_ld_wait();
-                    tc_fence_before();
-                    mbar_arrive(bar_sfree);              // S^T is in registers
-                    uint32_t pw[32];
-                    const float* lse2 = s_lse + (t % kSlots) * kTile + half * 64;
-                    const bool p_free = t == 0 || mbar_test(bar_pfree, (t - 1) & 1);
+                for (int j0 = w * 32 + (gt >> 3); j0 < it.n_sel; j0 += 128) {        // two rows a thread in flight
+                    float4 a[2][2];
+                    int n[2];
 #pragma unroll
-                    for (int g = 0; g < 10; ++g) {       // batches of eight: exponents of g, exponentials of g - 1, rounding of g - 2
-                        if (g < 8) {
-#pragma unroll
-                            for (int e = 8 * g; e < 8 * g + 8; e += 4) {
-                                const float4 l4 = *reinterpret_cast<const float4*>(lse2 + e);
-                                halves_of(fma_pair(pair_of(s[e], s[e + 1]), scale2, pair_of(l4.x, l4.y)), s[e], s[e + 1]);
-                                halves_of(fma_pair(pair_of(s[e + 2], s[e + 3]), scale2, pair_of(l4.z, l4.w)), s[e + 2], s[e + 3]);
-                            }
-                        }
-                        if (g >= 1 && g < 9) {
-#pragma unroll
-                            for (int e = 8 * g - 8; e < 8 * g; ++e) s[e] = fast_exp2(s[e]);
-                        }
-                        if (g >= 2) {
-#pragma unroll
-                            for (int e = 8 * g - 16; e < 8 * g - 8; e += 2) pw[e >> 1] = pack_bf16(s[e], s[e + 1]);
-                        }
+                    for (int e = 0; e < 2; ++e) {
+                        const int j = min(j0 + 64 * e, it.n_sel - 1);
+                        n[e] = sel ? __ldg(sel + j) : j;
+                        a[e][0] = __ldcg(acc + static_cast<size_t>(j) * P.H * (kDP / 4));
+                        a[e][1] = __ldcg(acc + static_cast<size_t>(j) * P.H * (kDP / 4) + 1);
                     }
-                    if (!key_valid) {                    // rows past n_sel hold zero keys: they must not count
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) pw[e] = 0u;
-                    }
-                    if (!__all_sync(0xffffffffu, p_free)) ok &= warp_wait(bar_pfree, (t - 1) & 1);      // the previous P^T has been read by phase B and by dV
-                    tc_fence_after();
-                    tmem_st32(tm + 448 + half * 32, pw);
-                    tmem_st_wait();
-                    tc_fence_before();
-                    mbar_arrive(bar_p);                  // dV may go, phase B may read P^T
-                    if (!ok) break;
-                }
-            }
-        } else {
-            // -------------------------------------------------------- phase B: dS^T --------------------------------------
-            const uint64_t minus1 = pair_of(-1.f, -1.f);
-            const bool owner = gt == 0;                  // the one thread that owns the bulk reductions of dQ
-            // dQ of query tile x of the item is in registers: to the fp32 staging tile, which one thread adds to the accumulator.
-            auto reduce_dq = [&](const Item& it, int x, const float (&v)[32]) {
-                if (owner) bulk_wait_group_read0();      // the reduction before, a tile ago, has read the staging tile
-                group_sync(2);
-                unsigned char* to = sDQ + half * kTileBytes + row * kRowBytes;
-                if (half * 32 < P.D) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) *reinterpret_cast<float4*>(to + (e ^ (row & 7)) * 16) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-                }
-                fence_proxy_async_smem();
-                group_sync(2);
-                if (owner) {
-                    tma_reduce_add_4d(&map_acc, sDQ, 0, it.h, x * kTile, it.b);
-                    if (P.D > 32) tma_reduce_add_4d(&map_acc, sDQ + kTileBytes, 32, it.h, x * kTile, it.b);
-                    bulk_commit_group();
+                    for (int e = 0; e < 2; ++e)
+                        if (j0 + 64 * e < it.n_sel)
+                            *reinterpret_cast<uint4*>(out + static_cast<size_t>(n[e]) * P.H * P.D) =
+                                make_uint4(pack2(a[e][0].x * P.scale, a[e][0].y * P.scale), pack2(a[e][0].z * P.scale, a[e][0].w * P.scale),
+                                           pack2(a[e][1].x * P.scale, a[e][1].y * P.scale), pack2(a[e][1].z * P.scale, a[e][1].w * P.scale));
                 }
             };
+            if (key0 >= it.n_sel) { t += n_q; convert_dq(); continue; }
+            const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
+            if (!boxes) {                                // this team's K and V rows, 32 a warp
+                const int x = (warp >> 2) & 1, g = (warp & 3) * 32;
+                copy_32_rows(sKV + (2 * w + x) * kTileBytes + g * kRowBytes, (x == 0 ? P.k : P.v) + it.b * P.sB + it.h * P.sH, P.sN, sel, key0 + g, it.n_sel, P.D);
+                cp_async_arrive(bar_kv_full + w);
+            }
+            const bool key_valid = key0 + row < it.n_sel;
+            bool s_ready = false;                        // a poll takes a hundred cycles to answer: polls go out ahead of where they are needed
 #pragma unroll 1
-            for (uint32_t i = 0; ok; ++i) {
-                const Item it = item_at(i);
-                if (it.n_sel < 0) break;
-                const int n_q = (it.n_sel + kTile - 1) / kTile;
-                const __nv_bfloat16* o_row = P.o + (static_cast<size_t>(it.b) * P.N * P.H + it.h) * P.D + c8 * 8;
+            for (int x = 0; x < n_q && ok; ++x, ++t) {
+                const int nh = steps_of(it, x), slot = t & 1;
 #pragma unroll 1
-                for (int x = 0; x < n_q; ++x, ++t) {
-                    float* dlt = s_delta + (t % kSlots) * kTile;
-                    if (!kMany) {                        // Delta of this query tile: eight threads a row of O (from memory) and dO (from the slot)
-                        uint4 o[4];
+                for (int hs = 0; hs < nh; ++hs, ++u) {
+                    const int q0 = hs * 64 + half * 32;  // this thread's queries of the tile
+                    const uint32_t lse = smem_u32(key_valid ? s_lse + slot * kTile + q0 : s_none), dlt = smem_u32(s_delta + slot * kTile + q0);
+                    if (hs == 0) ok &= warp_wait(bar_q_full + slot, (t >> 1) & 1);       // the row statistics come with the tile
+                    uint64_t l[16];                      // all asked for ahead: a load behind the tensor core's operands takes a hundred cycles
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int r = x * kTile + r8 + 32 * e;
-                            o[e] = r < it.n_sel && c8 * 8 < P.D ? __ldg(reinterpret_cast<const uint4*>(o_row + static_cast<size_t>(r) * P.H * P.D)) : make_uint4(0u, 0u, 0u, 0u);
-                        }
-                        ok &= warp_wait(bar_q_full + t % kSlots, (t / kSlots) & 1);
-                        const unsigned char* sdO = sQ + (t % kSlots) * 2 * kTileBytes + kTileBytes;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int r = r8 + 32 * e;
-                            const float part = sum8(dot8(o[e], *reinterpret_cast<const uint4*>(sdO + r * kRowBytes + ((c8 ^ (r & 7)) << 4))));
-                            if (c8 == 0) dlt[r] = part;
-                        }
-                        group_sync(2);
-                    }
-                    const bool have = mbar_test(bar_q_full + t % kSlots, (t / kSlots) & 1);
-                    ok &= warp_wait(bar_p, t & 1);
-                    if (!__all_sync(0xffffffffu, have)) ok &= warp_wait(bar_q_full + t % kSlots, (t / kSlots) & 1);
+                    for (int e = 0; e < 16; ++e) l[e] = lds_pair(lse + 8 * e);
+                    if (!__all_sync(0xffffffffu, s_ready)) ok &= warp_wait(bar_x + w, 0);
                     tc_fence_after();
-                    uint32_t pw[32];                     // this thread's 64 probabilities, bf16 pairs; then its dS^T
-                    tmem_ld32(tm + 448 + half * 32, reinterpret_cast<float*>(pw));
+                    float s[32], d[32];
+                    tmem_ld32(tm + half * 32, s);
                     tmem_ld_wait();
                     tc_fence_before();
-                    mbar_arrive(bar_pfree);
-                    ok &= warp_wait(bar_dp, t & 1);
+                    warp_arrive(bar_xfree + w);          // S^T is in registers: dP^T may be produced
+                    uint32_t pk[16];
+                    const bool dk_done = u == 0 || mbar_test(bar_dk + w, (u - 1) & 1);
+                    exp_step(s, pk, l, scale2);
+                    const bool dp_ready = mbar_test(bar_x + w, 1);
+                    if (!__all_sync(0xffffffffu, dk_done)) ok &= warp_wait(bar_dk + w, (u - 1) & 1);     // dV of the previous step has read P^T, dK its dS^T
                     tc_fence_after();
-                    uint64_t* bar_read = kMany ? bar_dsfree : bar_g;     // dK and dQ of a tile have read its dS^T
-                    const bool ds_free = t == 0 || mbar_test(bar_read, (t - 1) & 1);
-                    float dp[2][16];
-                    tmem_ld16(tm + 128 + half * 64, dp[0]);
+                    tmem_st16(tm + kColP + half * 16, pk);
+                    if (!__all_sync(0xffffffffu, dp_ready)) ok &= warp_wait(bar_x + w, 1);
+                    tc_fence_after();
+                    tmem_ld32(tm + half * 32, d);
+                    const bool g_done = hs > 0 || x == 0 || mbar_test(bar_g, (t - 1) & 1);
+                    if (!kMany && hs == 0) ok &= warp_wait(bar_delta + slot, (t >> 1) & 1);
+                    uint64_t dl[2][4];                   // Delta of eight queries, the next eight on their way
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {        // 16 queries at a time, the next ones on their way
-                        float4 da[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) da[e] = *reinterpret_cast<const float4*>(dlt + half * 64 + c * 16 + 4 * e);
-                        tmem_ld_wait();
-                        if (c < 3) tmem_ld16(tm + 128 + half * 64 + (c + 1) * 16, dp[(c + 1) & 1]);
-                        else { tc_fence_before(); mbar_arrive(bar_dpfree); }      // dP^T is in registers: the next one may be produced
-                        const float* d = dp[c & 1];
-#pragma unroll
-                        for (int e = 0; e < 16; e += 4) {
-                            const uint32_t w0 = pw[c * 8 + (e >> 1)], w1 = pw[c * 8 + (e >> 1) + 1];
-                            const uint64_t p01 = pair_of(__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xFFFF0000u));
-                            const uint64_t p23 = pair_of(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xFFFF0000u));
-                            float r0, r1, r2, r3;
-                            halves_of(mul_pair(p01, fma_pair(pair_of(da[e >> 2].x, da[e >> 2].y), minus1, pair_of(d[e], d[e + 1]))), r0, r1);
-                            halves_of(mul_pair(p23, fma_pair(pair_of(da[e >> 2].z, da[e >> 2].w), minus1, pair_of(d[e + 2], d[e + 3]))), r2, r3);
-                            pw[c * 8 + (e >> 1)] = pack_bf16(r0, r1);
-                            pw[c * 8 + (e >> 1) + 1] = pack_bf16(r2, r3);
-                        }
-                    }
-                    if (!__all_sync(0xffffffffu, ds_free)) ok &= warp_wait(bar_read, (t - 1) & 1);
-                    float dq[32];                        // few: dQ of the previous tile
-                    if (!kMany && x > 0) {
-                        tc_fence_after();
-                        tmem_ld32(tm + 384 + half * 32, dq);
-                        tmem_ld_wait();
-                        tc_fence_before();
-                        mbar_arrive(bar_dqfree);         // the next dQ may be produced
-                    }
-                    {
-                        unsigned char* to = sdSt + half * kTileBytes + row * kRowBytes;
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) *reinterpret_cast<uint4*>(to + ((q ^ (row & 7)) << 4)) = make_uint4(pw[4 * q], pw[4 * q + 1], pw[4 * q + 2], pw[4 * q + 3]);
-                    }
+                    for (int e = 0; e < 4; ++e) dl[0][e] = lds_pair(dlt + 8 * e);
+                    tmem_st_wait();
+                    tmem_ld_wait();
+                    tc_fence_before();
+                    warp_arrive(bar_xfree + w);          // dP^T is in registers, P^T in tensor memory: dV and the next S^T may go
+                    ds_step(s, d, pk, dl, dlt);
+                    if (!__all_sync(0xffffffffu, g_done)) ok &= warp_wait(bar_g, (t - 1) & 1);   // dQ of the previous tile has read the panels
+                    store_panel(panels + hs * kTileBytes, row, half, pk);
+                    s_ready = mbar_test(bar_x + w, 0);
                     fence_proxy_async_smem();
-                    mbar_arrive(bar_ds);                 // dQ and dK may go
-                    if (!kMany && x > 0) reduce_dq(it, x - 1, dq);
+                    warp_arrive(bar_ds + w);             // dK may go
+                    if (hs + 1 == nh && lane == 0) mbar_arrive(bar_tile + w);    // and dQ
                     if (!ok) break;
                 }
-                ok = group_sync_and(2, ok);
-                if (!ok) break;
-                const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
-                int nout[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int key = it.jt * kTile + r8 + 32 * e;
-                    nout[e] = key < it.n_sel ? (sel ? __ldg(sel + key) : key) : -1;
-                }
-                // dQ of the last tile
-                if (!kMany) {
-                    ok = warp_wait(bar_g, (t - 1) & 1);
-                    tc_fence_after();
-                }
-                if (kMany) {
-                } else if (n_q > 1) {
-                    float dq[32];
-                    tmem_ld32(tm + 384 + half * 32, dq);
-                    tmem_ld_wait();
-                    tc_fence_before();
-                    mbar_arrive(bar_dqfree);
-                    reduce_dq(it, n_q - 1, dq);
-                } else {                                 // nothing to accumulate: rounded and written here (key rows = query rows)
-                    stage_acc(sDQ, tm + 384, P.scale, row, half);
-                    tc_fence_before();
-                    mbar_arrive(bar_dqfree);
-                    group_sync(2);
-                    store_rows(sDQ, P.dq, nout, gt, P, it.b, it.h);
-                }
-                // dV and dK of the key tile, staged over dS^T
-                ok = warp_wait(bar_acc, i & 1);
-                tc_fence_after();
-#pragma unroll 1
-                for (int e = 0; e < 2; ++e) stage_acc(sdSt + e * kTileBytes, tm + 256 + e * 64, e == 0 ? 1.f : P.scale, row, half);
-                tc_fence_before();
-                mbar_arrive(bar_accfree);
-                ok = group_sync_and(2, ok);
-                if (!ok) break;
-#pragma unroll 1
-                for (int e = 0; e < 2; ++e) store_rows(sdSt + e * kTileBytes, e == 0 ? P.dv : P.dk, nout, gt, P, it.b, it.h);
-                group_sync(2);                           // the staging tiles are free
-                if (!kMany && n_q > 1) {         // dQ' of this (instance, head) is complete once all its key tiles are: the last one converts it
-                    if (owner) {
-                        bulk_wait_group0();              // this item's reductions have landed
-                        __threadfence();
-                        *s_flag = atomicAdd(P.tile_done + it.b * P.H + it.h, 1) == n_q - 1;
-                    }
-                    group_sync(2);
-                    if (*s_flag) {
-                        __threadfence();
-                        const int chunks_head = P.D / 8, sh = P.D > 32 ? 3 : 2;       // 16-byte output chunks per row
-#pragma unroll 2
-                        for (int e = gt; e < it.n_sel * chunks_head; e += kBwdGroup) {
-                            const int j = e >> sh, dc = e & (chunks_head - 1);
-                            const float4* acc = reinterpret_cast<const float4*>(P.dq_acc + ((static_cast<size_t>(it.b) * P.Ncap + j) * P.H + it.h) * kDP) + dc * 2;
-                            const float4 a0 = __ldcg(acc), a1 = __ldcg(acc + 1);
-                            const int n = sel ? __ldg(sel + j) : j;
-                            *reinterpret_cast<uint4*>(P.dq + ((static_cast<size_t>(it.b) * P.N + n) * P.H + it.h) * P.D + dc * 8) =
-                                make_uint4(pack2(a0.x * P.scale, a0.y * P.scale), pack2(a0.z * P.scale, a0.w * P.scale),
-                                           pack2(a1.x * P.scale, a1.y * P.scale), pack2(a1.z * P.scale, a1.w * P.scale));
-                        }
-                    }
-                    group_sync(2);                       // the flag is free
-                }
             }
-            if (!kMany && owner) bulk_wait_group0();     // the last dQ reductions have landed
+            ok = group_sync_and(id, ok);
+            if (!ok) break;
+            // dV and dK of the key tile, staged over dS^T
+            int nout[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int key = key0 + r8 + 32 * e;
+                nout[e] = key < it.n_sel ? (sel ? __ldg(sel + key) : key) : -1;
+            }
+            ok = warp_wait(bar_dk + w, (u - 1) & 1);
+            ok &= warp_wait(bar_g, (t - 1) & 1);
+            tc_fence_after();
+#pragma unroll 1
+            for (int e = 0; e < 2; ++e) stage_acc(panels + e * kTileBytes, tm + (e == 0 ? kColDv : kColDk), e == 0 ? 1.f : P.scale, row, half);
+            tc_fence_before();
+            warp_arrive(bar_accfree + w);
+            ok = group_sync_and(id, ok);
+            if (!ok) break;
+#pragma unroll 1
+            for (int e = 0; e < 2; ++e) store_rows(panels + e * kTileBytes, e == 0 ? P.dv : P.dk, nout, gt, P, it.b, it.h);
+            group_sync(id);                              // the staging tiles are free
+            convert_dq();
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     }
     }
+    if (!kMany && (warp >= 8 || n_t > 1))
+#pragma unroll 1
+        while (write_zero_row(P, zeros)) {}              // what is left
     if (!ok) set_status(P.status, VARDROP_ERR_TIMEOUT);
     tc_fence_before();
     __syncthreads();
@@ -1158,14 +1158,14 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
     P.dq = static_cast<__nv_bfloat16*>(dq); P.dk = static_cast<__nv_bfloat16*>(dk); P.dv = static_cast<__nv_bfloat16*>(dv);
     P.sel_idx = sel_idx; P.n_sel = sel_idx ? n_sel : nullptr;
     P.inv_idx = sel_idx ? inv_idx : nullptr;
-    P.tile_done = reinterpret_cast<int32_t*>(base + w.tile_done);
+    P.tile_done = reinterpret_cast<int32_t*>(base + w.delta);
     P.status = reinterpret_cast<int*>(base);
     P.sB = L.sB; P.sN = L.sN; P.sH = L.sH;
     P.B = c.B; P.N = c.N; P.Ncap = w.Ncap; P.H = c.H; P.D = c.D; P.S = attn_sel_rows(c);
     P.scale = scale; P.scale_log2 = scale * 1.4426950408889634f;
     const long long worst = static_cast<long long>(w.Ncap / kTile) * c.H * c.B;
     const int grid = static_cast<int>(worst < sm_count() ? worst : sm_count());          // one CTA per SM (all of tensor memory)
-    auto launch = [&](auto kernel, int threads, int& attr_dev) {
+    auto launch = [&](auto kernel, int& attr_dev) {
         int dev = 0;
         cudaGetDevice(&dev);
         if (attr_dev != dev) {
@@ -1173,10 +1173,10 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
             attr_dev = dev;
         }
         LaunchScope ls_(K_ATTN_BWD, stream);
-        return check_cuda(launch_chained(kernel, dim3(grid), dim3(threads), kBwdSmemBytes, stream, mq, mk, mv, mdo, macc, P), "attention: backward launch");
+        return check_cuda(launch_chained(kernel, dim3(grid), dim3(kBwdThreads), kBwdSmemBytes, stream, mq, mk, mv, mdo, macc, P), "attention: backward launch");
     };
     static thread_local int attr_few = -1, attr_many = -1;
-    if (int st = many ? launch(attn_bwd_kernel<true>, BwdShape<true>::kThreads, attr_many) : launch(attn_bwd_kernel<false>, BwdShape<false>::kThreads, attr_few)) return st;
+    if (int st = many ? launch(attn_bwd_kernel<true>, attr_many) : launch(attn_bwd_kernel<false>, attr_few)) return st;
     if (many) {
         ConvertParams F{};
         F.dq_acc = reinterpret_cast<const float4*>(base + w.dq_acc);

@@ -15,9 +15,8 @@ constexpr int kTileBytes = kTile * kRowBytes;   // 16 KiB
 
 struct AttnWs {
     size_t staged[4];         // [B, Ncap, H, D] bf16 copies of the kept rows of Q, K, V and of dO (selections of many tiles)
-    size_t delta;             // [B, H, Ncap] fp32
+    size_t delta;             // [B, H, Ncap] fp32; few tiles: [B, H] int32 counters instead
     size_t dq_acc;            // [B, Ncap, H, 64] fp32
-    size_t tile_done;         // [B, H] int32: key tiles of (b, h) whose backward work is complete
     size_t total;
     int Ncap;
 };
@@ -29,7 +28,7 @@ inline AttnWs attn_layout(const vardrop_attn_cfg& c) {
     for (size_t& s : w.staged) { s = o; o += align_up(static_cast<size_t>(c.B) * w.Ncap * c.H * kRowBytes, 1024); }
     w.delta = o; o += align_up(sizeof(float) * c.B * c.H * w.Ncap, 1024);
     w.dq_acc = o; o += align_up(static_cast<size_t>(c.B) * w.Ncap * c.H * kDP * sizeof(float), 1024);
-    w.tile_done = o; o += align_up(sizeof(int32_t) * c.B * c.H, 1024);
+    o += align_up(sizeof(int32_t) * c.B * c.H, 1024);         // reserved
     w.total = o;
     return w;
 }

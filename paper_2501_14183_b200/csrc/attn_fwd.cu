@@ -131,7 +131,7 @@ struct FwdParams {
     const int32_t* n_sel;   // [S] kept counts; NULL: all N tokens
     int* status;
     float4* dq_acc;         // [B, Ncap, H, 64] fp32: zeroed here where the backward pass will accumulate into it (NULL: the backward pass does)
-    int32_t* tile_done;     // [B, H] completion counters of the backward pass, zeroed here
+    int32_t* tile_done;     // few tiles: [B, H] completion counters of the backward pass, zeroed here
     long long sB, sN, sH;   // element strides of q, k, v
     int B, N, Ncap, H, D, S;
     float scale_log2;       // sm_scale * log2(e)
@@ -624,7 +624,6 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
             if (w >= it.n_act) continue;
             if (half == 0) {
                 const int qt = it.split ? it.qt : it.qt + w, h = it.split ? it.h + w : it.h;
-                if (qt == 0 && r == 0) P.tile_done[it.b * P.H + h] = 0;
                 if (P.dq_acc) {     // the backward pass adds per-key-tile pieces of dQ' into the accumulator: clear this tile's rows
                     float4* rows = P.dq_acc + ((static_cast<size_t>(it.b) * P.Ncap + qt * kTile + (r >> 4)) * P.H + h) * (kDP / 4) + (r & 15);
 #pragma unroll 1
@@ -800,7 +799,7 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
         const int32_t* idx = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? b : 0) * P.N : nullptr;
         const long long base = b * P.sB + h * P.sH;
         if (qt == 0 && tid == 0) P.tile_done[b * P.H + h] = 0;
-        if (n_kv > 1 && P.dq_acc) {             // the backward pass will add per-key-tile pieces of dQ' into the accumulator: clear this tile's rows
+        if ((n_kv > 2 || (n_kv == 2 && P.S > 1)) && P.dq_acc) {             // the backward pass adds per-key-tile pieces of dQ' into the accumulator (it completes dQ of two tiles in place, if no instance has more): clear this tile's rows
             float4* rows = P.dq_acc + ((static_cast<size_t>(b) * P.Ncap + qt * kTile + (tid >> 4)) * P.H + h) * (kDP / 4) + (tid & 15);
 #pragma unroll 1
             for (int x = 0; x < kDP / 4; ++x, rows += static_cast<size_t>(kTileFwdThreads / 16) * P.H * (kDP / 4))
@@ -1012,7 +1011,7 @@ int attn_fwd_launch(const void* q, const void* k, const void* v, const int32_t* 
     P.o = static_cast<__nv_bfloat16*>(o); P.lse = lse; P.sel_idx = sel_idx; P.n_sel = sel_idx ? n_sel : nullptr;
     P.status = reinterpret_cast<int*>(base);
     P.dq_acc = attn_fwd_clears(c, sel_idx) ? reinterpret_cast<float4*>(base + w.dq_acc) : nullptr;
-    P.tile_done = reinterpret_cast<int32_t*>(base + w.tile_done);
+    P.tile_done = reinterpret_cast<int32_t*>(base + w.delta);
     P.sB = L.sB; P.sN = L.sN; P.sH = L.sH;
     P.B = c.B; P.N = c.N; P.Ncap = w.Ncap; P.H = c.H; P.D = c.D; P.S = attn_sel_rows(c);
     const float scale = c.sm_scale > 0.f ? c.sm_scale : 1.f / sqrtf(static_cast<float>(c.D));
