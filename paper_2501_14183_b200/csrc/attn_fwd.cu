@@ -989,10 +989,8 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
 
 }  // namespace
 
-// Which kernel: the kept count is only known on the device, so the host goes by the largest it can be.  A selection keeps a fraction of
-// the variates (a tenth to a third in the paper's settings): up to 2048 variates that is a handful of tiles per head and instance.
-// Without one, up to three tiles: all of 384 variates take 10.4 us against 12.4 at B = 4 (27.9 and 27.2 at B = 32); at four it turns.
-static bool attn_fwd_few_tiles(const vardrop_attn_cfg& c, const int32_t* sel_idx) { return sel_idx ? c.N <= kManyTilesN : c.N <= 3 * kTile; }
+// Which kernel: with a selection as the backward pass (see attn_many_tiles).  Without one, up to three tiles: all of 384 variates take 10.4 us against 12.4 at B = 4 (27.9 and 27.2 at B = 32); at four it turns.
+static bool attn_fwd_few_tiles(const vardrop_attn_cfg& c, const int32_t* sel_idx) { return sel_idx ? !attn_many_tiles(c, sel_idx) : c.N <= 3 * kTile; }
 
 int attn_fwd_launch(const void* q, const void* k, const void* v, const int32_t* sel_idx, const int32_t* n_sel,
                     const vardrop_attn_cfg& c, void* o, float* lse, void* ws, cudaStream_t stream) {
