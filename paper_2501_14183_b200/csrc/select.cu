@@ -308,10 +308,15 @@ __global__ void __launch_bounds__(kTailThreads) select_sample_kernel(const Selec
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// Small problems (N <= 2048): one CTA per hash row does everything in shared memory with two bitonic sorts.
+// Small problems (N <= 2048): one CTA per hash row does everything in shared memory.
+//
+// More than 512, in few groups (the point of the method): the distinct keys are found with a hash table and ranked by counting, which gives the group ids; a
+// variate's place in its group is the number of equal keys in the 32-variate chunks before its own plus those below it in the chunk; its
+// sampling rank is counted over its group.  No sort.
+// Fewer, many groups, or a long one: two bitonic sorts.
 //   sort 1: (key, variate)                      -> members, group heads -> ids, offsets
 //   sort 2: (group id, Philox priority, rank j) -> position inside the group = sampling rank
-// then the kept flags are compacted with one scan.  No scratch in global memory, no atomics.
+// Then the kept flags are compacted with one scan.  No scratch in global memory, no global atomics.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kSmallMaxN = 2048;
 
@@ -381,26 +386,240 @@ __device__ __forceinline__ int block_scan_pair(int v0, int v1, int* warp_sums, i
     return v + base - v0 - v1;
 }
 
+// Most groups the counting path takes: ranking G keys is G^2 / 32 cycles, about half of what the sort of M items takes at this line.
+__host__ __device__ constexpr int small_max_groups(int M) { return M <= 64 ? 64 : M == 128 ? 128 : M == 256 ? 182 : M == 512 ? 256 : M == 1024 ? 362 : 512; }
+// Longest group whose sampling ranks are counted: 128 positions take some 4000 cycles, the second sort of 1024 items 8000 (of 512 items 4500).
+constexpr int kCountMaxGroup = 128, kSortCountMaxGroup = 64;
+
+// Shared memory of the counting path (the sorting path uses less, over it).
+struct SmallLayout {
+    int table, list, prio, size, off, count, slot_id, rank, quota, slot, place, member, entry, total;       // byte offsets
+};
+__host__ __device__ inline SmallLayout small_layout(int M) {
+    SmallLayout l{};
+    const int G = (small_max_groups(M) + 1) & ~1;
+    int o = 0;
+    l.table = o; o += 2 * M * 8;                   // [2M] keys
+    l.list = o; o += G * 8;                        // [G] distinct keys, in any order: the entries
+    l.prio = o; o += M * 4;                        // [M] priority by sorted position
+    l.size = o; o += G * 4;                        // [G] members of an entry
+    l.off = o; o += G * 4;                         // [G] sorted position of its first member
+    l.count = o; o += M / 32 * G * 2;              // [M / 32][G] members of an entry in a chunk; then in the chunks before it
+    l.slot_id = o; o += (2 * M + 2) * 2;           // [2M + 1] slot -> entry
+    l.rank = o; o += G * 2;                        // [G] group id of an entry
+    l.quota = o; o += G * 2;                       // [G] members of an entry to keep
+    l.slot = o; o += M * 2;                        // [M] by variate: its slot, then its entry
+    l.place = o; o += M;                           // [M] by variate: its place among the equal keys of its chunk
+    l.member = o; o += M * 2;                      // [M] by sorted position: variate
+    l.entry = o; o += M * 2;                       // [M] by sorted position: entry
+    l.total = (o + 15) & ~15;
+    return l;
+}
+
 // launched with M / 2 threads (M >= 64 a power of two, N <= M)
+//
+// What bounds it is latency: half a dozen short steps between barriers, each run once, at the speed of instruction fetch.  So the steps are
+// few (sizes and offsets come out of the ranking of the distinct keys, without scans) and their loops rolled, with what a variate
+// carries from step to step in shared memory.
+// Measured (events around the launch), counting | sorting: 862 variates in 52 groups of up to 72 12.8 | 15.5 us, in 146 groups 14.8 | 16.9;
+// 32 rows of 321 11.6 | 10.7, 21 8.6 | 8.7: up to 512 items it sorts.
+constexpr int kSortOnlyItems = 512;
+template <bool kCounting>
 __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const SelectParams P, int M) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    uint64_t* a = reinterpret_cast<uint64_t*>(sm_raw);            // [M] sorted keys, later sorted (group, priority, rank) codes
-    uint32_t* idx = reinterpret_cast<uint32_t*>(a + M);           // [M] variate by sorted position
-    int* gpos = reinterpret_cast<int*>(idx + M);                  // [M] group id by sorted position
-    int* off_s = gpos + M;                                        // [M + 1] group offsets
-    int* keep_s = off_s + M + 1;                                  // [M] kept flag by variate
     __shared__ int warp_sums[kSmallMaxN / 64];
+    __shared__ uint32_t keep_bits[kSmallMaxN / 32];
+    __shared__ int n_entries, all_ones;
+    const int s = blockIdx.x, N = P.N, tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
+    const SmallLayout L = small_layout(M);
+    const int G_max = small_max_groups(M), G_row = (G_max + 1) & ~1;
+    constexpr uint64_t kEmpty = ~0ull;             // marks a free slot; as a key it has a slot of its own behind the table's
+    uint64_t* table = reinterpret_cast<uint64_t*>(sm_raw + L.table);
+    uint64_t* list = reinterpret_cast<uint64_t*>(sm_raw + L.list);
+    uint32_t* prio = reinterpret_cast<uint32_t*>(sm_raw + L.prio);
+    int* size_s = reinterpret_cast<int*>(sm_raw + L.size);
+    int* first_s = reinterpret_cast<int*>(sm_raw + L.off);
+    uint32_t* count2 = reinterpret_cast<uint32_t*>(sm_raw + L.count);              // two entries a word
+    uint16_t* count = reinterpret_cast<uint16_t*>(sm_raw + L.count);
+    uint16_t* slot_id = reinterpret_cast<uint16_t*>(sm_raw + L.slot_id);
+    uint16_t* rank = reinterpret_cast<uint16_t*>(sm_raw + L.rank);
+    uint16_t* quota_s = reinterpret_cast<uint16_t*>(sm_raw + L.quota);
+    uint16_t* slot_s = reinterpret_cast<uint16_t*>(sm_raw + L.slot);
+    unsigned char* place_s = sm_raw + L.place;
+    uint16_t* member_s = reinterpret_cast<uint16_t*>(sm_raw + L.member);
+    uint16_t* entry_s = reinterpret_cast<uint16_t*>(sm_raw + L.entry);
+    if (kCounting) {
+        for (int i = tid; i < M; i += T) reinterpret_cast<uint4*>(table)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+#pragma unroll 1
+        for (int i = tid; i < M / 32 * (G_row / 2); i += T) count2[i] = 0u;
+#pragma unroll 1
+        for (int i = tid; i < G_row; i += T) size_s[i] = 0;
+        if (tid < M / 32) keep_bits[tid] = 0u;
+        if (tid == 0) { n_entries = 0; all_ones = 0; }
+        __syncthreads();
+    }
     chain_wait();
     chain_release();
-    const int s = blockIdx.x, N = P.N, tid = threadIdx.x;
     const uint64_t* keys = P.keys + static_cast<size_t>(s) * N;
     int32_t* members = P.members + static_cast<size_t>(s) * N;
     int32_t* gid = P.group_id + static_cast<size_t>(s) * N;
     int32_t* off = P.group_offsets + static_cast<size_t>(s) * (N + 1);
     int32_t* sel = P.sel_idx + static_cast<size_t>(s) * N;
     int32_t* inv = P.inv_idx + static_cast<size_t>(s) * N;
-    const int p0 = 2 * tid, p1 = 2 * tid + 1;                     // the two items / positions this thread owns
 
+    if (kCounting) {
+        // ---- the distinct keys: whoever takes a slot opens an entry --------------------------------------------
+#pragma unroll 1
+        for (int n = tid; n < N; n += T) {
+            const uint64_t key = keys[n];
+            int at = 2 * M;
+            bool mine;
+            if (key == kEmpty) {
+                mine = atomicExch(&all_ones, 1) == 0;
+            } else {
+                at = static_cast<int>((key * 0x9E3779B97F4A7C15ull) >> (64 - (31 - __clz(2 * M))));
+#pragma unroll 1
+                for (;;) {                             // at most half of the slots are ever taken
+                    uint64_t cur = *reinterpret_cast<volatile uint64_t*>(table + at);
+                    mine = false;
+                    if (cur == kEmpty) {
+                        cur = atomicCAS(reinterpret_cast<unsigned long long*>(table + at), kEmpty, key);
+                        mine = cur == kEmpty;
+                    }
+                    if (mine || cur == key) break;
+                    at = (at + 1) & (2 * M - 1);
+                }
+            }
+            if (mine) {
+                const int d = atomicAdd(&n_entries, 1);
+                if (d < G_max) { list[d] = key; slot_id[at] = static_cast<uint16_t>(d); }
+            }
+            slot_s[n] = static_cast<uint16_t>(at);
+        }
+        __syncthreads();
+        const int G = n_entries;
+        bool counting = G <= G_max;
+        if (counting) {
+            // equal keys within a chunk of 32 consecutive variates
+#pragma unroll 1
+            for (int n = tid; n - lane < N; n += T) {
+                const int d = n < N ? slot_id[slot_s[n]] : 0x10000 + lane;
+                const unsigned same = __match_any_sync(0xffffffffu, d);
+                if (n < N) {
+                    const int place = __popc(same & ((1u << lane) - 1u));
+                    slot_s[n] = static_cast<uint16_t>(d);
+                    place_s[n] = static_cast<unsigned char>(place);
+                    if (place == 0) {
+                        count[(n >> 5) * G_row + d] = static_cast<uint16_t>(__popc(same));
+                        atomicAdd(size_s + d, __popc(same));
+                    }
+                }
+            }
+            __syncthreads();
+            // entries 2 i and 2 i + 1: members in the chunks before each chunk
+            if (2 * tid < G) {
+                uint32_t run = 0;
+#pragma unroll 1
+                for (int c = 0; c < (N + 31) / 32; c += 4) {
+                    uint32_t v[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v[i] = c + i < M / 32 ? count2[(c + i) * (G_row / 2) + tid] : 0u;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (c + i < M / 32) count2[(c + i) * (G_row / 2) + tid] = run;
+                        run += v[i];
+                    }
+                }
+            }
+            // group id and first position of an entry: entries with smaller keys and their members, counted by `parts` lanes to an entry
+            int parts_log = 0;
+            while (parts_log < 5 && (G << (parts_log + 1)) <= T) ++parts_log;
+            int longest = 0;
+#pragma unroll 1
+            for (int base = 0; base < (G << parts_log); base += T) {
+                const int d = (base + tid) >> parts_log;
+                uint32_t below = 0, before = 0;
+                if (d < G) {
+                    const uint64_t mine = list[d];
+                    longest = max(longest, size_s[d]);
+#pragma unroll 4
+                    for (int e = tid & ((1 << parts_log) - 1); e < G; e += 1 << parts_log) {
+                        const uint32_t less = list[e] < mine ? 1u : 0u;
+                        below += less;
+                        before += less * static_cast<uint32_t>(size_s[e]);
+                    }
+                }
+                uint32_t both = below << 16 | before;          // below < 2^9, before <= 2^11
+#pragma unroll 1
+                for (int m = 1; m < 1 << parts_log; m <<= 1) both += __shfl_xor_sync(0xffffffffu, both, m);
+                if (d < G && (tid & ((1 << parts_log) - 1)) == 0) {
+                    rank[d] = static_cast<uint16_t>(both >> 16);
+                    first_s[d] = static_cast<int>(both & 0xFFFFu);
+                    quota_s[d] = static_cast<uint16_t>(quota_of(size_s[d], P.gs, P.rate_ppm));
+                }
+            }
+            counting = !__syncthreads_or(longest > kCountMaxGroup);
+        }
+        if (counting) {
+            // sorted positions
+#pragma unroll 1
+            for (int n = tid; n < N; n += T) {
+                const int d = slot_s[n], g = rank[d], first = first_s[d];
+                const int j = count[(n >> 5) * G_row + d] + place_s[n];
+                prio[first + j] = philox4x32_10_word0(static_cast<uint32_t>(j), static_cast<uint32_t>(g), static_cast<uint32_t>(s), P.step, P.seed_lo, P.seed_hi);
+                member_s[first + j] = static_cast<uint16_t>(n);
+                entry_s[first + j] = static_cast<uint16_t>(d);
+                gid[n] = g;
+            }
+            for (int d = tid; d < G; d += T) off[rank[d]] = first_s[d];
+            for (int i = G + tid; i <= N; i += T) off[i] = N;
+            if (tid == 0) P.n_groups[s] = G;
+            __syncthreads();
+            // sampling ranks, by sorted position: neighbours read the same priorities
+#pragma unroll 1
+            for (int p = tid; p < N; p += T) {
+                const int d = entry_s[p], begin = first_s[d], size = size_s[d], n = member_s[p];
+                members[p] = n;
+                const int quota = quota_s[d];
+                int below = 0;
+                if (quota < size) {
+                    const uint32_t mine = prio[p];
+#pragma unroll 8
+                    for (int o = begin; o < begin + size; ++o) {
+                        const uint32_t other = prio[o];
+                        below += (other < mine) | ((other == mine) & (o < p));
+                    }
+                }
+                if (below < quota) atomicOr(keep_bits + (n >> 5), 1u << (n & 31));
+            }
+            __syncthreads();
+            const uint32_t w0 = lane < M / 32 ? keep_bits[lane] : 0u, w1 = lane + 32 < M / 32 ? keep_bits[lane + 32] : 0u;
+            const int v0 = __popc(w0), v1 = __popc(w1);
+            const int total = __reduce_add_sync(0xffffffffu, v0 + v1);
+#pragma unroll 1
+            for (int n = tid; n - lane < N; n += T) {
+                const int c = n >> 5;
+                const int base = __reduce_add_sync(0xffffffffu, (lane < c ? v0 : 0) + (lane + 32 < c ? v1 : 0));
+                const uint32_t word = keep_bits[c];
+                const bool keep = (word >> lane) & 1u;
+                const int pos = base + __popc(word & ((1u << lane) - 1u));
+                if (keep) sel[pos] = n;
+                if (n < N) inv[n] = keep ? pos : -1;
+            }
+            for (int i = total + tid; i < N; i += T) sel[i] = -1;
+            if (tid == 0) P.n_sel[s] = total;
+            return;
+        }
+        __syncthreads();
+    }
+
+    // ---- the sorting path --------------------------------------------------------------------------------
+    uint64_t* a = reinterpret_cast<uint64_t*>(sm_raw);            // [M] sorted keys, later sorted (group, priority, rank) codes
+    uint32_t* idx = reinterpret_cast<uint32_t*>(a + M);           // [M] variate by sorted position
+    int* gpos = reinterpret_cast<int*>(idx + M);                  // [M] group id by sorted position
+    int* off_s = gpos + M;                                        // [M + 1] group offsets
+    int* keep_s = off_s + M + 1;                                  // [M] kept flag by variate
+    const int p0 = 2 * tid, p1 = 2 * tid + 1;                     // the two items / positions this thread owns
     uint64_t k0 = p0 < N ? keys[p0] : ~0ull, k1 = p1 < N ? keys[p1] : ~0ull;
     uint32_t n0 = p0, n1 = p1;
     // Keys of up to 53 bits (k <= 4 frequencies of 12 bits, say) leave room for the variate index below them: one 64-bit
@@ -425,8 +644,8 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
     // group heads -> dense ids and offsets
     const int h0 = (p0 < N) && (p0 == 0 || k0 != a[p0 - 1]);
     const int h1 = (p1 < N) && (k1 != k0);
-    int G = 0;
-    const int before = block_scan_pair(h0, h1, warp_sums, &G);
+    int groups = 0;
+    const int before = block_scan_pair(h0, h1, warp_sums, &groups);
     const int g0 = before + h0 - 1, g1 = before + h0 + h1 - 1;
     if (p0 < N) {
         gpos[p0] = g0;
@@ -440,8 +659,8 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
         members[p1] = n1;
         gid[n1] = g1;
     }
-    if (tid == 0) { off_s[G] = N; P.n_groups[s] = G; }
-    for (int i = G + tid; i <= N; i += blockDim.x) off[i] = N;
+    if (tid == 0) { off_s[groups] = N; P.n_groups[s] = groups; }
+    for (int i = groups + tid; i <= N; i += blockDim.x) off[i] = N;
     __syncthreads();
 
     // sampling rank: sort (group, priority, j)
@@ -458,12 +677,11 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
     }
     uint32_t d0 = 0, d1 = 0;
     __syncthreads();                                              // everyone is done reading the sorted keys in `a`
-    // Groups are usually small: a member's sampling rank is then the number of codes of its group below its own, counted over
-    // the group's few positions.  Only when some group is long does the second sort pay.
-    constexpr int kCountMaxGroup = 64;
+    // Where groups are small a member's sampling rank is the number of codes of its group below its own, counted over the group's
+    // few positions.  Only when some group is long does the second sort pay.
     const int size0 = p0 < N ? off_s[g0 + 1] - off_s[g0] : 0, size1 = p1 < N ? off_s[g1 + 1] - off_s[g1] : 0;
     a[p0] = c0; a[p1] = c1;
-    if (!__syncthreads_or(size0 > kCountMaxGroup || size1 > kCountMaxGroup)) {
+    if (!__syncthreads_or(size0 > kSortCountMaxGroup || size1 > kSortCountMaxGroup)) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int p = 2 * tid + e;
@@ -552,16 +770,18 @@ int select_launch(const uint64_t* keys, const vardrop_select_cfg& c, int32_t* gr
     if (c.N <= kSmallMaxN) {
         int M = 64;
         while (M < c.N) M <<= 1;
-        const size_t smem = static_cast<size_t>(M) * (8 + 4 + 4 + 4 + 4) + 16;
+        const size_t sorting = static_cast<size_t>(M) * (8 + 4 + 4 + 4 + 4) + 16, counting = small_layout(M).total;
+        const bool count = M > kSortOnlyItems;
+        const size_t smem = count && counting > sorting ? counting : sorting;
         static thread_local int attr_dev = -1;
         int dev = 0;
         cudaGetDevice(&dev);
         if (attr_dev != dev) {
-            if (int st = check_cuda(cudaFuncSetAttribute(select_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024), "select: smem attribute")) return st;
+            if (int st = check_cuda(cudaFuncSetAttribute(select_small_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024), "select: smem attribute")) return st;
             attr_dev = dev;
         }
         cudaError_t err;
-        { LaunchScope ls_(K_SELECT_SMALL, stream); err = launch_chained(select_small_kernel, dim3(c.S), dim3(M / 2), smem, stream, P, M); }
+        { LaunchScope ls_(K_SELECT_SMALL, stream); err = launch_chained(count ? select_small_kernel<true> : select_small_kernel<false>, dim3(c.S), dim3(M / 2), smem, stream, P, M); }
         return check_cuda(err, "select: launch");
     }
     if (int st = check_cuda(cudaMemsetAsync(base + w.zero_begin, 0, w.zero_bytes, stream), "select: clear counters")) return st;

@@ -60,6 +60,18 @@ def test_select_group_sizes_around_the_counting_limit():
             check(keys, gs, rate, seed=99, step=4)
 
 
+@pytest.mark.parametrize("N,G", [(64, 64), (65, 63), (255, 182), (256, 183), (512, 256), (513, 257), (1024, 362), (1000, 363), (2048, 512), (1500, 513), (2048, 16), (1100, 9)])
+def test_select_group_counts_around_the_counting_limit(N, G):
+    """Both sides of the largest number of groups whose keys are ranked by counting, and of the longest group (128 members) whose sampling ranks
+    are; one key is all ones, the mark of a free slot of the hash table."""
+    rng = np.random.default_rng(N * 7 + G)
+    values = np.unique(rng.integers(1, 1 << 60, 2 * G, dtype=np.uint64))[:G]
+    values[G // 2] = np.uint64(0xFFFFFFFFFFFFFFFF)
+    keys = values[np.concatenate([np.arange(G), rng.integers(0, G, N - G)])] if N > G else values.copy()
+    keys = keys[rng.permutation(N)]
+    check(np.stack([keys, keys[::-1]]), 0, 0.3, seed=N + G, step=2)
+
+
 def test_select_long_rows():
     """Rows beyond the one-CTA path: grouping with its working arrays in shared memory (up to 18432 variates), at that
     limit, and on the global arrays beyond it; several rows at once; one group only and all-distinct keys."""
