@@ -50,6 +50,16 @@ def test_pearson_parity_random(B, N, L):
     check(x)
 
 
+@pytest.mark.parametrize("B,N,L", [(2, 256, 64), (1, 257, 128), (3, 130, 129), (1, 600, 256), (2, 385, 257), (1, 129, 512), (1, 130, 516), (1, 140, 1024), (1, 40, 1028), (2, 300, 62)])
+def test_pearson_parity_at_tile_edges(B, N, L):
+    """Edges of the 128 x 256 units, windows on both sides of the lengths whose column tile stays in shared memory (128) and whose rows stay in
+    registers (4 to 1024 in steps of 4), many CTAs to an instance and many instances to a CTA."""
+    rng = np.random.default_rng(B * 100 + N + L)
+    x = rng.normal(size=(B, N, L)).astype(np.float32) + rng.normal(size=(B, N, 1)).astype(np.float32)
+    x[:, N - 1] = 0.95 * x[:, 0] + 0.05 * x[:, N - 1]
+    check(x, threshold=0.2)
+
+
 @pytest.mark.parametrize("name", ["tiny", "elec", "traffic", "long"])
 def test_pearson_parity_workloads(name):
     w = inputs.WORKLOADS[name]
