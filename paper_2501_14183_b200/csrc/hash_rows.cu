@@ -1,4 +1,4 @@
-// k-dominant frequency hashing (Algorithm 1), batch-mean scope, for the lookback lengths the paper's
+// k-dominant frequency hashing (Algorithm 1) for the lookback lengths the paper's
 // workloads use: a register-blocked two-pass FFT with every index and twiddle fixed at compile time.
 //
 // Work is laid out by hash row (one variate): a team of 1, 2 or 4 warps owns a row, each warp takes a
@@ -265,6 +265,48 @@ __device__ __forceinline__ float sqrt_fast(float v) {                      // sq
     return r;
 }
 
+// Pass 1 of the n_win staged windows of a warp.
+template <int L, int R1, int R2, int PC>
+__device__ __forceinline__ void first_pass(const float* stage, float2* exch, const float2* tw, int lane, int n_win) {
+    using Plan = RowsPlan<L, R1, R2, PC>;
+    constexpr int P2 = Plan::P2, PS = Plan::PS, LP = Plan::LP;
+    for (int t = lane; t < ((n_win + 1) >> 1) * R2; t += 32) {
+        const int p = t / R2, j2 = t - p * R2;
+        const bool two = 2 * p + 1 < n_win;
+        float2 v[R1], y[R1];
+        const float* s1 = stage + p * LP + j2;
+        const float* s2 = s1 + (two ? PC * LP : 0);
+        static_for<0, R1>([&](auto J) {
+            constexpr int j1 = decltype(J)::value;
+            v[j1].x = s1[j1 * R2];
+            v[j1].y = s2[j1 * R2];
+        });
+        if (!two) {
+            static_for<0, R1>([&](auto J) { v[decltype(J)::value].y = 0.f; });
+        }
+        dft<R1, 1, 1>(v, y);
+        float2* dst = exch + p * PS + j2;
+        dst[0] = y[0];
+        static_for<1, R1>([&](auto K) {
+            constexpr int k1 = decltype(K)::value;
+            const float2 w = tw[k1 * R2 + j2];
+            dst[k1 * P2] = make_float2(fmaf(-y[k1].y, w.y, y[k1].x * w.x), fmaf(y[k1].x, w.y, y[k1].y * w.x));
+        });
+    }
+}
+// Twiddles between the passes, by the whole CTA.
+template <int L, int R2>
+__device__ __forceinline__ void fill_twiddles(float2* tw) {
+    for (int m = threadIdx.x; m < L; m += kRowsThreads) {
+        const int k1 = m / R2, j2 = m - k1 * R2;
+        int e = (j2 * k1) % L;
+        if (2 * e > L) e -= L;                                               // angle folded to |e| <= L / 2
+        float s, c;
+        sincospif(2.f * static_cast<float>(e) / static_cast<float>(L), &s, &c);
+        tw[m] = make_float2(c, -s);
+    }
+}
+
 // kWide: candidate bins may lie anywhere up to L / 2; otherwise the band ends below R1 K2Q (the default low-pass band does), and
 // a lane evaluates, adds up and ranks only its K2Q lowest bins: the outputs of the second pass that no such bin or mirror term
 // reads are never computed.
@@ -286,14 +328,7 @@ __global__ void __launch_bounds__(kRowsThreads, MINB) hash_rows_kernel(const Row
         mbar_fence_init();
     }
 
-    for (int m = threadIdx.x; m < L; m += kRowsThreads) {
-        const int k1 = m / R2, j2 = m - k1 * R2;
-        int e = (j2 * k1) % L;
-        if (2 * e > L) e -= L;                                               // angle folded to |e| <= L / 2
-        float s, c;
-        sincospif(2.f * static_cast<float>(e) / static_cast<float>(L), &s, &c);
-        tw[m] = make_float2(c, -s);
-    }
+    fill_twiddles<L, R2>(tw);
     __syncthreads();
     chain_wait();
     chain_release();
@@ -342,30 +377,7 @@ __global__ void __launch_bounds__(kRowsThreads, MINB) hash_rows_kernel(const Row
             if (!__all_sync(0xffffffffu, mbar_wait(bar, landed)) && lane == 0) set_status(P.status, VARDROP_ERR_TIMEOUT);
             landed ^= 1u;
             // ---- pass 1 ---------------------------------------------------------------------------------------
-            for (int t = lane; t < n_pair * R2; t += 32) {
-                const int p = t / R2, j2 = t - p * R2;
-                const int b1 = c0 + 2 * p;
-                const bool two = b1 + 1 < b_hi;
-                float2 v[R1], y[R1];
-                const float* s1 = stage + p * LP + j2;
-                const float* s2 = s1 + (two ? PC * LP : 0);
-                static_for<0, R1>([&](auto J) {
-                    constexpr int j1 = decltype(J)::value;
-                    v[j1].x = s1[j1 * R2];
-                    v[j1].y = s2[j1 * R2];
-                });
-                if (!two) {
-                    static_for<0, R1>([&](auto J) { v[decltype(J)::value].y = 0.f; });
-                }
-                dft<R1, 1, 1>(v, y);
-                float2* dst = exch + p * PS + j2;
-                dst[0] = y[0];
-                static_for<1, R1>([&](auto K) {
-                    constexpr int k1 = decltype(K)::value;
-                    const float2 w = tw[k1 * R2 + j2];
-                    dst[k1 * P2] = make_float2(fmaf(-y[k1].y, w.y, y[k1].x * w.x), fmaf(y[k1].x, w.y, y[k1].y * w.x));
-                });
-            }
+            first_pass<L, R1, R2, PC>(stage, exch, tw, lane, n_win);
             __syncwarp();
             // the staged windows are consumed: bring in the next ones
             if (c0 + 2 * PC < b_hi) stage_windows(row, c0 + 2 * PC);
@@ -459,8 +471,157 @@ __global__ void __launch_bounds__(kRowsThreads, MINB) hash_rows_kernel(const Row
     }
 }
 
+// Per-instance scope: every window is a hash row of its own.  A warp takes 2 PC consecutive rows at a time (they lie one after the other), two a
+// transform as above, and ranks the two spectra of a transform among its R1 lanes.
+// What bounds it is instruction issue, as above; 10272 rows of 96 steps 5.8 us (14.5 with the transform in shared memory), 13792 of 192 7.5 (19.6),
+// 16000 of 336 14 (30.5), 6896 of 720 15.3 (29.4).
+template <int R1, class F>
+__device__ __forceinline__ unsigned group_reduce(unsigned v, int base, int k1, F f) {        // over the R1 lanes from `base` on
+    auto from = [&](unsigned x, int off) {
+        int to = k1 + off;
+        if (to >= R1) to -= R1;
+        return __shfl_sync(0xffffffffu, x, base + to);
+    };
+    constexpr int kThirds = R1 % 3 == 0 ? R1 / 3 : R1;
+    static_assert((kThirds & (kThirds - 1)) == 0, "R1 is a power of two, or three times one");
+#pragma unroll
+    for (int off = R1 / 2; off >= (R1 % 3 == 0 ? 3 : 1); off >>= 1) v = f(v, from(v, off));
+    if constexpr (R1 % 3 == 0) {
+        const unsigned a = from(v, 1), b = from(v, 2);
+        v = f(v, f(a, b));
+    }
+    return v;
+}
+
+template <int L, int R1, int R2, int PC, int MINB, bool kWide>
+__global__ void __launch_bounds__(kRowsThreads, MINB) hash_windows_kernel(const RowsParams P) {
+    using Plan = RowsPlan<L, R1, R2, PC>;
+    constexpr int P2 = Plan::P2, PS = Plan::PS, K2N = kWide ? Plan::K2N : Plan::K2Q, G2 = Plan::G2, LP = Plan::LP;
+    extern __shared__ __align__(16) unsigned char smem_rows[];
+    const int nf = P.nf, f_lo = P.f_lo, f_hi = P.f_lo + P.nf;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float2* tw = reinterpret_cast<float2*>(smem_rows);
+    float2* exch = reinterpret_cast<float2*>(smem_rows + Plan::off_exch) + static_cast<size_t>(warp) * Plan::exch_elems;
+    float* stage = reinterpret_cast<float*>(smem_rows + Plan::off_stage) + static_cast<size_t>(warp) * Plan::stage_elems;
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem_rows + Plan::off_bar) + warp;
+    if (lane == 0) {
+        mbar_init(bar, 1);
+        mbar_fence_init();
+    }
+    fill_twiddles<L, R2>(tw);
+    __syncthreads();
+    chain_wait();
+    chain_release();
+
+    const int grp = lane / R1, k1 = lane - grp * R1;
+    const bool lane_used = grp < G2;
+    const int base = lane_used ? lane - k1 : lane;
+    const int partner = lane_used ? base + (R1 - k1) % R1 : lane;
+    const int step = gridDim.x * kRowsWarps * 2 * PC;
+    uint32_t landed = 0;
+    auto stage_rows = [&](int row0) {
+        const int n = min(2 * PC, P.N - row0);
+        if (lane == 0) mbar_expect_tx(bar, static_cast<uint32_t>(n) * L * sizeof(float));
+        __syncwarp();
+        if (lane < n) bulk_load(stage + ((lane & 1) * PC + (lane >> 1)) * LP, P.x + static_cast<size_t>(row0 + lane) * L, L * sizeof(float), bar);
+    };
+    int row0 = (blockIdx.x * kRowsWarps + warp) * 2 * PC;
+    if (row0 < P.N) stage_rows(row0);
+    for (; row0 < P.N; row0 += step) {
+        const int n_win = min(2 * PC, P.N - row0), n_pair = (n_win + 1) >> 1;
+        if (!__all_sync(0xffffffffu, mbar_wait(bar, landed)) && lane == 0) set_status(P.status, VARDROP_ERR_TIMEOUT);
+        landed ^= 1u;
+        first_pass<L, R1, R2, PC>(stage, exch, tw, lane, n_win);
+        __syncwarp();
+        if (row0 + step < P.N) stage_rows(row0 + step);
+        for (int p0 = 0; p0 < n_pair; p0 += G2) {
+            const int p = p0 + grp;
+            const bool live = lane_used && p < n_pair;
+            const float2* src = exch + (live ? p : 0) * PS + (lane_used ? k1 : 0) * P2;
+            float2 v[R2], y[R2];
+            static_for<0, R2>([&](auto J) { v[decltype(J)::value] = src[decltype(J)::value]; });
+            dft<R2, 1, 1>(v, y);                                             // y[k2] = Z[k1 + R1 k2]
+            float amp[2][K2N];                                               // bin k1 + R1 k2 of the two rows
+            static_for<0, K2N>([&](auto K) {
+                constexpr int k2 = decltype(K)::value;
+                constexpr int far = R2 - 1 - k2, own = (R2 - k2) % R2;
+                float mx = __shfl_sync(0xffffffffu, y[far].x, partner), my = __shfl_sync(0xffffffffu, y[far].y, partner);
+                if (k1 == 0) { mx = y[own].x; my = y[own].y; }
+                const float re1 = y[k2].x + mx, im1 = y[k2].y - my;
+                const float re2 = y[k2].y + my, im2 = mx - y[k2].x;
+                amp[0][k2] = sqrtf(fmaf(re1, re1, im1 * im1));
+                amp[1][k2] = sqrtf(fmaf(re2, re2, im2 * im2));
+            });
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int row = row0 + 2 * p + e;
+                const bool mine = live && 2 * p + e < n_win;
+                bool bad = false;
+#pragma unroll
+                for (int i = 0; i < K2N; ++i) {
+                    const int bin = k1 + R1 * i;
+                    if (mine && bin >= f_lo && bin < f_hi) {
+                        bad |= !isfinite(amp[e][i]);
+                        if (P.amp_dbg) P.amp_dbg[static_cast<size_t>(row) * nf + bin - f_lo] = 0.5f * amp[e][i];
+                    } else {
+                        amp[e][i] = -1.f;                                    // not a candidate
+                    }
+                }
+                if (__any_sync(0xffffffffu, bad) && lane == 0) set_status(P.status, VARDROP_ERR_NONFINITE);
+                uint64_t key = 0;
+#pragma unroll 1
+                for (int rank = 0; rank < P.k; ++rank) {
+                    // the largest amplitude left, then the lowest bin that has it (as in the kernel above, among the transform's lanes)
+                    float top = -1.f;
+#pragma unroll
+                    for (int i = 0; i < K2N; ++i) top = fmaxf(top, amp[e][i]);
+                    const unsigned top_all = group_reduce<R1>(top >= 0.f ? __float_as_uint(top) + 1u : 0u, base, lane_used ? k1 : 0, [](unsigned a, unsigned b) { return max(a, b); });
+                    unsigned bin = 0xffffffffu;
+#pragma unroll
+                    for (int i = K2N - 1; i >= 0; --i)
+                        if (amp[e][i] >= 0.f && __float_as_uint(amp[e][i]) + 1u == top_all) bin = static_cast<unsigned>(k1 + R1 * i);
+                    const unsigned bin_all = group_reduce<R1>(bin, base, lane_used ? k1 : 0, [](unsigned a, unsigned b) { return min(a, b); });
+                    const int best = top_all ? static_cast<int>(bin_all) : f_lo;             // f_lo only with non-finite input
+#pragma unroll
+                    for (int i = 0; i < K2N; ++i)
+                        if (k1 + R1 * i == best) amp[e][i] = -1.f;
+                    if (mine && k1 == 0 && P.freqs) P.freqs[static_cast<size_t>(row) * P.k + rank] = best;
+                    key = (key << 12) | static_cast<uint64_t>(best);
+                }
+                if (mine && k1 == 0) P.keys[row] = key;
+            }
+        }
+        __syncwarp();
+    }
+}
+
+template <int L, int R1, int R2, int PC, int MINB, bool kWide>
+int launch_windows(const RowsParams& P, cudaStream_t stream) {
+    using Plan = RowsPlan<L, R1, R2, PC>;
+    const size_t smem = Plan::smem_bytes();
+    static thread_local int attr_dev = -1;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (attr_dev != dev) {
+        if (int st = check_cuda(cudaFuncSetAttribute(hash_windows_kernel<L, R1, R2, PC, MINB, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     static_cast<int>(smem)), "hash: smem attribute"))
+            return st;
+        attr_dev = dev;
+    }
+    const int rows_per_cta = kRowsWarps * 2 * PC;
+    const int want = (P.N + rows_per_cta - 1) / rows_per_cta;
+    int per_sm = static_cast<int>((220 * 1024) / (smem + 1024));
+    if (per_sm > 16) per_sm = 16;
+    if (per_sm < 1) per_sm = 1;
+    const int cap = sm_count() * per_sm;
+    cudaError_t err;
+    { LaunchScope ls_(K_HASH, stream); err = launch_chained(hash_windows_kernel<L, R1, R2, PC, MINB, kWide>, dim3(want < cap ? want : cap), dim3(kRowsThreads), smem, stream, P); }
+    return check_cuda(err, "hash: launch");
+}
+
 template <int L, int R1, int R2, int PC, int MINB, bool kWide>
 int launch_rows(const RowsParams& P, cudaStream_t stream) {
+    if (P.team == 0) return launch_windows<L, R1, R2, PC, MINB, kWide>(P, stream);
     using Plan = RowsPlan<L, R1, R2, PC>;
     const size_t smem = Plan::smem_bytes();
     static thread_local int attr_dev = -1;
@@ -489,7 +650,6 @@ int launch_rows(const RowsParams& P, cudaStream_t stream) {
 // Returns -1 when this length has no register-blocked plan (the caller then takes the shared-memory kernel).
 int hash_rows_launch(const float* x, const vardrop_hash_cfg& c, int f_lo, int f_hi, uint64_t* keys, int32_t* freqs, float* amp_dbg,
                      int* status, cudaStream_t stream) {
-    if (c.scope != 0) return -1;
     if (c.L != 96 && c.L != 192 && c.L != 336 && c.L != 720) return -1;
     RowsParams P{};
     P.x = x; P.keys = keys; P.freqs = freqs; P.amp_dbg = amp_dbg; P.status = status;
@@ -498,6 +658,11 @@ int hash_rows_launch(const float* x, const vardrop_hash_cfg& c, int f_lo, int f_
     int team = 1;
     while (team < kRowsWarps && static_cast<long long>(c.N) * team < 8ll * sm_count() && c.B >= 8 * team) team *= 2;
     P.team = team;
+    if (c.scope != 0) {                              // every (instance, variate) pair is a row of one window
+        P.team = 0;
+        P.B = 1;
+        P.N = c.B * c.N;
+    }
     if (reinterpret_cast<uintptr_t>(x) % 16 != 0) return fail(VARDROP_ERR_INVALID_ARG, "hash: x is not 16-byte aligned");
     int per = (c.B + team - 1) / team;
     P.per_member = per + (per & 1);
