@@ -31,6 +31,9 @@ int hash_launch(const float* x, const vardrop_hash_cfg& cfg, uint64_t* keys, int
 // hash_rows.cu: register-blocked plans for selected lookback lengths; -1 = no plan for this configuration
 int hash_rows_launch(const float* x, const vardrop_hash_cfg& cfg, int f_lo, int f_hi, uint64_t* keys, int32_t* freqs, float* amp_dbg,
                      int* status, cudaStream_t stream);
+// hash_dft.cu: the candidate bins as a matrix product; -1 = the transform in shared memory is better
+int hash_dft_launch(const float* x, const vardrop_hash_cfg& cfg, int f_lo, int f_hi, uint64_t* keys, int32_t* freqs, float* amp_dbg, int* status,
+                    cudaStream_t stream);
 int sm_count();       // multiprocessors of the current device
 
 // select.cu
