@@ -1078,31 +1078,41 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
 struct ConvertParams {
     const float4* dq_acc;    // [B, Ncap, H, 64] fp32
     uint4* dq;               // [B, N, H, D] bf16
-    const int32_t* inv_idx;  // [S, N]; NULL: identity
+    const int32_t* sel_idx;  // [S, N]; NULL: identity
     const int32_t* n_sel;    // [S]; NULL: N
     int N, Ncap, H, D, S;
     float scale;
 };
 
+// What bounds it is memory: kept rows only (dropped ones were zeroed by the main kernel), 16-byte results, two in flight a thread.  1423 of 8192
+// kept, B = 8, H = 8: 12.6 us, 15.5 when it looked every variate up (events around the launch).
 __global__ void __launch_bounds__(256) bwd_convert_kernel(const ConvertParams P) {
     chain_wait();
     chain_release();
-    const int b = blockIdx.y;
-    const int srow = P.S > 1 ? b : 0;
-    const int32_t* inv = P.inv_idx ? P.inv_idx + static_cast<size_t>(srow) * P.N : nullptr;
-    const int chunks_head = P.D / 8;
-    const int chunks_row = P.H * chunks_head;
-    const int total = P.N * chunks_row;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-        const int n = idx / chunks_row;
-        const int c = idx - n * chunks_row;
-        const int h = c / chunks_head, dc = c - h * chunks_head;
-        const int j = inv ? inv[n] : n;
-        if (j < 0) continue;                                     // dropped rows were zeroed by the main kernel
-        const float4* src = P.dq_acc + ((static_cast<size_t>(b) * P.Ncap + j) * P.H + h) * (kDP / 4) + dc * 2;
-        const float4 a = __ldcg(src), c2 = __ldcg(src + 1);
-        P.dq[static_cast<size_t>(b) * total + idx] = make_uint4(pack2(a.x * P.scale, a.y * P.scale), pack2(a.z * P.scale, a.w * P.scale),
-                                                                pack2(c2.x * P.scale, c2.y * P.scale), pack2(c2.z * P.scale, c2.w * P.scale));
+    const int b = blockIdx.y, srow = P.S > 1 ? b : 0;
+    const int n_sel = P.n_sel ? P.n_sel[srow] : P.N;
+    const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(srow) * P.N : nullptr;
+    const int sh = P.D > 32 ? 3 : 2, chunks_row = P.H << sh;        // 16-byte results per row
+    const int total = n_sel * chunks_row, stride = gridDim.x * blockDim.x;
+    const float4* acc = P.dq_acc + static_cast<size_t>(b) * P.Ncap * P.H * (kDP / 4);
+    uint4* dq = P.dq + static_cast<size_t>(b) * P.N * chunks_row;
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += 2 * stride) {
+        float4 a[2][2];
+        size_t to[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int at = min(idx + e * stride, total - 1);
+            const int j = small_div(at, chunks_row), c = at - j * chunks_row, h = c >> sh, dc = c & ((1 << sh) - 1);
+            to[e] = static_cast<size_t>(sel ? __ldg(sel + j) : j) * chunks_row + c;
+            const float4* src = acc + (static_cast<size_t>(j) * P.H + h) * (kDP / 4) + dc * 2;
+            a[e][0] = __ldcg(src);
+            a[e][1] = __ldcg(src + 1);
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            if (idx + e * stride < total)
+                dq[to[e]] = make_uint4(pack2(a[e][0].x * P.scale, a[e][0].y * P.scale), pack2(a[e][0].z * P.scale, a[e][0].w * P.scale),
+                                       pack2(a[e][1].x * P.scale, a[e][1].y * P.scale), pack2(a[e][1].z * P.scale, a[e][1].w * P.scale));
     }
 }
 
@@ -1181,7 +1191,7 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
         ConvertParams F{};
         F.dq_acc = reinterpret_cast<const float4*>(base + w.dq_acc);
         F.dq = static_cast<uint4*>(dq);
-        F.inv_idx = sel_idx ? inv_idx : nullptr;
+        F.sel_idx = sel_idx;
         F.n_sel = sel_idx ? n_sel : nullptr;
         F.N = c.N; F.Ncap = w.Ncap; F.H = c.H; F.D = c.D; F.S = attn_sel_rows(c); F.scale = scale;
         const long long work = static_cast<long long>(c.N) * c.H * (c.D / 8);
