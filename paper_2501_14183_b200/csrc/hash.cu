@@ -14,7 +14,6 @@ namespace vardrop {
 
 namespace {
 
-constexpr int kHashThreads = 256;
 constexpr int kMaxStages = 16;
 
 struct HashParams {
@@ -203,7 +202,8 @@ __device__ __forceinline__ void fft_first_stage(const HashParams& P, float2* __r
     }
 }
 
-__global__ void __launch_bounds__(kHashThreads) hash_kernel(const HashParams P) {
+template <int kMaxThreads>       // 512 or 256: the bound that costs the shorter passes no registers
+__global__ void __launch_bounds__(kMaxThreads) hash_kernel(const HashParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int L = P.L, nf = P.nf;
     const int max_win = P.rows_per_cta * P.chunk;           // windows per pass
@@ -371,8 +371,10 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     if (rem > 1 && P.n_stages == 0) push(1);
     for (int p = 11; rem > 1; p += 2) while (rem % p == 0) { push(p); rem /= p; }
 
-    // windows per pass: about 2048 complex points per buffer, an even count
-    int per_pass = 2 * (2048 / c.L);
+    // windows per pass: about 2048 complex points per buffer, an even count; three times that where the rows are fewer than two an SM, so that
+    // a row takes one pass (137 rows of 32 windows of 168 steps: 9.3 -> 7.4 us with 512 threads)
+    const bool few_rows = P.rows_total < 2 * sm_count();
+    int per_pass = 2 * ((few_rows ? 6144 : 2048) / c.L);
     if (per_pass < 2) per_pass = 2;
     if (per_pass > 64) per_pass = 64;
     if (P.win_per_row >= per_pass) {
@@ -396,12 +398,18 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     int dev = 0;
     cudaGetDevice(&dev);
     if (attr_done_dev != dev) {
-        if (int st = check_cuda(cudaFuncSetAttribute(hash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024), "hash: smem attribute")) return st;
+        if (int st = check_cuda(cudaFuncSetAttribute(hash_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024), "hash: smem attribute")) return st;
+        if (int st = check_cuda(cudaFuncSetAttribute(hash_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024), "hash: smem attribute")) return st;
         attr_done_dev = dev;
     }
     const int grid = (P.rows_total + P.rows_per_cta - 1) / P.rows_per_cta;
+    // Threads: a stage is a few hundred butterflies, and a CTA that is mostly idle in its last round keeps others from the SM: 128 instead of 256
+    // where that wastes less (16000 windows of 300 steps 23.1 -> 18.8 us, 4000 of 64 8.4 -> 5.6); 512 for a long pass when CTAs are few.
+    const int butterflies = max_fft * (c.L / P.radix[0]);
+    auto idle = [&](int t) { return (butterflies + t - 1) / t * t; };
+    const int threads = few_rows && butterflies > 256 ? 512 : butterflies <= 128 || 5 * idle(128) < 4 * idle(256) ? 128 : 256;
     cudaError_t err;
-    { LaunchScope ls_(K_HASH, stream); err = launch_chained(hash_kernel, dim3(grid), dim3(kHashThreads), smem, stream, P); }
+    { LaunchScope ls_(K_HASH, stream); err = launch_chained(threads > 256 ? hash_kernel<512> : hash_kernel<256>, dim3(grid), dim3(threads), smem, stream, P); }
     return check_cuda(err, "hash: launch");
 }
 
