@@ -302,6 +302,18 @@ __device__ __forceinline__ void store_panel(unsigned char* panel, int row, int h
         *reinterpret_cast<uint4*>(panel + row * kRowBytes + (((half * 4 + q) ^ (row & 7)) << 4)) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
 }
 
+// With a selection per instance, the i-th instance that keeps several tiles (`several`) or one; the whole warp looks.
+__device__ __forceinline__ int nth_instance(const BwdParams& P, int i, bool several) {
+#pragma unroll 1
+    for (int base = 0; base < P.S; base += 32) {
+        const int s = base + (threadIdx.x & 31), n = s < P.S ? __ldg(P.n_sel + s) : 0;
+        const unsigned mask = __ballot_sync(0xffffffffu, several ? n > kTile : n > 0 && n <= kTile);
+        if (i < __popc(mask)) return base + __fns(mask, 0, i + 1);
+        i -= __popc(mask);
+    }
+    return 0;
+}
+
 // ---------------------------------------------------------------------------------------------------------
 // single: a kept set of one tile
 // ---------------------------------------------------------------------------------------------------------
@@ -310,7 +322,8 @@ __device__ __forceinline__ void store_panel(unsigned char* panel, int row, int h
 // every path runs once or twice, so hand-offs between roles and unrolled code only lengthen it.
 // Team memory: Q, K, V, dO, dS^T (two 64-query panels); tensor memory (256 columns): S^T [0,128), dP^T [128,256); P^T (bf16) goes over the
 // first half of each 64-column half of S^T, dV and dK over dP^T, dQ over P^T once dV has read it.
-__device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigned char* tiles, float* stats, uint64_t* bar, uint32_t tm0, int team, int gt, bool& ok) {
+template <bool kMixed>
+__device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigned char* tiles, float* stats, uint64_t* bar, uint32_t tm0, int team, int gt, int first, int stride, int count, bool& ok) {
     unsigned char* sQ = tiles + team * 6 * kTileBytes;
     unsigned char* sdO = sQ + 3 * kTileBytes;           // Q, K, V, dO
     unsigned char* sdS = sQ + 4 * kTileBytes;
@@ -325,11 +338,11 @@ __device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigne
     if (half == 0) s_none[row] = -INFINITY;
     uint32_t t = 0;
 #pragma unroll 1
-    for (int item = blockIdx.x + team * gridDim.x; item < P.H * P.B && ok; item += 2 * gridDim.x, ++t) {
-        const int b = small_div(item, P.H), h = item - b * P.H;
-        const int n = P.S > 1 ? P.n_sel[b] : kept;
-        const int32_t* idx = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? b : 0) * P.N : nullptr;
-        if (n <= 0) { --t; continue; }
+    for (int item = first; item < count && ok; item += stride, ++t) {
+        const int bi = small_div(item, P.H), h = item - bi * P.H, b = kMixed ? nth_instance(P, bi, false) : bi;
+        const int n = kMixed ? P.n_sel[b] : kept;
+        const int32_t* idx = P.sel_idx ? P.sel_idx + static_cast<size_t>(kMixed ? b : 0) * P.N : nullptr;
+        if (n <= 0) { --t; continue; }                   // (nothing kept at all)
         // rows: every warp a quarter of Q or K, then of V or dO
 #pragma unroll 1
         for (int x = warp >> 2; x < 4; x += 2) {
@@ -468,7 +481,9 @@ __device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigne
 constexpr uint32_t kTeamCols = 224, kColP = 64, kColDv = 96, kColDk = 160, kColDq = 448;
 constexpr int kTeamWarps = 8;
 
-template <bool kMany>
+// kMixed: few tiles, a selection per instance, so that some instances may keep one tile and others several (its code costs the other calls 0.4 us
+// of instruction fetch).
+template <bool kMany, bool kMixed>
 __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                                                                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
                                                                   const __grid_constant__ CUtensorMap map_acc, const BwdParams P) {
@@ -552,16 +567,45 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     const uint32_t tmem = *tmem_slot;
     bool ok = true;
     int kept = 0, n_t = 0, per_item = 1, n_slots = 0, n_items = 0;
+    bool pipeline = true, singles = false;                     // this CTA has items of the pipeline; and, few, single-tile (head, instance) pairs
+    int s_first = 0, s_stride = 1, s_count = 0;                // a team's first of those, the next one, and how many there are
     auto begin = [&]() {
         chain_wait();
         chain_release();
         kept = largest_kept(P.n_sel, P.S, P.N);
         n_t = (kept + kTile - 1) / kTile;                      // tiles of the longest selection
+        // Instances with several tiles go through the pipeline, those with one by teams.
+        int several = n_t > 1 || kMany ? P.B : 0, one = P.B - several;
+        const int grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
+        int c = cta, takers = grid;                            // CTAs that take singles
+        if (kMixed) {
+            several = one = 0;
+#pragma unroll 1
+            for (int i = 0; i < P.S; i += 32) {
+                const int n = i + lane < P.S ? __ldg(P.n_sel + i + lane) : 0;
+                several += __popc(__ballot_sync(0xffffffffu, n > kTile));
+                one += __popc(__ballot_sync(0xffffffffu, n > 0 && n <= kTile));
+            }
+        }
         // Key tiles of an item: two, except that where every key tile can have a CTA of its own it gets one (1000 of 2000 kept, B = 1, H = 8:
         // 64 tiles).  Two tiles are always one item, whose dQ is complete in place: the forward pass does not clear the accumulator then.
-        per_item = n_t == 2 || n_t * P.H * P.B > static_cast<int>(gridDim.x) ? 2 : 1;
+        per_item = n_t == 2 || n_t * P.H * several > grid ? 2 : 1;
         n_slots = (n_t + per_item - 1) / per_item;
-        n_items = n_slots * P.H * P.B;                         // pipeline: (key tiles, head, instance); short instances skip some
+        n_items = n_slots * P.H * several;                     // pipeline: (key tiles, head, instance); short instances skip some
+        pipeline = kMany || (kMixed ? cta < n_items : n_t > 1);
+        if (!kMany) {
+            s_count = one * P.H;
+            if (kMixed && several && one) {
+                // Both kinds: the CTAs without items take the singles if their teams can (32 instances of about 120 kept, a few of them above 128: forward
+                // and backward 35 us with every instance in the pipeline, 29 so).
+                const bool apart = n_items < grid && 2 * (grid - n_items) >= s_count;
+                takers = apart ? grid - n_items : grid;
+                c = apart ? cta - n_items : (cta + grid - n_items % grid) % grid;
+            }
+            singles = kMixed ? c >= 0 && c < s_count : n_t <= 1;
+            s_first = c + (warp >= 16 ? takers : 0);
+            s_stride = 2 * takers;
+        }
     };
     auto item_at = [&](uint32_t i) {
         Item it;
@@ -573,6 +617,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     auto warp_arrive = [&](uint64_t* bar) {                    // all lanes are done
         __syncwarp();
         if (lane == 0) mbar_arrive(bar);
+    };
+    auto phase_sync = [&]() {                                  // between the pipeline's use of shared and tensor memory and the teams'
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
     };
     // first token of team w's key tile (n_sel: it has none)
     auto key0_of = [&](const Item& it, int w) { return w < per_item ? (it.jt + w) * kTile : it.n_sel; };
@@ -586,10 +635,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     // does not find it (a second backward for the same forward, or two forwards sharing the workspace before their backwards) would
     // add into stale state, so it reports the call instead of returning wrong gradients.
     if (blockIdx.x == 0 && tid == 0 && atomicExch(P.status + kWsPairingWord, 0) != 1) set_status(P.status, VARDROP_ERR_INVALID_ARG);
-    if (!kMany && n_t <= 1) {
-        if (warp < 2)                                    // (four warps at it hold the teams' loads up: 20 us against 18.8 at 119 of 321 kept)
-#pragma unroll 1
-            while (write_zero_row(P, zeros)) {}
+    if (!pipeline) {
+        // nothing to issue, load or drain: the teams work by themselves
     } else if (warp < 2) {
         // ------------------------------------------------------------ issue ---------------------------------------------
         const int w = warp;
@@ -681,10 +728,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             Item it{0, 0, 0, -1};
 #pragma unroll 1
             for (; it.n_sel < 0 && k < n_items; k += gridDim.x) {
-                const int hb = small_div(k, n_slots);
+                const int hb = small_div(k, n_slots), bi = small_div(hb, P.H);
                 it.jt = (k - hb * n_slots) * per_item;
-                it.b = small_div(hb, P.H);
-                it.h = hb - it.b * P.H;
+                it.h = hb - bi * P.H;
+                it.b = kMixed ? nth_instance(P, bi, true) : bi;
                 const int n = P.S > 1 ? P.n_sel[it.b] : kept;
                 if (it.jt * kTile < n) it.n_sel = n;
             }
@@ -931,13 +978,17 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         if (owner) bulk_wait_group0();                   // the last dQ reductions have landed
         asm volatile("cp.async.wait_all;" ::: "memory");
     }
+    if (!kMany && singles) {
+        if (kMixed && pipeline) phase_sync();
+        if (warp < 2)                                    // (four warps at it hold the teams' loads up: 20 us against 18.8 at 119 of 321 kept)
+#pragma unroll 1
+            while (write_zero_row(P, zeros)) {}
+    }
     } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kBwdBigRegs));
     begin();
     const int w = (warp - 8) >> 3, gt = tid & (kBwdGroup - 1);
-    if (!kMany && n_t <= 1) {
-        bwd_single(P, kept, sKV, reinterpret_cast<float*>(sDQ), bar_team + 2 * w, tmem + w * 256, w, gt, ok);
-    } else {
+    if (pipeline) {
         // ------------------------------------------------------------ teams ---------------------------------------------
         const int row = gt & (kTile - 1), half = gt >> 7, id = w + 1;
         const uint32_t tm = tmem + w * kTeamCols + (static_cast<uint32_t>((warp & 3) * 32) << 16);
@@ -1062,8 +1113,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     }
+    if (!kMany && singles) {
+        if (kMixed && pipeline) phase_sync();
+        bwd_single<kMixed>(P, kept, sKV, reinterpret_cast<float*>(sDQ), bar_team + 2 * w, tmem + w * 256, w, gt, s_first, s_stride, s_count, ok);
     }
-    if (!kMany && (warp >= 8 || n_t > 1))
+    }
+    if (!kMany && (warp >= 8 || pipeline || !singles))       // (a warp that zeroed rows while it waited may have some of its group left)
 #pragma unroll 1
         while (write_zero_row(P, zeros)) {}              // what is left
     if (!ok) set_status(P.status, VARDROP_ERR_TIMEOUT);
@@ -1185,8 +1240,11 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
         LaunchScope ls_(K_ATTN_BWD, stream);
         return check_cuda(launch_chained(kernel, dim3(grid), dim3(kBwdThreads), kBwdSmemBytes, stream, mq, mk, mv, mdo, macc, P), "attention: backward launch");
     };
-    static thread_local int attr_few = -1, attr_many = -1;
-    if (int st = many ? launch(attn_bwd_kernel<true>, attr_many) : launch(attn_bwd_kernel<false>, attr_few)) return st;
+    static thread_local int attr_few = -1, attr_mixed = -1, attr_many = -1;
+    if (int st = many                  ? launch(attn_bwd_kernel<true, false>, attr_many)
+                 : sel_idx && P.S > 1 ? launch(attn_bwd_kernel<false, true>, attr_mixed)
+                                      : launch(attn_bwd_kernel<false, false>, attr_few))
+        return st;
     if (many) {
         ConvertParams F{};
         F.dq_acc = reinterpret_cast<const float4*>(base + w.dq_acc);

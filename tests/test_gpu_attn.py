@@ -220,6 +220,37 @@ def test_attention_per_instance_selections():
         assert torch.isnan(o[b, c:].float()).all()
 
 
+@pytest.mark.parametrize("B,N,H,D,counts", [
+    (20, 140, 8, 64, [60 + 3 * i for i in range(20)][:19] + [140]),            # one instance of two tiles: its CTAs apart from the others
+    (24, 260, 8, 32, [100 + (37 * i) % 160 for i in range(24)]),               # many of two and three: every CTA both kinds
+    (3, 200, 1, 64, [129, 1, 128]), (2, 300, 2, 64, [130, 300])])
+def test_attention_instances_of_one_and_of_several_tiles(B, N, H, D, counts):
+    dev, ref = bf16_tokens(B, N, H, D, 1.0, seed=B + N)
+    q, k, v, d_o = dev
+    sels = [pick(N, c, seed=40 + i) for i, c in enumerate(counts)]
+    sel, inv = (torch.full((B, N), -1, dtype=torch.int32) for _ in range(2))
+    for b, s_ in enumerate(sels):
+        sel[b, :len(s_)] = torch.from_numpy(np.asarray(s_, dtype=np.int32))
+        inv[b, torch.from_numpy(np.asarray(s_, dtype=np.int64))] = torch.arange(len(s_), dtype=torch.int32)
+    sel, inv, n_sel = sel.cuda(), inv.cuda(), torch.tensor(counts, dtype=torch.int32, device="cuda")
+    cfg = vd.AttnCfg(B, N, H, D, 0.0, B)
+    ws = vd.alloc_ws(vd.vardrop_attn_workspace_bytes(cfg))
+    o, dq, dk, dv = (torch.full((B, N, H, D), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(4))
+    lse = torch.zeros((B, H, N), dtype=torch.float32, device="cuda")
+    for _ in range(2):                                                         # a workspace that has been used
+        vd.vardrop_attn_fwd(q, k, v, sel, n_sel, cfg, o, lse, ws)
+        vd.vardrop_attn_bwd(q, k, v, o, lse, d_o, sel, n_sel, inv, cfg, dq, dk, dv, ws)
+    torch.cuda.synchronize()
+    assert vd.ws_status(ws) == vd.OK
+    for b, s_ in enumerate(sels):
+        cut = [r[b:b + 1] for r in ref]
+        wq, wk, wv = oracle.attn_bwd(cut[0], cut[1], cut[2], cut[3][:, :len(s_)], s_)
+        for got, want, name in ((dq, wq, "dq"), (dk, wk, "dk"), (dv, wv, "dv")):
+            g = got[b:b + 1].double().cpu().numpy()
+            assert_attn_close(g, want, f"{name}[{b}]")
+            assert np.all(g[:, np.setdiff1d(np.arange(N), s_)] == 0.0)
+
+
 def run_strided(q, k, v, d_full, B, N, H, D, sel):
     """q, k, v are (possibly non-contiguous) views [B, N, H, D] with a contiguous head dimension; their strides go into the config."""
     assert q.stride() == k.stride() == v.stride() and q.stride(3) == 1
