@@ -120,8 +120,8 @@ struct BwdParams {
 
 constexpr int kBwdGroup = 256;
 constexpr int kBwdThreads = 256 + 2 * kBwdGroup;
-// Register split (setmaxnreg works on whole warpgroups): launched with 768 x 80 = 61440 registers; the first two warpgroups keep 56 a
-// thread, the teams take 88: 256 x 56 + 512 x 88 = 59392.
+// Register split (setmaxnreg works on whole warpgroups): launched with 768 x 80 = 61440 registers; the first two warpgroups keep 56 a thread, the
+// teams take 88: 256 x 56 + 512 x 88 = 59392.  (1423 of 8192 kept: 166 us with 64 and 80, 150 so, 156 with 48 and 96, whose loaders spill.)
 constexpr int kBwdSmallRegs = 56;
 constexpr int kBwdBigRegs = 88;
 constexpr uint32_t kBwdTmemCols = 512;
@@ -854,6 +854,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         const bool owner = row == 0;                     // the one thread that owns the bulk reductions
         const uint32_t idesc_mnmn = umma_idesc_bf16(128, P.D, 1, 1);       // A MN-major, B MN-major
         const uint64_t m_k = umma_desc_sw128(smem_u32(sKV), kTileBytes, 1024);
+        // Columns taken out at a time: with few key tiles these warps also hold Delta's loads and the output rows (862 variates, 200 kept:
+        // 43.4 us with 32, 41.5 with 16); with many the chain of loads is what they wait for (1423 of 8192 kept: 150 with 32, 157 with 16).
+        constexpr int kDrain = kMany ? 32 : 16;
         bool zeros_left = !kMany;
         uint32_t t = 0, t1 = 0;                          // query tiles so far, and those with a second key tile
 #pragma unroll 1
@@ -930,19 +933,20 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 if (warp == 4 && x + 1 == n_q && lane == 0) mbar_arrive(bar_kv_free);
                 tc_fence_after();
 #pragma unroll 1
-                for (int c = 0; c < P.D; c += 32) {
-                    float v[32];
-                    tmem_ld32(tm + c, v);
+                for (int c = 0; c < P.D; c += kDrain) {
+                    float v[kDrain];
+                    if constexpr (kMany) tmem_ld32(tm + c, v);
+                    else tmem_ld16(tm + c, v);
                     tmem_ld_wait();
                     if (!direct) {                       // fp32, 32-column panels of 128-byte swizzled rows
                         unsigned char* to = sDQ + (c >> 5) * kTileBytes + row * kRowBytes;
 #pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            *reinterpret_cast<float4*>(to + (e ^ (row & 7)) * 16) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+                        for (int e = 0; e < kDrain / 4; ++e)
+                            *reinterpret_cast<float4*>(to + (((c & 31) / 4 + e) ^ (row & 7)) * 16) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
                     } else {
                         unsigned char* to = sDQ + row * kRowBytes;
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
+                        for (int e = 0; e < kDrain / 8; ++e)
                             *reinterpret_cast<uint4*>(to + (((c >> 3) + e) ^ (row & 7)) * 16) =
                                 make_uint4(pack2(v[8 * e] * P.scale, v[8 * e + 1] * P.scale), pack2(v[8 * e + 2] * P.scale, v[8 * e + 3] * P.scale),
                                            pack2(v[8 * e + 4] * P.scale, v[8 * e + 5] * P.scale), pack2(v[8 * e + 6] * P.scale, v[8 * e + 7] * P.scale));
@@ -1048,7 +1052,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 for (int hs = 0; hs < nh; ++hs, ++u) {
                     const int q0 = hs * 64 + half * 32;  // this thread's queries of the tile
                     const uint32_t lse = smem_u32(key_valid ? s_lse + slot * kTile + q0 : s_none), dlt = smem_u32(s_delta + slot * kTile + q0);
-                    if (hs == 0) ok &= warp_wait(bar_q_full + slot, (t >> 1) & 1);       // the row statistics come with the tile
+                    if (hs == 0) {                       // the row statistics come with the tile
+                        if (x == 0) {                    // after an item it had no key tile in, a team may be two phases ahead of the slot's barrier,
+                                                         // which would let it through: its own scores come after the phase it wants
+                            ok &= warp_wait(bar_x + w, 0);
+                            s_ready = true;
+                        }
+                        ok &= warp_wait(bar_q_full + slot, (t >> 1) & 1);
+                    }
                     uint64_t l[16];                      // all asked for ahead: a load behind the tensor core's operands takes a hundred cycles
 #pragma unroll
                     for (int e = 0; e < 16; ++e) l[e] = lds_pair(lse + 8 * e);
