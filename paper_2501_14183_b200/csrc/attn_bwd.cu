@@ -1044,7 +1044,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 cp_async_arrive(bar_kv_full + w);
             }
             const bool key_valid = key0 + row < it.n_sel;
-            bool s_ready = false;                        // a poll takes a hundred cycles to answer: polls go out ahead of where they are needed
+            // After an item it had no key tile in, a team may be two phases ahead of a query slot's barrier, which would let it through: its own
+            // scores come after the phase it wants.
+            ok &= warp_wait(bar_x + w, 0);
+            bool s_ready = true;                         // a poll takes a hundred cycles to answer: polls go out ahead of where they are needed
 #pragma unroll 1
             for (int x = 0; x < n_q && ok; ++x, ++t) {
                 const int nh = steps_of(it, x), slot = t & 1;
@@ -1052,14 +1055,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 for (int hs = 0; hs < nh; ++hs, ++u) {
                     const int q0 = hs * 64 + half * 32;  // this thread's queries of the tile
                     const uint32_t lse = smem_u32(key_valid ? s_lse + slot * kTile + q0 : s_none), dlt = smem_u32(s_delta + slot * kTile + q0);
-                    if (hs == 0) {                       // the row statistics come with the tile
-                        if (x == 0) {                    // after an item it had no key tile in, a team may be two phases ahead of the slot's barrier,
-                                                         // which would let it through: its own scores come after the phase it wants
-                            ok &= warp_wait(bar_x + w, 0);
-                            s_ready = true;
-                        }
-                        ok &= warp_wait(bar_q_full + slot, (t >> 1) & 1);
-                    }
+                    if (hs == 0) ok &= warp_wait(bar_q_full + slot, (t >> 1) & 1);       // the row statistics come with the tile
                     uint64_t l[16];                      // all asked for ahead: a load behind the tensor core's operands takes a hundred cycles
 #pragma unroll
                     for (int e = 0; e < 16; ++e) l[e] = lds_pair(lse + 8 * e);
