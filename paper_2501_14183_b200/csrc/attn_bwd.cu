@@ -5,8 +5,9 @@
 // attn_bwd_kernel     one CTA per SM.  Scores are formed transposed (S^T = K Q^T, dP^T = V dO^T) so that a thread owns (part of) a key row
 //                     of tensor memory; P^T and dS^T feed dV += P^T dO, dK += dS^T Q and dQ_i = dS K.  Two shapes of the work:
 //                       single   a kept set of one tile: two teams of 256 threads, each a whole (head, instance) on its own, no hand-offs
-//                       pipeline several tiles: work items (128-key tile, head, instance), a warp role for each part of the work; dQ
-//                                is added into an fp32 accumulator by bulk reduce-adds
+//                       pipeline several tiles: work items (two neighbouring 128-key tiles, head, instance), a warp role for each part of
+//                                the work; dQ is written by the item (two tiles or fewer) or added into an fp32 accumulator by bulk
+//                                reduce-adds
 //                     The same kernel writes the zero rows of every dropped variate.
 // bwd_convert_kernel  many tiles: dQ' accumulator to bf16 rows of dq (fewer: by the CTA that finishes an (instance, head) pair).
 //
