@@ -172,6 +172,9 @@ constexpr int kFwdSmemBytes = 8192 /*barriers, row maxima and sums, alignment*/ 
                               kTileBytes /*O staging*/;
 constexpr int kFwdLoadWarps = 2;
 constexpr float kRescaleStep = 8.f;              // the reference maximum of a row moves only when the running maximum has grown by 2^8
+// Where it trails like that in the few-tile kernel it starts as the maximum over the row's first 64 keys: which keys it is taken over decides how
+// P is rounded to bf16, and so the last bits of O.
+__device__ __forceinline__ float first_reference(float m_first64, float m_rest) { return m_rest > m_first64 + kRescaleStep ? m_rest : m_first64; }
 
 // The arithmetic of the softmax, written as instructions that keep their order (volatile): left to itself the compiler places the
 // consumers of a pair of exponentials right behind it, and a warp then runs at the latency of the special-function unit (20 cycles
@@ -758,6 +761,10 @@ constexpr uint32_t kTileFwdTmemCols = 128;
 constexpr int kTileFwdSmemBytes = 1024 /*alignment*/ + 3 * kTileBytes /*Q, K, V*/;
 constexpr int kTileFwdPerSm = 4;
 
+// kLag: more than two tiles without a selection, where a row's reference maximum is that of its first 64 keys until the running maximum has outgrown
+// it by 2^8; O then goes back to tensor memory for the next P V to add to.  Otherwise it is the running maximum over whole key tiles, and the
+// tiles' parts of O are added up in registers.
+template <bool kLag>
 __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_kernel(const FwdParams P) {
     extern __shared__ unsigned char smem_dyn[];
     __shared__ uint64_t bar_s, bar_o;
@@ -834,10 +841,11 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
             ok = mbar_wait(&bar_s, t & 1);
             tc_fence_after();
             // ---- row maximum, 32 scores at a time ----
-            float m_tile = -INFINITY;
+            float m_first = -INFINITY, m_tile = -INFINITY;           // kLag: of the first 64 keys of the tile, of the others
 #pragma unroll 1
             for (int c = 0; c < n_keys; c += 32) {
                 float s[32];
+                if (kLag && c == 64) { m_first = m_tile; m_tile = -INFINITY; }
                 tmem_ld32(tm + c, s);
                 tmem_ld_wait();
                 if (n_keys - c < 32) {                                // ragged end: keys past n_sel never win the maximum
@@ -855,15 +863,34 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
                 }
                 m_tile = max3(m_tile, max3(mx[0], s[28], mx[1]), max3(max3(s[29], mx[2], s[30]), mx[3], s[31]));
             }
-            const float m_new = fmaxf(m_run, m_tile * P.scale_log2), alpha = fast_exp2(m_run - m_new);
+            float m_new, alpha;
+            if (kLag) {
+                if (n_keys <= 64) { m_first = m_tile; m_tile = -INFINITY; }
+                m_new = first_reference(j == 0 ? m_first * P.scale_log2 : first_reference(m_run, m_first * P.scale_log2), m_tile * P.scale_log2);
+                alpha = m_new == m_run ? 1.f : fast_exp2(m_run - m_new);
+                l_run *= alpha;
+            } else {
+                m_new = fmaxf(m_run, m_tile * P.scale_log2);
+                alpha = fast_exp2(m_run - m_new);
+            }
             m_run = m_new;
             // ---- P = exp2(S scale - maximum), rounded to bf16, over the columns of S that have been read ----
             const uint64_t shift2 = pair_of(-m_new, -m_new);
             uint64_t l2[2] = {pair_of(0.f, 0.f), pair_of(0.f, 0.f)};
+            auto l_sum = [&]() {
+                float a0, a1, a2, a3;
+                halves_of(l2[0], a0, a1);
+                halves_of(l2[1], a2, a3);
+                return (a0 + a1) + (a2 + a3);
+            };
 #pragma unroll 1
             for (int c = 0; c < n_keys; c += 32) {
                 float s[32];
                 uint32_t pk[16];
+                if (kLag && c == 64) {                   // 64 keys a sum
+                    l_run += l_sum();
+                    l2[0] = l2[1] = pair_of(0.f, 0.f);
+                }
                 tmem_ld32(tm + c, s);
                 tmem_ld_wait();
                 if (n_keys - c < 32) {
@@ -891,11 +918,18 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
                 }
                 tmem_st16(tm + (c >> 1), pk);            // keys 2 c' and 2 c' + 1 in column c'
             }
-            {
-                float a0, a1, a2, a3;
-                halves_of(l2[0], a0, a1);
-                halves_of(l2[1], a2, a3);
-                l_run = l_run * alpha + ((a0 + a1) + (a2 + a3));
+            if (kLag) {
+                l_run += l_sum();
+                if (j > 0) {                             // O so far, for P V to add to
+                    if (__any_sync(0xffffffffu, alpha != 1.f)) {
+#pragma unroll
+                        for (int d = 0; d < kDP; ++d) o_acc[d] *= alpha;
+                    }
+                    tmem_st32(tm + 64, reinterpret_cast<const uint32_t*>(o_acc));
+                    if (P.D > 32) tmem_st32(tm + 96, reinterpret_cast<const uint32_t*>(o_acc + 32));
+                }
+            } else {
+                l_run = l_run * alpha + l_sum();
             }
             asm volatile("cp.async.wait_group 0;" ::: "memory");         // V has landed
             fence_proxy_async_smem();
@@ -908,15 +942,15 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
                 if (elect_one()) {
 #pragma unroll 1
                     for (int ks = 0; ks < (n_keys + 15) >> 4; ++ks)
-                        tc_mma_bf16_ta(tmem + 64, tmem + ks * 8, umma_desc_advance(d_v, ks * 2048), idesc_o, ks > 0);
+                        tc_mma_bf16_ta(tmem + 64, tmem + ks * 8, umma_desc_advance(d_v, ks * 2048), idesc_o, (kLag && j > 0) || ks > 0);
                     tc_commit(&bar_o);
                 }
                 __syncwarp();
             }
             ok = mbar_wait(&bar_o, t & 1);
             tc_fence_after();
-            if (n_kv > 1) {
-                if (j == 0) {
+            if (kLag ? j + 1 < n_kv : n_kv > 1) {
+                if (kLag || j == 0) {
                     tmem_ld32(tm + 64, o_acc);
                     if (P.D > 32) tmem_ld32(tm + 96, o_acc + 32);
                     tmem_ld_wait();
@@ -1019,14 +1053,16 @@ int attn_fwd_launch(const void* q, const void* k, const void* v, const int32_t* 
     cudaGetDevice(&dev);
     if (attr_dev != dev) {
         if (int st = check_cuda(cudaFuncSetAttribute(attn_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmemBytes), "attention: smem attribute")) return st;
-        if (int st = check_cuda(cudaFuncSetAttribute(attn_fwd_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileFwdSmemBytes), "attention: smem attribute")) return st;
+        for (auto kernel : {attn_fwd_tile_kernel<false>, attn_fwd_tile_kernel<true>})
+            if (int st = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileFwdSmemBytes), "attention: smem attribute")) return st;
         attr_dev = dev;
     }
     const int n_t = w.Ncap / kTile;
     LaunchScope ls_(K_ATTN_FWD, stream);
     if (few) {
         const long long worst = static_cast<long long>(n_t) * c.H * c.B, cap = static_cast<long long>(kTileFwdPerSm) * sm_count();
-        return check_cuda(launch_chained(attn_fwd_tile_kernel, dim3(static_cast<unsigned>(worst < cap ? worst : cap)), dim3(kTileFwdThreads), kTileFwdSmemBytes, stream, P),
+        const bool lag = !sel_idx && c.N > 2 * kTile;
+        return check_cuda(launch_chained(lag ? attn_fwd_tile_kernel<true> : attn_fwd_tile_kernel<false>, dim3(static_cast<unsigned>(worst < cap ? worst : cap)), dim3(kTileFwdThreads), kTileFwdSmemBytes, stream, P),
                           "attention: forward launch");
     }
     const long long worst = (static_cast<long long>(n_t / 2) * c.H + (n_t & 1 ? (c.H + 1) / 2 : 0)) * c.B;

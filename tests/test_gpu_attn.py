@@ -129,6 +129,22 @@ def test_attention_large_tokens_relative_error(B, N, H, D, Ns, std):
         assert np.all(np.isfinite(got)) and err <= bound, f"{name}: max abs error {err:.3e} > {bound:.3e}"
 
 
+@pytest.mark.parametrize("B,N,H,D,Ns", [(2, 257, 2, 64, None), (1, 300, 2, 32, None), (2, 384, 1, 64, None)])
+def test_attention_probabilities_are_rounded_against_the_first_keys(B, N, H, D, Ns):
+    """P is rounded to bf16 relative to the maximum of a row's first 64 keys: with that rounding written out
+    O is met to its own last bits.  The bound: rows whose last bit falls the other way (fp32 sums, 1e-6 of an element, against a bf16 unit of
+    2^-8: one element in 2000) by one unit each, 2^-8 sqrt(1 / 2000) = 9e-5, times four.  Another reference shows as 2.5e-3."""
+    dev, _ = bf16_tokens(B, N, H, D, 0.3536, seed=N)
+    sel = None if Ns is None else pick(N, Ns, seed=N)
+    got = torch.from_numpy(run_attention(dev, B, N, H, D, sel)[0]).cuda()
+    idx = slice(None) if sel is None else torch.from_numpy(sel).long().cuda()
+    q, k, v = (t[:, idx].double().transpose(1, 2) for t in dev[:3])
+    s = q @ k.transpose(-1, -2) * (D ** -0.5 / np.log(2.0))
+    p = torch.exp2(s - s[..., :64].amax(dim=-1, keepdim=True))
+    want = (p.float().to(torch.bfloat16).double() @ v / p.sum(dim=-1, keepdim=True)).transpose(1, 2).float().to(torch.bfloat16).double()
+    assert float((got - want).norm() / want.norm()) <= 3.6e-4
+
+
 def test_attention_identity_selection_equals_all_token_path():
     B, N, H, D = 1, 200, 2, 64
     dev, _ = bf16_tokens(B, N, H, D, 1.0, seed=3)
