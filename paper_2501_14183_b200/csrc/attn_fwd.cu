@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
     uint64_t* bar_ofree = bar_l + kFwdTiles;       // [2] they and O have been read (128 arrivals): the next item may overwrite them
     uint64_t* bar_first = bar_ofree + kFwdTiles;    // the first item's row copies have landed
     uint64_t* bar_item = bar_first + 1;             // [8] entry of the item list is written
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_item + 8);
+    uint64_t* bar_stagger = bar_item + 8;           // P of tile 0's first step is in tensor memory; completes once
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_stagger + 1);
     float* s_max = reinterpret_cast<float*>(smem_dyn + 768);    // [tile][step parity][half][row] maxima of a step
     float* s_ref = s_max + kFwdTiles * 4 * kTile;               // [tile][row] reference maximum (log2 domain)
     float* s_sum = s_ref + kFwdTiles * kTile;                   // [tile][half][row] sums
@@ -285,6 +286,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
         }
         mbar_init(bar_first, kFwdThreads - 128);
         for (int i = 0; i < 8; ++i) mbar_init(bar_item + i, 1);
+        mbar_init(bar_stagger, 1);
         mbar_fence_init();
         if (boxes) {
             tma_prefetch_desc(&map_q);
@@ -508,7 +510,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                 wait_full(bar_kv_full + sn % kFwdStages, (sn / kFwdStages) & 1);
                 // The second tile starts a softmax later than the first: in step, both tiles' exponentials queue up and then both tiles'
                 // hand-offs leave the special-function unit idle (3400 cycles a step of 128 keys against 2600).  Not worth its delay for a few steps.
-                if (i == 0 && w == 1 && it.n_kv >= 4) ok &= warp_wait_relaxed(bar_p, 0);
+                // (On a barrier of one phase: bar_p may have gone two phases on by the time this warp's first stage has landed, and its third waits for
+                // a stage of the ring that this warp has yet to release.)
+                if (i == 0 && w == 1 && it.n_kv >= 4) ok &= warp_wait_relaxed(bar_stagger, 0);
                 issue_scores(a, sn % kFwdStages, min(kTile, it.n_sel));
                 if (it.n_kv == 1) tc_commit_w(bar_q_free + qb);
 #pragma unroll 1
@@ -522,6 +526,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                         if (j + 2 == it.n_kv) tc_commit_w(bar_q_free + qb);
                     }
                     ok &= warp_wait_relaxed(bar_p + w, t & 1);
+                    if (t == 0 && w == 0 && lane == 0) mbar_arrive(bar_stagger);
                     if (j == 0 && n_mine > 0) ok &= warp_wait_relaxed(bar_ofree + w, (n_mine - 1) & 1);     // O of the previous item has been read
                     tc_fence_after();
                     issue_pv(sn % kFwdStages, min(kTile, it.n_sel - j * kTile), j > 0);
