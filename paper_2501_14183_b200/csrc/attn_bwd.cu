@@ -493,11 +493,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     // while the previous kernel of the stream is still finishing.
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_dyn);
     uint64_t* bar_kv_full = bars;                   // [2] K, V of team w
-    uint64_t* bar_kv_free = bars + 2;               // every product of the item is done (both issue warps and the dQ warps)
+    uint64_t* bar_kv_free = bars + 2;               // every product of the item is done (both issue warps and the dQ warps), and both teams are in it
     uint64_t* bar_q_full = bars + 3;                // [2] slot holds a query tile
     uint64_t* bar_q_free = bars + 5;                // [2] every product reading the slot is done (both issue warps)
     uint64_t* bar_x = bars + 7;                     // [2] S^T, then dP^T of a step complete
     uint64_t* bar_xfree = bars + 9;                 // [2] S^T is in registers, then dP^T (and P^T in tensor memory)
+    uint64_t* bar_flag = bars + 11;                 // few: both teams have read whether the item was the last of its dQ' (16 warps)
     uint64_t* bar_ds = bars + 13;                   // [2] dS^T in shared memory
     uint64_t* bar_dk = bars + 15;                   // [2] dV and dK of a step done
     uint64_t* bar_tile = bars + 17;                 // [2] dS^T of the whole query tile in shared memory
@@ -545,7 +546,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             mbar_init(bar_accfree + w, kTeamWarps);
             mbar_init(bar_delta + w, 4);
         }
-        mbar_init(bar_kv_free, 3);
+        mbar_init(bar_kv_free, 5);
+        mbar_init(bar_flag, 2 * kTeamWarps);
         mbar_init(bar_g, 1);
         mbar_init(bar_conv, 1);
         mbar_init(bar_first, 128);
@@ -859,7 +861,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         // 43.4 us with 32, 41.5 with 16); with many the chain of loads is what they wait for (1423 of 8192 kept: 150 with 32, 157 with 16).
         constexpr int kDrain = kMany ? 32 : 16;
         bool zeros_left = !kMany;
-        uint32_t t = 0, t1 = 0;                          // query tiles so far, and those with a second key tile
+        uint32_t t = 0, t1 = 0, n_conv = 0;              // query tiles so far, those with a second key tile, items with an accumulated dQ'
 #pragma unroll 1
         for (uint32_t i = 0; ok; ++i) {
             const Item it = item_at(i);
@@ -976,6 +978,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             if (!kMany && !direct && owner) {            // dQ' of this (instance, head) is complete once all its items are: the teams of the last convert it
                 bulk_wait_group0();                      // this item's reductions have landed
                 __threadfence();
+                if (n_conv > 0) ok &= mbar_wait_relaxed(bar_flag, (n_conv - 1) & 1);      // the teams have read the previous item's
+                ++n_conv;
                 *s_flag = atomicAdd(P.tile_done + it.b * P.H + it.h, 1) == (n_q - 1) / per_item;
                 mbar_arrive(bar_conv);
             }
@@ -1013,7 +1017,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 ok &= warp_wait_relaxed(bar_conv, n_conv & 1);
                 ++n_conv;
                 const int c8 = gt & 7;
-                if (!*s_flag || c8 * 8 >= P.D) return;
+                const bool last = *s_flag != 0;
+                warp_arrive(bar_flag);
+                if (!last || c8 * 8 >= P.D) return;
                 __threadfence();
                 const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
                 const float4* acc = reinterpret_cast<const float4*>(P.dq_acc + (static_cast<size_t>(it.b) * P.Ncap * P.H + it.h) * kDP) + c8 * 2;
@@ -1037,7 +1043,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                                            pack2(a[e][1].x * P.scale, a[e][1].y * P.scale), pack2(a[e][1].z * P.scale, a[e][1].w * P.scale));
                 }
             };
-            if (key0 >= it.n_sel) { t += n_q; convert_dq(); continue; }
+            if (key0 >= it.n_sel) {                      // no key tile: nothing else ties this team to the others' pace, and it waits by parity
+                if (boxes && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
+                group_sync(id);
+                if (gt == 0) mbar_arrive(bar_kv_free);
+                t += n_q;
+                convert_dq();
+                continue;
+            }
             const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
             if (!boxes) {                                // this team's K and V rows, 32 a warp
                 const int x = (warp >> 2) & 1, g = (warp & 3) * 32;
@@ -1048,6 +1061,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             // After an item it had no key tile in, a team may be two phases ahead of a query slot's barrier, which would let it through: its own
             // scores come after the phase it wants.
             ok &= warp_wait(bar_x + w, 0);
+            if (gt == 0) mbar_arrive(bar_kv_free);       // (the scores come after the phase before)
             bool s_ready = true;                         // a poll takes a hundred cycles to answer: polls go out ahead of where they are needed
 #pragma unroll 1
             for (int x = 0; x < n_q && ok; ++x, ++t) {

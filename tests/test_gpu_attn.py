@@ -91,11 +91,11 @@ def test_attention_selected_at_path_boundaries(B, N, H, D, Ns):
 @pytest.mark.parametrize("B,N,H,D,Ns", [(1, 2048, 1, 64, 130), (2, 2049, 1, 64, 1), (1, 2049, 2, 32, 128), (1, 2049, 1, 64, 129), (1, 2300, 3, 64, 384), (1, 257, 2, 64, None), (1, 384, 2, 64, None),
                                         (1, 1024, 2, 64, 256), (1, 1025, 2, 64, 300), (16, 1025, 2, 32, 257), (32, 2048, 1, 32, 700),
                                         (10, 600, 8, 32, None), (8, 2049, 8, 32, 600),
-                                        (2, 600, 2, 64, None), (2, 2049, 2, 64, 700), (3, 880, 3, 64, None)])
+                                        (2, 600, 2, 64, None), (2, 2049, 2, 64, 700), (3, 880, 3, 64, None), (24, 600, 8, 32, 300)])
 def test_attention_at_the_many_tile_boundary(B, N, H, D, Ns):
     """Both sides of the largest N whose selections count as few tiles (2048, or 1024 with few heads and
     instances; without a selection 256, in the forward pass 384): one kept row, full tiles, remainders; an odd number of key
-    tiles with several items a block, so that a team without a key tile in one item has one in the next; blocks whose first item is the odd last
+    tiles with several items a block, so that a team without a key tile in one item has one in the next, or in none of its block's items; blocks whose first item is the odd last
     tiles of two heads over five and more key tiles (the second of which starts a softmax later than the first)."""
     check_case(B, N, H, D, None if Ns is None else pick(N, Ns, seed=N + Ns), 1.0, seed=N + 3 * (Ns or 0))
 
