@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     // while the previous kernel of the stream is still finishing.
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_dyn);
     uint64_t* bar_kv_full = bars;                   // [2] K, V of team w
-    uint64_t* bar_kv_free = bars + 2;               // every product of the item is done (both issue warps and the dQ warps), and both teams are in it
+    uint64_t* bar_kv_free = bars + 2;               // every product of the item is done (both issue warps and the dQ warps)
     uint64_t* bar_q_full = bars + 3;                // [2] slot holds a query tile
     uint64_t* bar_q_free = bars + 5;                // [2] every product reading the slot is done (both issue warps)
     uint64_t* bar_x = bars + 7;                     // [2] S^T, then dP^T of a step complete
@@ -509,11 +509,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     uint64_t* bar_item = bars + 25;                 // [8] entry of the item list is written
     uint64_t* bar_team = bars + 33;                 // [2][2] single: scores, gradients
     uint64_t* bar_conv = bars + 37;                 // few: whether this item was the last of its dQ' is known
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
+    uint64_t* bar_skip = bars + 38;                 // [2] team w is in an item that it has no key tile in
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 40);
     int* s_flag = reinterpret_cast<int*>(tmem_slot + 1);
-    ZeroRows zeros{s_flag + 1, 0, 0u};
+    ZeroRows zeros{s_flag + 1, 0, 0u};                              // (the word after that counts the flags written)
     struct alignas(16) Item { int jt, h, b, n_sel; };               // n_sel < 0 ends the list
-    Item* s_item = reinterpret_cast<Item*>(smem_dyn + 320);         // [8]
+    Item* s_item = reinterpret_cast<Item*>(smem_dyn + 336);         // [8]
     float* s_lse = reinterpret_cast<float*>(smem_dyn + 512);        // [2][128] minus the lse of the slot's rows, log2 domain
     float* s_delta = s_lse + 2 * kTile;                             // [2][128] their Delta
     float* s_none = s_delta + 2 * kTile;                            // [128] minus the lse for key rows that do not exist: -inf throughout
@@ -545,8 +546,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             mbar_init(bar_tile + w, kTeamWarps);
             mbar_init(bar_accfree + w, kTeamWarps);
             mbar_init(bar_delta + w, 4);
+            mbar_init(bar_skip + w, 1);
         }
-        mbar_init(bar_kv_free, 5);
+        mbar_init(bar_kv_free, 3);
         mbar_init(bar_flag, 2 * kTeamWarps);
         mbar_init(bar_g, 1);
         mbar_init(bar_conv, 1);
@@ -563,7 +565,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         tma_prefetch_desc(&map_acc);
     }
     if (tid < kTile) s_none[tid] = -INFINITY;
-    if (tid == 0) *zeros.taken = 0;
+    if (tid == 0) s_flag[1] = s_flag[2] = 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -610,11 +612,19 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             s_stride = 2 * takers;
         }
     };
-    auto item_at = [&](uint32_t i) {
-        Item it;
-        ok &= warp_wait_relaxed(bar_item + (i & 7), (i >> 3) & 1);
+    // A role of several warps shares a named barrier, which nothing bounds: a warp whose wait gives up leaves only behind such a barrier, where the
+    // others learn of it.  The teams wait for their next item ahead of the last barrier of the current one; the dQ warps all pass a barrier at the end
+    // of the list, so that one that only took it for the end meets the others.  (8192 variates, 1423 kept: with a barrier of their own at every item
+    // 257 us instead of 252.)
+    auto item_wait = [&](uint32_t i) { ok &= warp_wait_relaxed(bar_item + (i & 7), (i >> 3) & 1); };
+    auto item_read = [&](uint32_t i) {
         const int4 x = *reinterpret_cast<const int4*>(s_item + (i & 7));
-        it.jt = x.x; it.h = x.y; it.b = x.z; it.n_sel = ok ? x.w : -1;
+        return Item{x.x, x.y, x.z, x.w};
+    };
+    auto item_at = [&](uint32_t i) {                           // -1 for an item that did not come
+        item_wait(i);
+        Item it = item_read(i);
+        if (!ok) it.n_sel = -1;
         return it;
     };
     auto warp_arrive = [&](uint64_t* bar) {                    // all lanes are done
@@ -623,7 +633,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     };
     auto phase_sync = [&]() {                                  // between the pipeline's use of shared and tensor memory and the teams'
         tc_fence_before();
-        __syncthreads();
+        ok = __syncthreads_and(ok);
         tc_fence_after();
     };
     // first token of team w's key tile (n_sel: it has none)
@@ -661,6 +671,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                     ok &= warp_wait_relaxed(bar_q_full + (t & 1), (t >> 1) & 1);
                     warp_arrive(bar_q_free + (t & 1));
                 }
+                ok &= warp_wait_relaxed(bar_skip + w, (i - ai) & 1);
                 warp_arrive(bar_kv_free);
                 continue;
             }
@@ -861,11 +872,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         // 43.4 us with 32, 41.5 with 16); with many the chain of loads is what they wait for (1423 of 8192 kept: 150 with 32, 157 with 16).
         constexpr int kDrain = kMany ? 32 : 16;
         bool zeros_left = !kMany;
-        uint32_t t = 0, t1 = 0, n_conv = 0;              // query tiles so far, those with a second key tile, items with an accumulated dQ'
+        uint32_t t = 0, t1 = 0;                          // query tiles so far, and those with a second key tile
 #pragma unroll 1
-        for (uint32_t i = 0; ok; ++i) {
+        for (uint32_t i = 0;; ++i) {
             const Item it = item_at(i);
-            if (it.n_sel < 0) break;
+            if (it.n_sel < 0) { ok = drain_sync_and(ok); break; }
             const int n_q = (it.n_sel + kTile - 1) / kTile;
             const bool two = key0_of(it, 1) < it.n_sel;
             const bool direct = !kMany && n_q <= per_item;      // dQ is complete here
@@ -978,8 +989,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             if (!kMany && !direct && owner) {            // dQ' of this (instance, head) is complete once all its items are: the teams of the last convert it
                 bulk_wait_group0();                      // this item's reductions have landed
                 __threadfence();
-                if (n_conv > 0) ok &= mbar_wait_relaxed(bar_flag, (n_conv - 1) & 1);      // the teams have read the previous item's
-                ++n_conv;
+                const int n = s_flag[2]++;               // items with an accumulated dQ' before this one
+                if (n > 0 && !mbar_wait_relaxed(bar_flag, (n - 1) & 1)) set_status(P.status, VARDROP_ERR_TIMEOUT);     // the teams have read that one's flag
                 *s_flag = atomicAdd(P.tile_done + it.b * P.H + it.h, 1) == (n_q - 1) / per_item;
                 mbar_arrive(bar_conv);
             }
@@ -1005,16 +1016,18 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         unsigned char* panels = sdS + 2 * w * kTileBytes;
         const uint64_t scale2 = pair_of(P.scale_log2, P.scale_log2);
         uint32_t t = 0, u = 0, n_conv = 0;               // query tiles, steps of this team, items with an accumulated dQ' so far
+        item_wait(0);
+        ok = group_sync_and(id, ok);
 #pragma unroll 1
         for (uint32_t i = 0; ok; ++i) {
-            const Item it = item_at(i);
+            const Item it = item_read(i);
             if (it.n_sel < 0) break;
             const int n_q = (it.n_sel + kTile - 1) / kTile, key0 = key0_of(it, w);
             if (!boxes && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
             // dQ' of an (instance, head) of more than two tiles: both teams of the CTA that brought its last part
             auto convert_dq = [&]() {
                 if (kMany || n_q <= per_item) return;
-                ok &= warp_wait_relaxed(bar_conv, n_conv & 1);
+                if (!warp_wait_relaxed(bar_conv, n_conv & 1)) set_status(P.status, VARDROP_ERR_TIMEOUT);
                 ++n_conv;
                 const int c8 = gt & 7;
                 const bool last = *s_flag != 0;
@@ -1045,8 +1058,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             };
             if (key0 >= it.n_sel) {                      // no key tile: nothing else ties this team to the others' pace, and it waits by parity
                 if (boxes && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
-                group_sync(id);
-                if (gt == 0) mbar_arrive(bar_kv_free);
+                item_wait(i + 1);
+                ok = group_sync_and(id, ok);
+                if (gt == 0) mbar_arrive(bar_skip + w);
                 t += n_q;
                 convert_dq();
                 continue;
@@ -1061,7 +1075,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             // After an item it had no key tile in, a team may be two phases ahead of a query slot's barrier, which would let it through: its own
             // scores come after the phase it wants.
             ok &= warp_wait(bar_x + w, 0);
-            if (gt == 0) mbar_arrive(bar_kv_free);       // (the scores come after the phase before)
             bool s_ready = true;                         // a poll takes a hundred cycles to answer: polls go out ahead of where they are needed
 #pragma unroll 1
             for (int x = 0; x < n_q && ok; ++x, ++t) {
@@ -1119,7 +1132,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 const int key = key0 + r8 + 32 * e;
                 nout[e] = key < it.n_sel ? (sel ? __ldg(sel + key) : key) : -1;
             }
-            ok = warp_wait(bar_dk + w, (u - 1) & 1);
+            ok &= warp_wait(bar_dk + w, (u - 1) & 1);
             ok &= warp_wait(bar_g, (t - 1) & 1);
             tc_fence_after();
 #pragma unroll 1
@@ -1130,7 +1143,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             if (!ok) break;
 #pragma unroll 1
             for (int e = 0; e < 2; ++e) store_rows(panels + e * kTileBytes, e == 0 ? P.dv : P.dk, nout, gt, P, it.b, it.h);
-            group_sync(id);                              // the staging tiles are free
+            item_wait(i + 1);
+            ok = group_sync_and(id, ok);                 // the staging tiles are free
             convert_dq();
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
