@@ -225,8 +225,10 @@ __device__ __forceinline__ void tile_sync(int w) {
     if (w == 0) asm volatile("bar.sync 2, 256;" ::: "memory");
     else asm volatile("bar.sync 3, 256;" ::: "memory");
 }
-// barrier among the 128 threads of the finishing warpgroup
-__device__ __forceinline__ void finish_group_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+__device__ __forceinline__ void tile_arrive(int w) {
+    if (w == 0) asm volatile("bar.arrive 2, 256;" ::: "memory");
+    else asm volatile("bar.arrive 3, 256;" ::: "memory");
+}
 
 __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q,
                                                                    const __grid_constant__ CUtensorMap map_k,
@@ -556,11 +558,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
     } else if (warp < 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFwdOtherRegs));
         // ---------------------------------------------------------------- O / l, rounded to bf16 ------------------
-        // through a staging tile, so that whole 128-byte rows are written
+        // through a staging tile, so that whole 128-byte rows are written; a warp writes the rows it has staged
         const int r = tid & (kFwdGroupThreads - 1);
         const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
         uint32_t t0 = 0, t1 = 0, n0 = 0, n1 = 0;        // steps and items of the two softmax warpgroups so far
-        const int c = r & 7;
+        const int c = r & 7, r0 = (r & ~31) + (lane >> 3);
         begin();
         load_first();
 #pragma unroll 1
@@ -594,22 +596,22 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                 tc_fence_before();
                 mbar_arrive(bar_ofree + w);                  // O, maximum and sum are in registers or in the staging tile
                 if (row < it.n_sel) P.lse[(static_cast<size_t>(it.b) * P.H + h) * P.N + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
-                finish_group_sync();
+                __syncwarp();
                 if (c * 8 < P.D) {
-                    __nv_bfloat16* out = P.o + ((static_cast<size_t>(it.b) * P.N + qt * kTile + (r >> 3)) * P.H + h) * P.D + c * 8;
-                    const unsigned char* from = stage + (r >> 3) * kRowBytes + ((c ^ ((r >> 3) & 7)) << 4);
-                    const int left = it.n_sel - qt * kTile - (r >> 3);       // rows 16 apart, as long as they exist
+                    __nv_bfloat16* out = P.o + ((static_cast<size_t>(it.b) * P.N + qt * kTile + r0) * P.H + h) * P.D + c * 8;
+                    const unsigned char* from = stage + r0 * kRowBytes;
+                    const int left = it.n_sel - qt * kTile - r0;             // rows 4 apart, as long as they exist
 #pragma unroll 1
-                    for (int x = 0; x < kTile / 16; x += 4) {
+                    for (int x = 0; x < 8; x += 4) {
                         uint4 v[4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(from + (x + u) * 16 * kRowBytes);
+                        for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(from + (x + u) * 4 * kRowBytes + ((c ^ ((r0 + 4 * u) & 7)) << 4));
 #pragma unroll
                         for (int u = 0; u < 4; ++u)
-                            if ((x + u) * 16 < left) *reinterpret_cast<uint4*>(out + static_cast<size_t>(x + u) * 16 * P.H * P.D) = v[u];
+                            if ((x + u) * 4 < left) *reinterpret_cast<uint4*>(out + static_cast<size_t>(x + u) * 4 * P.H * P.D) = v[u];
                     }
                 }
-                finish_group_sync();                         // the staging tile is free
+                __syncwarp();                                // its rows of the staging tile are free
             }
             t0 += it.n_kv; ++n0;
             if (it.n_act > 1) { t1 += it.n_kv; ++n1; }
@@ -745,7 +747,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
         }
     }
 
-    if (!ok) set_status(P.status, VARDROP_ERR_TIMEOUT);
+    if (!ok) {
+        set_status(P.status, VARDROP_ERR_TIMEOUT);
+        // A softmax warp whose wait gave up has left by itself, and nothing bounds a named barrier: it arrives once more in passing.  The others reach
+        // at most one more: the scores of the step behind that one wait for this warp's arrivals too.
+        if (warp >= 8) tile_arrive((warp - 8) >> 3);
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kFwdTmemCols);
