@@ -250,7 +250,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
     uint64_t* bar_first = bar_ofree + kFwdTiles;    // the first item's row copies have landed
     uint64_t* bar_item = bar_first + 1;             // [8] entry of the item list is written
     uint64_t* bar_stagger = bar_item + 8;           // P of tile 0's first step is in tensor memory; completes once
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_stagger + 1);
+    uint64_t* bar_skip = bar_stagger + 1;           // [2] tile 1's softmax warps (8), its issue warp are in an item without a second tile
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_skip + 2);
     float* s_max = reinterpret_cast<float*>(smem_dyn + 768);    // [tile][step parity][half][row] maxima of a step
     float* s_ref = s_max + kFwdTiles * 4 * kTile;               // [tile][row] reference maximum (log2 domain)
     float* s_sum = s_ref + kFwdTiles * kTile;                   // [tile][half][row] sums
@@ -289,6 +290,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
         mbar_init(bar_first, kFwdThreads - 128);
         for (int i = 0; i < 8; ++i) mbar_init(bar_item + i, 1);
         mbar_init(bar_stagger, 1);
+        mbar_init(bar_skip, kFwdTileThreads / 32);
+        mbar_init(bar_skip + 1, 1);
         mbar_fence_init();
         if (boxes) {
             tma_prefetch_desc(&map_q);
@@ -543,6 +546,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                 ++n_mine;
             } else {                                     // nothing to compute in this item: keep up with its barriers
                 ok &= warp_wait_relaxed(bar_q_full + qb, (n_done >> 1) & 1);
+                ok &= warp_wait_relaxed(bar_skip, (n_done - n_mine) & 1);      // its softmax warps are here too
+                if (lane == 0) mbar_arrive(bar_skip + 1);
                 tc_commit_w(bar_q_free + qb);
 #pragma unroll 1
                 for (int l = 0; l < it.n_kv * per_step && ok; ++l) {
@@ -631,7 +636,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
         for (uint32_t i = 0; ok; ++i) {
             const Item it = item_at(i);
             if (it.n_act < 0) break;
-            if (w >= it.n_act) continue;
+            if (w >= it.n_act) {                        // nothing else ties the warps of a tile that an item lacks to the others' pace, and they wait by parity
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_skip);
+                ok = warp_wait_relaxed(bar_skip + 1, (i - n_mine) & 1);
+                continue;
+            }
             if (half == 0) {
                 const int qt = it.split ? it.qt : it.qt + w, h = it.split ? it.h + w : it.h;
                 if (P.dq_acc) {     // the backward pass adds per-key-tile pieces of dQ' into the accumulator: clear this tile's rows
