@@ -172,8 +172,8 @@ constexpr int kFwdSmemBytes = 8192 /*barriers, row maxima and sums, alignment*/ 
                               kTileBytes /*O staging*/;
 constexpr int kFwdLoadWarps = 2;
 constexpr float kRescaleStep = 8.f;              // the reference maximum of a row moves only when the running maximum has grown by 2^8
-// Where it trails like that in the few-tile kernel it starts as the maximum over the row's first 64 keys: which keys it is taken over decides how
-// P is rounded to bf16, and so the last bits of O.
+// It starts as the maximum over the row's first 64 keys: which keys it is taken over decides how P is rounded to bf16, and so the last bits of O
+// (which calls without a selection keep whichever kernel serves them).
 __device__ __forceinline__ float first_reference(float m_first64, float m_rest) { return m_rest > m_first64 + kRescaleStep ? m_rest : m_first64; }
 
 // The arithmetic of the softmax, written as instructions that keep their order (volatile): left to itself the compiler places the
@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                 tile_sync(w);
                 const float m_tile = fmaxf(m_mine, ex[(half ^ 1) * kTile]);
                 if (j == 0) {
-                    m_ref = m_tile;
+                    m_ref = first_reference(ex[0], m_tile);
                 } else {
                     // O accumulates in tensor memory against m_ref.  It is rescaled only when a row's maximum has outgrown m_ref by
                     // 2^8 (probabilities then stay below 256, exact enough in bf16 and far from overflow); each half takes its

@@ -131,9 +131,9 @@ def test_attention_large_tokens_relative_error(B, N, H, D, Ns, std):
         assert np.all(np.isfinite(got)) and err <= bound, f"{name}: max abs error {err:.3e} > {bound:.3e}"
 
 
-@pytest.mark.parametrize("B,N,H,D,Ns", [(2, 257, 2, 64, None), (1, 300, 2, 32, None), (2, 384, 1, 64, None)])
+@pytest.mark.parametrize("B,N,H,D,Ns", [(2, 257, 2, 64, None), (1, 300, 2, 32, None), (2, 384, 1, 64, None), (1, 385, 2, 64, None), (1, 862, 1, 64, None), (1, 2049, 2, 64, 300)])
 def test_attention_probabilities_are_rounded_against_the_first_keys(B, N, H, D, Ns):
-    """P is rounded to bf16 relative to the maximum of a row's first 64 keys: with that rounding written out
+    """P is rounded to bf16 relative to the maximum of a row's first 64 keys, whichever kernel serves the call: with that rounding written out
     O is met to its own last bits.  The bound: rows whose last bit falls the other way (fp32 sums, 1e-6 of an element, against a bf16 unit of
     2^-8: one element in 2000) by one unit each, 2^-8 sqrt(1 / 2000) = 9e-5, times four.  Another reference shows as 2.5e-3."""
     dev, _ = bf16_tokens(B, N, H, D, 0.3536, seed=N)
