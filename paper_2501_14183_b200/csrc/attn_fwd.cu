@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
     uint32_t t = 0;                                     // key tiles of this CTA so far: parity of bar_s and bar_o
 
 #pragma unroll 1
-    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int hb = small_div(item, n_t), qt = item - hb * n_t, b = small_div(hb, P.H), h = hb - b * P.H;
         const int n_sel = P.S > 1 ? P.n_sel[b] : kept, n_kv = (n_sel + kTile - 1) / kTile;
         if (qt >= n_kv) continue;
@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
                 }
                 __syncwarp();
             }
-            ok = mbar_wait(&bar_s, t & 1);
+            ok &= mbar_wait(&bar_s, t & 1);
             tc_fence_after();
             // ---- row maximum, 32 scores at a time ----
             float m_first = -INFINITY, m_tile = -INFINITY;           // kLag: of the first 64 keys of the tile, of the others
@@ -957,8 +957,8 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
             fence_proxy_async_smem();
             tmem_st_wait();
             tc_fence_before();
-            ok = __syncthreads_and(ok);                  // (a wait gave up somewhere in the CTA: stop)
-            if (!ok) break;
+            ok = __syncthreads_and(ok);
+            if (!ok) { item = n_items; break; }          // a wait gave up somewhere in the CTA: stop
             if (warp == 0) {
                 tc_fence_after();
                 if (elect_one()) {
@@ -969,7 +969,7 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
                 }
                 __syncwarp();
             }
-            ok = mbar_wait(&bar_o, t & 1);
+            ok &= mbar_wait(&bar_o, t & 1);              // (agreed on at the next such barrier: no thread leaves by itself)
             tc_fence_after();
             if (kLag ? j + 1 < n_kv : n_kv > 1) {
                 if (kLag || j == 0) {
@@ -999,7 +999,7 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
             tc_fence_before();
             if (j + 1 < n_kv) __syncthreads();           // the next step's S goes over these columns
         }
-        if (!ok) break;
+        if (item == n_items) break;
         // ---- O / l, rounded to bf16, through Q's tile so that whole rows are written ----
         {
             const float inv_l = 1.f / l_run;
