@@ -275,14 +275,15 @@ __global__ void __launch_bounds__(kPearsonThreads, 1) pearson_max_kernel(const _
         // two threads a row, 128 of the 256 columns each
         const int row = tid & (kTile - 1), half = (warp - 4) >> 2;
         const uint32_t tm = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + half * kTile;
+        // (These warps share a named barrier, which nothing bounds: one whose wait gives up goes on to it, without work or further waits, and all leave there.)
         int taken = 0;                                               // units of the current instance
         uint32_t i = 0;
 #pragma unroll 1
-        for (long long u = u0; u < u1 && ok; ++u, ++i) {
+        for (long long u = u0; u < u1; ++u, ++i) {
             const Unit x = unit_at(u);
             const int v = x.ti * kTile + row;
             float best = -2.f;
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_acc + (i & 1), (i >> 1) & 1));
+            ok = ok && __all_sync(0xffffffffu, mbar_wait(bar_acc + (i & 1), (i >> 1) & 1));
             tc_fence_after();
 #pragma unroll 1
             for (int c = 0; c < kTile && ok; c += 32) {
@@ -304,7 +305,7 @@ __global__ void __launch_bounds__(kPearsonThreads, 1) pearson_max_kernel(const _
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_accfree + (i & 1));
+            if (lane == 0 && ok) mbar_arrive(bar_accfree + (i & 1));
             if (v < P.N && best > -2.f) atomic_max_float(P.max_rho + static_cast<size_t>(x.b) * P.N + v, best);
             ++taken;
             if (u + 1 == u1 || (x.ti + 1 == row_tiles && x.tj + 1 == col_tiles)) {           // the run leaves this instance
