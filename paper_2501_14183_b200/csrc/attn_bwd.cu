@@ -1229,7 +1229,7 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
         R.sel_idx = sel_idx;
         R.sB = L.sB; R.sN = L.sN; R.sH = L.sH;
         R.n_sel = sel_idx ? n_sel : nullptr;
-        R.N = c.N; R.Ncap = w.Ncap; R.H = c.H; R.D = c.D; R.S = attn_sel_rows(c);
+        R.N = c.N; R.Ncap = w.Ncap; R.H = c.H; R.D = c.D; R.S = attn_sel_rows(c, sel_idx);
         const long long work = static_cast<long long>(w.Ncap) * c.H * 8;
         int gx = static_cast<int>((work + 255) / 256);
         const int cap = max(1, 8 * sm_count() / c.B);              // about eight CTAs per SM in total
@@ -1262,7 +1262,7 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
     P.tile_done = reinterpret_cast<int32_t*>(base + w.delta);
     P.status = reinterpret_cast<int*>(base);
     P.sB = L.sB; P.sN = L.sN; P.sH = L.sH;
-    P.B = c.B; P.N = c.N; P.Ncap = w.Ncap; P.H = c.H; P.D = c.D; P.S = attn_sel_rows(c);
+    P.B = c.B; P.N = c.N; P.Ncap = w.Ncap; P.H = c.H; P.D = c.D; P.S = attn_sel_rows(c, sel_idx);
     P.scale = scale; P.scale_log2 = scale * 1.4426950408889634f;
     const long long worst = static_cast<long long>(w.Ncap / kTile) * c.H * c.B;
     const int grid = static_cast<int>(worst < sm_count() ? worst : sm_count());          // one CTA per SM (all of tensor memory)
@@ -1287,7 +1287,7 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
         F.dq = static_cast<uint4*>(dq);
         F.sel_idx = sel_idx;
         F.n_sel = sel_idx ? n_sel : nullptr;
-        F.N = c.N; F.Ncap = w.Ncap; F.H = c.H; F.D = c.D; F.S = attn_sel_rows(c); F.scale = scale;
+        F.N = c.N; F.Ncap = w.Ncap; F.H = c.H; F.D = c.D; F.S = attn_sel_rows(c, sel_idx); F.scale = scale;
         const long long work = static_cast<long long>(c.N) * c.H * (c.D / 8);
         int gx = static_cast<int>((work + 255) / 256);
         const int cap = max(1, 8 * sm_count() / c.B);

@@ -152,8 +152,8 @@ inline bool attn_many_tiles(const vardrop_attn_cfg& c, const int32_t* sel_idx) {
 // prep launch follows; without a selection the forward pass may be inference, and the prep launch does it.
 inline bool attn_fwd_clears(const vardrop_attn_cfg& c, const int32_t* sel_idx) { return sel_idx != nullptr || !attn_many_tiles(c, sel_idx); }
 
-// Number of selection rows: one shared by the batch, or one per instance.
-inline int attn_sel_rows(const vardrop_attn_cfg& c) { return c.S > 1 ? c.S : 1; }
+// Number of selection rows: one shared by the batch (or none at all), or one per instance.
+inline int attn_sel_rows(const vardrop_attn_cfg& c, const int32_t* sel_idx) { return sel_idx && c.S > 1 ? c.S : 1; }
 
 // Kept count that sizes the work: of the one selection, the largest of several (each warp looks on its own), or N.
 __device__ __forceinline__ int largest_kept(const int32_t* n_sel, int S, int N) {

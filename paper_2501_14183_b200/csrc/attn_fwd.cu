@@ -1067,7 +1067,7 @@ int attn_fwd_launch(const void* q, const void* k, const void* v, const int32_t* 
     P.dq_acc = attn_fwd_clears(c, sel_idx) ? reinterpret_cast<float4*>(base + w.dq_acc) : nullptr;
     P.tile_done = reinterpret_cast<int32_t*>(base + w.delta);
     P.sB = L.sB; P.sN = L.sN; P.sH = L.sH;
-    P.B = c.B; P.N = c.N; P.Ncap = w.Ncap; P.H = c.H; P.D = c.D; P.S = attn_sel_rows(c);
+    P.B = c.B; P.N = c.N; P.Ncap = w.Ncap; P.H = c.H; P.D = c.D; P.S = attn_sel_rows(c, sel_idx);
     const float scale = c.sm_scale > 0.f ? c.sm_scale : 1.f / sqrtf(static_cast<float>(c.D));
     P.scale_log2 = scale * 1.4426950408889634f;
     static thread_local int attr_dev = -1;

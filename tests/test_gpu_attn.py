@@ -271,6 +271,27 @@ def test_attention_instances_of_one_and_of_several_tiles(B, N, H, D, counts):
             assert np.all(g[:, np.setdiff1d(np.arange(N), s_)] == 0.0)
 
 
+@pytest.mark.parametrize("N", [100, 300, 400])
+def test_attention_of_all_tokens_takes_a_configuration_for_selections_per_instance(N):
+    """S = B in the configuration and no selection: every token, as with S = 1."""
+    B, H, D = 3, 2, 64
+    (q, k, v, d_o), _ = bf16_tokens(B, N, H, D, 0.5, seed=N)
+    runs = []
+    for S in (1, B):
+        cfg = vd.AttnCfg(B, N, H, D, 0.0, S)
+        ws = vd.alloc_ws(vd.vardrop_attn_workspace_bytes(cfg))
+        o, dq, dk, dv = (torch.zeros_like(q) for _ in range(4))
+        lse = torch.zeros((B, H, N), device="cuda")
+        vd.vardrop_attn_fwd(q, k, v, None, None, cfg, o, lse, ws)
+        vd.vardrop_attn_bwd(q, k, v, o, lse, d_o, None, None, None, cfg, dq, dk, dv, ws)
+        torch.cuda.synchronize()
+        assert vd.ws_status(ws) == vd.OK
+        runs.append((o, lse, dk, dv, dq))
+    for a, b in zip(runs[0][:4], runs[1][:4]):
+        assert torch.equal(a, b)
+    np.testing.assert_allclose(runs[0][4].float().cpu().numpy(), runs[1][4].float().cpu().numpy(), rtol=0, atol=2e-3)      # dq: fp32 adds in no fixed order
+
+
 def run_strided(q, k, v, d_full, B, N, H, D, sel):
     """q, k, v are (possibly non-contiguous) views [B, N, H, D] with a contiguous head dimension; their strides go into the config."""
     assert q.stride() == k.stride() == v.stride() and q.stride(3) == 1
