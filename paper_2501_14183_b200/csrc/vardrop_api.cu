@@ -56,6 +56,7 @@ LaunchScope::LaunchScope(int id, cudaStream_t stream) : id_(id), stream_(stream)
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (!g_prof_on.load(std::memory_order_relaxed)) return;
     std::lock_guard<std::mutex> lock(g_prof_mutex);
+    if (!g_prof_on.load(std::memory_order_relaxed)) return;                // disarmed in between
     std::pair<cudaEvent_t, cudaEvent_t> ev;
     if (!g_prof_free.empty()) {
         ev = g_prof_free.back();
