@@ -312,8 +312,8 @@ __global__ void __launch_bounds__(kTailThreads) select_sample_kernel(const Selec
 //
 // More than 512, in few groups (the point of the method): the distinct keys are found with a hash table and ranked by counting, which gives the group ids; a
 // variate's place in its group is the number of equal keys in the 32-variate chunks before its own plus those below it in the chunk; its
-// sampling rank is counted over its group.  No sort.
-// Fewer, many groups, or a long one: two bitonic sorts.
+// sampling rank is counted over its group, or, with a long group, found by sorting (group, priority, place).
+// Fewer variates, or many groups: two bitonic sorts.
 //   sort 1: (key, variate)                      -> members, group heads -> ids, offsets
 //   sort 2: (group id, Philox priority, rank j) -> position inside the group = sampling rank
 // Then the kept flags are compacted with one scan.  No scratch in global memory, no global atomics.
@@ -386,9 +386,11 @@ __device__ __forceinline__ int block_scan_pair(int v0, int v1, int* warp_sums, i
     return v + base - v0 - v1;
 }
 
-// Most groups the counting path takes: ranking G keys is G^2 / 32 cycles, about half of what the sort of M items takes at this line.
-__host__ __device__ constexpr int small_max_groups(int M) { return M <= 64 ? 64 : M == 128 ? 128 : M == 256 ? 182 : M == 512 ? 256 : M == 1024 ? 362 : 512; }
-// Longest group whose sampling ranks are counted: 128 positions take some 4000 cycles, the second sort of 1024 items 8000 (of 512 items 4500).
+// Most groups the counting path takes.  Ranking G keys is G^2 / 32 cycles; the sort does not depend on G.  Counting | sorting, 862 variates: 60 groups
+// 7.2 | 8.8 us, 130 8.0 | 8.6, 160 8.4 | 8.7, 200 10.3 | 8.7; 2048 variates: 100 11.7 | 18.6, 300 15.6 | 17.6, 362 17.5 | 17.6, 420 19.8 | 17.6.  A call
+// with more has paid for the table when it comes to sort: 862 distinct keys 9.4 us instead of 8.3, 2048 18.6 instead of 16.8.
+__host__ __device__ constexpr int small_max_groups(int M) { return M <= 1024 ? 160 : 360; }
+// Longest group whose sampling ranks are counted: 128 positions take some 4000 cycles, the sort of 1024 codes 8000.
 constexpr int kCountMaxGroup = 128, kSortCountMaxGroup = 64;
 
 // Shared memory of the counting path (the sorting path uses less, over it).
@@ -421,8 +423,8 @@ __host__ __device__ inline SmallLayout small_layout(int M) {
 // What bounds it is latency: half a dozen short steps between barriers, each run once, at the speed of instruction fetch.  So the steps are
 // few (sizes and offsets come out of the ranking of the distinct keys, without scans) and their loops rolled, with what a variate
 // carries from step to step in shared memory.
-// Measured (events around the launch), counting | sorting: 862 variates in 52 groups of up to 72 12.8 | 15.5 us, in 146 groups 14.8 | 16.9;
-// 32 rows of 321 11.6 | 10.7, 21 8.6 | 8.7: up to 512 items it sorts.
+// Measured, counting | sorting: 862 variates in one group 9.2 | 11.6 us, in 16 groups 7.5 | 11.8, in 60 7.2 | 8.8; 2048 in one 15.8 | 24.3; events around
+// the launch, 32 rows of 321 11.6 | 10.7, 21 8.6 | 8.7: up to 512 items it sorts.
 constexpr int kSortOnlyItems = 512;
 template <bool kCounting>
 __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const SelectParams P, int M) {
@@ -471,9 +473,10 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
         // ---- the distinct keys: whoever takes a slot opens an entry --------------------------------------------
 #pragma unroll 1
         for (int n = tid; n < N; n += T) {
+            if (n >= T && *reinterpret_cast<volatile int*>(&n_entries) > G_max) break;       // too many already: to the sort
             const uint64_t key = keys[n];
             int at = 2 * M;
-            bool mine;
+            bool mine = false;
             if (key == kEmpty) {
                 mine = atomicExch(&all_ones, 1) == 0;
             } else {
@@ -481,7 +484,6 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
 #pragma unroll 1
                 for (;;) {                             // at most half of the slots are ever taken
                     uint64_t cur = *reinterpret_cast<volatile uint64_t*>(table + at);
-                    mine = false;
                     if (cur == kEmpty) {
                         cur = atomicCAS(reinterpret_cast<unsigned long long*>(table + at), kEmpty, key);
                         mine = cur == kEmpty;
@@ -498,8 +500,7 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
         }
         __syncthreads();
         const int G = n_entries;
-        bool counting = G <= G_max;
-        if (counting) {
+        if (G <= G_max) {
             // equal keys within a chunk of 32 consecutive variates
 #pragma unroll 1
             for (int n = tid; n - lane < N; n += T) {
@@ -558,9 +559,7 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
                     quota_s[d] = static_cast<uint16_t>(quota_of(size_s[d], P.gs, P.rate_ppm));
                 }
             }
-            counting = !__syncthreads_or(longest > kCountMaxGroup);
-        }
-        if (counting) {
+            const bool long_group = __syncthreads_or(longest > kCountMaxGroup);
             // sorted positions
 #pragma unroll 1
             for (int n = tid; n < N; n += T) {
@@ -571,26 +570,56 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
                 entry_s[first + j] = static_cast<uint16_t>(d);
                 gid[n] = g;
             }
-            for (int d = tid; d < G; d += T) off[rank[d]] = first_s[d];
+            uint32_t* by_rank = reinterpret_cast<uint32_t*>(list);       // first position | quota << 16 of a group (the keys are no longer read)
+            for (int d = tid; d < G; d += T) {
+                off[rank[d]] = first_s[d];
+                by_rank[rank[d]] = static_cast<uint32_t>(first_s[d]) | static_cast<uint32_t>(quota_s[d]) << 16;
+            }
             for (int i = G + tid; i <= N; i += T) off[i] = N;
             if (tid == 0) P.n_groups[s] = G;
             __syncthreads();
-            // sampling ranks, by sorted position: neighbours read the same priorities
+            if (!long_group) {
+                // sampling ranks, by sorted position: neighbours read the same priorities
 #pragma unroll 1
-            for (int p = tid; p < N; p += T) {
-                const int d = entry_s[p], begin = first_s[d], size = size_s[d], n = member_s[p];
-                members[p] = n;
-                const int quota = quota_s[d];
-                int below = 0;
-                if (quota < size) {
-                    const uint32_t mine = prio[p];
+                for (int p = tid; p < N; p += T) {
+                    const int d = entry_s[p], begin = first_s[d], size = size_s[d], n = member_s[p];
+                    members[p] = n;
+                    const int quota = quota_s[d];
+                    int below = 0;
+                    if (quota < size) {
+                        const uint32_t mine = prio[p];
 #pragma unroll 8
-                    for (int o = begin; o < begin + size; ++o) {
-                        const uint32_t other = prio[o];
-                        below += (other < mine) | ((other == mine) & (o < p));
+                        for (int o = begin; o < begin + size; ++o) {
+                            const uint32_t other = prio[o];
+                            below += (other < mine) | ((other == mine) & (o < p));
+                        }
+                    }
+                    if (below < quota) atomicOr(keep_bits + (n >> 5), 1u << (n & 31));
+                }
+            } else {
+                // some group is long: the codes (group, priority, place) are sorted, over the hash table's slots
+                uint64_t c[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int p = 2 * tid + e;
+                    c[e] = ~0ull;
+                    if (p < N) {
+                        const int d = entry_s[p];
+                        members[p] = member_s[p];
+                        c[e] = static_cast<uint64_t>(rank[d]) << 43 | static_cast<uint64_t>(prio[p]) << 11 | static_cast<uint64_t>(p - first_s[d]);
                     }
                 }
-                if (below < quota) atomicOr(keep_bits + (n >> 5), 1u << (n & 31));
+                uint32_t none0 = 0, none1 = 0;
+                bitonic_sort_regs<false>(c[0], none0, c[1], none1, table, nullptr, M);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int q = 2 * tid + e;
+                    if (q < N) {
+                        const uint32_t group = by_rank[c[e] >> 43];
+                        const int begin = static_cast<int>(group & 0xFFFFu), n = member_s[begin + static_cast<int>(c[e] & 2047u)];
+                        if (q - begin < static_cast<int>(group >> 16)) atomicOr(keep_bits + (n >> 5), 1u << (n & 31));
+                    }
+                }
             }
             __syncthreads();
             const uint32_t w0 = lane < M / 32 ? keep_bits[lane] : 0u, w1 = lane + 32 < M / 32 ? keep_bits[lane + 32] : 0u;
@@ -610,7 +639,6 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
             if (tid == 0) P.n_sel[s] = total;
             return;
         }
-        __syncthreads();
     }
 
     // ---- the sorting path --------------------------------------------------------------------------------

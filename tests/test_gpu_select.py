@@ -60,16 +60,27 @@ def test_select_group_sizes_around_the_counting_limit():
             check(keys, gs, rate, seed=99, step=4)
 
 
-@pytest.mark.parametrize("N,G", [(64, 64), (65, 63), (255, 182), (256, 183), (512, 256), (513, 257), (1024, 362), (1000, 363), (2048, 512), (1500, 513), (2048, 16), (1100, 9)])
+@pytest.mark.parametrize("N,G", [(64, 64), (65, 63), (255, 182), (256, 183), (512, 256), (513, 159), (513, 257), (862, 160), (1024, 160), (1000, 161), (1024, 362), (1000, 363),
+                                 (1025, 360), (2048, 360), (1500, 361), (2048, 512), (1500, 513), (2048, 16), (1100, 9), (513, 1), (862, 2), (1024, 3), (2048, 1)])
 def test_select_group_counts_around_the_counting_limit(N, G):
-    """Both sides of the largest number of groups whose keys are ranked by counting, and of the longest group (128 members) whose sampling ranks
-    are; one key is all ones, the mark of a free slot of the hash table."""
+    """Up to 512 variates, which are sorted; from 513 on both sides of the largest number of groups whose keys are ranked by counting (160, from 1025
+    variates 360), and groups on both sides of 128 members, beyond which the sampling ranks are sorted; one key is all ones, the mark of a
+    free slot of the hash table."""
     rng = np.random.default_rng(N * 7 + G)
     values = np.unique(rng.integers(1, 1 << 60, 2 * G, dtype=np.uint64))[:G]
     values[G // 2] = np.uint64(0xFFFFFFFFFFFFFFFF)
     keys = values[np.concatenate([np.arange(G), rng.integers(0, G, N - G)])] if N > G else values.copy()
     keys = keys[rng.permutation(N)]
     check(np.stack([keys, keys[::-1]]), 0, 0.3, seed=N + G, step=2)
+
+
+@pytest.mark.parametrize("sizes", [[128] * 5, [129, 128, 128, 128, 1], [300, 213], [1, 1, 1000], [128, 600, 128, 100, 1], [2000, 48], [700, 700, 648]])
+def test_select_group_lengths_around_the_counting_limit(sizes):
+    """From 513 variates: a longest group of 128 members, whose sampling ranks are counted, and longer ones, which are sorted."""
+    keys = np.concatenate([np.full(n, 7919 * (i + 3) % 1000, dtype=np.uint64) for i, n in enumerate(sizes)])
+    keys = keys[np.random.default_rng(len(keys)).permutation(len(keys))]
+    for gs, rate in ((10, 1.0), (0, 0.3), (0, 1.0), (150, 0.9)):
+        check(np.stack([keys, keys[::-1]]), gs, rate, seed=17, step=3)
 
 
 def test_select_long_rows():
