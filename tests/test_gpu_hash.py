@@ -82,6 +82,19 @@ def test_hash_rows_of_one_window_and_large_prime_factors(B, N, L, k, scope, wide
     np.testing.assert_allclose(ga, abar, rtol=2e-5, atol=2e-5 * abar.max())
 
 
+@pytest.mark.parametrize("B,N,L,scope", [(8, 1000, 442, 1), (8, 1000, 391, 0), (8, 1000, 961, 1), (32, 137, 1012, 0), (8, 1000, 130, 1), (1, 200, 1021, 0), (8, 1000, 858, 1), (8, 1000, 715, 1)])
+def test_hash_amplitudes_of_lengths_with_large_prime_factors(B, N, L, scope):
+    """As close to fp64 as the transform in shared memory is, whichever kernel serves the length.  The bound: an amplitude is a sum of L / 2 products
+    taken 16 at a time and then block by block, some sqrt(16 + L / 32) / 2 roundings of 2^-25 of the spectrum, and about as much again from the
+    folded windows and the table: 2^-25 sqrt(48) = 2.1e-7 at L = 1021, where one chain of L / 2 reaches 3.4e-7; the transform needs 1e-7
+    to 1.7e-7."""
+    x = random_periodic(B, N, L, 3, seed=L)
+    _, _, got = run_hash(x, 3, scope=scope)
+    want = np.abs(np.fft.rfft(x.astype(np.float64), axis=-1))[..., 1:(L // 2 + 2) // 2]
+    want = want.mean(axis=0, keepdims=True) if scope == 0 else want
+    assert np.linalg.norm(got - want) <= 2.1e-7 * np.linalg.norm(want)
+
+
 def test_hash_random_configurations():
     """Seeded random draws of (B, N, L, k, scope): the register-blocked transforms (L = 96, 192, 336, 720) with every team
     size, and the generic kernel at window lengths of any factorisation (odd, prime, powers of two)."""
