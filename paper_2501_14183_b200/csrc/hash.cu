@@ -337,6 +337,28 @@ int hash_validate(const vardrop_hash_cfg& c, int* f_lo, int* f_hi) {
     return VARDROP_OK;
 }
 
+HashSplit hash_split(const vardrop_hash_cfg& c) {
+    HashSplit s;
+    s.rows_total = c.scope == 0 ? c.N : c.B * c.N;
+    s.win_per_row = c.scope == 0 ? c.B : 1;
+    // windows per pass: about 2048 complex points per buffer, an even count; three times that where the rows are fewer than two an SM, so that
+    // a row takes one pass (137 rows of 32 windows of 168 steps: 9.3 -> 7.4 us with 512 threads)
+    s.few_rows = s.rows_total < 2 * sm_count();
+    int per_pass = 2 * ((s.few_rows ? 6144 : 2048) / c.L);
+    if (per_pass < 2) per_pass = 2;
+    if (per_pass > 64) per_pass = 64;
+    if (s.win_per_row >= per_pass) {
+        s.rows_per_cta = 1;
+        s.chunk = per_pass;
+    } else {
+        s.chunk = s.win_per_row;
+        s.rows_per_cta = per_pass / s.win_per_row;
+        // keep at least a few CTAs per SM in flight
+        while (s.rows_per_cta > 1 && (s.rows_total + s.rows_per_cta - 1) / s.rows_per_cta < 592) s.rows_per_cta = (s.rows_per_cta + 1) / 2;
+    }
+    return s;
+}
+
 int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32_t* freqs, float* amp_dbg, int* status,
                 cudaStream_t stream) {
     int f_lo, f_hi;
@@ -352,8 +374,10 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     HashParams P{};
     P.x = x; P.keys = keys; P.freqs = freqs; P.amp_dbg = amp_dbg; P.status = status;
     P.B = c.B; P.N = c.N; P.L = c.L; P.k = c.k; P.f_lo = f_lo; P.nf = f_hi - f_lo; P.scope = c.scope;
-    P.rows_total = c.scope == 0 ? c.N : c.B * c.N;
-    P.win_per_row = c.scope == 0 ? c.B : 1;
+    const HashSplit split = hash_split(c);
+    P.rows_total = split.rows_total; P.win_per_row = split.win_per_row;
+    P.rows_per_cta = split.rows_per_cta; P.chunk = split.chunk;
+    const bool few_rows = split.few_rows;
 
     // radix plan: fours first, then a two, then the odd primes; prime factors above 7 come last as plain-sum stages (behind
     // a copy-in stage when there is no small factor to read the windows with)
@@ -371,21 +395,6 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     if (rem > 1 && P.n_stages == 0) push(1);
     for (int p = 11; rem > 1; p += 2) while (rem % p == 0) { push(p); rem /= p; }
 
-    // windows per pass: about 2048 complex points per buffer, an even count; three times that where the rows are fewer than two an SM, so that
-    // a row takes one pass (137 rows of 32 windows of 168 steps: 9.3 -> 7.4 us with 512 threads)
-    const bool few_rows = P.rows_total < 2 * sm_count();
-    int per_pass = 2 * ((few_rows ? 6144 : 2048) / c.L);
-    if (per_pass < 2) per_pass = 2;
-    if (per_pass > 64) per_pass = 64;
-    if (P.win_per_row >= per_pass) {
-        P.rows_per_cta = 1;
-        P.chunk = per_pass;
-    } else {
-        P.chunk = P.win_per_row;
-        P.rows_per_cta = per_pass / P.win_per_row;
-        // keep at least a few CTAs per SM in flight
-        while (P.rows_per_cta > 1 && (P.rows_total + P.rows_per_cta - 1) / P.rows_per_cta < 592) P.rows_per_cta = (P.rows_per_cta + 1) / 2;
-    }
     P.div_L = make_fastdiv(c.L);
     P.div_L4 = make_fastdiv(c.L >= 4 ? c.L / 4 : 1);
     P.div_nf = make_fastdiv(P.nf);

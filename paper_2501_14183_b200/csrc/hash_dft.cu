@@ -312,20 +312,15 @@ int launch_dft(const DftParams& P, cudaStream_t stream) {
 // Returns -1 where the transform in shared memory is the better one (or the sums do not fit).
 int hash_dft_launch(const float* x, const vardrop_hash_cfg& c, int f_lo, int f_hi, uint64_t* keys, int32_t* freqs, float* amp_dbg, int* status,
                     cudaStream_t stream) {
-    int rem = c.L, prime = 1;                    // the largest prime factor
-    for (int p = 2; p * p <= rem; ++p)
-        while (rem % p == 0) { rem /= p; prime = p; }
-    if (rem > 1) prime = rem;
-    // The transform in shared memory spends p multiply-adds a point on a prime factor p > 7, this one nf a point, at a better rate but with more to
-    // set up.  Measured, there | here: 1000 windows of 313 steps 45 | 19 us, 16000 of 130 20 | 11.5, 16000 of 1021 5690 | 310, 50 of 1021 121 | 51;
-    // without such a factor it is the other way round (16000 of 300 23 | 58).
-    const double plain = static_cast<double>(c.B) * c.N * c.L * prime;
-    if (prime <= 7 || plain < 2.0e7 || c.L > 500 + 48 * prime) return -1;
+    int large = 0;                               // sum of the prime factors above 7, which the transform takes as plain sums
+    for (int rem = c.L, p = 2; rem > 1; ++p)
+        while (rem % p == 0) { rem /= p; large += p > 7 ? p : 0; }
+    if (large == 0) return -1;                   // (16000 windows of 300 steps: 23 us there, 58 here)
     DftParams P{};
     P.x = x; P.keys = keys; P.freqs = freqs; P.amp_dbg = amp_dbg; P.status = status;
     P.N = c.N; P.L = c.L; P.k = c.k; P.f_lo = f_lo; P.nf = f_hi - f_lo; P.scope = c.scope;
-    P.rows_total = c.scope == 0 ? c.N : c.B * c.N;
-    P.win_per_row = c.scope == 0 ? c.B : 1;
+    const HashSplit there = hash_split(c);
+    P.rows_total = there.rows_total; P.win_per_row = there.win_per_row;
     const bool narrow = P.nf <= 32;
     P.tiles = (P.nf + (narrow ? 31 : 63)) / (narrow ? 32 : 64);
     // 64 windows a CTA, or 16 where that leaves SMs idle, and then the bin tiles over a cluster as well
@@ -338,6 +333,21 @@ int hash_dft_launch(const float* x, const vardrop_hash_cfg& c, int f_lo, int f_h
     const long long groups = (P.rows_total + P.rows_per_cta - 1) / P.rows_per_cta;
     P.split = 1;
     while (P.split < 8 && P.split < P.tiles && groups * P.split < 2ll * sm_count()) P.split *= 2;
+    // What either costs, in microseconds: rounds of CTAs, each its blocks and rows here (the first of a cluster ranks for all), its complex transforms
+    // there (plain sums over an even length read shared memory with bank conflicts).  The terms are fitted to 1100 measured calls of 33 to 1021 steps,
+    // 100 to 32000 windows and three bands: the choice so made costs about 1 % more than the better of the two.  Where it turns, there | here: 4384 windows of 715 = 5 11 13 steps 41 | 63 us, of 391 = 17 23 37 | 25, of 1021 1642 | 86; 100 of 313 14 | 21, of 1021 107 | 50.
+    auto rounds = [](long long ctas, int at_once) { return static_cast<double>((ctas + at_once - 1) / at_once); };
+    const int passes_there = (there.win_per_row + there.chunk - 1) / there.chunk;
+    const int transforms = there.rows_per_cta > 1 ? (there.rows_per_cta * there.chunk + 1) / 2 : passes_there * ((there.chunk + 1) / 2);
+    const double cost_there = 4.3 + rounds((there.rows_total + there.rows_per_cta - 1) / there.rows_per_cta, sm_count()) * transforms * c.L *
+                                       ((c.L & 1 ? 1.17e-4 : 1.5e-4) * large + 1.1e-3);
+    const int passes = (P.win_per_row + P.chunk - 1) / P.chunk, blocks = ((c.L - 1) / 2 + kStep - 1) / kStep;
+    const double work = static_cast<double>((P.tiles + P.split - 1) / P.split) * passes * blocks;
+    const double cost = W == 16 ? (narrow ? 3.2 + rounds(groups * P.split, 3 * sm_count()) * (1.24 * work + 0.42 * P.rows_per_cta)
+                                          : 4.0 + rounds(groups * P.split, 3 * sm_count()) * (1.32 * work + 0.22 * P.rows_per_cta))
+                                : (narrow ? 4.5 + rounds(groups * P.split, 2 * sm_count()) * (1.24 * work + 0.07 * P.rows_per_cta)
+                                          : 6.1 + rounds(groups * P.split, sm_count()) * (1.365 * work + 0.048 * P.rows_per_cta) + (P.split > 1 ? 0.25 * P.rows_per_cta : 0.0));
+    if (cost >= cost_there) return -1;
     if (W == 64) return narrow ? launch_dft<64, 32>(P, stream) : launch_dft<64, 64>(P, stream);
     return narrow ? launch_dft<16, 32>(P, stream) : launch_dft<16, 64>(P, stream);
 }

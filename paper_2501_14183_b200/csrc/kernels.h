@@ -28,6 +28,13 @@ int hash_validate(const vardrop_hash_cfg& cfg, int* f_lo, int* f_hi);
 int hash_launch(const float* x, const vardrop_hash_cfg& cfg, uint64_t* keys, int32_t* freqs, float* amp_dbg, int* status,
                 cudaStream_t stream);
 
+// how the transform in shared memory shares a call out: windows of a row per pass, rows to a CTA
+struct HashSplit {
+    int rows_total, win_per_row, rows_per_cta, chunk;
+    bool few_rows;
+};
+HashSplit hash_split(const vardrop_hash_cfg& cfg);
+
 // hash_rows.cu: register-blocked plans for selected lookback lengths; -1 = no plan for this configuration
 int hash_rows_launch(const float* x, const vardrop_hash_cfg& cfg, int f_lo, int f_hi, uint64_t* keys, int32_t* freqs, float* amp_dbg,
                      int* status, cudaStream_t stream);
