@@ -95,6 +95,21 @@ def test_hash_amplitudes_of_lengths_with_large_prime_factors(B, N, L, scope):
     assert np.linalg.norm(got - want) <= 2.1e-7 * np.linalg.norm(want)
 
 
+@pytest.mark.parametrize("B,N,L", [(1, 21, 96), (4, 100, 96), (2, 137, 192), (3, 50, 336), (2, 60, 720), (2, 40, 168), (2, 40, 143)])
+def test_hash_per_instance_rows_do_not_disturb_each_other(B, N, L):
+    """Up to about a thousand windows: a variate a hundred thousand times smaller than its neighbours has its own rounding errors only (a few 2^-24 of
+    its spectrum), and one of all zeros has amplitudes of zero, which rank lowest bin first."""
+    x = np.random.default_rng(L).normal(size=(B, N, L)).astype(np.float32)
+    x[:, 1::2] *= 1e5
+    x[:, 4::8] = 0.0
+    _, gf, ga = run_hash(x, 3, scope=1)
+    want = np.abs(np.fft.rfft(x.astype(np.float64), axis=-1))[..., 1:(L // 2 + 2) // 2]
+    live = np.setdiff1d(np.arange(N), np.arange(4, N, 8))
+    err = np.linalg.norm(ga - want, axis=-1) / np.maximum(np.linalg.norm(want, axis=-1), 1e-30)
+    assert err[:, live].max() <= 1e-6
+    assert np.all(ga[:, 4::8] == 0.0) and np.all(gf[:, 4::8] == np.array([1, 2, 3]))
+
+
 def test_hash_random_configurations():
     """Seeded random draws of (B, N, L, k, scope): the register-blocked transforms (L = 96, 192, 336, 720) with every team
     size, and the generic kernel at window lengths of any factorisation (odd, prime, powers of two)."""
