@@ -413,10 +413,13 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     }
     const int grid = (P.rows_total + P.rows_per_cta - 1) / P.rows_per_cta;
     // Threads: a stage is a few hundred butterflies, and a CTA that is mostly idle in its last round keeps others from the SM: 128 instead of 256
-    // where that wastes less (16000 windows of 300 steps 23.1 -> 18.8 us, 4000 of 64 8.4 -> 5.6); 512 for a long pass when CTAs are few.
-    const int butterflies = max_fft * (c.L / P.radix[0]);
-    auto idle = [&](int t) { return (butterflies + t - 1) / t * t; };
-    const int threads = few_rows && butterflies > 256 ? 512 : butterflies <= 128 || 5 * idle(128) < 4 * idle(256) ? 128 : 256;
+    // where that wastes less (16000 windows of 300 steps 23.1 -> 18.8 us, 4000 of 64 8.4 -> 5.6); 512 for a long pass when CTAs are few.  Not with many
+    // rows to a CTA, which its warps rank one after the other (27584 rows of one window of 32 steps: 17.9 us with 256 threads, 27.7 with 128), nor
+    // where the CTAs are few anyway (1920 of 600 steps 10.8 | 13.7; with fewer than one an SM a stage of plain sums has a task for every output).
+    const int tasks = max_fft * (P.radix[P.n_stages - 1] > 7 && grid < sm_count() ? c.L : c.L / P.radix[0]);
+    auto idle = [&](int t) { return (tasks + t - 1) / t * t; };
+    const bool small = tasks <= 128 || (grid >= 8 * sm_count() && 5 * idle(128) < 4 * idle(256));
+    const int threads = few_rows && tasks > 256 ? 512 : small && P.rows_per_cta <= 4 ? 128 : 256;
     cudaError_t err;
     { LaunchScope ls_(K_HASH, stream); err = launch_chained(threads > 256 ? hash_kernel<512> : hash_kernel<256>, dim3(grid), dim3(threads), smem, stream, P); }
     return check_cuda(err, "hash: launch");
