@@ -83,8 +83,8 @@ def test_attention_all_tokens(B, N, H, D):
 @pytest.mark.parametrize("B,N,H,D,Ns", [(1, 512, 2, 64, 200), (1, 513, 2, 64, 200), (1, 512, 2, 64, 256), (1, 512, 1, 64, 384),
                                         (1, 512, 1, 64, 512), (1, 640, 2, 32, 384), (2, 1100, 1, 64, 640)])
 def test_attention_selected_at_path_boundaries(B, N, H, D, Ns):
-    """Both sides of the largest N whose kept rows are gathered by the tile loads themselves (512), kept counts that fill
-    whole tiles exactly (two, three, four tiles on the gathered path; three and five on the staged one), head size 32."""
+    """Kept counts that fill two to five whole tiles exactly, one just past a tile, head size 32: the few-tile kernels, and at 1100 variates (two
+    heads and instances in all) the many-tile ones."""
     check_case(B, N, H, D, pick(N, Ns, seed=N * 3 + Ns), 1.0, seed=N + 11 * Ns)
 
 
@@ -101,7 +101,7 @@ def test_attention_at_the_many_tile_boundary(B, N, H, D, Ns):
 
 
 def test_attention_random_configurations():
-    """Seeded random draws of (B, N, H, D, kept count, value scale): gathered, staged and all-token paths, one to six tiles.
+    """Seeded random draws of (B, N, H, D, kept count, value scale), with a selection (few-tile kernels) and of all tokens, one to six tiles.
     Value scales stay at or below 1: the absolute tolerance is stated for unit-scale tokens (bf16 rounding of P and dS is
     relative, so gradients of larger tokens carry proportionally larger absolute errors)."""
     rng = np.random.default_rng(2025)
@@ -167,9 +167,10 @@ def test_attention_forward_is_deterministic():
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[3], b[3]) and np.array_equal(a[4], b[4])
 
 
-@pytest.mark.parametrize("B,N,H,D,Ns", [(2, 300, 2, 64, 260), (2, 600, 2, 64, 300), (1, 700, 2, 64, None), (2, 321, 2, 64, 97)])
+@pytest.mark.parametrize("B,N,H,D,Ns", [(2, 300, 2, 64, 260), (2, 600, 2, 64, 300), (1, 700, 2, 64, None), (2, 321, 2, 64, 97), (1, 2100, 2, 64, 200),
+                                        (2, 2100, 2, 32, 400)])
 def test_attention_backward_is_reproducible(B, N, H, D, Ns):
-    """Gathered, staged and all-token paths with several tiles: every gradient is bit for bit the same from run to run while
+    """Few tiles, many tiles with a selection and of all tokens: every gradient is bit for bit the same from run to run while
     no (instance, head) pair has more than two key tiles' worth of additions per accumulator row (two fp32 addends commute);
     with more tiles dq may differ in the last bits only.  Guards the shared-memory hand-offs inside the backward kernel."""
     dev, _ = bf16_tokens(B, N, H, D, 1.0, seed=N + (Ns or 0))
@@ -243,7 +244,9 @@ def test_attention_per_instance_selections():
 @pytest.mark.parametrize("B,N,H,D,counts", [
     (20, 140, 8, 64, [60 + 3 * i for i in range(20)][:19] + [140]),            # one instance of two tiles: its CTAs apart from the others
     (24, 260, 8, 32, [100 + (37 * i) % 160 for i in range(24)]),               # many of two and three: every CTA both kinds
-    (3, 200, 1, 64, [129, 1, 128]), (2, 300, 2, 64, [130, 300])])
+    (3, 200, 1, 64, [129, 1, 128]), (2, 300, 2, 64, [130, 300]), (3, 300, 2, 64, [0, 128, 260]),
+    # the many-tile kernels: nothing kept, one row, whole tiles, odd and even tile counts, more items than blocks
+    (5, 2100, 4, 64, [0, 1, 256, 300, 700]), (9, 1030, 3, 32, [5, 130, 257, 384, 640, 128, 900, 1, 129]), (16, 2060, 8, 32, [100 + 37 * i for i in range(16)])])
 def test_attention_instances_of_one_and_of_several_tiles(B, N, H, D, counts):
     dev, ref = bf16_tokens(B, N, H, D, 1.0, seed=B + N)
     q, k, v, d_o = dev
@@ -264,6 +267,11 @@ def test_attention_instances_of_one_and_of_several_tiles(B, N, H, D, counts):
     assert vd.ws_status(ws) == vd.OK
     for b, s_ in enumerate(sels):
         cut = [r[b:b + 1] for r in ref]
+        if len(s_) == 0:
+            assert not dq[b].any() and not dk[b].any() and not dv[b].any()
+            continue
+        wo, _ = oracle.attn_fwd(cut[0], cut[1], cut[2], s_)
+        assert_attn_close(o[b:b + 1, :len(s_)].double().cpu().numpy(), wo, f"o[{b}]")
         wq, wk, wv = oracle.attn_bwd(cut[0], cut[1], cut[2], cut[3][:, :len(s_)], s_)
         for got, want, name in ((dq, wq, "dq"), (dk, wk, "dk"), (dv, wv, "dv")):
             g = got[b:b + 1].double().cpu().numpy()
@@ -319,11 +327,12 @@ def run_strided(q, k, v, d_full, B, N, H, D, sel):
 
 
 @pytest.mark.parametrize("layout", ["fused_qkv", "padded_heads", "padded_tokens", "token_slice"])
-@pytest.mark.parametrize("B,N,H,D,Ns", [(2, 300, 2, 64, 140), (1, 700, 2, 64, 300), (2, 200, 3, 64, None), (1, 600, 2, 64, None), (2, 90, 2, 32, 50)])
+@pytest.mark.parametrize("B,N,H,D,Ns", [(2, 300, 2, 64, 140), (1, 700, 2, 64, 300), (2, 200, 3, 64, None), (1, 600, 2, 64, None), (2, 90, 2, 32, 50),
+                                        (1, 2100, 2, 64, 300), (2, 1100, 3, 32, 140)])
 def test_attention_strided_qkv(layout, B, N, H, D, Ns):
     """q, k, v as views of larger buffers (the element strides of the configuration): slices of a fused [B, N, 3, H, D] projection,
-    heads padded to D + 8, tokens padded by 8 elements (no row view: the library stages), and a slice along N of a longer
-    sequence.  Results must match the oracle run on contiguous copies."""
+    heads padded to D + 8, tokens padded by 8 elements, and a slice along N of a longer sequence; with few tiles, with many (rows laid out
+    from the strided tensors ahead of the backward pass) and of all tokens.  Results must match the oracle run on contiguous copies."""
     dev, ref = bf16_tokens(B, N, H, D, 0.5, seed=N + H)
     gen = torch.Generator(device="cuda").manual_seed(5)
     junk = lambda *shape: (torch.rand(shape, device="cuda", generator=gen) * 8 - 4).to(torch.bfloat16)       # what lies between the rows

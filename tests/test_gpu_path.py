@@ -227,8 +227,8 @@ class Guarded:
 
 @pytest.mark.parametrize("name,N", [("elec", None), ("traffic", None), ("scale", 2304)])
 def test_no_write_outside_any_output_or_workspace(name, N):
-    """Every output and every workspace of a whole step sits between guard margins: gathered, staged and many-tile launch shapes
-    (the Scale shape cut to 2304 variates keeps the three-kernel selection and the four-warpgroup attention kernels in play)."""
+    """Every output and every workspace of a whole step sits between guard margins: few-tile and many-tile launch shapes
+    (the Scale shape cut to 2304 variates keeps the three-kernel selection and the many-tile attention kernels in play)."""
     w = inputs.WORKLOADS[name]
     N = w.N if N is None else N
     B = min(w.B, 4)
