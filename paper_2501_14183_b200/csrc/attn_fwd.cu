@@ -148,15 +148,15 @@ struct FwdParams {
 //                    the next one (done by the softmax warpgroups it was 5000 cycles an item, more than a step and a half of seven)
 //   warps 8-23       four softmax warpgroups, two to a query tile: one thread per row and 64-key half of a step
 // The limit is the special-function unit: 16 exponentials a cycle and SM make 1024 cycles per 128 x 128 scores where the products
-// need 614 (N = 128 scores at 64 cycles, N = 64 P V at 45 with P in tensor memory).  What it takes to get near it:
+// need 512 (N = 128 scores at 64 cycles, N = 64 P V at 32 with P in tensor memory).  What it takes to get near it:
 //   - a softmax thread never waits for a product: it copies its scores to registers and frees their columns at once, so the next
 //     S = Q K^T runs under the exponentials, and P has columns of its own, so P V of the step before does too;
 //   - four warps a scheduler: what surrounds the exponentials of one (tensor-memory loads, maximum, hand-offs: as long as the
 //     exponentials themselves) runs under those of the others (two threads a row share its reference maximum through shared memory);
 //   - little code: a warp's step is some 300 instructions (one thread per row made it 1300, and short items, which run every path
 //     once, then spend their time on instruction fetch).
-// Measured: 8192 variates, B = 8, 1245 us (1528 with one thread per row and the staged form), 862 variates, B = 32, 98 us (120); 1423 kept
-// of 8192 76 us and no gather launch (94 + 20).
+// Measured, events around the launch: 8192 variates, B = 8, 1380 us (1528 with one thread per row and the staged form), 862 variates, B = 32, 104 us
+// (120); 1423 kept of 8192 83 us and no gather launch (94 + 20).  Back to back the last two take 98 and 75.
 // Tensor memory of tile w (256 columns): S 128 | P 64 | O 64.
 constexpr int kFwdTiles = 2;                     // query tiles of an item
 constexpr int kFwdGroupThreads = 128;
