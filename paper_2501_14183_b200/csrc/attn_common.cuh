@@ -28,7 +28,6 @@ inline AttnWs attn_layout(const vardrop_attn_cfg& c) {
     for (size_t& s : w.staged) { s = o; o += align_up(static_cast<size_t>(c.B) * w.Ncap * c.H * kRowBytes, 1024); }
     w.delta = o; o += align_up(sizeof(float) * c.B * c.H * w.Ncap, 1024);
     w.dq_acc = o; o += align_up(static_cast<size_t>(c.B) * w.Ncap * c.H * kDP * sizeof(float), 1024);
-    o += align_up(sizeof(int32_t) * c.B * c.H, 1024);         // reserved
     w.total = o;
     return w;
 }

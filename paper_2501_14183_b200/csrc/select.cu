@@ -32,7 +32,6 @@ struct SelectParams {
     int32_t *group_id, *group_offsets, *members, *n_groups, *sel_idx, *n_sel, *inv_idx;
     // workspace
     int* status;
-    unsigned int* done1;   // [S]
     unsigned int* done2;   // [S]
     int32_t* lt;           // [S, N]
     int32_t* eq;           // [S, N]
@@ -388,7 +387,7 @@ __device__ __forceinline__ int block_scan_pair(int v0, int v1, int* warp_sums, i
 
 // Most groups the counting path takes.  Ranking G keys is G^2 / 32 cycles; the sort does not depend on G.  Counting | sorting, 862 variates: 60 groups
 // 7.2 | 8.8 us, 130 8.0 | 8.6, 160 8.4 | 8.7, 200 10.3 | 8.7; 2048 variates: 100 11.7 | 18.6, 300 15.6 | 17.6, 362 17.5 | 17.6, 420 19.8 | 17.6.  A call
-// with more has paid for the table when it comes to sort: 862 distinct keys 9.4 us instead of 8.3, 2048 18.6 instead of 16.8.
+// with more has paid for the table when it comes to sort: 862 distinct keys 9.7 us instead of 8.1, 2048 19.1 instead of 16.6.
 __host__ __device__ constexpr int small_max_groups(int M) { return M <= 1024 ? 160 : 360; }
 // Longest group whose sampling ranks are counted: 128 positions take some 4000 cycles, the sort of 1024 codes 8000.
 constexpr int kCountMaxGroup = 128, kSortCountMaxGroup = 64;
@@ -573,7 +572,7 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
             uint32_t* by_rank = reinterpret_cast<uint32_t*>(list);       // first position | quota << 16 of a group (the keys are no longer read)
             for (int d = tid; d < G; d += T) {
                 off[rank[d]] = first_s[d];
-                by_rank[rank[d]] = static_cast<uint32_t>(first_s[d]) | static_cast<uint32_t>(quota_s[d]) << 16;
+                if (long_group) by_rank[rank[d]] = static_cast<uint32_t>(first_s[d]) | static_cast<uint32_t>(quota_s[d]) << 16;
             }
             for (int i = G + tid; i <= N; i += T) off[i] = N;
             if (tid == 0) P.n_groups[s] = G;
@@ -748,13 +747,12 @@ __global__ void __launch_bounds__(kSmallMaxN / 2) select_small_kernel(const Sele
 }
 
 struct SelectWs {
-    size_t done1, done2, lt, eq, prio, keep, total, zero_begin, zero_bytes;
+    size_t done2, lt, eq, prio, keep, total, zero_begin, zero_bytes;
 };
 SelectWs select_layout(int S, int N) {
     SelectWs w;
     size_t o = kWsHeaderBytes;
     w.zero_begin = o;
-    w.done1 = o; o += align_up(sizeof(unsigned int) * S, 16);
     w.done2 = o; o += align_up(sizeof(unsigned int) * S, 16);
     w.lt = o;    o += align_up(sizeof(int32_t) * S * N, 16);
     w.eq = o;    o += align_up(sizeof(int32_t) * S * N, 16);
@@ -784,7 +782,6 @@ int select_launch(const uint64_t* keys, const vardrop_select_cfg& c, int32_t* gr
     P.keys = keys; P.group_id = group_id; P.group_offsets = group_offsets; P.members = members; P.n_groups = n_groups;
     P.sel_idx = sel_idx; P.n_sel = n_sel; P.inv_idx = inv_idx;
     P.status = reinterpret_cast<int*>(base);
-    P.done1 = reinterpret_cast<unsigned int*>(base + w.done1);
     P.done2 = reinterpret_cast<unsigned int*>(base + w.done2);
     P.lt = reinterpret_cast<int32_t*>(base + w.lt);
     P.eq = reinterpret_cast<int32_t*>(base + w.eq);
