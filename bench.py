@@ -302,6 +302,8 @@ def kernel_work(w, n_sel, selected=True):
     return {
         "hash_kernel": (w.B * w.N * w.L * 4 + w.N * (8 + 4 * w.k), None),
         "select_small_kernel": (w.N * (8 + 6 * 4), None),
+        "select_place_kernel": (w.N * (2 * 8 + 4), None),
+        "select_cluster_kernel": (w.N * (8 + 6 * 4), None),
         "select_count_kernel": (w.N * (8 + 4 * 4), None),
         "select_group_kernel": (w.N * 6 * 4, None),
         "select_sample_kernel": (w.N * 4 * 4, None),

@@ -49,7 +49,7 @@ std::vector<std::pair<cudaEvent_t, cudaEvent_t>> g_prof_events[K_COUNT];   // pa
 std::vector<std::pair<cudaEvent_t, cudaEvent_t>> g_prof_free;              // pairs ready for reuse
 const char* const g_kernel_names[K_COUNT] = {"hash_kernel", "select_small_kernel", "select_count_kernel", "select_group_kernel", "select_sample_kernel",
                                              "attn_fwd_kernel", "bwd_prep_kernel", "attn_bwd_kernel", "bwd_convert_kernel", "pearson_normalize_kernel",
-                                             "pearson_max_kernel", "gather_rows_kernel"};
+                                             "pearson_max_kernel", "gather_rows_kernel", "select_place_kernel", "select_cluster_kernel"};
 }  // namespace
 
 LaunchScope::LaunchScope(int id, cudaStream_t stream) : id_(id), stream_(stream), stop_(nullptr) {

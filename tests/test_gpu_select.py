@@ -83,6 +83,31 @@ def test_select_group_lengths_around_the_counting_limit(sizes):
         check(np.stack([keys, keys[::-1]]), gs, rate, seed=17, step=3)
 
 
+@pytest.mark.parametrize("N,size", [(60, 60), (64, 64), (65, 65), (500, 64), (862, 60), (1000, 300), (1024, 700), (1025, 64), (1500, 1500), (2000, 60), (3000, 700)])
+def test_select_equal_priorities_rank_by_place(N, size):
+    """Members 13 and 36 of the first group draw the same 32-bit priority under this seed and step (found by search): with the quota
+    between them the earlier one is kept.  Short groups, which count their ranks, and long ones, in every size range."""
+    seed, step = 77, 3689518
+    rank = {60: 21, 64: 23, 65: 23, 300: 113, 700: 256, 1500: 548}[size]       # members of lower priority
+    keys = np.concatenate([np.full(size, 5, dtype=np.uint64), 6 + np.arange(N - size, dtype=np.uint64) // 20])
+    keys = keys[np.random.default_rng(N).permutation(N)]
+    for gs in (rank, rank + 1, rank + 2):
+        check(keys, gs, 1.0, seed=seed, step=step)
+
+
+@pytest.mark.parametrize("N", [2, 63, 64, 65, 128, 129, 256, 257, 512, 513, 1023, 1024, 1025, 1026, 2047, 2048, 2049, 2368, 2369, 4096, 4097, 4736, 4737, 8191, 8192, 8193])
+def test_select_group_shapes_at_the_size_limits(N):
+    """Both sides of the sizes at which a path, its tables or a CTA's share change: few and many groups, some of 64 and 65 members (ranks counted, and
+    found by buckets), long ones that reach over several CTAs' positions, all distinct."""
+    rng = np.random.default_rng(N)
+    for sizes in ([N], [1] * N, [64, 65] * (N // 129) + [N % 129], [N // 2, N // 3, N - N // 2 - N // 3], [9] * (N // 9) + [N % 9]):
+        sizes = [n for n in sizes if n > 0]
+        values = rng.permutation(np.unique(rng.integers(0, 1 << 56, 2 * len(sizes), dtype=np.uint64)))[:len(sizes)]
+        keys = np.repeat(values, sizes)[rng.permutation(N)]
+        check(keys, 0, 0.3, seed=N, step=1)
+        check(np.stack([keys, keys[::-1]]), 40, 1.0, seed=N, step=2)
+
+
 def test_select_long_rows():
     """Rows beyond the one-CTA path: grouping with its working arrays in shared memory (up to 18432 variates), at that
     limit, and on the global arrays beyond it; several rows at once; one group only and all-distinct keys."""
