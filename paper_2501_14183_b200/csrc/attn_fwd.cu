@@ -774,7 +774,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
 // With one or two tiles per head and instance the step is a chain of latencies (kept count, row indices, rows, scores, softmax, P V,
 // rows out), each a few hundred cycles, and every path runs once or twice, at the speed of instruction fetch.  So: no roles and no
 // hand-offs but __syncthreads, rolled loops over 32 scores (the scores stay in tensor memory and are read twice), one stage, 48 KB
-// and 128 columns a CTA, so that four CTAs share an SM and fill each other's waits.
+// and 128 columns a CTA, so that four CTAs share an SM and fill each other's waits.  The next key tile's K comes in under the softmax, its V
+// under the step after (all of 321 variates, B = 32: 30.1 -> 29.1 us a call).
 // B = 32, H = 8, D = 64: 119 kept 7.1 us back to back (10 in the persistent kernel of the first form), 200 kept 15.3 us without a gather
 // launch (19 and a gather of 16).
 // Tensor memory: S 128; P (bf16) over S's columns 0 .. 63 as they are consumed, P V into columns 64 .. 127.
@@ -834,17 +835,20 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
             for (int x = 0; x < kDP / 4; ++x, rows += static_cast<size_t>(kTileFwdThreads / 16) * P.H * (kDP / 4))
                 *rows = make_float4(0.f, 0.f, 0.f, 0.f);                 // 16 consecutive threads clear one 256-byte row
         }
+        // every warp copies its 32 rows of a tile
+        auto load_rows = [&](unsigned char* tile, const __nv_bfloat16* from, int t0) {
+            copy_32_rows(tile + warp * 32 * kRowBytes, from + base, P.sN, idx, t0 * kTile + warp * 32, n_sel, P.D);
+        };
+        load_rows(sQ, P.q, qt);
+        load_rows(sK, P.k, 0);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        load_rows(sV, P.v, 0);
+        asm volatile("cp.async.commit_group;" ::: "memory");
         float o_acc[kDP];                                // more than one key tile: the sum over the tiles before the current one
         float m_run = -INFINITY, l_run = 0.f;
 #pragma unroll 1
         for (int j = 0; j < n_kv; ++j, ++t) {
             const int n_keys = min(kTile, n_sel - j * kTile);
-#pragma unroll 1
-            for (int x = j == 0 ? 0 : 1; x < 3; ++x) {   // Q (once), K, V: every warp copies its 32 rows
-                copy_32_rows(sQ + x * kTileBytes + warp * 32 * kRowBytes, (x == 0 ? P.q : x == 1 ? P.k : P.v) + base, P.sN, idx,
-                             (x == 0 ? qt : j) * kTile + warp * 32, n_sel, P.D);
-                if (x > 0) asm volatile("cp.async.commit_group;" ::: "memory");
-            }
             asm volatile("cp.async.wait_group 1;" ::: "memory");         // Q and K have landed
             fence_proxy_async_smem();
             tc_fence_before();
@@ -862,6 +866,11 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
             }
             ok &= mbar_wait(&bar_s, t & 1);
             tc_fence_after();
+            const bool more = j + 1 < n_kv;
+            if (more) {                                  // K has been read: the next one comes in under the softmax
+                load_rows(sK, P.k, j + 1);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            }
             // ---- row maximum, 32 scores at a time ----
             float m_first = -INFINITY, m_tile = -INFINITY;           // kLag: of the first 64 keys of the tile, of the others
 #pragma unroll 1
@@ -953,7 +962,8 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
             } else {
                 l_run = l_run * alpha + l_sum();
             }
-            asm volatile("cp.async.wait_group 0;" ::: "memory");         // V has landed
+            if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");         // V has landed
+            else asm volatile("cp.async.wait_group 0;" ::: "memory");
             fence_proxy_async_smem();
             tmem_st_wait();
             tc_fence_before();
@@ -971,6 +981,10 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
             }
             ok &= mbar_wait(&bar_o, t & 1);              // (agreed on at the next such barrier: no thread leaves by itself)
             tc_fence_after();
+            if (more) {                                  // and V
+                load_rows(sV, P.v, j + 1);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            }
             if (kLag ? j + 1 < n_kv : n_kv > 1) {
                 if (kLag || j == 0) {
                     tmem_ld32(tm + 64, o_acc);
