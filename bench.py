@@ -309,7 +309,7 @@ def kernel_work(w, n_sel, selected=True):
         "select_sample_kernel": (w.N * 4 * 4, None),
         # (with many key tiles and a selection the forward pass also clears the dQ' accumulator, 64 floats a row and head; without one the prep kernel does)
         "attn_fwd_kernel": (3 * kept * row + kept * row + kept * w.H * 4 + (kept * w.H * 64 * 4 if selected and n_sel > 256 else 0), 4.0 * w.B * w.H * n_sel * n_sel * w.D),
-        "bwd_prep_kernel": ((5 * kept * row + 4 * kept * row if selected else 2 * kept * row + kept * w.H * 64 * 4) + kept * w.H * 4, None),
+        "bwd_prep_kernel": ((3 * kept * row + 2 * kept * row if selected else 2 * kept * row + kept * w.H * 64 * 4) + kept * w.H * 4, None),
         "attn_bwd_kernel": (5 * kept * row + kept * w.H * 4 + grads, 10.0 * w.B * w.H * n_sel * n_sel * w.D),
         "bwd_convert_kernel": (kept * row + kept * w.H * 64 * 4, None),
     }

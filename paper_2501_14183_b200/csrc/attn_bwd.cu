@@ -43,10 +43,10 @@ __device__ __forceinline__ float sum8(float v) {       // over the eight lanes o
 struct PrepParams {
     const uint4* o;         // [B, N, H, D] bf16
     const uint4* d_o;       // [B, N, H, D] bf16
-    const __nv_bfloat16 *q, *k, *v;
+    const __nv_bfloat16* q;
     float* delta;           // [B, H, Ncap]
     float4* dq_acc;         // [B, Ncap, H, 64] fp32; NULL: cleared by the forward pass
-    uint4* staged[4];       // [B, Ncap, H, D] bf16 copies of the kept rows of Q, K, V, and of dO: with a selection
+    uint4* staged[2];       // [B, Ncap, H, D] bf16 copies of the kept rows of Q, and of dO: with a selection
     const int32_t* sel_idx; // [S, N]; NULL: identity, nothing is staged
     const int32_t* n_sel;   // [S] kept counts; NULL: N
     long long sB, sN, sH;
@@ -54,8 +54,9 @@ struct PrepParams {
 };
 
 // One thread per 16-byte chunk of a (token, head) row of 64; the 8 threads of a row reduce Delta by shuffles.  With a selection the rows
-// that the main kernel reads again for every key tile are laid out here once, zeros up to the tile's end (rows of dO past the kept ones
-// may hold anything), so that it takes boxes: row copies by its two loader warps bound it at 1423 kept tokens (250 us against 170).
+// that the main kernel reads again for every pair of key tiles (Q, dO) are laid out here once, zeros up to the tile's end (rows of dO past the
+// kept ones may hold anything), so that it takes boxes: row copies by its two loader warps bound it at 1423 kept tokens (250 us against 170).
+// K and V it reads once, as rows, and under the end of the item before (laid out here too, a step of 8192 variates took 311.8 us instead of 304.6).
 __global__ void __launch_bounds__(256) bwd_prep_kernel(const PrepParams P) {
     chain_wait();
     chain_release();
@@ -70,21 +71,16 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const PrepParams P) {
         const int i = small_div(idx, chunks_row);
         const int c = idx - i * chunks_row;
         const int h = c >> 3, dc = c & 7;
-        uint4 vo = make_uint4(0u, 0u, 0u, 0u), vd = vo, vq = vo, vk = vo, vv = vo;
+        uint4 vo = make_uint4(0u, 0u, 0u, 0u), vd = vo, vq = vo;
         if (i < n_sel && dc < src_chunks_head) {
             const size_t src = (static_cast<size_t>(b) * P.N + i) * (P.H * src_chunks_head) + h * src_chunks_head + dc;
             vo = __ldg(P.o + src);
             vd = __ldg(P.d_o + src);
-            if (sel) {
-                const long long from = b * P.sB + __ldg(sel + i) * P.sN + h * P.sH + dc * 8;
-                vq = __ldg(reinterpret_cast<const uint4*>(P.q + from));
-                vk = __ldg(reinterpret_cast<const uint4*>(P.k + from));
-                vv = __ldg(reinterpret_cast<const uint4*>(P.v + from));
-            }
+            if (sel) vq = __ldg(reinterpret_cast<const uint4*>(P.q + (b * P.sB + __ldg(sel + i) * P.sN + h * P.sH + dc * 8)));
         }
         if (sel && dc < src_chunks_head) {
             const size_t to = ((static_cast<size_t>(b) * P.Ncap + i) * P.H + h) * src_chunks_head + dc;
-            P.staged[0][to] = vq; P.staged[1][to] = vk; P.staged[2][to] = vv; P.staged[3][to] = vd;
+            P.staged[0][to] = vq; P.staged[1][to] = vd;
         }
         const float part = sum8(dot8(vo, vd));
         if (dc == 0) P.delta[(static_cast<size_t>(b) * P.H + h) * P.Ncap + i] = part;
@@ -533,14 +529,15 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         if (tid == 0) set_status(P.status, VARDROP_ERR_CUDA);
         return;
     }
-    const bool boxes = kMany || P.sel_idx == nullptr;
+    const bool boxes = kMany || P.sel_idx == nullptr;          // Q and dO come as boxes, or as rows
+    const bool kv_rows = P.sel_idx != nullptr;                 // K and V, which an item reads once, as rows wherever there is a selection
     if (warp == 0) {
         tmem_alloc(tmem_slot, kBwdTmemCols);
         tmem_relinquish();
     }
     if (tid == 0) {
         for (int w = 0; w < 2; ++w) {
-            mbar_init(bar_kv_full + w, boxes ? 1 : kBwdGroup);      // a box: one announcing arrival; row copies: every thread of the team
+            mbar_init(bar_kv_full + w, kv_rows ? kBwdGroup : 1);    // a box: one announcing arrival; row copies: every thread of the team
             mbar_init(bar_q_full + w, boxes ? 1 : 66);              // row copies: every loader lane, and one of each loader for the statistics
             mbar_init(bar_q_free + w, 2);
             mbar_init(bar_x + w, 1);
@@ -562,8 +559,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         mbar_fence_init();
         if (boxes) {
             tma_prefetch_desc(&map_q);
-            tma_prefetch_desc(&map_k);
-            tma_prefetch_desc(&map_v);
+            if (!kv_rows) {
+                tma_prefetch_desc(&map_k);
+                tma_prefetch_desc(&map_v);
+            }
             tma_prefetch_desc(&map_do);
         }
         tma_prefetch_desc(&map_acc);
@@ -680,6 +679,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 continue;
             }
             ok &= warp_wait_relaxed(bar_kv_full + w, ai & 1);
+            if (kMany && kv_rows) fence_proxy_async_smem();      // (otherwise with the slot's rows)
             auto wait_slot = [&](uint32_t tt) {
                 ok &= warp_wait_relaxed(bar_q_full + (tt & 1), (tt >> 1) & 1);
                 if (!boxes) fence_proxy_async_smem();    // rows written by asynchronous copies are read by the tensor core
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                         tma_load_4d(sQ + slot * 2 * kTileBytes + kTileBytes, &map_do, bar_q_full + slot, 0, it.h, x * kTile, it.b);
                     }
                     __syncwarp();
-                    if (x == 0) {                        // the first query tile comes in under the item before; K and V replace that one's
+                    if (x == 0 && !kv_rows) {            // the first query tile comes in under the item before; K and V replace that one's
                         ok = warp_wait_relaxed(bar_kv_free, (i & 1) ^ 1);
                         if (!ok) break;
                         if (lane == 0) {
@@ -1020,6 +1020,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         unsigned char* panels = sdS + 2 * w * kTileBytes;
         const uint64_t scale2 = pair_of(P.scale_log2, P.scale_log2);
         uint32_t t = 0, u = 0, n_conv = 0;               // query tiles, steps of this team, items with an accumulated dQ' so far
+        auto load_kv = [&](const Item& it) {             // this team's K and V rows, 32 a warp
+            const int x = (warp >> 2) & 1, g = (warp & 3) * 32;
+            copy_32_rows(sKV + (2 * w + x) * kTileBytes + g * kRowBytes, (x == 0 ? P.k : P.v) + it.b * P.sB + it.h * P.sH, P.sN,
+                         P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N, key0_of(it, w) + g, it.n_sel, P.D);
+            cp_async_arrive(bar_kv_full + w);
+        };
+        bool loaded = false;                             // many: this item's were asked for under the end of the item before
         item_wait(0);
         ok = group_sync_and(id, ok);
 #pragma unroll 1
@@ -1027,7 +1034,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             const Item it = item_read(i);
             if (it.n_sel < 0) break;
             const int n_q = (it.n_sel + kTile - 1) / kTile, key0 = key0_of(it, w);
-            if (!boxes && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
+            if (kv_rows && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
             // dQ' of an (instance, head) of more than two tiles: both teams of the CTA that brought its last part
             auto convert_dq = [&]() {
                 if (kMany || n_q <= per_item) return;
@@ -1061,20 +1068,17 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 }
             };
             if (key0 >= it.n_sel) {                      // no key tile: nothing else ties this team to the others' pace, and it waits by parity
-                if (boxes && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
+                if (!kv_rows && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
                 item_wait(i + 1);
                 ok = group_sync_and(id, ok);
                 if (gt == 0) mbar_arrive(bar_skip + w);
+                if (kMany) loaded = false;
                 t += n_q;
                 convert_dq();
                 continue;
             }
             const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
-            if (!boxes) {                                // this team's K and V rows, 32 a warp
-                const int x = (warp >> 2) & 1, g = (warp & 3) * 32;
-                copy_32_rows(sKV + (2 * w + x) * kTileBytes + g * kRowBytes, (x == 0 ? P.k : P.v) + it.b * P.sB + it.h * P.sH, P.sN, sel, key0 + g, it.n_sel, P.D);
-                cp_async_arrive(bar_kv_full + w);
-            }
+            if (kv_rows && !(kMany && loaded)) load_kv(it);
             const bool key_valid = key0 + row < it.n_sel;
             // After an item it had no key tile in, a team may be two phases ahead of a query slot's barrier, which would let it through: its own
             // scores come after the phase it wants.
@@ -1139,6 +1143,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             ok &= warp_wait(bar_dk + w, (u - 1) & 1);
             ok &= warp_wait(bar_g, (t - 1) & 1);
             tc_fence_after();
+            if (kMany && kv_rows) {                      // every product that reads this team's K and V is done: the next item's come in under what follows
+                item_wait(i + 1);
+                const Item next = item_read(i + 1);
+                loaded = __all_sync(0xffffffffu, ok && next.n_sel >= 0 && key0_of(next, w) < next.n_sel);
+                if (loaded) load_kv(next);
+            }
 #pragma unroll 1
             for (int e = 0; e < 2; ++e) stage_acc(panels + e * kTileBytes, tm + (e == 0 ? kColDv : kColDk), e == 0 ? 1.f : P.scale, row, half);
             tc_fence_before();
@@ -1233,8 +1243,8 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
         R.o = static_cast<const uint4*>(o); R.d_o = static_cast<const uint4*>(d_o);
         R.delta = reinterpret_cast<float*>(base + w.delta);
         R.dq_acc = attn_fwd_clears(c, sel_idx) ? nullptr : reinterpret_cast<float4*>(base + w.dq_acc);
-        R.q = static_cast<const __nv_bfloat16*>(q); R.k = static_cast<const __nv_bfloat16*>(k); R.v = static_cast<const __nv_bfloat16*>(v);
-        for (int i = 0; i < 4; ++i) R.staged[i] = reinterpret_cast<uint4*>(base + w.staged[i]);
+        R.q = static_cast<const __nv_bfloat16*>(q);
+        for (int i = 0; i < 2; ++i) R.staged[i] = reinterpret_cast<uint4*>(base + w.staged[i]);
         R.sel_idx = sel_idx;
         R.sB = L.sB; R.sN = L.sN; R.sH = L.sH;
         R.n_sel = sel_idx ? n_sel : nullptr;
@@ -1250,8 +1260,8 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
 
     CUtensorMap mq{}, mk{}, mv{}, mdo{}, macc;
     if (many && sel_idx) {
-        CUtensorMap* const maps[4] = {&mq, &mk, &mv, &mdo};
-        for (int i = 0; i < 4; ++i)
+        CUtensorMap* const maps[2] = {&mq, &mdo};
+        for (int i = 0; i < 2; ++i)
             if (int st = make_tile_map(maps[i], base + w.staged[i], c.D, c.B, w.Ncap, c.H, w.Ncap * HD, HD, c.D)) return st;
     } else if (!sel_idx) {
         if (int st = make_tile_map(&mq, q, c.D, c.B, c.N, c.H, L.sB, L.sN, L.sH)) return st;

@@ -14,7 +14,7 @@ constexpr int kRowBytes = kDP * 2;  // one (token, head) row of bf16: 128 bytes 
 constexpr int kTileBytes = kTile * kRowBytes;   // 16 KiB
 
 struct AttnWs {
-    size_t staged[4];         // [B, Ncap, H, D] bf16 copies of the kept rows of Q, K, V and of dO (selections of many tiles)
+    size_t staged[2];         // [B, Ncap, H, D] bf16 copies of the kept rows of Q and of dO (selections of many tiles)
     size_t delta;             // [B, H, Ncap] fp32; few tiles: [B, H] int32 counters instead
     size_t dq_acc;            // [B, Ncap, H, 64] fp32
     size_t total;
