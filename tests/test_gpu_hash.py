@@ -82,6 +82,16 @@ def test_hash_rows_of_one_window_and_large_prime_factors(B, N, L, k, scope, wide
     np.testing.assert_allclose(ga, abar, rtol=2e-5, atol=2e-5 * abar.max())
 
 
+@pytest.mark.parametrize("L", [6, 8, 9, 10, 18, 24, 36, 45, 48, 54, 60, 64, 70, 72, 81, 90, 100, 128, 144, 162, 250, 256, 270, 300, 360, 432, 500, 512, 539, 630, 726, 875, 960, 1000, 1024, 4000])
+def test_hash_amplitudes_of_every_radix(L):
+    """Plans of the transform in shared memory with each radix (2 to 10) as first, middle and last stage.  The bound: a stage rounds each value a few times
+    at 2^-25, at most five stages to a length: 2^-24 of the spectrum per stage of four roundings, and a little for the table and the sum."""
+    x = random_periodic(3, 5, L, 1, seed=L) + np.random.default_rng(L).normal(0, 1, size=(3, 5, L)).astype(np.float32)
+    _, _, got = run_hash(x, 1, 0, L // 2 + 1)
+    want = np.abs(np.fft.rfft(x.astype(np.float64), axis=-1)).mean(axis=0, keepdims=True)
+    assert np.linalg.norm(got.reshape(want.shape) - want) <= 3e-7 * np.linalg.norm(want)
+
+
 @pytest.mark.parametrize("B,N,L,scope", [(8, 1000, 442, 1), (8, 1000, 391, 0), (8, 1000, 961, 1), (32, 137, 1012, 0), (8, 1000, 130, 1), (1, 200, 1021, 0), (8, 1000, 858, 1), (8, 1000, 715, 1)])
 def test_hash_amplitudes_of_lengths_with_large_prime_factors(B, N, L, scope):
     """As close to fp64 as the transform in shared memory is, whichever kernel serves the length.  The bound: an amplitude is a sum of L / 2 products
