@@ -166,7 +166,7 @@ int vardrop_select(const uint64_t* keys, const vardrop_select_cfg* cfg, int32_t*
  * Same arguments, outputs and results as vardrop_select, minus ws / ws_bytes.
  * Limit: S * N <= 16384; larger problems return VARDROP_ERR_UNSUPPORTED (use vardrop_select).
  * It never calls cudaMalloc, cudaFree or any allocating routine.  For N <= 2048 it issues one kernel launch
- * and the built-in array is not touched; for larger N it issues one cudaMemsetAsync and three kernel
+ * and the built-in array is not touched; up to 8192 it issues two, for larger N one cudaMemsetAsync and three kernel
  * launches on `stream`, all working in that array.
  * The first call on each device looks up the array's device address (cudaGetSymbolAddress, with that
  * device current) and caches it; make that first call outside any stream capture.

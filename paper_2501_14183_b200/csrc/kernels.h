@@ -48,7 +48,7 @@ int sm_count();       // multiprocessors of the current device
 size_t select_workspace_bytes(const vardrop_select_cfg& cfg);
 int select_validate(const vardrop_select_cfg& cfg);
 int select_launch(const uint64_t* keys, const vardrop_select_cfg& cfg, int32_t* group_id, int32_t* group_offsets, int32_t* members,
-                  int32_t* n_groups, int32_t* sel_idx, int32_t* n_sel, int32_t* inv_idx, void* ws, cudaStream_t stream);
+                  int32_t* n_groups, int32_t* sel_idx, int32_t* n_sel, int32_t* inv_idx, void* ws, cudaStream_t stream, bool one_cta = false);
 
 // allocation-free variant: scratch is a fixed array inside the module
 constexpr int kStaticMaxRows = 16384;                 // largest S * N it accepts

@@ -1121,7 +1121,7 @@ int select_validate(const vardrop_select_cfg& c) {
 size_t select_workspace_bytes(const vardrop_select_cfg& c) { return select_layout(c.S, c.N).total; }
 
 int select_launch(const uint64_t* keys, const vardrop_select_cfg& c, int32_t* group_id, int32_t* group_offsets, int32_t* members,
-                  int32_t* n_groups, int32_t* sel_idx, int32_t* n_sel, int32_t* inv_idx, void* ws, cudaStream_t stream) {
+                  int32_t* n_groups, int32_t* sel_idx, int32_t* n_sel, int32_t* inv_idx, void* ws, cudaStream_t stream, bool one_cta) {
     const SelectWs w = select_layout(c.S, c.N);
     char* base = static_cast<char*>(ws);
     SelectParams P{};
@@ -1141,7 +1141,8 @@ int select_launch(const uint64_t* keys, const vardrop_select_cfg& c, int32_t* gr
     P.step = c.step;
     // From 1025 variates two launches over more SMs are faster than one CTA a row until the rows' pairs of keys are many.  2000 variates in
     // 160 | 600 groups, two launches 11.2 | 11.5 us for one row, 16.5 | 16.1 for four, 20 | 20 for eight, 42 | 41 for 32; one CTA a row 10 | 27 throughout.
-    const bool small = c.N <= 1024 || (c.N <= kSmallMaxN && static_cast<double>(c.N) * c.N * c.S > kSmallPairs);
+    // (one_cta: the caller's scratch is shared by calls that may overlap, and may not be touched up to 2048 variates.)
+    const bool small = c.N <= 1024 || (c.N <= kSmallMaxN && (one_cta || static_cast<double>(c.N) * c.N * c.S > kSmallPairs));
     if (small) {
         auto launch = [&](auto m) {
             constexpr int kM = decltype(m)::value;
@@ -1256,7 +1257,7 @@ int select_static_launch(const uint64_t* keys, const vardrop_select_cfg& c, int3
         }
         ptr = dev_ptr[dev];
     }
-    return select_launch(keys, c, group_id, group_offsets, members, n_groups, sel_idx, n_sel, inv_idx, ptr, stream);
+    return select_launch(keys, c, group_id, group_offsets, members, n_groups, sel_idx, n_sel, inv_idx, ptr, stream, true);
 }
 
 }  // namespace vardrop

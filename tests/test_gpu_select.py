@@ -51,7 +51,7 @@ def test_select_degenerate_groups():
 
 
 def test_select_group_sizes_around_the_counting_limit():
-    """The one-CTA path ranks members by counting inside groups of up to 64 and sorts when some group is longer: both sides of it."""
+    """Members are ranked by counting inside groups of up to 64 and by buckets of their priorities in longer ones: both sides of it."""
     rng = np.random.default_rng(11)
     for sizes in ([64, 64, 64], [65, 64, 64], [64, 1, 63, 2], [300, 5, 5, 5], [1] * 40 + [64]):
         keys = np.concatenate([np.full(n, 100 + 7 * i, dtype=np.uint64) for i, n in enumerate(sizes)])
@@ -63,9 +63,9 @@ def test_select_group_sizes_around_the_counting_limit():
 @pytest.mark.parametrize("N,G", [(64, 64), (65, 63), (255, 182), (256, 183), (512, 256), (513, 159), (513, 257), (862, 160), (1024, 160), (1000, 161), (1024, 362), (1000, 363),
                                  (1025, 360), (2048, 360), (1500, 361), (2048, 512), (1500, 513), (2048, 16), (1100, 9), (513, 1), (862, 2), (1024, 3), (2048, 1)])
 def test_select_group_counts_around_the_counting_limit(N, G):
-    """Up to 512 variates, which are sorted; from 513 on both sides of the largest number of groups whose keys are ranked by counting (160, from 1025
-    variates 360), and groups on both sides of 128 members, beyond which the sampling ranks are sorted; one key is all ones, the mark of a
-    free slot of the hash table."""
+    """Few and many distinct keys in every size range: up to 512 variates all of them have entries in the hash table, up to 1024 as long as they are
+    no more than 512 (then they are sorted), above that all pairs are compared; one key is all ones, the mark of a free slot of the table and
+    not a number where keys are compared as doubles."""
     rng = np.random.default_rng(N * 7 + G)
     values = np.unique(rng.integers(1, 1 << 60, 2 * G, dtype=np.uint64))[:G]
     values[G // 2] = np.uint64(0xFFFFFFFFFFFFFFFF)
@@ -76,7 +76,7 @@ def test_select_group_counts_around_the_counting_limit(N, G):
 
 @pytest.mark.parametrize("sizes", [[128] * 5, [129, 128, 128, 128, 1], [300, 213], [1, 1, 1000], [128, 600, 128, 100, 1], [2000, 48], [700, 700, 648]])
 def test_select_group_lengths_around_the_counting_limit(sizes):
-    """From 513 variates: a longest group of 128 members, whose sampling ranks are counted, and longer ones, which are sorted."""
+    """Long groups, whose sampling ranks come from buckets of their priorities, alone and among others, on one CTA and over several."""
     keys = np.concatenate([np.full(n, 7919 * (i + 3) % 1000, dtype=np.uint64) for i, n in enumerate(sizes)])
     keys = keys[np.random.default_rng(len(keys)).permutation(len(keys))]
     for gs, rate in ((10, 1.0), (0, 0.3), (0, 1.0), (150, 0.9)):
@@ -108,8 +108,18 @@ def test_select_group_shapes_at_the_size_limits(N):
         check(np.stack([keys, keys[::-1]]), 40, 1.0, seed=N, step=2)
 
 
+@pytest.mark.parametrize("S,N,G", [(18, 1025, 100), (9, 1500, 360), (8, 2048, 361), (6, 2000, 3), (6, 2048, 2048), (8, 2047, 200), (5, 2048, 1), (5, 2048, 31)])
+def test_select_many_rows_of_1025_to_2048(S, N, G):
+    """With this many rows one CTA a row takes them, two variates a thread: few and many distinct keys, more than the table takes, long groups."""
+    rng = np.random.default_rng(N + G)
+    values = rng.permutation(np.unique(rng.integers(0, 1 << 60, 2 * G, dtype=np.uint64)))[:G]
+    rows = np.stack([values[np.concatenate([np.arange(G), rng.integers(0, G, N - G)])][rng.permutation(N)] for _ in range(S)])
+    check(rows, 0, 0.3, seed=N, step=1)
+    check(rows, 12, 1.0, seed=G, step=2)
+
+
 def test_select_long_rows():
-    """Rows beyond the one-CTA path: grouping with its working arrays in shared memory (up to 18432 variates), at that
+    """Rows beyond the cluster's: grouping with its working arrays in shared memory (up to 18432 variates), at that
     limit, and on the global arrays beyond it; several rows at once; one group only and all-distinct keys."""
     for N, G in ((18432, 700), (18433, 50), (24000, 3000)):
         check(inputs.make_keys(N, G, k=4, f_hi=169, seed=N), 10, 1.0, seed=42, step=2)
@@ -125,7 +135,7 @@ def test_select_long_rows():
 
 
 def test_select_middle_rows():
-    """Rows of 2049 .. 8192 variates: ragged sizes, keys that differ in all 64 bits or in a single one, one group, two groups
+    """Rows of 2049 .. 8192 variates (all pairs and a cluster): ragged sizes, keys that differ in all 64 bits or in a single one, one group, two groups
     of very different size, many equal groups of 512, 20 and 2 members, several rows at once."""
     rng = np.random.default_rng(5)
     wide = rng.integers(0, 2**63, size=5000, dtype=np.uint64) * np.uint64(2) + rng.integers(0, 2, size=5000, dtype=np.uint64)
@@ -149,7 +159,7 @@ def test_select_middle_rows():
 
 def test_select_random_configurations():
     """Seeded random draws of (N, rows, groups, gs, rate, k) on both sides of every size limit of the kernels
-    (2048: one-CTA path; 18432: grouping in shared memory; 65536: the largest N)."""
+    (1024: one-CTA path; 8192: all pairs and a cluster; 18432: grouping in shared memory; 65536: the largest N)."""
     rng = np.random.default_rng(123)
     for it in range(24):
         N = int(rng.choice([63, 64, 65, 700, 2047, 2048, 2049, 4096, 8192, 18432, 18433, 30000, 65536]))

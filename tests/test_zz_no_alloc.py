@@ -81,3 +81,19 @@ def test_static_variant_rejects_sizes_beyond_its_scratch():
     torch.cuda.synchronize()
     for name in NAMES:
         assert torch.equal(out[name], want[name]), name
+
+
+@pytest.mark.parametrize("N,G", [(1025, 60), (2048, 300), (2048, 700)])
+def test_static_variant_leaves_its_scratch_alone_up_to_2048_variates(N, G):
+    """One launch, which works in shared memory: calls on different streams may overlap (with a workspace of its own a call of this size takes two)."""
+    kt = torch.from_numpy(inputs.make_keys(N, G, k=4, f_hi=85, seed=N).reshape(1, -1).view(np.int64)).cuda()
+    cfg = vd.SelectCfg(1, N, 0, 0.2, 11, 1)
+    out = vd.alloc_select_outputs(cfg)
+    before = vd.vardrop_launch_count()
+    without_workspace(kt, cfg, out)
+    assert vd.vardrop_launch_count() == before + 1
+    want = with_workspace(kt, cfg)
+    assert vd.vardrop_launch_count() == before + 3
+    torch.cuda.synchronize()
+    for name in NAMES:
+        assert torch.equal(out[name], want[name]), name
