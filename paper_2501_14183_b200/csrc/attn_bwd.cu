@@ -485,7 +485,9 @@ constexpr int kTeamWarps = 8;
 // dropped ones: every warp then helps with what is left.  B = 32, H = 8, 2049 variates, 102 kept 116 -> 71 us, forward and backward, 204 kept 140 -> 97;
 // 4096, 204 kept, B = 8 73 -> 48.  Where the items take longer the code alone costs something: 8192, 1423 kept 254 -> 262.
 constexpr int kHelpZerosN = 6144;
-template <bool kMany, bool kMixed, bool kHelp>
+// kKvRows: many tiles, with a selection: K and V come as rows.  (Decided when the kernel runs, the same code without one was 1 to 3 % slower: 862 tokens,
+// B = 6, 105.1 -> 107.2 us forward and backward.)
+template <bool kMany, bool kMixed, bool kHelp, bool kKvRows>
 __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                                                                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
                                                                   const __grid_constant__ CUtensorMap map_acc, const BwdParams P) {
@@ -532,7 +534,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         return;
     }
     const bool boxes = kMany || P.sel_idx == nullptr;          // Q and dO come as boxes, or as rows
-    const bool kv_rows = P.sel_idx != nullptr;                 // K and V, which an item reads once, as rows wherever there is a selection
+    const bool kv_rows = kMany ? kKvRows : P.sel_idx != nullptr;       // K and V, which an item reads once, as rows wherever there is a selection
     if (warp == 0) {
         tmem_alloc(tmem_slot, kBwdTmemCols);
         tmem_relinquish();
@@ -1302,11 +1304,13 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
         LaunchScope ls_(K_ATTN_BWD, stream);
         return check_cuda(launch_chained(kernel, dim3(grid), dim3(kBwdThreads), kBwdSmemBytes, stream, mq, mk, mv, mdo, macc, P), "attention: backward launch");
     };
-    static thread_local int attr_few = -1, attr_mixed = -1, attr_many = -1, attr_help = -1;
+    static thread_local int attr_few = -1, attr_mixed = -1, attr_many = -1, attr_rows = -1, attr_help = -1;
     const bool help = sel_idx && c.N <= kHelpZerosN;
-    if (int st = many                  ? (help ? launch(attn_bwd_kernel<true, false, true>, attr_help) : launch(attn_bwd_kernel<true, false, false>, attr_many))
-                 : sel_idx && P.S > 1 ? launch(attn_bwd_kernel<false, true, false>, attr_mixed)
-                                      : launch(attn_bwd_kernel<false, false, false>, attr_few))
+    if (int st = many                  ? (help      ? launch(attn_bwd_kernel<true, false, true, true>, attr_help)
+                                         : sel_idx ? launch(attn_bwd_kernel<true, false, false, true>, attr_rows)
+                                                   : launch(attn_bwd_kernel<true, false, false, false>, attr_many))
+                 : sel_idx && P.S > 1 ? launch(attn_bwd_kernel<false, true, false, false>, attr_mixed)
+                                      : launch(attn_bwd_kernel<false, false, false, false>, attr_few))
         return st;
     if (many) {
         ConvertParams F{};
