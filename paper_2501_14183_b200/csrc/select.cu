@@ -848,7 +848,8 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
 //                         of one to seven microseconds for the whole GPU, and nothing has to be cleared or exchanged
 // select_cluster_kernel   a cluster of eight CTAs per hash row, each with an eighth of the positions (n_loc, a multiple of 32), a thread to a
 //                         position: group heads, ids, priorities, sampling ranks, compaction
-// What bounds the second is latency: a few short steps and three barriers of the cluster.  One CTA with several variates a thread is bound by its
+// What bounds the second is latency: a few short steps and three barriers of the cluster (a fourth, that says that all of its CTAs run, is
+// arrived at where the kernel begins and waited for behind the keys' loads).  One CTA with several variates a thread is bound by its
 // instruction rate (2000 variates in 100 groups 9.4 us, in 500 27; so 11 in either), sorting an eighth of the keys in every CTA of the cluster and
 // searching the eight lists took 31 us for 8192.  In a training step: 8192 variates 43.8 us by the three launches below and their clear -> 20.8; 3000
 // 22.5 -> 11.5; 1200 12.9 (one CTA) -> 8.3.
@@ -940,8 +941,11 @@ __global__ void __launch_bounds__(kPlaceThreads) select_place_kernel(const Selec
     }
 }
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 // address of this CTA's shared variable `p` in CTA `cta` of the cluster
 __device__ __forceinline__ uint32_t peer_addr(const void* p, int cta) {
@@ -966,6 +970,7 @@ __global__ void __launch_bounds__(M) select_cluster_kernel(const SelectParams P,
     const int r = blockIdx.x, s = blockIdx.y, N = P.N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int lo = r * n_loc, cnt = max(0, min(n_loc, N - lo)), p = lo + tid;
     const bool mine = tid < cnt;
+    cluster_arrive();                                          // this CTA runs: its shared memory may be written (the others wait for it ahead of their first store)
     kept[tid] = 0;
 #pragma unroll 1
     for (int i = tid; i < kMaxLong * kBuckets; i += M) long_groups.hist[i] = 0;
@@ -997,6 +1002,7 @@ __global__ void __launch_bounds__(M) select_cluster_kernel(const SelectParams P,
     int heads = 0;
     const int heads_before = warp_prefix(&heads);
     const uint32_t with_heads = __ballot_sync(0xffffffffu, lane < kWarps && bits[lane < kWarps ? lane : 0] != 0u);       // warps that hold a head
+    cluster_wait();                                            // every CTA of the cluster runs (the launch chain and the keys' loads hide it)
     if (tid < kClusterCtas) {
         int first = N, last = -1;                              // the CTA's first and last head
         if (with_heads) {

@@ -70,3 +70,32 @@ def test_host_side_validation_needs_no_gpu(lib):
     assert st == vd.ERR_INVALID_ARG and b"x is NULL" in lib.vardrop_last_error()
     st = lib.vardrop_attn_fwd(None, None, None, None, None, C.byref(vd.AttnCfg(1, 8, 1, 48, 0.0)), None, None, None, 0, None)
     assert st == vd.ERR_UNSUPPORTED
+
+
+def kernel_bodies():
+    """(file, name, text without comments) of every __global__ function."""
+    csrc = os.path.join(ROOT, "paper_2501_14183_b200", "csrc")
+    for fn in sorted(os.listdir(csrc)):
+        if not fn.endswith(".cu"):
+            continue
+        text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(os.path.join(csrc, fn)).read(), flags=re.S)
+        for m in re.finditer(r"__global__[^;{]*?\b(\w+_kernel)\s*\([^{;]*\)\s*\{", text):
+            depth, end = 1, m.end()
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[end], 0)
+                end += 1
+            yield fn, m.group(1), text[m.end():end]
+
+
+def test_peers_shared_memory_is_reached_behind_a_cluster_barrier():
+    """A CTA's shared memory may only be reached from another one of its cluster once it runs, which nothing but a barrier of the cluster says: in the
+    text of a kernel one is waited for ahead of the first remote access."""
+    seen = []
+    for fn, name, body in kernel_bodies():
+        remote = re.search(r"\bpeer_(addr|store\d)\s*\(|\bfirst_cta_addr\s*\(|(ld|st|red|atom)\.shared::cluster", body)
+        if not remote:
+            continue
+        seen.append(name)
+        barrier = re.search(r"\bcluster_(sync|wait)\s*\(\)", body)
+        assert barrier and barrier.start() < remote.start(), f"{fn}: {name}"
+    assert set(seen) == {"select_cluster_kernel", "hash_dft_kernel"}
