@@ -5,17 +5,16 @@
 // per-instance scope) and all the windows that feed them, so the mean over the batch never leaves the SM
 // and is summed in ascending instance order.  Two real windows ride one complex transform
 // (z = x1 + i x2; X1_f = (Z_f + conj Z_{L-f}) / 2, X2_f = (Z_f - conj Z_{L-f}) / 2i), which is evaluated by
-// a Stockham autosort mixed-radix FFT (radices 4, 2, 3, 5, 7; larger prime factors as plain sums) whose butterflies are spread over the
-// whole CTA.  Twiddles are produced once per CTA with sincospif on an angle reduced to half a turn with integers.
+// a Stockham autosort mixed-radix FFT (radices of up to 10 made of 2, 3, 5 and 7; larger prime factors as plain sums) whose butterflies
+// are spread over the whole CTA.  Twiddles are produced once per CTA with sincospif on an angle reduced to half a turn with integers.
 #include "common.cuh"
 #include "dft_codelets.cuh"
+#include "hash_plan.h"
 #include "kernels.h"
 
 namespace vardrop {
 
 namespace {
-
-constexpr int kMaxStages = 16;
 
 struct HashParams {
     const float* x;
@@ -156,7 +155,30 @@ __device__ __forceinline__ void fft_first_stage(const HashParams& P, float2* __r
     }
 }
 
-template <int kMaxThreads>       // 512 or 256: the bound that costs the shorter passes no registers
+// f(Int<radix>{}) for a radix that has a codelet, f(Int<1>{}) for any other.
+template <bool kWide, class F>
+__device__ __forceinline__ void with_radix(int radix, F f) {
+    switch (radix) {
+        case 2: return f(Int<2>{});
+        case 3: return f(Int<3>{});
+        case 4: return f(Int<4>{});
+        case 5: return f(Int<5>{});
+        case 7: return f(Int<7>{});
+    }
+    if constexpr (kWide) {
+        switch (radix) {
+            case 6: return f(Int<6>{});
+            case 8: return f(Int<8>{});
+            case 9: return f(Int<9>{});
+            case 10: return f(Int<10>{});
+        }
+    }
+    f(Int<1>{});
+}
+
+// kMaxThreads: 512 or 256, the bound that costs the shorter passes no registers.
+// kWide: with radices 6 and 8 to 10, which take 56 registers instead of 48 (with 256 threads four CTAs an SM instead of five).
+template <int kMaxThreads, bool kWide>
 __global__ void __launch_bounds__(kMaxThreads) hash_kernel(const HashParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int L = P.L, nf = P.nf;
@@ -187,32 +209,14 @@ __global__ void __launch_bounds__(kMaxThreads) hash_kernel(const HashParams P) {
         // ---- mixed-radix Stockham FFT, ping-pong between the two buffers; the first stage reads global memory --
         float2* cur = buf0;
         float2* oth = buf1;
-        switch (P.radix[0]) {
-            case 2: fft_first_stage<2>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            case 3: fft_first_stage<3>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            case 4: fft_first_stage<4>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            case 5: fft_first_stage<5>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            case 7: fft_first_stage<7>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            case 6: fft_first_stage<6>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            case 8: fft_first_stage<8>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            case 9: fft_first_stage<9>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            case 10: fft_first_stage<10>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;
-            default: fft_first_stage<1>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); break;      // plain copy-in: every factor is a large prime
-        }
+        with_radix<kWide>(P.radix[0], [&](auto r) { fft_first_stage<decltype(r)::value>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); });     // (1: plain copy-in, every factor is a large prime)
         __syncthreads();
         for (int s = 1; s < P.n_stages; ++s) {
-            switch (P.radix[s]) {
-                case 2: fft_stage<2>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                case 3: fft_stage<3>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                case 4: fft_stage<4>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                case 5: fft_stage<5>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                case 7: fft_stage<7>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                case 6: fft_stage<6>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                case 8: fft_stage<8>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                case 9: fft_stage<9>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                case 10: fft_stage<10>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]); break;
-                default: fft_stage_any(cur, oth, tw, n_fft, L, P.radix[s], P.div_lr[s], P.div_ns[s]); break;
-            }
+            with_radix<kWide>(P.radix[s], [&](auto r) {
+                constexpr int R = decltype(r)::value;
+                if constexpr (R > 1) fft_stage<R>(cur, oth, tw, n_fft, L, P.div_lr[s], P.div_ns[s]);
+                else fft_stage_any(cur, oth, tw, n_fft, L, P.radix[s], P.div_lr[s], P.div_ns[s]);
+            });
             __syncthreads();
             float2* tmp = cur; cur = oth; oth = tmp;
         }
@@ -341,40 +345,13 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     P.rows_per_cta = split.rows_per_cta; P.chunk = split.chunk;
     const bool few_rows = split.few_rows;
 
-    // radix plan: radices of up to 10 made of the factors 2, 3, 5, 7; prime factors above 7 come last as plain-sum stages (behind
-    // a copy-in stage when there is no small factor to read the windows with)
-    int rem = c.L, ns = 1;
-    P.n_stages = 0;
-    auto push = [&](int r) {
-        P.radix[P.n_stages] = r;
-        P.div_lr[P.n_stages] = make_fastdiv(c.L / r);
-        P.div_ns[P.n_stages] = make_fastdiv(ns);
-        ns *= r;
-        ++P.n_stages;
-    };
-    // (fewest stages: each is a pass over shared memory and a barrier.  u twos go with a five to a radix of 10, v with a three to 6; the twos left make
-    // eights, the threes nines.  With fours and primes only, 32 windows of 168 steps, 137 rows: 7.4 us, 7.05 so; 16 of 250, 862 rows 17.8 -> 14.5; 8 of
-    // 1000, 200 rows 12.0 -> 10.1.)
-    int exps[4] = {0, 0, 0, 0};
-    const int primes[4] = {2, 3, 5, 7};
-    for (int i = 0; i < 4; ++i) for (; rem % primes[i] == 0; rem /= primes[i]) ++exps[i];
-    int tens = 0, sixes = 0, fewest = 99;
-    for (int u = 0; u <= min(exps[0], exps[2]); ++u)
-        for (int v = 0; v <= min(exps[0] - u, exps[1]); ++v) {
-            const int stages = u + v + (exps[0] - u - v + 2) / 3 + (exps[1] - v + 1) / 2;      // (and the fives and sevens)
-            if (stages - u < fewest) { fewest = stages - u; tens = u; sixes = v; }             // (a ten takes a five's place)
-        }
-    int twos = exps[0] - tens - sixes, threes = exps[1] - sixes;
-    for (int i = 0; i < tens; ++i) push(10);
-    for (; threes >= 2; threes -= 2) push(9);
-    for (; twos >= 3; twos -= 3) push(8);
-    for (int i = 0; i < sixes; ++i) push(6);
-    if (twos > 0) push(2 * twos);
-    if (threes == 1) push(3);
-    for (int i = tens; i < exps[2]; ++i) push(5);
-    for (int i = 0; i < exps[3]; ++i) push(7);
-    if (rem > 1 && P.n_stages == 0) push(1);
-    for (int p = 11; rem > 1; p += 2) while (rem % p == 0) { push(p); rem /= p; }
+    const RadixPlan plan = radix_plan(c.L);
+    P.n_stages = plan.n;
+    for (int i = 0, ns = 1; i < plan.n; ns *= plan.radix[i++]) {
+        P.radix[i] = plan.radix[i];
+        P.div_lr[i] = make_fastdiv(c.L / plan.radix[i]);
+        P.div_ns[i] = make_fastdiv(ns);
+    }
 
     P.div_L = make_fastdiv(c.L);
     P.div_L4 = make_fastdiv(c.L >= 4 ? c.L / 4 : 1);
@@ -384,14 +361,6 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     const int max_fft = (P.rows_per_cta * P.chunk + 1) / 2;
     const size_t smem = sizeof(float2) * (static_cast<size_t>(c.L) + 2ull * max_fft * c.L) + sizeof(float) * P.rows_per_cta * P.nf;
     if (smem > 200 * 1024) return fail(VARDROP_ERR_UNSUPPORTED, "hash: shared memory plan of %zu bytes does not fit", smem);
-    static thread_local int attr_done_dev = -1;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (attr_done_dev != dev) {
-        if (int st = check_cuda(cudaFuncSetAttribute(hash_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024), "hash: smem attribute")) return st;
-        if (int st = check_cuda(cudaFuncSetAttribute(hash_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024), "hash: smem attribute")) return st;
-        attr_done_dev = dev;
-    }
     const int grid = (P.rows_total + P.rows_per_cta - 1) / P.rows_per_cta;
     // Threads: a stage is a few hundred butterflies, and a CTA that is mostly idle in its last round keeps others from the SM: 128 instead of 256
     // where that wastes less (16000 windows of 300 steps 23.1 -> 18.8 us, 4000 of 64 8.4 -> 5.6); 512 for a long pass when CTAs are few.  Not with many
@@ -401,9 +370,19 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     auto idle = [&](int t) { return (tasks + t - 1) / t * t; };
     const bool small = tasks <= 128 || (grid >= 8 * sm_count() && 5 * idle(128) < 4 * idle(256));
     const int threads = few_rows && tasks > 256 ? 512 : small && P.rows_per_cta <= 4 ? 128 : 256;
-    cudaError_t err;
-    { LaunchScope ls_(K_HASH, stream); err = launch_chained(threads > 256 ? hash_kernel<512> : hash_kernel<256>, dim3(grid), dim3(threads), smem, stream, P); }
-    return check_cuda(err, "hash: launch");
+    auto launch = [&](auto kernel, int& attr_dev) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (attr_dev != dev) {
+            if (int st = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024), "hash: smem attribute")) return st;
+            attr_dev = dev;
+        }
+        LaunchScope ls_(K_HASH, stream);
+        return check_cuda(launch_chained(kernel, dim3(grid), dim3(threads), smem, stream, P), "hash: launch");
+    };
+    static thread_local int attr_256 = -1, attr_512 = -1, attr_wide_256 = -1, attr_wide_512 = -1;
+    return plan.wide ? (threads > 256 ? launch(hash_kernel<512, true>, attr_wide_512) : launch(hash_kernel<256, true>, attr_wide_256))
+                : (threads > 256 ? launch(hash_kernel<512, false>, attr_512) : launch(hash_kernel<256, false>, attr_256));
 }
 
 }  // namespace vardrop

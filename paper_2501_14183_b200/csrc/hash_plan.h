@@ -1,0 +1,69 @@
+// Host-side plan of the transform in shared memory (hash_kernel): the radices of a length.  Plain C++, no CUDA.
+#pragma once
+
+#include <initializer_list>
+
+namespace vardrop {
+
+constexpr int kMaxStages = 16;
+
+// Radices in the order of the stages.  Prime factors above 7 come last, as stages of plain sums (behind a copy-in stage, radix 1, when there is
+// no small factor to read the windows with).
+struct RadixPlan {
+    int n = 0, radix[kMaxStages] = {};
+    bool wide = false;                           // has radices of 6 and 8 to 10
+    bool sums = false;                           // has stages of plain sums
+    void push(int r) { radix[n++] = r; }
+    void push_sums(int rem) {
+        if (rem > 1 && n == 0) push(1);
+        for (int p = 11; rem > 1; p += 2)
+            for (; rem % p == 0; rem /= p) { push(p); sums = true; }
+    }
+};
+
+inline RadixPlan fours_and_primes(int L) {
+    RadixPlan plan;
+    for (int r : {4, 2, 3, 5, 7})
+        for (; L % r == 0; L /= r) plan.push(r);
+    plan.push_sums(L);
+    return plan;
+}
+
+// Fewest stages: u twos go with a five to a radix of 10, v with a three to 6; the threes left make nines, the twos eights (and fours, where an eight
+// would leave a single two: a stage more of two-point butterflies, and larger errors).
+inline RadixPlan radices_to_ten(int L) {
+    int exps[4] = {0, 0, 0, 0};
+    const int primes[4] = {2, 3, 5, 7};
+    for (int i = 0; i < 4; ++i)
+        for (; L % primes[i] == 0; L /= primes[i]) ++exps[i];
+    int tens = 0, sixes = 0, fewest = 99;
+    for (int u = 0; u <= exps[0] && u <= exps[2]; ++u)
+        for (int v = 0; u + v <= exps[0] && v <= exps[1]; ++v) {
+            const int stages = v + (exps[0] - u - v + 2) / 3 + (exps[1] - v + 1) / 2;      // (a ten takes a five's place)
+            if (stages < fewest) { fewest = stages; tens = u; sixes = v; }
+        }
+    int twos = exps[0] - tens - sixes, threes = exps[1] - sixes;
+    RadixPlan plan;
+    plan.wide = true;
+    for (int i = 0; i < tens; ++i) plan.push(10);
+    for (; threes >= 2; threes -= 2) plan.push(9);
+    for (; twos >= 3 && twos != 4; twos -= 3) plan.push(8);
+    for (int i = 0; i < sixes; ++i) plan.push(6);
+    for (; twos >= 2; twos -= 2) plan.push(4);
+    if (twos == 1) plan.push(2);
+    if (threes == 1) plan.push(3);
+    for (int i = tens; i < exps[2]; ++i) plan.push(5);
+    for (int i = 0; i < exps[3]; ++i) plan.push(7);
+    plan.push_sums(L);
+    return plan;
+}
+
+// A stage is a pass over shared memory and a barrier, but the radices above 7 cost registers: they are taken where they save a stage.
+// (Back to back, with fours and primes and with them: 137 rows of 32 windows of 168 steps 6.6 -> 6.1 us, 862 of 16 of 250 16.7 -> 13.2, 200 of 8 of 1000
+// 11.1 -> 9.2.  2500 rows of 4 of 140 steps, which save none: 8.1, and 11.9 with 8 more registers.)
+inline RadixPlan radix_plan(int L) {
+    const RadixPlan narrow = fours_and_primes(L), wide = radices_to_ten(L);
+    return wide.n < narrow.n ? wide : narrow;
+}
+
+}  // namespace vardrop

@@ -3,6 +3,7 @@ structs match the header's layout."""
 import ctypes as C
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -99,3 +100,37 @@ def test_peers_shared_memory_is_reached_behind_a_cluster_barrier():
         barrier = re.search(r"\bcluster_(sync|wait)\s*\(\)", body)
         assert barrier and barrier.start() < remote.start(), f"{fn}: {name}"
     assert set(seen) == {"select_cluster_kernel", "hash_dft_kernel"}
+
+
+@pytest.fixture(scope="module")
+def plan_lib(tmp_path_factory):
+    """The host-side plan of the transform, which is plain C++."""
+    d = tmp_path_factory.mktemp("plan")
+    src = d / "plan.cpp"
+    src.write_text('#include "hash_plan.h"\nusing namespace vardrop;\n'
+                   'static int put(const RadixPlan& p, int* r) { for (int i = 0; i < p.n; ++i) r[i] = p.radix[i]; return p.n; }\n'
+                   'extern "C" int plan(int L, int* r, int* wide, int* sums) { RadixPlan p = radix_plan(L); *wide = p.wide; *sums = p.sums; return put(p, r); }\n'
+                   'extern "C" int narrow(int L, int* r) { return put(fours_and_primes(L), r); }\n')
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", f"-I{ROOT}/paper_2501_14183_b200/csrc", "-o", str(d / "plan.so"), str(src)])
+    return C.CDLL(str(d / "plan.so"))
+
+
+def radix_plans(plan_lib):
+    for L in range(2, 8193):
+        r, n, wide, sums = (C.c_int * 16)(), (C.c_int * 16)(), C.c_int(), C.c_int()
+        count = plan_lib.plan(L, r, C.byref(wide), C.byref(sums))
+        yield L, list(r[:count]), list(n[:plan_lib.narrow(L, n)]), bool(wide.value), bool(sums.value)
+
+
+def test_radix_plan_of_every_length(plan_lib):
+    """The product of the radices is the length; radices 6 and 8 to 10, which cost every call of their kernel registers, only where they save a stage; no
+    two-point stage where a four and a four do as well as an eight and a two."""
+    for L, radices, narrow, wide, sums in radix_plans(plan_lib):
+        prod = 1
+        for r in radices:
+            prod *= r
+        assert prod == L, L
+        assert wide == any(r in (6, 8, 9, 10) for r in radices), L
+        assert len(radices) < len(narrow) if wide else radices == narrow, (L, radices, narrow)
+        assert not (8 in radices and 2 in radices), (L, radices)
+        assert sums == (radices[-1] > 10), L
