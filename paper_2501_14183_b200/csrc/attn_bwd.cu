@@ -320,7 +320,7 @@ __device__ __forceinline__ int nth_instance(const BwdParams& P, int i, bool seve
 // Team memory: Q, K, V, dO, dS^T (two 64-query panels); tensor memory (256 columns): S^T [0,128), dP^T [128,256); P^T (bf16) goes over the
 // first half of each 64-column half of S^T, dV and dK over dP^T, dQ over P^T once dV has read it.
 template <bool kMixed>
-__device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigned char* tiles, float* stats, uint64_t* bar, uint32_t tm0, int team, int gt, int first, int stride, int count, uint64_t* bar_rows, bool& ok) {
+__device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigned char* tiles, float* stats, uint64_t* bar, uint32_t tm0, int team, int gt, int first, int stride, int count, bool& ok) {
     unsigned char* sQ = tiles + team * 6 * kTileBytes;
     unsigned char* sdO = sQ + 3 * kTileBytes;           // Q, K, V, dO
     unsigned char* sdS = sQ + 4 * kTileBytes;
@@ -339,7 +339,7 @@ __device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigne
         const int bi = small_div(item, P.H), h = item - bi * P.H, b = kMixed ? nth_instance(P, bi, false) : bi;
         const int n = kMixed ? P.n_sel[b] : kept;
         const int32_t* idx = P.sel_idx ? P.sel_idx + static_cast<size_t>(kMixed ? b : 0) * P.N : nullptr;
-        if (n <= 0) { --t; continue; }                   // (nothing kept at all: so for every item)
+        if (n <= 0) { --t; continue; }                   // (nothing kept at all)
         // rows: every warp a quarter of Q or K, then of V or dO
 #pragma unroll 1
         for (int x = warp >> 2; x < 4; x += 2) {
@@ -377,7 +377,6 @@ __device__ __forceinline__ void bwd_single(const BwdParams& P, int kept, unsigne
         fence_proxy_async_smem();
         tc_fence_before();
         group_sync(id);
-        if (t == 0 && team == 0 && gt == 0) mbar_arrive(bar_rows);
         if (warp == 0) {
             tc_fence_after();
             if (elect_one()) {
@@ -518,7 +517,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     ZeroRows zeros{s_flag + 1, 0, 0u};                              // (the word after that counts the flags written)
     struct alignas(16) Item { int jt, h, b, n_sel; };               // n_sel < 0 ends the list
     Item* s_item = reinterpret_cast<Item*>(smem_dyn + 336);         // [8]
-    uint64_t* bar_rows = reinterpret_cast<uint64_t*>(smem_dyn + 464);          // single: the rows of team 0's first item are in
     float* s_lse = reinterpret_cast<float*>(smem_dyn + 512);        // [2][128] minus the lse of the slot's rows, log2 domain
     float* s_delta = s_lse + 2 * kTile;                             // [2][128] their Delta
     float* s_none = s_delta + 2 * kTile;                            // [128] minus the lse for key rows that do not exist: -inf throughout
@@ -557,7 +555,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         mbar_init(bar_flag, 2 * kTeamWarps);
         mbar_init(bar_g, 1);
         mbar_init(bar_conv, 1);
-        mbar_init(bar_rows, 1);
         mbar_init(bar_first, 128);
         for (int i = 0; i < 8; ++i) mbar_init(bar_item + i, 1);
         for (int i = 0; i < 4; ++i) mbar_init(bar_team + i, 1);
@@ -1009,13 +1006,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     }
     if (!kMany && singles) {
         if (kMixed && pipeline) phase_sync();
-        if (warp < 2) {
-            // Behind the first rows: zero rows ahead of them held the loads up (119 of 321 kept, B = 32: step 35.4 us, 35.0 so; with four warps at it the
-            // backward 20 us against 18.8).
-            if (kept > 0 && s_first < s_count) ok &= warp_wait_relaxed(bar_rows, 0);
+        if (warp < 2)                                    // (four warps at it hold the teams' loads up: 20 us against 18.8 at 119 of 321 kept)
 #pragma unroll 1
             while (write_zero_row(P, zeros)) {}
-        }
     }
     } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kBwdBigRegs));
@@ -1174,7 +1167,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     }
     if (!kMany && singles) {
         if (kMixed && pipeline) phase_sync();
-        bwd_single<kMixed>(P, kept, sKV, reinterpret_cast<float*>(sDQ), bar_team + 2 * w, tmem + w * 256, w, gt, s_first, s_stride, s_count, bar_rows, ok);
+        bwd_single<kMixed>(P, kept, sKV, reinterpret_cast<float*>(sDQ), bar_team + 2 * w, tmem + w * 256, w, gt, s_first, s_stride, s_count, ok);
     }
     }
     if constexpr (kHelp) {                                   // (the loading warp that began has none of its group left)
