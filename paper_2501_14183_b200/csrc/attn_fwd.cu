@@ -774,8 +774,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
 // With one or two tiles per head and instance the step is a chain of latencies (kept count, row indices, rows, scores, softmax, P V,
 // rows out), each a few hundred cycles, and every path runs once or twice, at the speed of instruction fetch.  So: no roles and no
 // hand-offs but __syncthreads, rolled loops over 32 scores (the scores stay in tensor memory and are read twice), one stage, 48 KB
-// and 128 columns a CTA, so that four CTAs share an SM and fill each other's waits.  The next key tile's K comes in under the softmax, its V
-// under the step after (all of 321 variates, B = 32: 30.1 -> 29.1 us a call).
+// and 128 columns a CTA, so that four CTAs share an SM and fill each other's waits.
 // B = 32, H = 8, D = 64: 119 kept 7.1 us back to back (10 in the persistent kernel of the first form), 200 kept 15.3 us without a gather
 // launch (19 and a gather of 16).
 // Tensor memory: S 128; P (bf16) over S's columns 0 .. 63 as they are consumed, P V into columns 64 .. 127.
@@ -785,8 +784,10 @@ constexpr int kTileFwdSmemBytes = 1024 /*alignment*/ + 3 * kTileBytes /*Q, K, V*
 constexpr int kTileFwdPerSm = 4;
 
 // kLag: more than two tiles without a selection, where a row's reference maximum is that of its first 64 keys until the running maximum has outgrown
-// it by 2^8; O then goes back to tensor memory for the next P V to add to.  Otherwise it is the running maximum over whole key tiles, and the
-// tiles' parts of O are added up in registers.
+// it by 2^8; O then goes back to tensor memory for the next P V to add to; and the next key tile's K comes in under the softmax, its V under the step
+// after (all of 321 variates, B = 32: 28.2 -> 27.6 us back to back).  Otherwise it is the running maximum over whole key tiles, and the tiles' parts
+// of O are added up in registers; a second tile's rows come when the first is done (under its softmax, the code of it cost calls of one and
+// two tiles 1 to 4 %: 128 variates, B = 32 5.98 -> 6.15, 555 of 1500 kept, B = 32 65.6 -> 66.8).
 template <bool kLag>
 __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_kernel(const FwdParams P) {
     extern __shared__ unsigned char smem_dyn[];
@@ -849,6 +850,13 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
 #pragma unroll 1
         for (int j = 0; j < n_kv; ++j, ++t) {
             const int n_keys = min(kTile, n_sel - j * kTile);
+            if (!kLag && j > 0) {
+#pragma unroll 1
+                for (int x = 1; x < 3; ++x) {            // K, V
+                    load_rows(sQ + x * kTileBytes, x == 1 ? P.k : P.v, j);
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                }
+            }
             asm volatile("cp.async.wait_group 1;" ::: "memory");         // Q and K have landed
             fence_proxy_async_smem();
             tc_fence_before();
@@ -866,7 +874,7 @@ __global__ void __launch_bounds__(kTileFwdThreads, kTileFwdPerSm) attn_fwd_tile_
             }
             ok &= mbar_wait(&bar_s, t & 1);
             tc_fence_after();
-            const bool more = j + 1 < n_kv;
+            const bool more = kLag && j + 1 < n_kv;
             if (more) {                                  // K has been read: the next one comes in under the softmax
                 load_rows(sK, P.k, j + 1);
                 asm volatile("cp.async.commit_group;" ::: "memory");
