@@ -380,16 +380,16 @@ __device__ __noinline__ bool long_group_keeps(const LongGroups<kMax>& G, const u
 // Small problems (N <= 1024, or 2048 with many rows): one CTA per hash row does everything in shared memory.
 //
 // The distinct keys are found with a hash table and ranked against each other, which gives the group ids and offsets; a bitmap of its
-// members per distinct key gives a variate's place in its group; the sampling rank of a member is counted over its group.  More than 512 (of 2048: 360)
-// distinct keys are sorted instead:
+// members per distinct key gives a variate's place in its group; the sampling rank of a member is counted over its group.  More distinct keys than a
+// few hundred (small_max_groups) are sorted instead:
 //   sort 1: (key, variate)                      -> members, group heads -> ids, offsets
 //   sort 2: (group id, Philox priority, rank j) -> position inside the group = sampling rank
 // Then the kept flags are compacted.  No scratch in global memory, no global atomics.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kSmallMaxN = 2048;
 
-// Bitonic sort of M (a power of two >= 64) items by the first M / 2 threads of the CTA (all of them call it).  Thread t keeps items 2t and
-// 2t + 1 in registers.
+// Bitonic sort of M (a power of two >= 64) items by M / 2 threads, which are all that is left of the CTA.  Thread t keeps items 2t and 2t + 1 in
+// registers.
 // Compare-exchange distance j = 1 stays inside the thread, j = 2 .. 32 goes through warp shuffles (the partner of item
 // i is item i ^ j = slot (i & 1) of lane t ^ (j / 2)), and only j >= 64 passes through shared memory.
 // Items are (key, payload) pairs ordered by key, then payload; kPayload = false sorts bare keys.
@@ -406,12 +406,10 @@ __device__ __forceinline__ void bitonic_sort_regs(uint64_t& k0, uint32_t& p0, ui
         const bool up = ((2 * t) & k) == 0;              // the same for both items of the thread once k >= 2
         int j = k >> 1;
         for (; j >= 64; j >>= 1) {                       // partners live in another warp
-            if (2 * t < M) {
-                sk[2 * t] = k0; sk[2 * t + 1] = k1;
-                if (kPayload) { sp[2 * t] = p0; sp[2 * t + 1] = p1; }
-            }
+            sk[2 * t] = k0; sk[2 * t + 1] = k1;
+            if (kPayload) { sp[2 * t] = p0; sp[2 * t + 1] = p1; }
             __syncthreads();
-            const int l = ((2 * t) ^ j) & (M - 1);
+            const int l = (2 * t) ^ j;
             const uint64_t ok0 = sk[l], ok1 = sk[l + 1];
             const uint32_t op0 = kPayload ? sp[l] : 0u, op1 = kPayload ? sp[l + 1] : 0u;
             __syncthreads();
@@ -434,10 +432,11 @@ __device__ __forceinline__ void bitonic_sort_regs(uint64_t& k0, uint32_t& p0, ui
     }
 }
 
-// exclusive scan of two values per thread (positions 2 tid and 2 tid + 1) over the CTA; returns the exclusive prefix
+// exclusive scan of two values per thread (positions 2 tid and 2 tid + 1) over the CTA's first kThreads threads; returns the exclusive prefix
 // of position 2 tid and the total
+template <int kThreads>
 __device__ __forceinline__ int block_scan_pair(int v0, int v1, int* warp_sums, int* total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int v = v0 + v1;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -448,7 +447,8 @@ __device__ __forceinline__ int block_scan_pair(int v0, int v1, int* warp_sums, i
     if (lane == 31) warp_sums[warp] = v;
     __syncthreads();
     int base = 0, tot = 0;
-    for (int w = 0; w < n_warps; ++w) {
+#pragma unroll 1
+    for (int w = 0; w < kThreads / 32; ++w) {
         const int sw = warp_sums[w];
         if (w < warp) base += sw;
         tot += sw;
@@ -457,9 +457,10 @@ __device__ __forceinline__ int block_scan_pair(int v0, int v1, int* warp_sums, i
     return v + base - v0 - v1;
 }
 
-// Most distinct keys the table path takes: all of up to 512; beyond that their bitmaps fill shared memory, and ranking G keys is G^2 / 4 cycles.
-// (A call with more has paid for the table when it comes to sort.)
-__host__ __device__ constexpr int small_max_groups(int M) { return M <= 512 ? M : M <= 1024 ? 512 : 360; }
+// Most distinct keys the table path takes: ranking G keys is G^2 / 4 cycles, the sort does not depend on G.  Table | sort: 200 variates, 100 keys 3.9 | 5.2 us,
+// 200 6.2 | 5.4; 512, 256 keys 6.4 | 6.6, 512 13.8 | 7.0; 600, 300 keys 8.0 | 9.3; 862, 431 keys 11.7 | 10.0; above 1024 variates the bitmaps fill shared
+// memory first.  (A call with more has paid for the table when it comes to sort: 512 variates, all distinct, 4.9 us by sorting alone.)
+__host__ __device__ constexpr int small_max_groups(int M) { return M <= 128 ? M : M <= 256 ? 160 : M <= 512 ? 256 : M <= 1024 ? 352 : 360; }
 
 // Shared memory of the table path (the sorting path uses less, over it).
 struct SmallLayout {
@@ -496,8 +497,8 @@ template <int M>
 __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const SelectParams P) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     constexpr int T = M < 1024 ? M : 1024, kItems = M / T;
-    constexpr bool kSort = M > 512;
     constexpr SmallLayout L = small_layout(M);
+    constexpr bool kSort = small_max_groups(M) < M;
     constexpr int G_max = small_max_groups(M), W = M >> 5, pitch = W | 1, pitch2 = (W / 2) | 1;
     constexpr int kMaxLong = M / (kCountMaxGroup + 1) + 1;
     static_assert(G_max * pitch * 4 >= (M + 7 * G_max + 8) * 2 || M <= kCountMaxGroup, "candidates fit the place of the bitmaps");
@@ -553,7 +554,7 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
 #pragma unroll
     for (int e = 0; e < kItems; ++e) {
         at[e] = 2 * M;
-        if (tid + e * T >= N) continue;
+        if (tid + e * T >= N || (kSort && e > 0 && *reinterpret_cast<volatile int*>(&n_entries) > G_max)) continue;         // (too many already: to the sort)
         bool mine = false;
         if (key[e] == kEmpty) {
             mine = atomicExch(&all_ones, 1) == 0;
@@ -734,7 +735,9 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
         return;
     }
     if constexpr (kSort) {
-    // ---- the sorting path --------------------------------------------------------------------------------
+    // ---- the sorting path: two items a thread, the rest of the threads are done ----------------------------
+    constexpr int kSortThreads = M / 2;
+    if (tid >= kSortThreads) return;               // (whole warps; a barrier waits for those that have not left)
     uint64_t* a = reinterpret_cast<uint64_t*>(sm_raw);            // [M] sorted keys, later sorted (group, priority, rank) codes
     uint32_t* idx = reinterpret_cast<uint32_t*>(a + M);           // [M] variate by sorted position
     int* gpos = reinterpret_cast<int*>(idx + M);                  // [M] group id by sorted position
@@ -759,15 +762,15 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
     } else {
         bitonic_sort_regs<true>(k0, n0, k1, n1, a, idx, M);
     }
-    if (p0 < M) { a[p0] = k0; a[p1] = k1; idx[p0] = n0; idx[p1] = n1; }
+    a[p0] = k0; a[p1] = k1; idx[p0] = n0; idx[p1] = n1;
     __syncthreads();
 
     // group heads -> dense ids and offsets
     const int h0 = (p0 < N) && (p0 == 0 || k0 != a[p0 - 1]);
     const int h1 = (p1 < N) && (k1 != k0);
     int groups = 0;
-    const int before = block_scan_pair(h0, h1, warp_sums, &groups);
-    const int g0 = before + h0 - 1, g1 = before + h0 + h1 - 1;
+    const int heads_before = block_scan_pair<kSortThreads>(h0, h1, warp_sums, &groups);
+    const int g0 = heads_before + h0 - 1, g1 = heads_before + h0 + h1 - 1;
     if (p0 < N) {
         gpos[p0] = g0;
         if (h0) { off_s[g0] = p0; off[g0] = p0; }
@@ -781,7 +784,7 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
         gid[n1] = g1;
     }
     if (tid == 0) { off_s[groups] = N; P.n_groups[s] = groups; }
-    for (int i = groups + tid; i <= N; i += blockDim.x) off[i] = N;
+    for (int i = groups + tid; i <= N; i += kSortThreads) off[i] = N;
     __syncthreads();
 
     // sampling rank: sort (group, priority, j)
@@ -801,7 +804,7 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
     // Where groups are small a member's sampling rank is the number of codes of its group below its own, counted over the group's
     // few positions.  Only when some group is long does the second sort pay.
     const int size0 = p0 < N ? off_s[g0 + 1] - off_s[g0] : 0, size1 = p1 < N ? off_s[g1 + 1] - off_s[g1] : 0;
-    if (p0 < M) { a[p0] = c0; a[p1] = c1; }
+    a[p0] = c0; a[p1] = c1;
     if (!__syncthreads_or(size0 > kCountMaxGroup || size1 > kCountMaxGroup)) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
@@ -833,10 +836,10 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
     // compaction in ascending variate order
     const int kp0 = p0 < N ? keep_s[p0] : 0, kp1 = p1 < N ? keep_s[p1] : 0;
     int total = 0;
-    int pos = block_scan_pair(kp0, kp1, warp_sums, &total);
+    int pos = block_scan_pair<kSortThreads>(kp0, kp1, warp_sums, &total);
     if (p0 < N) { if (kp0) { sel[pos] = p0; inv[p0] = pos; ++pos; } else inv[p0] = -1; }
     if (p1 < N) { if (kp1) { sel[pos] = p1; inv[p1] = pos; } else inv[p1] = -1; }
-    for (int i = total + tid; i < N; i += blockDim.x) sel[i] = -1;
+    for (int i = total + tid; i < N; i += kSortThreads) sel[i] = -1;
     if (tid == 0) P.n_sel[s] = total;
     }
 }
@@ -1151,8 +1154,7 @@ int select_launch(const uint64_t* keys, const vardrop_select_cfg& c, int32_t* gr
     const bool small = c.N <= 1024 || (c.N <= kSmallMaxN && (one_cta || static_cast<double>(c.N) * c.N * c.S > kSmallPairs));
     if (small) {
         auto launch = [&](auto m) {
-            constexpr int kM = decltype(m)::value;
-            constexpr int sorting = kM > 512 ? kM * (8 + 4 + 4 + 4 + 4) + 16 : 0, table = small_layout(kM).total, smem = table > sorting ? table : sorting;
+            constexpr int kM = decltype(m)::value, sorting = small_max_groups(kM) < kM ? kM * (8 + 4 + 4 + 4 + 4) + 16 : 0, table = small_layout(kM).total, smem = table > sorting ? table : sorting;
             static thread_local int attr_dev = -1;
             int dev = 0;
             cudaGetDevice(&dev);

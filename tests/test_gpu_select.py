@@ -61,10 +61,10 @@ def test_select_group_sizes_around_the_counting_limit():
 
 
 @pytest.mark.parametrize("N,G", [(64, 64), (65, 63), (255, 182), (256, 183), (512, 256), (513, 159), (513, 257), (862, 160), (1024, 160), (1000, 161), (1024, 362), (1000, 363),
-                                 (1025, 360), (2048, 360), (1500, 361), (2048, 512), (1500, 513), (2048, 16), (1100, 9), (513, 1), (862, 2), (1024, 3), (2048, 1)])
+                                 (129, 129), (200, 160), (256, 161), (512, 257), (513, 352), (1024, 353), (1025, 360), (2048, 360), (1500, 361), (2048, 512), (1500, 513), (2048, 16), (1100, 9), (513, 1), (862, 2), (1024, 3), (2048, 1)])
 def test_select_group_counts_around_the_counting_limit(N, G):
-    """Few and many distinct keys in every size range: up to 512 variates all of them have entries in the hash table, up to 1024 as long as they are
-    no more than 512 (then they are sorted), above that all pairs are compared; one key is all ones, the mark of a free slot of the table and
+    """Few and many distinct keys in every size range: up to 128 variates all of them have entries in the hash table, up to 256, 512 and 1024 as long as they are
+    no more than 160, 256 and 352 (then they are sorted), above that all pairs are compared; one key is all ones, the mark of a free slot of the table and
     not a number where keys are compared as doubles."""
     rng = np.random.default_rng(N * 7 + G)
     values = np.unique(rng.integers(1, 1 << 60, 2 * G, dtype=np.uint64))[:G]
