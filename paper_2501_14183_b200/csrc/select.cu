@@ -859,7 +859,7 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kClusterCtas = 8;
 constexpr int kClusterMaxN = 8192;
-constexpr double kSmallPairs = 1.8e7;
+constexpr int kTwoLaunchRows = 4;                // from 1025 to 2048 variates: hash rows up to which the two launches are taken
 constexpr int kPlaceThreads = 1024;
 
 // What bounds it is the integer and comparison rate (64 results a cycle and SM).  Sixteen lanes hold kV variates each, the half warps of the CTA compare them with different keys, two a shared-memory load.  Keys are compared as
@@ -1148,10 +1148,12 @@ int select_launch(const uint64_t* keys, const vardrop_select_cfg& c, int32_t* gr
     P.seed_lo = static_cast<uint32_t>(c.seed & 0xFFFFFFFFu);
     P.seed_hi = static_cast<uint32_t>(c.seed >> 32);
     P.step = c.step;
-    // From 1025 variates two launches over more SMs are faster than one CTA a row until the rows' pairs of keys are many.  2000 variates in
-    // 160 | 600 groups, two launches 11.2 | 11.5 us for one row, 16.5 | 16.1 for four, 20 | 20 for eight, 42 | 41 for 32; one CTA a row 10 | 27 throughout.
+    // From 1025 variates two launches over more SMs do not depend on the groups, and take as long as one CTA a row does with few groups until the rows
+    // are many.  In 40 | 200 | all groups, one CTA a row takes 6.4 | 8.1 | 18 us at 1025 variates and 8.4 | 10 | 20 at 2048, with any number of rows;
+    // two launches take, at 1025, 7.1 | 6.5 | 5.5 for one row, 9.3 | 8.7 | 7.4 for four, 11.8 | 10.6 | 9.1 for eight; at 2048 8.0 | 7.5 | 6.4 for one,
+    // 11.9 | 11.0 | 10.1 for four.
     // (one_cta: the caller's scratch is shared by calls that may overlap, and may not be touched up to 2048 variates.)
-    const bool small = c.N <= 1024 || (c.N <= kSmallMaxN && (one_cta || static_cast<double>(c.N) * c.N * c.S > kSmallPairs));
+    const bool small = c.N <= 1024 || (c.N <= kSmallMaxN && (one_cta || c.S > kTwoLaunchRows));
     if (small) {
         auto launch = [&](auto m) {
             constexpr int kM = decltype(m)::value, sorting = small_max_groups(kM) < kM ? kM * (8 + 4 + 4 + 4 + 4) + 16 : 0, table = small_layout(kM).total, smem = table > sorting ? table : sorting;

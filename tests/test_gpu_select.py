@@ -118,6 +118,15 @@ def test_select_many_rows_of_1025_to_2048(S, N, G):
     check(rows, 12, 1.0, seed=G, step=2)
 
 
+@pytest.mark.parametrize("S,N,launches", [(1, 1024, 1), (32, 1024, 1), (1, 1025, 2), (4, 1025, 2), (5, 1025, 1), (8, 1500, 1), (4, 2048, 2), (5, 2048, 1), (32, 2048, 1), (1, 2049, 2), (32, 2049, 2)])
+def test_select_launches_by_rows(S, N, launches):
+    """From 1025 to 2048 variates two launches as long as they take no longer than one CTA a row does with few groups."""
+    keys = np.stack([inputs.make_keys(N, 40, k=4, f_hi=169, seed=s) for s in range(S)])
+    before = vd.vardrop_launch_count()
+    check(keys, 0, 0.2, seed=N, step=1)
+    assert vd.vardrop_launch_count() == before + launches
+
+
 def test_select_long_rows():
     """Rows beyond the cluster's: grouping with its working arrays in shared memory (up to 18432 variates), at that
     limit, and on the global arrays beyond it; several rows at once; one group only and all-distinct keys."""
