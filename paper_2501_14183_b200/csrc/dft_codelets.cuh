@@ -50,6 +50,16 @@ struct Turn {                                   // cos and sin of 2 pi NUM / DEN
     static constexpr float s = static_cast<float>(ct::sin_turn(NUM, DEN));
 };
 
+// m2 = 2 m for the angle 2 pi m / L, folded to |m| <= L / 2.
+__device__ __forceinline__ float folded_half_turns(int m, int L) { return static_cast<float>(2 * (2 * m > L ? m - L : m)); }
+// cos and sin of pi m2 / L to their last bit; turn: m2 / L to a rounding or two.  What it is off by (known exactly from its product with L) is put in after.
+__device__ __forceinline__ float2 cos_sin_turn(float m2, float turn, int L, float inv_L) {
+    const float rest = fmaf(-turn, static_cast<float>(L), m2) * (3.14159265f * inv_L);
+    float s, c;
+    sincospif(turn, &s, &c);
+    return make_float2(fmaf(-s, rest, c), fmaf(c, rest, s));
+}
+
 template <int I>
 struct Int {
     static constexpr int value = I;

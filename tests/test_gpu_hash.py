@@ -92,6 +92,16 @@ def test_hash_amplitudes_of_every_radix(L):
     assert np.linalg.norm(got.reshape(want.shape) - want) <= 3e-7 * np.linalg.norm(want)
 
 
+@pytest.mark.parametrize("L,bound", [(112, 7.00e-8), (324, 8.09e-8), (648, 8.62e-8), (729, 9.19e-8), (784, 8.16e-8), (1024, 7.46e-8)])
+def test_hash_amplitudes_with_radices_above_7(L, bound):
+    """No further from fp64 than stages of fours and primes are: the bound is what those measure on these inputs (with a table whose angles are rounded), and
+    a thousandth.  Lengths at which an eight and a two, or nines with that table, were 1 to 3 % above it."""
+    x = random_periodic(2, 600, L, 1, seed=L) + np.random.default_rng(L).normal(0, 1, size=(2, 600, L)).astype(np.float32)
+    _, _, got = run_hash(x, 1, 0, L // 2 + 1)
+    want = np.abs(np.fft.rfft(x.astype(np.float64), axis=-1)).mean(axis=0, keepdims=True)
+    assert np.linalg.norm(got.reshape(want.shape) - want) <= bound * np.linalg.norm(want)
+
+
 @pytest.mark.parametrize("B,N,L,scope", [(8, 1000, 442, 1), (8, 1000, 391, 0), (8, 1000, 961, 1), (32, 137, 1012, 0), (8, 1000, 130, 1), (1, 200, 1021, 0), (8, 1000, 858, 1), (8, 1000, 715, 1)])
 def test_hash_amplitudes_of_lengths_with_large_prime_factors(B, N, L, scope):
     """As close to fp64 as the transform in shared memory is, whichever kernel serves the length.  The bound: an amplitude is a sum of L / 2 products
