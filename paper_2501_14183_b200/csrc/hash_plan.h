@@ -59,11 +59,13 @@ inline RadixPlan radices_to_ten(int L) {
 }
 
 // A stage is a pass over shared memory and a barrier, but the radices above 7 cost registers: they are taken where they save a stage.
-// (Back to back, with fours and primes and with them: 137 rows of 32 windows of 168 steps 6.6 -> 6.1 us, 862 of 16 of 250 16.7 -> 13.2, 200 of 8 of 1000
-// 11.1 -> 9.2.  2500 rows of 4 of 140 steps, which save none: 8.1, and 11.9 with 8 more registers.)
+// (Between other launches, with fours and primes and with them: 137 rows of 32 windows of 168 steps 6.5 -> 6.0 us, 862 of 16 of 250 16.6 -> 11.0, 200 of 8 of
+// 1000 11.2 -> 9.1.  2500 rows of 4 of 140 steps, which save none: 8.0, and 11.9 with 8 more registers.)
+// Not two eights for three fours: their stores conflict eight ways (862 rows of 16 of 64 steps 5.3 us, 5.7 so), and the error is 1 % larger.
 inline RadixPlan radix_plan(int L) {
     const RadixPlan narrow = fours_and_primes(L), wide = radices_to_ten(L);
-    return wide.n < narrow.n ? wide : narrow;
+    const bool eights = wide.n == 2 && wide.radix[0] == 8 && wide.radix[1] == 8;
+    return wide.n < narrow.n && !eights ? wide : narrow;
 }
 
 }  // namespace vardrop

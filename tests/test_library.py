@@ -124,7 +124,7 @@ def radix_plans(plan_lib):
 
 def test_radix_plan_of_every_length(plan_lib):
     """The product of the radices is the length; radices 6 and 8 to 10, which cost every call of their kernel registers, only where they save a stage; no
-    two-point stage where a four and a four do as well as an eight and a two."""
+    two-point stage where a four and a four do as well as an eight and a two; not two eights, slower and less exact than three fours."""
     for L, radices, narrow, wide, sums in radix_plans(plan_lib):
         prod = 1
         for r in radices:
@@ -132,5 +132,5 @@ def test_radix_plan_of_every_length(plan_lib):
         assert prod == L, L
         assert wide == any(r in (6, 8, 9, 10) for r in radices), L
         assert len(radices) < len(narrow) if wide else radices == narrow, (L, radices, narrow)
-        assert not (8 in radices and 2 in radices), (L, radices)
+        assert not (8 in radices and 2 in radices) and radices != [8, 8], (L, radices)
         assert sums == (radices[-1] > 10), L
