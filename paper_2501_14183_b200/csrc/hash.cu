@@ -183,8 +183,10 @@ __device__ __forceinline__ void with_radix(int radix, F f) {
 // kWide: with radices 6 and 8 to 10, which take 56 registers instead of 40 (with 256 threads four CTAs an SM instead of six).
 // kSums: with the stage of plain sums.  Its kernel takes the table's angles from the quotient instead of the product with 1 / L: the compiler then lays that
 // stage out the better way (862 rows of 16 windows of 676 steps 170 -> 150 us).
-template <int kMaxThreads, bool kWide, bool kSums>
-__global__ void __launch_bounds__(kMaxThreads) hash_kernel(const HashParams P) {
+// kCtas: held to registers for so many CTAs an SM, where they are more than four (2500 rows of 4 of 384 steps 18.4 -> 15.9 us; where they are fewer the
+// other is up to 9 % faster).
+template <int kMaxThreads, bool kWide, bool kSums, int kCtas = 0>
+__global__ void __launch_bounds__(kMaxThreads, kCtas) hash_kernel(const HashParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int L = P.L, nf = P.nf;
     const int max_win = P.rows_per_cta * P.chunk;           // windows per pass
@@ -347,7 +349,6 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     const HashSplit split = hash_split(c);
     P.rows_total = split.rows_total; P.win_per_row = split.win_per_row;
     P.rows_per_cta = split.rows_per_cta; P.chunk = split.chunk;
-    const bool few_rows = split.few_rows;
 
     const RadixPlan plan = radix_plan(c.L);
     P.n_stages = plan.n;
@@ -367,14 +368,7 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     const size_t smem = sizeof(float2) * (static_cast<size_t>(c.L) + 2ull * max_fft * c.L) + sizeof(float) * P.rows_per_cta * P.nf;
     if (smem > 200 * 1024) return fail(VARDROP_ERR_UNSUPPORTED, "hash: shared memory plan of %zu bytes does not fit", smem);
     const int grid = (P.rows_total + P.rows_per_cta - 1) / P.rows_per_cta;
-    // Threads: a stage is a few hundred butterflies, and a CTA that is mostly idle in its last round keeps others from the SM: 128 instead of 256
-    // where that wastes less (16000 windows of 300 steps 23.1 -> 18.8 us, 4000 of 64 8.4 -> 5.6); 512 for a long pass when CTAs are few.  Not with many
-    // rows to a CTA, which its warps rank one after the other (27584 rows of one window of 32 steps: 17.9 us with 256 threads, 27.7 with 128), nor
-    // where the CTAs are few anyway (1920 of 600 steps 10.8 | 13.7; with fewer than one an SM a stage of plain sums has a task for every output).
-    const int tasks = max_fft * (P.radix[P.n_stages - 1] > 7 && grid < sm_count() ? c.L : c.L / P.radix[0]);
-    auto idle = [&](int t) { return (tasks + t - 1) / t * t; };
-    const bool small = tasks <= 128 || (grid >= 8 * sm_count() && 5 * idle(128) < 4 * idle(256));
-    const int threads = few_rows && tasks > 256 ? 512 : small && P.rows_per_cta <= 4 ? 128 : 256;
+    const int threads = hash_threads(plan, c.L, max_fft, P.rows_per_cta, grid, static_cast<int>(smem), split.few_rows, sm_count());
     auto launch = [&](auto kernel, int& attr_dev) {
         int dev = 0;
         cudaGetDevice(&dev);
@@ -387,8 +381,8 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
     };
     auto pick = [&](auto sums) {
         constexpr bool kSums = decltype(sums)::value;
-        static thread_local int attr_256 = -1, attr_512 = -1, attr_wide_256 = -1, attr_wide_512 = -1;
-        if (plan.wide) return threads > 256 ? launch(hash_kernel<512, true, kSums>, attr_wide_512) : launch(hash_kernel<256, true, kSums>, attr_wide_256);
+        static thread_local int attr_256 = -1, attr_512 = -1, attr_wide = -1, attr_wide_256 = -1;
+        if (plan.wide) return threads == 256 && grid > 4 * sm_count() ? launch(hash_kernel<256, true, kSums, 5>, attr_wide_256) : launch(hash_kernel<512, true, kSums>, attr_wide);
         return threads > 256 ? launch(hash_kernel<512, false, kSums>, attr_512) : launch(hash_kernel<256, false, kSums>, attr_256);
     };
     return plan.sums ? pick(std::true_type{}) : pick(std::false_type{});

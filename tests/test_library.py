@@ -110,13 +110,14 @@ def plan_lib(tmp_path_factory):
     src.write_text('#include "hash_plan.h"\nusing namespace vardrop;\n'
                    'static int put(const RadixPlan& p, int* r) { for (int i = 0; i < p.n; ++i) r[i] = p.radix[i]; return p.n; }\n'
                    'extern "C" int plan(int L, int* r, int* wide, int* sums) { RadixPlan p = radix_plan(L); *wide = p.wide; *sums = p.sums; return put(p, r); }\n'
-                   'extern "C" int narrow(int L, int* r) { return put(fours_and_primes(L), r); }\n')
+                   'extern "C" int narrow(int L, int* r) { return put(fours_and_primes(L), r); }\n'
+                   'extern "C" int threads(int L, int n, int rows, int ctas, int smem, int few, int sms) { return hash_threads(radix_plan(L), L, n, rows, ctas, smem, few, sms); }\n')
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", f"-I{ROOT}/paper_2501_14183_b200/csrc", "-o", str(d / "plan.so"), str(src)])
     return C.CDLL(str(d / "plan.so"))
 
 
-def radix_plans(plan_lib):
-    for L in range(2, 8193):
+def radix_plans(plan_lib, longest=8192):
+    for L in range(2, longest + 1):
         r, n, wide, sums = (C.c_int * 16)(), (C.c_int * 16)(), C.c_int(), C.c_int()
         count = plan_lib.plan(L, r, C.byref(wide), C.byref(sums))
         yield L, list(r[:count]), list(n[:plan_lib.narrow(L, n)]), bool(wide.value), bool(sums.value)
@@ -134,3 +135,22 @@ def test_radix_plan_of_every_length(plan_lib):
         assert len(radices) < len(narrow) if wide else radices == narrow, (L, radices, narrow)
         assert not (8 in radices and 2 in radices) and radices != [8, 8], (L, radices)
         assert sums == (radices[-1] > 10), L
+
+
+def test_threads_of_the_transform(plan_lib):
+    """The threads of a CTA go by the stage with the most butterflies (the first, of the largest radix, has the fewest), by the rounds that the CTAs take, and not
+    by a last radix above 7, which is no stage of plain sums."""
+    sms, kb = 148, 20 * 1024
+    threads = lambda L, transforms, rows, ctas, smem, few: plan_lib.threads(L, transforms, rows, ctas, smem, few, sms)  # noqa: E731
+    assert threads(960, 1, 1, 100, kb, 1) == 512 and threads(1024, 1, 1, 100, kb, 1) == 256          # 8 8 3 5: 320 butterflies; 8 8 4 4: 256
+    assert threads(300, 1, 1, 100, kb, 1) == 128 and threads(1000, 1, 1, 100, kb, 1) == 256          # 10 6 5: 60; 10 10 10: 100
+    assert threads(90, 8, 1, 862, kb, 0) == 128 and threads(112, 8, 1, 1000, kb, 0) == 128           # one round, where 256 threads take two
+    assert threads(1000, 2, 1, 862, 2 * kb, 0) == 256 and threads(384, 4, 2, 1250, 28 * 1024, 0) == 256     # two rounds of either
+    for L, radices, _, wide, sums in radix_plans(plan_lib, 1024):
+        most = max(L if r > 10 else L // r for r in radices)
+        for transforms in (1, 2, 8):
+            for ctas in (30, 200, 500, 700, 1000, 5000):
+                t = threads(L, transforms, 1, ctas, kb, int(ctas < 2 * sms))
+                assert t in (128, 256, 512) and (t < 512 or ctas <= 2 * sms)
+                if wide and ctas <= 2 * sms:
+                    assert min(512, transforms * most) / 2 <= t <= max(128, 4 * transforms * most), (L, transforms, ctas, t)
