@@ -9,6 +9,7 @@ import pytest
 
 from paper_2501_14183_b200 import binding as vd
 from paper_2501_14183_b200 import build as lib_build
+from util import RADIX_LENGTHS
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -154,3 +155,12 @@ def test_threads_of_the_transform(plan_lib):
                 assert t in (128, 256, 512) and (t < 512 or ctas <= 2 * sms)
                 if wide and ctas <= 2 * sms:
                     assert min(512, transforms * most) / 2 <= t <= max(128, 4 * transforms * most), (L, transforms, ctas, t)
+
+
+def test_radix_lengths_cover_every_radix_at_every_place(plan_lib):
+    """Lengths with a prime factor above 7 do not count: the matrix product may take them."""
+    places = set()
+    for L, radices, _, _, sums in radix_plans(plan_lib, 4000):
+        if L in RADIX_LENGTHS and not sums and len(radices) > 1:
+            places |= {(radices[0], "first"), (radices[-1], "last")} | {(r, "middle") for r in radices[1:-1]}
+    assert places == {(r, at) for r in range(2, 11) for at in ("first", "middle", "last")}

@@ -12,6 +12,10 @@ ATTN_MAX_ABS = 2e-2
 ATTN_MEAN_ABS = 2e-3
 RANK_GAP = 1e-3
 
+# Lengths whose transform in shared memory has, between them, each radix from 2 to 10 as first, middle and last stage (test_library.py holds them to it).
+RADIX_LENGTHS = [6, 8, 9, 10, 14, 18, 20, 21, 24, 27, 32, 35, 36, 40, 42, 45, 48, 49, 54, 60, 64, 70, 72, 81, 90, 100, 126, 128, 135, 144, 162, 175, 240, 250, 256, 270, 300, 343, 360,
+                 432, 500, 512, 539, 630, 700, 726, 875, 960, 1000, 1024, 4000]
+
 
 def gap_filtered_windows(x: np.ndarray, k: int, f_lo: int = 0, f_hi: int = 0, scope: int = 0):
     """Returns (x', keys, freqs, abar, n_replaced): variates whose hash is decided by a relative amplitude gap below
