@@ -335,7 +335,9 @@ int hash_dft_launch(const float* x, const vardrop_hash_cfg& c, int f_lo, int f_h
     while (P.split < 8 && P.split < P.tiles && groups * P.split < 2ll * sm_count()) P.split *= 2;
     // What either costs, in microseconds: rounds of CTAs, each its blocks and rows here (the first of a cluster ranks for all), its complex transforms
     // there (plain sums over an even length read shared memory with bank conflicts).  The terms are fitted to 1100 measured calls of 33 to 1021 steps,
-    // 100 to 32000 windows and three bands: the choice so made costs about 1 % more than the better of the two.  Where it turns, there | here: 4384 windows of 715 = 5 11 13 steps 41 | 63 us, of 391 = 17 23 37 | 25, of 1021 1642 | 86; 100 of 313 14 | 21, of 1021 107 | 50.
+    // 100 to 32000 windows and three bands, with stages of fours and primes there: the choice so made costs about 1 % more than the better of the two.  With
+    // the stages that some lengths save since (radix_plan), 484 calls of 70 such lengths: 2.0 % more, and 1.6 % by terms fitted to those.  Where it turns, there | here: 4384
+    // windows of 715 = 5 11 13 steps 41 | 63 us, of 391 = 17 23 37 | 25, of 1021 1642 | 86; 100 of 313 14 | 21, of 1021 107 | 50.
     auto rounds = [](long long ctas, int at_once) { return static_cast<double>((ctas + at_once - 1) / at_once); };
     const int passes_there = (there.win_per_row + there.chunk - 1) / there.chunk;
     const int transforms = there.rows_per_cta > 1 ? (there.rows_per_cta * there.chunk + 1) / 2 : passes_there * ((there.chunk + 1) / 2);

@@ -491,8 +491,8 @@ __host__ __device__ constexpr SmallLayout small_layout(int M) {
 // issue rate, and for a few dozen variates their latency.  So the steps are dependent accesses of shared memory without searches (the bitmaps
 // give places, a group's priorities are read eight at a time), ranked keys are held four to a thread, and the sizes of the tables are constants
 // of the instantiation (as arguments, index arithmetic and loop remainders were half of the instructions).
-// Back to back, with the bitonic sort (up to 512) or the counts per chunk and searches (above) of before: 321 variates 7.7 -> 4.6 us, 862 in 54 groups
-// 10.0 -> 6.6, in 148 10.8 -> 6.9, all distinct 12.8 -> 9.6; 32 rows of 321 7.7 -> 4.9.
+// Between other launches, with the bitonic sort (up to 512) or the counts per chunk and searches (above) of before: 321 variates in 26 groups 5.4 -> 3.4 us, 862
+// in 71 7.1 -> 4.9, in 172 10.0 -> 6.0; all distinct 321 4.9 -> 6.2, 862 10.1 -> 10.6; 32 rows of 321 in 26 5.6 -> 3.5.
 template <int M>
 __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const SelectParams P) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -678,7 +678,8 @@ __global__ void __launch_bounds__(M < 1024 ? M : 1024) select_small_kernel(const
                 if (p >= N) continue;
                 const int n = static_cast<int>(at_pos[p] & 0xFFFFu), d = static_cast<int>(at_pos[p] >> 16);
                 const uint2 f = info[d];
-                const int size = static_cast<int>(f.x >> 16), quota = static_cast<int>(f.y & 0xFFFFu), start = static_cast<int>(f.y >> 16), j = p - static_cast<int>(f.x & 0xFFFFu);
+                const int size = static_cast<int>(f.x >> 16), quota = static_cast<int>(f.y & 0xFFFFu);
+                const int start = static_cast<int>(f.y >> 16), j = p - static_cast<int>(f.x & 0xFFFFu);
                 members[p] = n;
                 bool keep = quota == size;
                 if (!keep && size <= kCountMaxGroup) {
@@ -862,10 +863,10 @@ constexpr int kClusterMaxN = 8192;
 constexpr int kTwoLaunchRows = 4;                // from 1025 to 2048 variates: hash rows up to which the two launches are taken
 constexpr int kPlaceThreads = 1024;
 
-// What bounds it is the integer and comparison rate (64 results a cycle and SM).  Sixteen lanes hold kV variates each, the half warps of the CTA compare them with different keys, two a shared-memory load.  Keys are compared as
-// doubles, whose bit patterns order like the values as long as none is negative, infinite or not a number: one instruction, on a pipe of its own,
-// where two 64-bit integers take two that share theirs with the counting (8192 variates 12.0 -> 10.4 us).  Keys of up to five 12-bit bins are such
-// numbers; others are compared as integers.
+// What bounds it is the integer and comparison rate (64 results a cycle and SM).  Sixteen lanes hold kV variates each, the half warps of the CTA compare them
+// with different keys, two a shared-memory load.  Keys are compared as doubles, whose bit patterns order like the values as long as none is
+// negative, infinite or not a number: one instruction, on a pipe of its own, where two 64-bit integers take two that share theirs with the counting
+// (8192 variates 12.0 -> 10.4 us).  Keys of up to five 12-bit bins are such numbers; others are compared as integers.
 template <int kV>
 __global__ void __launch_bounds__(kPlaceThreads) select_place_kernel(const SelectParams P) {
     extern __shared__ __align__(16) uint64_t s_keys[];         // [N rounded up to 2]
@@ -1156,7 +1157,8 @@ int select_launch(const uint64_t* keys, const vardrop_select_cfg& c, int32_t* gr
     const bool small = c.N <= 1024 || (c.N <= kSmallMaxN && (one_cta || c.S > kTwoLaunchRows));
     if (small) {
         auto launch = [&](auto m) {
-            constexpr int kM = decltype(m)::value, sorting = small_max_groups(kM) < kM ? kM * (8 + 4 + 4 + 4 + 4) + 16 : 0, table = small_layout(kM).total, smem = table > sorting ? table : sorting;
+            constexpr int kM = decltype(m)::value, table = small_layout(kM).total;
+            constexpr int sorting = small_max_groups(kM) < kM ? kM * (8 + 4 + 4 + 4 + 4) + 16 : 0, smem = table > sorting ? table : sorting;
             static thread_local int attr_dev = -1;
             int dev = 0;
             cudaGetDevice(&dev);
