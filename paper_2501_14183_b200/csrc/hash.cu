@@ -184,7 +184,7 @@ __device__ __forceinline__ void with_radix(int radix, F f) {
 // kSums: with the stage of plain sums.  Its kernel takes the table's angles from the quotient instead of the product with 1 / L: the compiler then lays that
 // stage out the better way (862 rows of 16 windows of 676 steps 170 -> 150 us).
 // kCtas: held to registers for so many CTAs an SM, where they are more than four (2500 rows of 4 of 384 steps 18.4 -> 15.9 us; where they are fewer the
-// other is up to 9 % faster).
+// other is up to 9 % faster), or for six with plain sums where five take a second round (862 rows of 16 of 924 steps 118 -> 105 us, 2500 of 4 of 165 17.4 -> 15.6).
 template <int kMaxThreads, bool kWide, bool kSums, int kCtas = 0>
 __global__ void __launch_bounds__(kMaxThreads, kCtas) hash_kernel(const HashParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -215,7 +215,8 @@ __global__ void __launch_bounds__(kMaxThreads, kCtas) hash_kernel(const HashPara
         // ---- mixed-radix Stockham FFT, ping-pong between the two buffers; the first stage reads global memory --
         float2* cur = buf0;
         float2* oth = buf1;
-        with_radix<kWide, kSums>(P.radix[0], [&](auto r) { fft_first_stage<decltype(r)::value>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); });     // (1: plain copy-in, every factor is a large prime)
+        // (radix 1: plain copy-in, every factor is a large prime)
+        with_radix<kWide, kSums>(P.radix[0], [&](auto r) { fft_first_stage<decltype(r)::value>(P, cur, n_win, row0, b0, cw, P.div_lr[0]); });
         __syncthreads();
         for (int s = 1; s < P.n_stages; ++s) {
             with_radix<kWide, kSums>(P.radix[s], [&](auto r) {
@@ -383,6 +384,10 @@ int hash_launch(const float* x, const vardrop_hash_cfg& c, uint64_t* keys, int32
         constexpr bool kSums = decltype(sums)::value;
         static thread_local int attr_256 = -1, attr_512 = -1, attr_wide = -1, attr_wide_256 = -1;
         if (plan.wide) return threads == 256 && grid > 4 * sm_count() ? launch(hash_kernel<256, true, kSums, 5>, attr_wide_256) : launch(hash_kernel<512, true, kSums>, attr_wide);
+        if constexpr (kSums) {                             // six CTAs an SM instead of five, where that is one round instead of two
+            static thread_local int attr_six = -1;
+            if (threads == 256 && grid > 5 * sm_count() && grid <= 6 * sm_count() && 6 * (smem + 1024) <= 228 * 1024) return launch(hash_kernel<256, false, true, 6>, attr_six);
+        }
         return threads > 256 ? launch(hash_kernel<512, false, kSums>, attr_512) : launch(hash_kernel<256, false, kSums>, attr_256);
     };
     return plan.sums ? pick(std::true_type{}) : pick(std::false_type{});

@@ -70,8 +70,8 @@ def test_hash_parity_small(B, N, L, k, scope):
     # every window a row: rows that do not fill a warp's set, one row, each planned length, both band widths
     (1, 1, 96, 3, 1, False), (3, 37, 96, 5, 1, True), (1, 47, 192, 3, 1, False), (2, 35, 192, 2, 1, True), (7, 9, 336, 4, 1, True), (1, 3, 720, 5, 1, True), (40, 130, 96, 3, 1, False),
     # large prime factors: 16 and 64 windows a CTA, 32 and 64 bins a tile, tiles over a cluster, more instances than a pass takes, even and odd lengths
-    # (and two small ones: the transform in shared memory with 512 and with 128 threads)
-    (70, 40, 97, 3, 0, False), (32, 37, 168, 3, 0, False), (12, 400, 75, 3, 0, False), (1, 900, 151, 3, 0, False), (3, 40, 622, 4, 0, False), (5, 300, 131, 3, 1, False), (1, 30, 1021, 5, 0, True), (6, 170, 202, 2, 0, True), (2, 23, 994, 3, 1, False)])
+    # (and two small ones: the transform in shared memory with 512 and with 128 threads; and one with six CTAs of 256 to an SM)
+    (70, 40, 97, 3, 0, False), (32, 37, 168, 3, 0, False), (12, 400, 75, 3, 0, False), (1, 900, 151, 3, 0, False), (3, 40, 622, 4, 0, False), (5, 300, 131, 3, 1, False), (1, 30, 1021, 5, 0, True), (6, 170, 202, 2, 0, True), (2, 23, 994, 3, 1, False), (4, 2500, 165, 3, 0, False)])
 def test_hash_rows_of_one_window_and_large_prime_factors(B, N, L, k, scope, wide):
     band = (0, L // 2 + 1) if wide else (0, 0)
     x = random_periodic(B, N, L, k, seed=B * 1000 + N * 10 + L)
