@@ -299,6 +299,7 @@ def kernel_work(w, n_sel, selected=True):
     kept = w.B * n_sel
     full = w.B * w.N
     grads = 3 * (full if selected else kept) * row                  # dq, dk, dv come back in the full layout
+    many = w.N > (2048 if selected else 256)                        # dq and the zero rows come from the convert kernel then, Delta from the prep kernel
     return {
         "hash_kernel": (w.B * w.N * w.L * 4 + w.N * (8 + 4 * w.k), None),
         "select_small_kernel": (w.N * (8 + 6 * 4), None),
@@ -310,8 +311,8 @@ def kernel_work(w, n_sel, selected=True):
         # (with many key tiles and a selection the forward pass also clears the dQ' accumulator, 64 floats a row and head; without one the prep kernel does)
         "attn_fwd_kernel": (3 * kept * row + kept * row + kept * w.H * 4 + (kept * w.H * 64 * 4 if selected and n_sel > 256 else 0), 4.0 * w.B * w.H * n_sel * n_sel * w.D),
         "bwd_prep_kernel": ((3 * kept * row + 2 * kept * row if selected else 2 * kept * row + kept * w.H * 64 * 4) + kept * w.H * 4, None),
-        "attn_bwd_kernel": (5 * kept * row + kept * w.H * 4 + grads, 10.0 * w.B * w.H * n_sel * n_sel * w.D),
-        "bwd_convert_kernel": (kept * row + kept * w.H * 64 * 4, None),
+        "attn_bwd_kernel": (4 * kept * row + 2 * kept * w.H * 4 + 2 * kept * row if many else 5 * kept * row + kept * w.H * 4 + grads, 10.0 * w.B * w.H * n_sel * n_sel * w.D),
+        "bwd_convert_kernel": (kept * row + kept * w.H * 64 * 4 + (3 * (full - kept) * row if selected else 0), None),
     }
 
 

@@ -11,7 +11,7 @@ HERE = Path(__file__).resolve().parent
 CSRC = HERE / "csrc"
 LIB = HERE / "libvardrop.so"
 MARSHAL = HERE / "_marshal.so"
-SOURCES = ["vardrop_api.cu", "hash.cu", "hash_rows.cu", "hash_dft.cu", "select.cu", "attn_fwd.cu", "attn_bwd.cu", "pearson.cu", "gather_rows.cu"]
+SOURCES = ["vardrop_api.cu", "hash.cu", "hash_rows.cu", "hash_dft.cu", "select.cu", "attn_fwd.cu", "attn_bwd.cu", "attn_bwd_many.cu", "pearson.cu", "gather_rows.cu"]
 
 
 def _nvcc() -> str:

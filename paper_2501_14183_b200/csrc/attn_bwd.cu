@@ -1,171 +1,33 @@
-// Attention backward over the kept variate tokens and the scatter of the gradients to the full layout.
+// Attention backward over few key tiles of kept variate tokens (attn_bwd_many.cu: many) and the scatter of the gradients to the full layout.
 //
-// bwd_prep_kernel     many tiles: Delta_i = sum_d dO'_id O'_id, the kept rows laid out as tiles (selection), and the cleared dQ' accumulator
-//                     (no selection: with one the forward pass clears it).
 // attn_bwd_kernel     one CTA per SM.  Scores are formed transposed (S^T = K Q^T, dP^T = V dO^T) so that a thread owns (part of) a key row
 //                     of tensor memory; P^T and dS^T feed dV += P^T dO, dK += dS^T Q and dQ_i = dS K.  Two shapes of the work:
 //                       single   a kept set of one tile: two teams of 256 threads, each a whole (head, instance) on its own, no hand-offs
 //                       pipeline several tiles: work items (two neighbouring 128-key tiles, head, instance), a warp role for each part of
 //                                the work; dQ is written by the item (two tiles or fewer) or added into an fp32 accumulator by bulk
-//                                reduce-adds
+//                                reduce-adds and converted by the CTA that finishes an (instance, head) pair
 //                     The same kernel writes the zero rows of every dropped variate.
-// bwd_convert_kernel  many tiles: dQ' accumulator to bf16 rows of dq (fewer: by the CTA that finishes an (instance, head) pair).
 //
 // Each row of dq / dk / dv is written exactly once.
-#include "attn_common.cuh"
+#include "attn_bwd.cuh"
 
 namespace vardrop {
 
 namespace {
 
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
-__device__ __forceinline__ float2 unpack2(uint32_t w) {
-    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w));
-}
-__device__ __forceinline__ float dot8(uint4 a, uint4 g) {
-    const float2 a0 = unpack2(a.x), a1 = unpack2(a.y), a2 = unpack2(a.z), a3 = unpack2(a.w);
-    const float2 g0 = unpack2(g.x), g1 = unpack2(g.y), g2 = unpack2(g.z), g3 = unpack2(g.w);
-    return a0.x * g0.x + a0.y * g0.y + a1.x * g1.x + a1.y * g1.y + a2.x * g2.x + a2.y * g2.y + a3.x * g3.x + a3.y * g3.y;
-}
-__device__ __forceinline__ float sum8(float v) {       // over the eight lanes of a row
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    v += __shfl_xor_sync(0xffffffffu, v, 4);
-    return v;
-}
-
-// ---------------------------------------------------------------------------------------------------------
-// prep
-// ---------------------------------------------------------------------------------------------------------
-struct PrepParams {
-    const uint4* o;         // [B, N, H, D] bf16
-    const uint4* d_o;       // [B, N, H, D] bf16
-    const __nv_bfloat16* q;
-    float* delta;           // [B, H, Ncap]
-    float4* dq_acc;         // [B, Ncap, H, 64] fp32; NULL: cleared by the forward pass
-    uint4* staged[2];       // [B, Ncap, H, D] bf16 copies of the kept rows of Q, and of dO: with a selection
-    const int32_t* sel_idx; // [S, N]; NULL: identity, nothing is staged
-    const int32_t* n_sel;   // [S] kept counts; NULL: N
-    long long sB, sN, sH;
-    int N, Ncap, H, D, S;
-};
-
-// One thread per 16-byte chunk of a (token, head) row of 64; the 8 threads of a row reduce Delta by shuffles.  With a selection the rows
-// that the main kernel reads again for every pair of key tiles (Q, dO) are laid out here once, zeros up to the tile's end (rows of dO past the
-// kept ones may hold anything), so that it takes boxes: row copies by its two loader warps bound it at 1423 kept tokens (250 us against 170).
-// K and V it reads once, as rows, and under the end of the item before (laid out here too, a step of 8192 variates took 311.8 us instead of 304.6).
-__global__ void __launch_bounds__(256) bwd_prep_kernel(const PrepParams P) {
-    chain_wait();
-    chain_release();
-    const int b = blockIdx.y;
-    const int n_sel = P.n_sel ? P.n_sel[P.S > 1 ? b : 0] : P.N;
-    const int n_fill = min(P.Ncap, (n_sel + kTile - 1) / kTile * kTile);
-    const int chunks_row = P.H * 8;
-    const int src_chunks_head = P.D / 8;
-    const int total = n_fill * chunks_row;            // a multiple of 8; blockDim is a multiple of 8
-    const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? b : 0) * P.N : nullptr;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-        const int i = small_div(idx, chunks_row);
-        const int c = idx - i * chunks_row;
-        const int h = c >> 3, dc = c & 7;
-        uint4 vo = make_uint4(0u, 0u, 0u, 0u), vd = vo, vq = vo;
-        if (i < n_sel && dc < src_chunks_head) {
-            const size_t src = (static_cast<size_t>(b) * P.N + i) * (P.H * src_chunks_head) + h * src_chunks_head + dc;
-            vo = __ldg(P.o + src);
-            vd = __ldg(P.d_o + src);
-            if (sel) vq = __ldg(reinterpret_cast<const uint4*>(P.q + (b * P.sB + __ldg(sel + i) * P.sN + h * P.sH + dc * 8)));
-        }
-        if (sel && dc < src_chunks_head) {
-            const size_t to = ((static_cast<size_t>(b) * P.Ncap + i) * P.H + h) * src_chunks_head + dc;
-            P.staged[0][to] = vq; P.staged[1][to] = vd;
-        }
-        const float part = sum8(dot8(vo, vd));
-        if (dc == 0) P.delta[(static_cast<size_t>(b) * P.H + h) * P.Ncap + i] = part;
-        if (P.dq_acc) {
-            const size_t dst = (static_cast<size_t>(b) * P.Ncap + i) * chunks_row + c;
-            P.dq_acc[2 * dst] = make_float4(0.f, 0.f, 0.f, 0.f);
-            P.dq_acc[2 * dst + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------------------------------------
 // main
 // ---------------------------------------------------------------------------------------------------------
-struct BwdParams {
-    const __nv_bfloat16 *q, *k, *v;   // read by the row copies of a selection (boxes go through the tensor maps)
-    const __nv_bfloat16* d_o;         // [B, N, H, D]
-    const __nv_bfloat16* o;           // [B, N, H, D] forward output (rows 0 .. n_sel-1), for Delta
-    const float* lse;       // [B, H, N]
-    const float* delta;     // [B, H, Ncap] many tiles: Delta (few: computed here from o and dO)
-    float* dq_acc;          // [B, Ncap, H, 64]
-    __nv_bfloat16* dq;      // [B, N, H, D]
-    __nv_bfloat16* dk;
-    __nv_bfloat16* dv;
-    const int32_t* sel_idx; // [S, N]; NULL: identity
-    const int32_t* inv_idx; // [S, N]; NULL: identity (nothing dropped)
-    int32_t* tile_done;     // few tiles: [B, H] items whose part of dQ' has landed; zeroed by the forward pass
-    const int32_t* n_sel;   // [S]; NULL: N
-    int* status;
-    long long sB, sN, sH;   // element strides of q, k, v
-    int B, N, Ncap, H, D, S;
-    float scale, scale_log2;
-};
-
 constexpr int kBwdGroup = 256;
 constexpr int kBwdThreads = 256 + 2 * kBwdGroup;
 // Register split (setmaxnreg works on whole warpgroups): launched with 768 x 80 = 61440 registers; the first two warpgroups keep 56 a thread, the
-// teams take 88: 256 x 56 + 512 x 88 = 59392.  (1423 of 8192 kept: 166 us with 64 and 80, 150 so, 156 with 48 and 96, whose loaders spill.)
+// teams take 88: 256 x 56 + 512 x 88 = 59392.
 constexpr int kBwdSmallRegs = 56;
 constexpr int kBwdBigRegs = 88;
 constexpr uint32_t kBwdTmemCols = 512;
 constexpr int kBwdHeader = 3072;       // barriers, item list, row statistics
 constexpr int kBwdSmemBytes = kBwdHeader + 4 * kTileBytes /*K, V of two key tiles*/ + 4 * kTileBytes /*two slots of Q, dO*/ +
                               4 * kTileBytes /*dS^T of two key tiles*/ + 2 * kTileBytes /*dQ tile, fp32, two 32-column halves*/;
-
-// The arithmetic between the products, as instructions that keep their order: left to itself the compiler puts the consumers of a pair
-// of exponentials right behind it and a warp runs at the latency of the special-function unit instead of its rate.
-__device__ __forceinline__ uint64_t pair_of(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void halves_of(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma_pair(uint64_t a, uint64_t b, uint64_t c) {      // two IEEE fp32 results per issue slot
-    uint64_t d;
-    asm volatile("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t mul_pair(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm volatile("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ float fast_exp2(float x) {      // special-function unit; exp2(-inf) = 0
-    float y;
-    asm volatile("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    uint32_t d;
-    asm volatile("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-    return d;
-}
-
-// A pair of floats from shared memory, issued here.  Read by all lanes alike, 8 bytes take 0.6 cycles of the shared-memory pipe, 16 bytes 2.1.
-__device__ __forceinline__ uint64_t lds_pair(uint32_t addr) {
-    uint64_t v;
-    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr));
-    return v;
-}
-
-// every lane of the warp waits; the result is the same in all of them
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity)); }
-// the same with a sleep between polls
-__device__ __forceinline__ bool warp_wait_relaxed(uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait_relaxed(bar, parity)); }
 
 // named barrier among 256 threads (id 1 or 2), with an and-reduction of ok
 __device__ __forceinline__ bool group_sync_and(int id, bool ok) {
@@ -194,45 +56,6 @@ __device__ __forceinline__ bool drain_sync_and(bool ok) {     // the same among 
 }
 __device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, 256;" ::"r"(id) : "memory"); }
 
-// Zero rows of dq, dk, dv for every dropped variate, by whichever warps of the CTA have nothing else to do: they take the CTA's rows eight at
-// a time from a shared counter, look them up in inv_idx, and write one dropped row a call, 512 bytes a store instruction.  One row at a time,
-// between other work: written in one go by every CTA at once they fill the memory's queues, and row loads behind them took 10000 cycles (200
-// of 862 kept).
-struct ZeroRows {
-    int* taken;                         // groups of eight rows taken so far, by all warps of the CTA
-    int base;
-    unsigned mask;                      // dropped rows of the current group still to write
-};
-__device__ __forceinline__ bool write_zero_row(const BwdParams& P, ZeroRows& z) {      // false: none left
-    const int lane = threadIdx.x & 31;
-    if (!P.inv_idx) return false;
-#pragma unroll 1
-    while (z.mask == 0) {
-        int g = 0;
-        if (lane == 0) g = atomicAdd(z.taken, 1);
-        z.base = (blockIdx.x + __shfl_sync(0xffffffffu, g, 0) * gridDim.x) * 8;
-        if (z.base >= P.B * P.N) return false;
-        const int r = z.base + lane;
-        bool dropped = false;
-        if (lane < 8 && r < P.B * P.N) {
-            const int b = small_div(r, P.N), n = r - b * P.N;
-            dropped = __ldg(P.inv_idx + static_cast<size_t>(P.S > 1 ? b : 0) * P.N + n) < 0;
-        }
-        z.mask = __ballot_sync(0xffffffffu, dropped);
-    }
-    const int chunks_row = P.H * (P.D / 8);                    // 16-byte chunks per (instance, variate) row
-    const size_t row0 = static_cast<size_t>(z.base + __ffs(z.mask) - 1) * chunks_row;
-    z.mask &= z.mask - 1;
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll 1
-    for (int c = lane; c < chunks_row; c += 32) {
-        reinterpret_cast<uint4*>(P.dq)[row0 + c] = zero;
-        reinterpret_cast<uint4*>(P.dk)[row0 + c] = zero;
-        reinterpret_cast<uint4*>(P.dv)[row0 + c] = zero;
-    }
-    return true;
-}
-
 // This thread's 32 columns (half `half`) of its row of a 64-column accumulator, scaled and rounded, to a bf16 staging tile.
 __device__ __forceinline__ void stage_acc(unsigned char* tile, uint32_t tm, float mul, int row, int half) {
     unsigned char* rowp = tile + row * kRowBytes;
@@ -255,48 +78,6 @@ __device__ __forceinline__ void store_rows(const unsigned char* tile, __nv_bfloa
 #pragma unroll
     for (int x = 0; x < 4; ++x)
         if (n[x] >= 0) *reinterpret_cast<uint4*>(out + static_cast<size_t>(n[x]) * P.H * P.D) = *reinterpret_cast<const uint4*>(from + x * 32 * kRowBytes);
-}
-
-// P^T = exp2(S^T scale - lse) of a thread's 32 queries, in place, and as bf16: batches of eight (exponents of g, exponentials of g - 1,
-// rounding of g - 2) keep the special-function unit at its rate.
-__device__ __forceinline__ void exp_step(float (&s)[32], uint32_t (&pk)[16], const uint64_t (&l)[16], uint64_t scale2) {
-#pragma unroll
-    for (int g = 0; g < 6; ++g) {
-        if (g < 4) {
-#pragma unroll
-            for (int e = 8 * g; e < 8 * g + 8; e += 2) halves_of(fma_pair(pair_of(s[e], s[e + 1]), scale2, l[e >> 1]), s[e], s[e + 1]);
-        }
-        if (g >= 1 && g < 5) {
-#pragma unroll
-            for (int e = 8 * g - 8; e < 8 * g; ++e) s[e] = fast_exp2(s[e]);
-        }
-        if (g >= 2) {
-#pragma unroll
-            for (int e = 8 * g - 16; e < 8 * g - 8; e += 2) pk[e >> 1] = pack_bf16(s[e], s[e + 1]);
-        }
-    }
-}
-// dS^T = P^T o (dP^T - Delta) as bf16; Delta of eight queries is in registers, the next eight on their way.
-__device__ __forceinline__ void ds_step(const float (&s)[32], float (&d)[32], uint32_t (&pk)[16], uint64_t (&dl)[2][4], uint32_t dlt) {
-    const uint64_t minus1 = pair_of(-1.f, -1.f);
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        if (g < 3) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) dl[(g + 1) & 1][e] = lds_pair(dlt + 32 * g + 32 + 8 * e);
-        }
-#pragma unroll
-        for (int e = 8 * g; e < 8 * g + 8; e += 2) {
-            halves_of(mul_pair(pair_of(s[e], s[e + 1]), fma_pair(dl[g & 1][(e >> 1) & 3], minus1, pair_of(d[e], d[e + 1]))), d[e], d[e + 1]);
-            pk[e >> 1] = pack_bf16(d[e], d[e + 1]);
-        }
-    }
-}
-// Four 16-byte chunks (32 queries) of a row of a 64-query panel.
-__device__ __forceinline__ void store_panel(unsigned char* panel, int row, int half, const uint32_t (&pk)[16]) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<uint4*>(panel + row * kRowBytes + (((half * 4 + q) ^ (row & 7)) << 4)) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
 }
 
 // With a selection per instance, the i-th instance that keeps several tiles (`several`) or one; the whole warp looks.
@@ -480,13 +261,7 @@ constexpr int kTeamWarps = 8;
 
 // kMixed: few tiles, a selection per instance, so that some instances may keep one tile and others several (its code costs the other calls 0.4 us
 // of instruction fetch).
-// kHelp: many tiles, but a selection of up to kHelpZerosN variates, whose kept tiles may be done long before one warp has written the zero rows of the
-// dropped ones: every warp then helps with what is left.  B = 32, H = 8, 2049 variates, 102 kept 116 -> 71 us, forward and backward, 204 kept 140 -> 97;
-// 4096, 204 kept, B = 8 73 -> 48.  Where the items take longer the code alone costs something: 8192, 1423 kept 254 -> 262.
-constexpr int kHelpZerosN = 6144;
-// kKvRows: many tiles, with a selection: K and V come as rows.  (Decided when the kernel runs, the same code without one was 1 to 3 % slower: 862 tokens,
-// B = 6, 105.1 -> 107.2 us forward and backward.)
-template <bool kMany, bool kMixed, bool kHelp, bool kKvRows>
+template <bool kMixed>
 __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                                                                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
                                                                   const __grid_constant__ CUtensorMap map_acc, const BwdParams P) {
@@ -531,15 +306,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         if (tid == 0) set_status(P.status, VARDROP_ERR_CUDA);
         return;
     }
-    const bool boxes = kMany || P.sel_idx == nullptr;          // Q and dO come as boxes, or as rows
-    const bool kv_rows = kMany ? kKvRows : P.sel_idx != nullptr;       // K and V, which an item reads once, as rows wherever there is a selection
+    const bool boxes = P.sel_idx == nullptr;                   // operand tiles come as boxes, or as rows
     if (warp == 0) {
         tmem_alloc(tmem_slot, kBwdTmemCols);
         tmem_relinquish();
     }
     if (tid == 0) {
         for (int w = 0; w < 2; ++w) {
-            mbar_init(bar_kv_full + w, kv_rows ? kBwdGroup : 1);    // a box: one announcing arrival; row copies: every thread of the team
+            mbar_init(bar_kv_full + w, boxes ? 1 : kBwdGroup);    // a box: one announcing arrival; row copies: every thread of the team
             mbar_init(bar_q_full + w, boxes ? 1 : 66);              // row copies: every loader lane, and one of each loader for the statistics
             mbar_init(bar_q_free + w, 2);
             mbar_init(bar_x + w, 1);
@@ -561,10 +335,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         mbar_fence_init();
         if (boxes) {
             tma_prefetch_desc(&map_q);
-            if (!kv_rows) {
-                tma_prefetch_desc(&map_k);
-                tma_prefetch_desc(&map_v);
-            }
+            tma_prefetch_desc(&map_k);
+            tma_prefetch_desc(&map_v);
             tma_prefetch_desc(&map_do);
         }
         tma_prefetch_desc(&map_acc);
@@ -585,7 +357,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         kept = largest_kept(P.n_sel, P.S, P.N);
         n_t = (kept + kTile - 1) / kTile;                      // tiles of the longest selection
         // Instances with several tiles go through the pipeline, those with one by teams.
-        int several = n_t > 1 || kMany ? P.B : 0, one = P.B - several;
+        int several = n_t > 1 ? P.B : 0, one = P.B - several;
         const int grid = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
         int c = cta, takers = grid;                            // CTAs that take singles
         if (kMixed) {
@@ -602,20 +374,18 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         per_item = n_t == 2 || n_t * P.H * several > grid ? 2 : 1;
         n_slots = (n_t + per_item - 1) / per_item;
         n_items = n_slots * P.H * several;                     // pipeline: (key tiles, head, instance); short instances skip some
-        pipeline = kMany || (kMixed ? cta < n_items : n_t > 1);
-        if (!kMany) {
-            s_count = one * P.H;
-            if (kMixed && several && one) {
-                // Both kinds: the CTAs without items take the singles if their teams can (32 instances of about 120 kept, a few of them above 128: forward
-                // and backward 35 us with every instance in the pipeline, 29 so).
-                const bool apart = n_items < grid && 2 * (grid - n_items) >= s_count;
-                takers = apart ? grid - n_items : grid;
-                c = apart ? cta - n_items : (cta + grid - n_items % grid) % grid;
-            }
-            singles = kMixed ? c >= 0 && c < s_count : n_t <= 1;
-            s_first = c + (warp >= 16 ? takers : 0);
-            s_stride = 2 * takers;
+        pipeline = kMixed ? cta < n_items : n_t > 1;
+        s_count = one * P.H;
+        if (kMixed && several && one) {
+            // Both kinds: the CTAs without items take the singles if their teams can (32 instances of about 120 kept, a few of them above 128: forward
+            // and backward 35 us with every instance in the pipeline, 29 so).
+            const bool apart = n_items < grid && 2 * (grid - n_items) >= s_count;
+            takers = apart ? grid - n_items : grid;
+            c = apart ? cta - n_items : (cta + grid - n_items % grid) % grid;
         }
+        singles = kMixed ? c >= 0 && c < s_count : n_t <= 1;
+        s_first = c + (warp >= 16 ? takers : 0);
+        s_stride = 2 * takers;
     };
     // A role of several warps shares a named barrier, which nothing bounds: a warp whose wait gives up leaves only behind such a barrier, where the
     // others learn of it.  The teams wait for their next item ahead of the last barrier of the current one; the dQ warps all pass a barrier at the end
@@ -681,7 +451,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 continue;
             }
             ok &= warp_wait_relaxed(bar_kv_full + w, ai & 1);
-            if (kMany && kv_rows) fence_proxy_async_smem();      // (otherwise with the slot's rows)
             auto wait_slot = [&](uint32_t tt) {
                 ok &= warp_wait_relaxed(bar_q_full + (tt & 1), (tt >> 1) & 1);
                 if (!boxes) fence_proxy_async_smem();    // rows written by asynchronous copies are read by the tensor core
@@ -761,10 +530,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             }
             __syncwarp();
         };
-        if (kMany && part == 1) {                        // boxes are one warp's work: the other writes the zero rows
-#pragma unroll 1
-            while (write_zero_row(P, zeros)) {}
-        }
         uint32_t t = 0;
         if (part == 0) publish(0);
 #pragma unroll 1
@@ -775,21 +540,18 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             const int n_q = (it.n_sel + kTile - 1) / kTile;
             // Row statistics of a query tile travel with it: asked for ahead of the wait for the slot, four rows a lane.
             const float* lse_row = P.lse + (static_cast<size_t>(it.b) * P.H + it.h) * P.N;
-            const float* delta_row = kMany ? P.delta + (static_cast<size_t>(it.b) * P.H + it.h) * P.Ncap : nullptr;
-            float st_lse[4], st_delta[4];
+            float st_lse[4];
             auto stats_load = [&](int tile) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int r = tile * kTile + e * 32 + lane;
                     st_lse[e] = part == 0 && r < it.n_sel ? __ldg(lse_row + r) : INFINITY;
-                    if (kMany) st_delta[e] = r < it.n_sel ? __ldg(delta_row + r) : 0.f;
                 }
             };
             auto stats_store = [&](uint32_t slot) {      // minus the lse in the log2 domain: -inf switches a missing query off
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     if (part == 0) s_lse[slot * kTile + e * 32 + lane] = st_lse[e] * -1.4426950408889634f;
-                    if (kMany) s_delta[slot * kTile + e * 32 + lane] = st_delta[e];
                 }
                 __syncwarp();
             };
@@ -807,7 +569,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                         tma_load_4d(sQ + slot * 2 * kTileBytes + kTileBytes, &map_do, bar_q_full + slot, 0, it.h, x * kTile, it.b);
                     }
                     __syncwarp();
-                    if (x == 0 && !kv_rows) {            // the first query tile comes in under the item before; K and V replace that one's
+                    if (x == 0) {                        // the first query tile comes in under the item before; K and V replace that one's
                         ok = warp_wait_relaxed(bar_kv_free, (i & 1) ^ 1);
                         if (!ok) break;
                         if (lane == 0) {
@@ -874,10 +636,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         const bool owner = row == 0;                     // the one thread that owns the bulk reductions
         const uint32_t idesc_mnmn = umma_idesc_bf16(128, P.D, 1, 1);       // A MN-major, B MN-major
         const uint64_t m_k = umma_desc_sw128(smem_u32(sKV), kTileBytes, 1024);
-        // Columns taken out at a time: with few key tiles these warps also hold Delta's loads and the output rows (862 variates, 200 kept:
-        // 43.4 us with 32, 41.5 with 16); with many the chain of loads is what they wait for (1423 of 8192 kept: 150 with 32, 157 with 16).
-        constexpr int kDrain = kMany ? 32 : 16;
-        bool zeros_left = !kMany;
+        // Columns taken out at a time: these warps also hold Delta's loads and the output rows (862 variates, 200 kept: 43.4 us with 32, 41.5 with 16).
+        constexpr int kDrain = 16;
+        bool zeros_left = true;
         uint32_t t = 0, t1 = 0;                          // query tiles so far, and those with a second key tile
 #pragma unroll 1
         for (uint32_t i = 0;; ++i) {
@@ -885,7 +646,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             if (it.n_sel < 0) { ok = drain_sync_and(ok); break; }
             const int n_q = (it.n_sel + kTile - 1) / kTile;
             const bool two = key0_of(it, 1) < it.n_sel;
-            const bool direct = !kMany && n_q <= per_item;      // dQ is complete here
+            const bool direct = n_q <= per_item;              // dQ is complete here
             const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
             const int c8 = row & 7, r8 = row >> 3;
             const size_t compact = (static_cast<size_t>(it.b) * P.N * P.H + it.h) * P.D;
@@ -914,10 +675,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 }
                 warp_arrive(bar_delta + (tt & 1));
             };
-            if (!kMany) delta_of(0, t);
+            delta_of(0, t);
 #pragma unroll 1
             for (int x = 0; x < n_q; ++x, ++t) {
-                if (!kMany && x + 1 < n_q) delta_of(x + 1, t + 1);
+                if (x + 1 < n_q) delta_of(x + 1, t + 1);
                 while (zeros_left && warp != 4 && !__all_sync(0xffffffffu, mbar_test(bar_tile, t & 1))) {       // nothing else to do
                     zeros_left = write_zero_row(P, zeros);
                     __nanosleep(100);
@@ -955,8 +716,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
 #pragma unroll 1
                 for (int c = 0; c < P.D; c += kDrain) {
                     float v[kDrain];
-                    if constexpr (kMany) tmem_ld32(tm + c, v);
-                    else tmem_ld16(tm + c, v);
+                    tmem_ld16(tm + c, v);
                     tmem_ld_wait();
                     if (!direct) {                       // fp32, 32-column panels of 128-byte swizzled rows
                         unsigned char* to = sDQ + (c >> 5) * kTileBytes + row * kRowBytes;
@@ -992,7 +752,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 }
             }
             if (!ok) break;
-            if (!kMany && !direct && owner) {            // dQ' of this (instance, head) is complete once all its items are: the teams of the last convert it
+            if (!direct && owner) {                     // dQ' of this (instance, head) is complete once all its items are: the teams of the last convert it
                 bulk_wait_group0();                      // this item's reductions have landed
                 __threadfence();
                 const int n = s_flag[2]++;               // items with an accumulated dQ' before this one
@@ -1004,7 +764,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         if (owner) bulk_wait_group0();                   // the last dQ reductions have landed
         asm volatile("cp.async.wait_all;" ::: "memory");
     }
-    if (!kMany && singles) {
+    if (singles) {
         if (kMixed && pipeline) phase_sync();
         if (warp < 2)                                    // (four warps at it hold the teams' loads up: 20 us against 18.8 at 119 of 321 kept)
 #pragma unroll 1
@@ -1028,7 +788,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                          P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N, key0_of(it, w) + g, it.n_sel, P.D);
             cp_async_arrive(bar_kv_full + w);
         };
-        bool loaded = false;                             // many: this item's were asked for under the end of the item before
         item_wait(0);
         ok = group_sync_and(id, ok);
 #pragma unroll 1
@@ -1036,10 +795,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             const Item it = item_read(i);
             if (it.n_sel < 0) break;
             const int n_q = (it.n_sel + kTile - 1) / kTile, key0 = key0_of(it, w);
-            if (kv_rows && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
+            if (!boxes && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
             // dQ' of an (instance, head) of more than two tiles: both teams of the CTA that brought its last part
             auto convert_dq = [&]() {
-                if (kMany || n_q <= per_item) return;
+                if (n_q <= per_item) return;
                 if (!warp_wait_relaxed(bar_conv, n_conv & 1)) set_status(P.status, VARDROP_ERR_TIMEOUT);
                 ++n_conv;
                 const int c8 = gt & 7;
@@ -1070,17 +829,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 }
             };
             if (key0 >= it.n_sel) {                      // no key tile: nothing else ties this team to the others' pace, and it waits by parity
-                if (!kv_rows && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
+                if (boxes && i > 0) ok &= warp_wait_relaxed(bar_kv_free, (i - 1) & 1);
                 item_wait(i + 1);
                 ok = group_sync_and(id, ok);
                 if (gt == 0) mbar_arrive(bar_skip + w);
-                if (kMany) loaded = false;
                 t += n_q;
                 convert_dq();
                 continue;
             }
             const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N : nullptr;
-            if (kv_rows && !(kMany && loaded)) load_kv(it);
+            if (!boxes) load_kv(it);
             const bool key_valid = key0 + row < it.n_sel;
             // After an item it had no key tile in, a team may be two phases ahead of a query slot's barrier, which would let it through: its own
             // scores come after the phase it wants.
@@ -1115,7 +873,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                     tc_fence_after();
                     tmem_ld32(tm + half * 32, d);
                     const bool g_done = hs > 0 || x == 0 || mbar_test(bar_g, (t - 1) & 1);
-                    if (!kMany && hs == 0) ok &= warp_wait(bar_delta + slot, (t >> 1) & 1);
+                    if (hs == 0) ok &= warp_wait(bar_delta + slot, (t >> 1) & 1);
                     uint64_t dl[2][4];                   // Delta of eight queries, the next eight on their way
 #pragma unroll
                     for (int e = 0; e < 4; ++e) dl[0][e] = lds_pair(dlt + 8 * e);
@@ -1145,12 +903,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             ok &= warp_wait(bar_dk + w, (u - 1) & 1);
             ok &= warp_wait(bar_g, (t - 1) & 1);
             tc_fence_after();
-            if (kMany && kv_rows) {                      // every product that reads this team's K and V is done: the next item's come in under what follows
-                item_wait(i + 1);
-                const Item next = item_read(i + 1);
-                loaded = __all_sync(0xffffffffu, ok && next.n_sel >= 0 && key0_of(next, w) < next.n_sel);
-                if (loaded) load_kv(next);
-            }
 #pragma unroll 1
             for (int e = 0; e < 2; ++e) stage_acc(panels + e * kTileBytes, tm + (e == 0 ? kColDv : kColDk), e == 0 ? 1.f : P.scale, row, half);
             tc_fence_before();
@@ -1165,17 +917,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     }
-    if (!kMany && singles) {
+    if (singles) {
         if (kMixed && pipeline) phase_sync();
         bwd_single<kMixed>(P, kept, sKV, reinterpret_cast<float*>(sDQ), bar_team + 2 * w, tmem + w * 256, w, gt, s_first, s_stride, s_count, ok);
     }
     }
-    if constexpr (kHelp) {                                   // (the loading warp that began has none of its group left)
-        ZeroRows rest{zeros.taken, 0, 0u};
-#pragma unroll 1
-        while (write_zero_row(P, rest)) {}
-    }
-    if (!kMany && (warp >= 8 || pipeline || !singles))       // (a warp that zeroed rows while it waited may have some of its group left)
+    if (warp >= 8 || pipeline || !singles)       // (a warp that zeroed rows while it waited may have some of its group left)
 #pragma unroll 1
         while (write_zero_row(P, zeros)) {}              // what is left
     if (!ok) set_status(P.status, VARDROP_ERR_TIMEOUT);
@@ -1184,107 +931,24 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     if (warp == 0) tmem_dealloc(tmem, kBwdTmemCols);
 }
 
-// ---------------------------------------------------------------------------------------------------------
-// dq from the accumulator (paths with many key tiles)
-// ---------------------------------------------------------------------------------------------------------
-struct ConvertParams {
-    const float4* dq_acc;    // [B, Ncap, H, 64] fp32
-    uint4* dq;               // [B, N, H, D] bf16
-    const int32_t* sel_idx;  // [S, N]; NULL: identity
-    const int32_t* n_sel;    // [S]; NULL: N
-    int N, Ncap, H, D, S;
-    float scale;
-};
-
-// What bounds it is memory: kept rows only (dropped ones were zeroed by the main kernel), 16-byte results, two in flight a thread.  1423 of 8192
-// kept, B = 8, H = 8: 12.6 us, 15.5 when it looked every variate up (events around the launch).
-__global__ void __launch_bounds__(256) bwd_convert_kernel(const ConvertParams P) {
-    chain_wait();
-    chain_release();
-    const int b = blockIdx.y, srow = P.S > 1 ? b : 0;
-    const int n_sel = P.n_sel ? P.n_sel[srow] : P.N;
-    const int32_t* sel = P.sel_idx ? P.sel_idx + static_cast<size_t>(srow) * P.N : nullptr;
-    const int sh = P.D > 32 ? 3 : 2, chunks_row = P.H << sh;        // 16-byte results per row
-    const int total = n_sel * chunks_row, stride = gridDim.x * blockDim.x;
-    const float4* acc = P.dq_acc + static_cast<size_t>(b) * P.Ncap * P.H * (kDP / 4);
-    uint4* dq = P.dq + static_cast<size_t>(b) * P.N * chunks_row;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += 2 * stride) {
-        float4 a[2][2];
-        size_t to[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int at = min(idx + e * stride, total - 1);
-            const int j = small_div(at, chunks_row), c = at - j * chunks_row, h = c >> sh, dc = c & ((1 << sh) - 1);
-            to[e] = static_cast<size_t>(sel ? __ldg(sel + j) : j) * chunks_row + c;
-            const float4* src = acc + (static_cast<size_t>(j) * P.H + h) * (kDP / 4) + dc * 2;
-            a[e][0] = __ldcg(src);
-            a[e][1] = __ldcg(src + 1);
-        }
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-            if (idx + e * stride < total)
-                dq[to[e]] = make_uint4(pack2(a[e][0].x * P.scale, a[e][0].y * P.scale), pack2(a[e][0].z * P.scale, a[e][0].w * P.scale),
-                                       pack2(a[e][1].x * P.scale, a[e][1].y * P.scale), pack2(a[e][1].z * P.scale, a[e][1].w * P.scale));
-    }
-}
-
 }  // namespace
 
 int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* d_o,
                     const int32_t* sel_idx, const int32_t* n_sel, const int32_t* inv_idx, const vardrop_attn_cfg& c, void* dq,
                     void* dk, void* dv, void* ws, cudaStream_t stream) {
+    if (attn_many_tiles(c, sel_idx)) return attn_bwd_many_launch(q, k, v, o, lse, d_o, sel_idx, n_sel, inv_idx, c, dq, dk, dv, ws, stream);
     const AttnWs w = attn_layout(c);
     const QkvLayout L = qkv_layout(c);
-    char* base = static_cast<char*>(ws);
-    const float scale = c.sm_scale > 0.f ? c.sm_scale : 1.f / sqrtf(static_cast<float>(c.D));
-    const long long HD = static_cast<long long>(c.H) * c.D;
-    // With many key tiles Delta is precomputed by a small kernel (every key tile's CTA would otherwise recompute it from O).
-    const bool many = attn_many_tiles(c, sel_idx);
-    if (many) {
-        PrepParams R{};
-        R.o = static_cast<const uint4*>(o); R.d_o = static_cast<const uint4*>(d_o);
-        R.delta = reinterpret_cast<float*>(base + w.delta);
-        R.dq_acc = attn_fwd_clears(c, sel_idx) ? nullptr : reinterpret_cast<float4*>(base + w.dq_acc);
-        R.q = static_cast<const __nv_bfloat16*>(q);
-        for (int i = 0; i < 2; ++i) R.staged[i] = reinterpret_cast<uint4*>(base + w.staged[i]);
-        R.sel_idx = sel_idx;
-        R.sB = L.sB; R.sN = L.sN; R.sH = L.sH;
-        R.n_sel = sel_idx ? n_sel : nullptr;
-        R.N = c.N; R.Ncap = w.Ncap; R.H = c.H; R.D = c.D; R.S = attn_sel_rows(c, sel_idx);
-        const long long work = static_cast<long long>(w.Ncap) * c.H * 8;
-        int gx = static_cast<int>((work + 255) / 256);
-        const int cap = max(1, 8 * sm_count() / c.B);              // about eight CTAs per SM in total
-        if (gx > cap) gx = cap;
-        cudaError_t perr;
-        { LaunchScope ls_(K_BWD_PREP, stream); perr = launch_chained(bwd_prep_kernel, dim3(gx, c.B), dim3(256), 0, stream, R); }
-        if (int st = check_cuda(perr, "attention: backward prep launch")) return st;
-    }
-
+    const BwdParams P = bwd_params(q, k, v, o, lse, d_o, sel_idx, n_sel, inv_idx, c, dq, dk, dv, ws);
     CUtensorMap mq{}, mk{}, mv{}, mdo{}, macc;
-    if (many && sel_idx) {
-        CUtensorMap* const maps[2] = {&mq, &mdo};
-        for (int i = 0; i < 2; ++i)
-            if (int st = make_tile_map(maps[i], base + w.staged[i], c.D, c.B, w.Ncap, c.H, w.Ncap * HD, HD, c.D)) return st;
-    } else if (!sel_idx) {
+    const long long HD = static_cast<long long>(c.H) * c.D;
+    if (!sel_idx) {
         if (int st = make_tile_map(&mq, q, c.D, c.B, c.N, c.H, L.sB, L.sN, L.sH)) return st;
         if (int st = make_tile_map(&mk, k, c.D, c.B, c.N, c.H, L.sB, L.sN, L.sH)) return st;
         if (int st = make_tile_map(&mv, v, c.D, c.B, c.N, c.H, L.sB, L.sN, L.sH)) return st;
         if (int st = make_tile_map(&mdo, d_o, c.D, c.B, c.N, c.H, c.N * HD, HD, c.D)) return st;
     }
-    if (int st = make_acc_map(&macc, base + w.dq_acc, c.B, w.Ncap, c.H)) return st;
-    BwdParams P{};
-    P.q = static_cast<const __nv_bfloat16*>(q); P.k = static_cast<const __nv_bfloat16*>(k); P.v = static_cast<const __nv_bfloat16*>(v);
-    P.d_o = static_cast<const __nv_bfloat16*>(d_o); P.o = static_cast<const __nv_bfloat16*>(o);
-    P.lse = lse; P.delta = many ? reinterpret_cast<const float*>(base + w.delta) : nullptr;
-    P.dq_acc = reinterpret_cast<float*>(base + w.dq_acc);
-    P.dq = static_cast<__nv_bfloat16*>(dq); P.dk = static_cast<__nv_bfloat16*>(dk); P.dv = static_cast<__nv_bfloat16*>(dv);
-    P.sel_idx = sel_idx; P.n_sel = sel_idx ? n_sel : nullptr;
-    P.inv_idx = sel_idx ? inv_idx : nullptr;
-    P.tile_done = reinterpret_cast<int32_t*>(base + w.delta);
-    P.status = reinterpret_cast<int*>(base);
-    P.sB = L.sB; P.sN = L.sN; P.sH = L.sH;
-    P.B = c.B; P.N = c.N; P.Ncap = w.Ncap; P.H = c.H; P.D = c.D; P.S = attn_sel_rows(c, sel_idx);
-    P.scale = scale; P.scale_log2 = scale * 1.4426950408889634f;
+    if (int st = make_acc_map(&macc, static_cast<char*>(ws) + w.dq_acc, c.B, w.Ncap, c.H)) return st;
     const long long worst = static_cast<long long>(w.Ncap / kTile) * c.H * c.B;
     const int grid = static_cast<int>(worst < sm_count() ? worst : sm_count());          // one CTA per SM (all of tensor memory)
     auto launch = [&](auto kernel, int& attr_dev) {
@@ -1297,30 +961,8 @@ int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, 
         LaunchScope ls_(K_ATTN_BWD, stream);
         return check_cuda(launch_chained(kernel, dim3(grid), dim3(kBwdThreads), kBwdSmemBytes, stream, mq, mk, mv, mdo, macc, P), "attention: backward launch");
     };
-    static thread_local int attr_few = -1, attr_mixed = -1, attr_many = -1, attr_rows = -1, attr_help = -1;
-    const bool help = sel_idx && c.N <= kHelpZerosN;
-    if (int st = many                  ? (help      ? launch(attn_bwd_kernel<true, false, true, true>, attr_help)
-                                         : sel_idx ? launch(attn_bwd_kernel<true, false, false, true>, attr_rows)
-                                                   : launch(attn_bwd_kernel<true, false, false, false>, attr_many))
-                 : sel_idx && P.S > 1 ? launch(attn_bwd_kernel<false, true, false, false>, attr_mixed)
-                                      : launch(attn_bwd_kernel<false, false, false, false>, attr_few))
-        return st;
-    if (many) {
-        ConvertParams F{};
-        F.dq_acc = reinterpret_cast<const float4*>(base + w.dq_acc);
-        F.dq = static_cast<uint4*>(dq);
-        F.sel_idx = sel_idx;
-        F.n_sel = sel_idx ? n_sel : nullptr;
-        F.N = c.N; F.Ncap = w.Ncap; F.H = c.H; F.D = c.D; F.S = attn_sel_rows(c, sel_idx); F.scale = scale;
-        const long long work = static_cast<long long>(c.N) * c.H * (c.D / 8);
-        int gx = static_cast<int>((work + 255) / 256);
-        const int cap = max(1, 8 * sm_count() / c.B);
-        if (gx > cap) gx = cap;
-        cudaError_t cerr;
-        { LaunchScope ls_(K_BWD_CONVERT, stream); cerr = launch_chained(bwd_convert_kernel, dim3(gx, c.B), dim3(256), 0, stream, F); }
-        if (int st = check_cuda(cerr, "attention: backward convert launch")) return st;
-    }
-    return VARDROP_OK;
+    static thread_local int attr_few = -1, attr_mixed = -1;
+    return sel_idx && P.S > 1 ? launch(attn_bwd_kernel<true>, attr_mixed) : launch(attn_bwd_kernel<false>, attr_few);
 }
 
 }  // namespace vardrop

@@ -113,9 +113,8 @@ __device__ __forceinline__ void copy_tile_rows(unsigned char* tile, const __nv_b
 }
 // One warp's share of a tile when the whole CTA loads: 32 rows from tok0 on.  (Two loader warps need some 500 cycles a tile, bound by
 // the latency of their address chains; a dozen warps bring the first tiles of a CTA in together.)
-__device__ __forceinline__ void copy_32_rows(unsigned char* rows, const __nv_bfloat16* base, long long sN, const int32_t* idx, int tok0, int n_valid, int D) {
-    const int lane = threadIdx.x & 31, chunk = lane & 7, slot = tok0 + lane;
-    const int pick = slot < n_valid ? (idx ? __ldg(idx + slot) : slot) : -1;
+__device__ __forceinline__ void copy_32_picked(unsigned char* rows, const __nv_bfloat16* base, long long sN, int pick, int D) {      // pick: this lane's row, -1: none
+    const int lane = threadIdx.x & 31, chunk = lane & 7;
     const uint32_t live = chunk * 8 < D ? 16u : 0u;
     const __nv_bfloat16* src = base + (live ? chunk * 8 : 0);
     const uint32_t dst = smem_u32(rows) + (lane >> 3) * kRowBytes + (static_cast<uint32_t>(chunk ^ (lane >> 3)) << 4);
@@ -124,6 +123,10 @@ __device__ __forceinline__ void copy_32_rows(unsigned char* rows, const __nv_bfl
         const int n = __shfl_sync(0xffffffffu, pick, 4 * it + (lane >> 3));
         cp_async16((dst ^ ((it & 1) * 64u)) + it * 4 * kRowBytes, src + static_cast<long long>(max(n, 0)) * sN, n >= 0 ? live : 0u);
     }
+}
+__device__ __forceinline__ void copy_32_rows(unsigned char* rows, const __nv_bfloat16* base, long long sN, const int32_t* idx, int tok0, int n_valid, int D) {
+    const int slot = tok0 + (threadIdx.x & 31);
+    copy_32_picked(rows, base, sN, slot < n_valid ? (idx ? __ldg(idx + slot) : slot) : -1, D);
 }
 // Quotient of 0 <= a by 1 <= d in a few instructions (an integer division is some forty dependent ones); the correction loops run
 // more than once only for quotients beyond 2^22.

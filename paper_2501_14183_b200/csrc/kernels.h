@@ -73,5 +73,7 @@ int attn_fwd_launch(const void* q, const void* k, const void* v, const int32_t* 
 int attn_bwd_launch(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* d_o,
                     const int32_t* sel_idx, const int32_t* n_sel, const int32_t* inv_idx, const vardrop_attn_cfg& cfg, void* dq,
                     void* dk, void* dv, void* ws, cudaStream_t stream);
+int attn_bwd_many_launch(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* d_o, const int32_t* sel_idx,
+                         const int32_t* n_sel, const int32_t* inv_idx, const vardrop_attn_cfg& cfg, void* dq, void* dk, void* dv, void* ws, cudaStream_t stream);
 
 }  // namespace vardrop

@@ -131,6 +131,24 @@ def test_attention_large_tokens_relative_error(B, N, H, D, Ns, std):
         assert np.all(np.isfinite(got)) and err <= bound, f"{name}: max abs error {err:.3e} > {bound:.3e}"
 
 
+@pytest.mark.parametrize("N,H,D,Ns", [(257, 2, 64, None), (700, 1, 32, None), (2049, 2, 64, 130), (1030, 1, 32, 257), (300, 1, 64, 200)])
+def test_attention_scores_far_below_zero(N, H, D, Ns):
+    """Every score near -128 sqrt(D / 64): the exponential of minus a row's log-sum-exp, which a key that does not exist would get, is infinite, and the last
+    key tile has such keys.  The bound: as for large tokens."""
+    dev, _ = bf16_tokens(2, N, H, D, 0.3536, seed=N)
+    dev = [dev[0] + 4.0, dev[1] - 4.0, *dev[2:]]
+    ref = [t.double().cpu().numpy() for t in dev]
+    sel = None if Ns is None else pick(N, Ns, seed=N)
+    o, lse, dq, dk, dv, status, _ = run_attention(dev, 2, N, H, D, sel)
+    assert status == vd.OK
+    wo, wl = oracle.attn_fwd(ref[0], ref[1], ref[2], sel)
+    wq, wk, wv = oracle.attn_bwd(ref[0], ref[1], ref[2], ref[3][:, :Ns or N], sel)
+    for got, want, name in ((o, wo, "o"), (lse, wl, "lse"), (dq, wq, "dq"), (dk, wk, "dk"), (dv, wv, "dv")):
+        bound = 2e-2 * max(1.0, float(np.abs(want).max()))
+        err = float(np.abs(got - want).max())
+        assert np.all(np.isfinite(got)) and err <= bound, f"{name}: max abs error {err:.3e} > {bound:.3e}"
+
+
 @pytest.mark.parametrize("B,N,H,D,Ns", [(2, 257, 2, 64, None), (1, 300, 2, 32, None), (2, 384, 1, 64, None), (1, 385, 2, 64, None), (1, 862, 1, 64, None), (1, 2049, 2, 64, 300)])
 def test_attention_probabilities_are_rounded_against_the_first_keys(B, N, H, D, Ns):
     """P is rounded to bf16 relative to the maximum of a row's first 64 keys, whichever kernel serves the call: with that rounding written out
