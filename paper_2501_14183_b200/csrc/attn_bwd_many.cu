@@ -72,15 +72,15 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const PrepParams P) {
 // main
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kManyThreads = 896;
-// Register split (setmaxnreg works on whole warpgroups): launched with 896 x 72 = 64512 registers; the teams take 80, the
-// others keep 56: 384 x 56 + 512 x 80 = 62464.
+// Register split (setmaxnreg works on whole warpgroups): launched with 896 x 72 = 64512 registers; the first warpgroup keeps 56 a
+// thread, the two that take results out 64, the teams take 80: 128 x 56 + 256 x 64 + 512 x 80 = 64512.
 constexpr int kManySmallRegs = 56;
+constexpr int kManyOutRegs = 64;
 constexpr int kManyBigRegs = 80;
 constexpr uint32_t kManyTmemCols = 512;
 constexpr int kManyStages = 3;         // ring of (Q, dO) tiles
 constexpr int kManyTeamWarps = 8;
-constexpr int kManyRowsBytes = 1024;   // a warp's way out for rows of dV, dK: 32 rows of 16 columns
-constexpr int kManyHeader = 8192 + 8 * kManyRowsBytes;         // barriers, item list, row statistics; rows on their way out
+constexpr int kManyHeader = 7168;      // barriers, item list, row statistics
 constexpr int kManySmemBytes = kManyHeader + 3 * kTileBytes /*K of two items, V*/ + 2 * kManyStages * kTileBytes /*ring*/ + 2 * kTileBytes /*dS^T, two 64-query panels*/ +
                                2 * kTileBytes /*staging: dQ as fp32, two 32-column panels; dV, dK as bf16*/;
 
@@ -137,7 +137,7 @@ __device__ __forceinline__ bool group_sync_and(int id, bool ok) {     // barrier
 // 64 w to 64 w + 63 of every query tile.
 //   warp 0       issues S^T = K Q^T and dV += P^T dO of both teams (all lanes run the issue code, an elected lane executes a group of products)
 //   warp 1       issues dP^T = V dO^T and dK += dS^T Q of both teams
-//   warp 2       issues dQ = dS K of a query tile once both teams have handed over their dS^T
+//   warp 2       issues dQ = dS K of a query tile once both teams have handed over their dS^T; copies K and V of the next item to tensor memory
 //   warp 3       loads K, V of the items (boxes) and a ring of (Q, dO) tiles with their row statistics; decodes the items
 //   warps 4-7    columns 0 to 31 of dQ from tensor memory into the accumulator; dV of a finished item; K rows of a selection
 //   warps 8-11   columns 32 to 63; dK of a finished item; V rows of a selection
@@ -151,7 +151,7 @@ __device__ __forceinline__ bool group_sync_and(int id, bool ok) {     // barrier
 //     (64 broadcast loads a row and step), and without their registers nothing spills.
 //   - The tensor core runs the products of one thread in order: S^T of the next query tile goes over P^T right behind the dV that reads it, dP^T over dS^T
 //     behind dK, so a team hands over three times a step and waits for neither.
-//   - At the end of an item the issuing warps copy the next K and V and go on; the teams never leave the steps.
+//   - At the end of an item the next K and V are copied in behind the last products that read the old ones; the teams never leave the steps.
 // Two 128-key tiles a CTA, a team each, with K and V from shared memory (before this), took 3500 cycles for as many scores: forward and backward, B = 8, H = 8,
 // 8192 variates 4820 -> 4570 us, 1423 of 8192 kept 258 -> 243; 700 of 8192 171 -> 120; B = 32, 862 variates 347 -> 328.
 // Tensor memory: K 32 | V 32 | dV 64 | dK 64 | dQ 64 | team 0: S^T, P^T 64, dP^T, dS^T 64 | team 1.
@@ -182,14 +182,14 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
     uint64_t* bar_dk_free = bars + 24;
     uint64_t* bar_gfree = bars + 25;                // dQ of a query tile in registers
     uint64_t* bar_panel = bars + 26;                // [2] dS^T in shared memory
-    uint64_t* bar_item = bars + 28;                 // [8] entry of the item list is written
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 36);
+    uint64_t* bar_kv = bars + 28;                   // [2] K, V of an item in tensor memory
+    uint64_t* bar_item = bars + 30;                 // [8] entry of the item list is written
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
     struct alignas(16) Item { int jt, h, b, n_sel; };               // n_sel < 0 ends the list
     Item* s_item = reinterpret_cast<Item*>(smem_dyn + 320);         // [8]
     uint4* s_ones = reinterpret_cast<uint4*>(smem_dyn + 512);       // [3][8] bf16 rows that pick -lse, -Delta, nothing
     uint4* s_stats = s_ones + 24;                                   // [kManyStages][128] -lse / scale of the slot's rows in three bf16 terms, -Delta in three
-    unsigned char* s_rows = smem_dyn + 8192;                        // a piece of each warp that takes results out
-    static_assert(512 + (24 + kManyStages * kTile) * sizeof(uint4) <= 8192, "header too small");
+    static_assert(512 + (24 + kManyStages * kTile) * sizeof(uint4) <= kManyHeader, "header too small");
     unsigned char* sK = smem_dyn + kManyHeader;                     // K of two items
     unsigned char* sV = sK + 2 * kTileBytes;
     unsigned char* sQ = sV + kTileBytes;                            // slots of (Q tile, dO tile)
@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             mbar_init(bar_p + w, kManyTeamWarps);
             mbar_init(bar_ds + w, kManyTeamWarps);
             mbar_init(bar_panel + w, kManyTeamWarps);
+            mbar_init(bar_kv + w, 1);
         }
         mbar_init(bar_v_full, kRows ? 128 : 1);
         mbar_init(bar_v_free, 1);
@@ -277,7 +278,6 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
         // Warp 0: S^T from K and Q, dV from P^T and dO.  Warp 1: dP^T from V and dO, dK from dS^T and Q.  One body: `first` is the product that opens a
         // step, `second` the one that adds up.
         const uint32_t idesc_first = umma_idesc_bf16(128, 64, 0, 0), idesc_second = umma_idesc_bf16(128, P.D, 0, 1);
-        const uint64_t d_kv = umma_desc_sw128(smem_u32(warp == 0 ? sK : sV), 16, 1024);
         const uint64_t d_q = umma_desc_sw128(smem_u32(sQ) + (warp == 0 ? 0 : kTileBytes), 16, 1024);                 // operand of the first product
         const uint64_t m_q = umma_desc_sw128(smem_u32(sQ) + (warp == 0 ? kTileBytes : 0), kTileBytes, 1024);         // of the second
         const uint32_t c_kv = tmem + (warp == 0 ? kColK : kColV), c_acc = tmem + (warp == 0 ? kColDv : kColDk), c_team = tmem + kColTeam + warp * 64;
@@ -287,18 +287,6 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
         uint64_t* bar_done = warp == 0 ? bar_dv_done : bar_dk_done;
         uint64_t* bar_free = warp == 0 ? bar_dv_free : bar_dk_free;
         uint32_t t = 0, st = 0, ph = 0, sn = 0, pn = 0;        // query tiles so far, their slot; slot of the tile whose first products come next
-        auto copy_kv = [&](uint32_t i) {                       // this item's K or V to tensor memory
-            ok &= warp == 0 ? warp_wait_relaxed(bar_k_full + (i & 1), (i >> 1) & 1) : warp_wait_relaxed(bar_v_full, i & 1);
-            if (kRows) fence_proxy_async_smem();               // rows written by asynchronous copies are read by the tensor core
-            tc_fence_after();
-            if (elect_one()) {
-                const uint64_t from = umma_desc_advance(d_kv, warp == 0 ? (i & 1) * kTileBytes : 0);
-#pragma unroll 1
-                for (int ks = 0; ks < P.D / 16; ++ks) tc_copy_128x256b(c_kv + ks * 8, umma_desc_advance(from, ks * 32));
-                if (warp == 1) tc_commit(bar_v_free);
-            }
-            __syncwarp();
-        };
         auto wait_slot = [&]() {
             ok &= warp_wait_relaxed(bar_q_full + sn, pn);
             tc_fence_after();
@@ -320,7 +308,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
         };
         Item it = item_at(0);
         if (it.n_sel >= 0) {
-            copy_kv(0);
+            ok &= warp_wait(bar_kv + warp, 0);
             wait_slot();
             first(0);
             first(1);
@@ -352,10 +340,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
                     __syncwarp();
                     if (!more) continue;
                     if (w == 0) {
-                        if (last) {                            // the first products of both teams, the last to read this K (V), are done
-                            ok &= warp_wait(bar_first + 1, t & 1);
-                            copy_kv(i + 1);
-                        }
+                        if (last) ok &= warp_wait(bar_kv + warp, (i + 1) & 1);
                         wait_slot();
                     }
                     first(w);
@@ -367,19 +352,43 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
     } else if (warp == 2) {
         const uint32_t idesc_mnmn = umma_idesc_bf16(128, P.D, 1, 1);       // A MN-major, B MN-major
         const uint64_t a_ds = umma_desc_sw128(smem_u32(sdS), kTileBytes, 1024), b_k = umma_desc_sw128(smem_u32(sK), kTileBytes, 1024);
+        const uint64_t k_from = umma_desc_sw128(smem_u32(sK), 16, 1024), v_from = umma_desc_sw128(smem_u32(sV), 16, 1024);
+        auto copy_kv = [&](uint32_t i, bool v) {               // an item's K or V to tensor memory
+            ok &= v ? warp_wait_relaxed(bar_v_full, i & 1) : warp_wait_relaxed(bar_k_full + (i & 1), (i >> 1) & 1);
+            if (kRows) fence_proxy_async_smem();               // rows written by asynchronous copies are read by the tensor core
+            tc_fence_after();
+            if (elect_one()) {
+                const uint64_t from = v ? v_from : umma_desc_advance(k_from, (i & 1) * kTileBytes);
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks)
+                    if (ks < 2 || P.D > 32) tc_copy_128x256b(tmem + (v ? kColV : kColK) + ks * 8, umma_desc_advance(from, ks * 32));
+                tc_commit(bar_kv + (v ? 1 : 0));
+                if (v) tc_commit(bar_v_free);
+            }
+            __syncwarp();
+        };
         uint32_t t = 0;
+        Item it = item_at(0);
+        if (it.n_sel >= 0) {
+            copy_kv(0, false);
+            copy_kv(0, true);
+        }
 #pragma unroll 1
-        for (uint32_t i = 0; ok; ++i) {
-            const Item it = item_at(i);
-            if (it.n_sel < 0) break;
+        for (uint32_t i = 0; ok && it.n_sel >= 0; ++i) {
             const int n_q = (it.n_sel + kTile - 1) / kTile;
             const uint64_t bk = umma_desc_advance(b_k, (i & 1) * kTileBytes);
+            it = item_at(i + 1);
 #pragma unroll 1
             for (int x = 0; x < n_q && ok; ++x, ++t) {
+                if (x + 1 == n_q && it.n_sel >= 0) {           // the last products that read this K (V) are both teams' first ones of this tile
+                    ok &= warp_wait(bar_s + 1, t & 1);
+                    copy_kv(i + 1, false);
+                    ok &= warp_wait(bar_dp + 1, t & 1);
+                    copy_kv(i + 1, true);
+                }
                 if (t > 0) ok &= warp_wait_relaxed(bar_gfree, (t - 1) & 1);
                 ok &= warp_wait(bar_panel, t & 1);
                 ok &= warp_wait(bar_panel + 1, t & 1);
-                if (kRows && x == 0) fence_proxy_async_smem();             // K's rows
                 tc_fence_after();
                 if (elect_one()) {                       // dQ = dS K, dS the transposed view of dS^T
 #pragma unroll
@@ -476,9 +485,9 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
     }
     } else if (warp < 12) {
         // ------------------------------------------------------------ dQ; dV, dK of an item -----------------------------
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kManySmallRegs));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kManyOutRegs));
         begin();
-        const int g = (warp >> 2) - 1, id = 1 + g, row = tid & (kTile - 1), c8 = row & 7, r8 = row >> 3;
+        const int g = (warp >> 2) - 1, id = 1 + g, row = tid & (kTile - 1);
         const uint32_t tm = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const bool owner = row == 0, columns = g * 32 < P.D;     // the one thread of the warpgroup that owns its bulk reductions; there are such columns
         unsigned char* panel = sOut + g * kTileBytes;            // this warpgroup's staging panel of 128-byte swizzled rows
@@ -504,47 +513,49 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             const Item it = item_at(i);
             if (it.n_sel < 0) { ok = group_sync_and(id, ok); break; }
             const int n_q = (it.n_sel + kTile - 1) / kTile;
-            // dV or dK of the item's keys, a warp's 32 rows through its piece of shared memory, 16 columns at a time, two lanes a row
+            // dV or dK of the item's keys: a warp's 32 rows through its part of the panel, eight lanes a row
             auto rows_out = [&](uint32_t col, uint64_t* done, uint64_t* freed, float mul, __nv_bfloat16* dst) {
-                const int32_t* sel = P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N;
-                unsigned char* piece = s_rows + (warp - 4) * kManyRowsBytes;
-                __nv_bfloat16* out[2];
-                bool live[2];
+                int n[8];                                // variates of this lane's rows, -1: none
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int key = it.jt * kTile + (warp & 3) * 32 + 16 * e + (lane >> 1);
-                    live[e] = key < it.n_sel;
-                    const int n = live[e] ? (kRows ? __ldg(sel + key) : key) : 0;
-                    out[e] = dst + ((static_cast<size_t>(it.b) * P.N + n) * P.H + it.h) * P.D + (lane & 1) * 8;
+                for (int e = 0; e < 8; ++e) {
+                    const int key = it.jt * kTile + (warp & 3) * 32 + 4 * e + (lane >> 3);
+                    n[e] = key < it.n_sel ? (kRows ? __ldg(P.sel_idx + static_cast<size_t>(P.S > 1 ? it.b : 0) * P.N + key) : key) : -1;
                 }
+                panel_free();
                 ok &= warp_wait_relaxed(done, i & 1);
                 tc_fence_after();
 #pragma unroll 1
-                for (int c = 0; c < P.D; c += 16) {
-                    float v[16];
-                    tmem_ld16(tm + col + c, v);
+                for (int c = 0; c < P.D; c += 32) {
+                    float v[32];
+                    tmem_ld32(tm + col + c, v);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int q = 0; q < 2; ++q)
-                        *reinterpret_cast<uint4*>(piece + lane * 32 + ((q ^ ((lane >> 2) & 1)) << 4)) =
+                    for (int q = 0; q < 4; ++q)
+                        *reinterpret_cast<uint4*>(rowp + (((c / 8 + q) ^ (row & 7)) << 4)) =
                             make_uint4(pack2(v[8 * q + 0] * mul, v[8 * q + 1] * mul), pack2(v[8 * q + 2] * mul, v[8 * q + 3] * mul),
                                        pack2(v[8 * q + 4] * mul, v[8 * q + 5] * mul), pack2(v[8 * q + 6] * mul, v[8 * q + 7] * mul));
-                    __syncwarp();
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int r = 16 * e + (lane >> 1);
-                        if (live[e]) *reinterpret_cast<uint4*>(out[e] + c) = *reinterpret_cast<const uint4*>(piece + r * 32 + (((lane & 1) ^ ((r >> 2) & 1)) << 4));
-                    }
-                    __syncwarp();
                 }
                 tc_fence_before();
-                warp_arrive(freed);
+                warp_arrive(freed);                      // the next item's products wait for these columns
+                const int c8 = lane & 7;
+                if (c8 * 8 < P.D) {
+                    __nv_bfloat16* out = dst + (static_cast<size_t>(it.b) * P.N * P.H + it.h) * P.D + c8 * 8;
+                    const unsigned char* from = panel + ((warp & 3) * 32 + (lane >> 3)) * kRowBytes;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (n[e] >= 0)
+                            *reinterpret_cast<uint4*>(out + static_cast<size_t>(n[e]) * P.H * P.D) =
+                                *reinterpret_cast<const uint4*>(from + 4 * e * kRowBytes + ((c8 ^ ((4 * e + (lane >> 3)) & 7)) << 4));
+                }
             };
             // The next item's rows ahead of anything that waits for this one's products: those of its last query tile come behind them.
             if (kRows) load_rows(i + 1, item_at(i + 1));
 #pragma unroll 1
             for (int x = 0; x < n_q && ok; ++x, ++t) {
-                if (g == 0 && x + 1 == n_q) rows_out(kColDv, bar_dv_done, bar_dv_free, 1.f, P.dv);      // complete ahead of the item's last dQ
+                if (x + 1 == n_q) {                      // complete ahead of the item's last dQ, and about when it is
+                    if (g == 0) rows_out(kColDv, bar_dv_done, bar_dv_free, 1.f, P.dv);
+                    else rows_out(kColDk, bar_dk_done, bar_dk_free, P.scale, P.dk);
+                }
                 panel_free();
                 ok &= warp_wait_relaxed(bar_g, t & 1);
                 tc_fence_after();
@@ -567,8 +578,6 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
                     bulk_commit_group();
                 }
             }
-            if (!ok) break;
-            if (g == 1) rows_out(kColDk, bar_dk_done, bar_dk_free, P.scale, P.dk);
             if (!ok) break;
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
