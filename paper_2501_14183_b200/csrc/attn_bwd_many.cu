@@ -93,10 +93,10 @@ __device__ __forceinline__ void tc_copy_128x256b(uint32_t taddr, uint64_t desc) 
 __device__ __forceinline__ uint64_t umma_desc_plain(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
     return umma_desc_sw128(smem_addr, lbo_bytes, sbo_bytes) & ~(7ull << 61);
 }
-// x as three bf16 terms (24 bits), each in the low half of a word
+// x as three bf16 terms (24 bits), each in the low half of a word; one that is not finite as a single one
 __device__ __forceinline__ void split3(float x, uint32_t& a, uint32_t& b, uint32_t& c) {
     const __nv_bfloat16 h = __float2bfloat16_rn(x);
-    const float r = x - __bfloat162float(h);
+    const float r = fabsf(x) < INFINITY ? x - __bfloat162float(h) : 0.f;
     const __nv_bfloat16 m = __float2bfloat16_rn(r);
     a = __bfloat16_as_ushort(h);
     b = __bfloat16_as_ushort(m);
@@ -153,7 +153,7 @@ __device__ __forceinline__ bool group_sync_and(int id, bool ok) {     // barrier
 //     behind dK, so a team hands over three times a step and waits for neither.
 //   - At the end of an item the next K and V are copied in behind the last products that read the old ones; the teams never leave the steps.
 // Two 128-key tiles a CTA, a team each, with K and V from shared memory (before this), took 3500 cycles for as many scores: forward and backward, B = 8, H = 8,
-// 8192 variates 4820 -> 4570 us, 1423 of 8192 kept 258 -> 243; 700 of 8192 171 -> 120; B = 32, 862 variates 347 -> 328.
+// 8192 variates 4810 -> 4560 us, 1423 of 8192 kept 258 -> 235; 700 of 8192 171 -> 109; B = 32, 862 variates 346 -> 321.
 // Tensor memory: K 32 | V 32 | dV 64 | dK 64 | dQ 64 | team 0: S^T, P^T 64, dP^T, dS^T 64 | team 1.
 constexpr uint32_t kColK = 0, kColV = 32, kColDv = 64, kColDk = 128, kColDq = 192, kColTeam = 256;
 
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
         mbar_init(bar_v_full, kRows ? 128 : 1);
         mbar_init(bar_v_free, 1);
         for (int s = 0; s < kManyStages; ++s) {
-            mbar_init(bar_q_full + s, 1);
+            mbar_init(bar_q_full + s, 2);                     // the boxes' announcing arrival, the statistics
             mbar_init(bar_q_free + s, 2);
         }
         mbar_init(bar_g, 1);
@@ -431,6 +431,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             }
             __syncwarp();
         };
+        const float inv_scale = 1.f / P.scale;
         uint32_t st = 0, ph = 0;
         publish(0);
         Item next = item_at(0);
@@ -457,27 +458,24 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             stats_load(0);
 #pragma unroll 1
             for (int x = 0; x < n_q; ++x) {
-                uint4 terms[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    uint32_t l[3], d[3];
-                    split3(__fdividef(-st_lse[e], P.scale), l[0], l[1], l[2]);
-                    split3(-st_delta[e], d[0], d[1], d[2]);
-                    terms[e] = make_uint4(l[0] | l[1] << 16, l[2] | d[0] << 16, d[1] | d[2] << 16, 0u);
-                }
-                stats_load(x + 1);
                 ok = warp_wait_relaxed(bar_q_free + st, ph ^ 1);
                 if (!ok) break;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) s_stats[st * kTile + e * 32 + lane] = terms[e];
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
+                if (lane == 0) {                         // the tiles first: the products wait for them a step ahead of anything the statistics are for
                     mbar_expect_tx(bar_q_full + st, 2 * kTileBytes);
                     tma_load_4d(sQ + st * 2 * kTileBytes, &map_q, bar_q_full + st, 0, it.h, x * kTile, it.b);
                     tma_load_4d(sQ + st * 2 * kTileBytes + kTileBytes, &map_do, bar_q_full + st, 0, it.h, x * kTile, it.b);
                 }
                 __syncwarp();
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    uint32_t l[3], d[3];
+                    split3(-st_lse[e] * inv_scale, l[0], l[1], l[2]);
+                    split3(-st_delta[e], d[0], d[1], d[2]);
+                    s_stats[st * kTile + e * 32 + lane] = make_uint4(l[0] | l[1] << 16, l[2] | d[0] << 16, d[1] | d[2] << 16, 0u);
+                }
+                fence_proxy_async_smem();
+                warp_arrive(bar_q_full + st);
+                stats_load(x + 1);
                 next_slot(st, ph);
                 if (!kRows && x == (n_q > 1 ? 1 : 0) && next.n_sel >= 0) load_kv(i + 1, next);
             }
@@ -668,7 +666,8 @@ __global__ void __launch_bounds__(256) bwd_convert_kernel(const ConvertParams P)
         const int lane = threadIdx.x & 31, rows = P.B * P.N, row_chunks = P.H * (P.D / 8);
         const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
         // Eight CTAs fit an SM.  The first ones come in where the main kernel has an item less; they take as many rows more as an item is long (2700 cycles a
-        // query tile, 25 bytes written a cycle and SM).
+        // query tile, 25 bytes written a cycle and SM), as long as the late ones keep the early ones' part of an even share (with the early ones taking all they
+        // have time for: 2400 of 8192 kept 522 -> 520 us forward and backward, but 300 of 3000, B = 2 32.7 -> 33.1, 102 of 2049, B = 32 66.0 -> 67.2).
         const int kept = largest_kept(P.n_sel, P.S, P.N), n_t = (kept + kTile - 1) / kTile, n_long = n_t * P.H * P.B % P.main_grid;
         const int ctas = static_cast<int>(gridDim.x * gridDim.y), cta = static_cast<int>(blockIdx.y * gridDim.x + blockIdx.x);
         const int n_early = n_long ? min(ctas, 8 * (P.main_grid - n_long)) : 0;
