@@ -153,7 +153,7 @@ __device__ __forceinline__ bool group_sync_and(int id, bool ok) {     // barrier
 //     behind dK, so a team hands over three times a step and waits for neither.
 //   - At the end of an item the next K and V are copied in behind the last products that read the old ones; the teams never leave the steps.
 // Two 128-key tiles a CTA, a team each, with K and V from shared memory (before this), took 3500 cycles for as many scores: forward and backward, B = 8, H = 8,
-// 8192 variates 4810 -> 4560 us, 1423 of 8192 kept 258 -> 235; 700 of 8192 171 -> 109; B = 32, 862 variates 346 -> 321.
+// 8192 variates 4810 -> 4560 us, 1423 of 8192 kept 258 -> 243 (by events), 700 of 8192 171 -> 120; B = 32, 862 variates 346 -> 321.
 // Tensor memory: K 32 | V 32 | dV 64 | dK 64 | dQ 64 | team 0: S^T, P^T 64, dP^T, dS^T 64 | team 1.
 constexpr uint32_t kColK = 0, kColV = 32, kColDv = 64, kColDk = 128, kColDq = 192, kColTeam = 256;
 
