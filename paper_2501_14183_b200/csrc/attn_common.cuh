@@ -144,7 +144,7 @@ __device__ __forceinline__ int small_div(int a, int d) {
 // operand tiles and the conversion of dQ' from launches of their own): the kept count is only known on the device, so the host goes by the
 // largest it can be.  A selection keeps a fraction of the variates (a tenth to a third in the paper's settings); up to kManyTilesN variates that
 // is a handful of tiles.  With few heads and instances a tile's latency counts for more than the launches, and the line lies lower.  Forward and
-// backward, B = 8, H = 8, few | many: 200 of 2000 kept 31 | 48 us, 400 57 | 56, 1000 153 | 130; B = 1: 400 of 2000 42 | 40, 1000 86 | 63.
+// backward, B = 8, H = 8, few | many: 200 of 2000 kept 29 | 34 us, 400 56 | 48, 1000 153 | 115; B = 1: 110 of 1100 14 | 20, 200 of 2000 23 | 24, 400 41 | 31, 1000 85 | 44.
 constexpr int kManyTilesN = 2048, kManyTilesSmallN = 1024, kSmallHeads = 32;
 inline bool attn_many_tiles(const vardrop_attn_cfg& c, const int32_t* sel_idx) {
     return sel_idx ? c.N > (c.B * c.H < kSmallHeads ? kManyTilesSmallN : kManyTilesN) : c.N > 2 * kTile;
