@@ -80,7 +80,7 @@ constexpr int kManyBigRegs = 80;
 constexpr uint32_t kManyTmemCols = 512;
 constexpr int kManyStages = 3;         // ring of (Q, dO) tiles
 constexpr int kManyTeamWarps = 8;
-constexpr int kManyHeader = 7168;      // barriers, item list, row statistics
+constexpr int kManyHeader = 13312;     // barriers, item list, row statistics
 constexpr int kManySmemBytes = kManyHeader + 3 * kTileBytes /*K of two items, V*/ + 2 * kManyStages * kTileBytes /*ring*/ + 2 * kTileBytes /*dS^T, two 64-query panels*/ +
                                2 * kTileBytes /*staging: dQ as fp32, two 32-column panels; dV, dK as bf16*/;
 
@@ -93,7 +93,7 @@ __device__ __forceinline__ void tc_copy_128x256b(uint32_t taddr, uint64_t desc) 
 __device__ __forceinline__ uint64_t umma_desc_plain(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
     return umma_desc_sw128(smem_addr, lbo_bytes, sbo_bytes) & ~(7ull << 61);
 }
-// x as three bf16 terms (24 bits), each in the low half of a word; one that is not finite as a single one
+// x as three bf16 terms (24 bits), each in the low half of a word; one that is not finite as a single one.  (Below 1.7e38 in magnitude no term rounds to infinity.)
 __device__ __forceinline__ void split3(float x, uint32_t& a, uint32_t& b, uint32_t& c) {
     const __nv_bfloat16 h = __float2bfloat16_rn(x);
     const float r = fabsf(x) < INFINITY ? x - __bfloat162float(h) : 0.f;
@@ -148,7 +148,9 @@ __device__ __forceinline__ bool group_sync_and(int id, bool ok) {     // barrier
 //   - A operands come from tensor memory wherever they can (K and V copied there once an item, P^T, dS^T): a product of N = 64 then takes 32 cycles
 //     instead of 48, 1600 a step instead of 1920, and the shared-memory pipe 2200 instead of 2800.
 //   - -lse / scale and -Delta of a query are three bf16 terms each (24 bits) of a fifth k-step of S^T and dP^T, against rows of ones: no thread reads them
-//     (64 broadcast loads a row and step), and without their registers nothing spills.
+//     (64 broadcast loads a row and step), and without their registers nothing spills.  Each product has rows of its own and meets them with ones and with the
+//     zeros behind the terms only: a row of both, picked from by ones and zeros, takes a Delta that is not finite into S^T (0 times infinity), and so into every
+//     column of dV.  (6 KB more of shared memory; no difference in time that shows.)
 //   - The tensor core runs the products of one thread in order: S^T of the next query tile goes over P^T right behind the dV that reads it, dP^T over dS^T
 //     behind dK, so a team hands over three times a step and waits for neither.
 //   - At the end of an item the next K and V are copied in behind the last products that read the old ones; the teams never leave the steps.
@@ -187,9 +189,9 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
     struct alignas(16) Item { int jt, h, b, n_sel; };               // n_sel < 0 ends the list
     Item* s_item = reinterpret_cast<Item*>(smem_dyn + 320);         // [8]
-    uint4* s_ones = reinterpret_cast<uint4*>(smem_dyn + 512);       // [3][8] bf16 rows that pick -lse, -Delta, nothing
-    uint4* s_stats = s_ones + 24;                                   // [kManyStages][128] -lse / scale of the slot's rows in three bf16 terms, -Delta in three
-    static_assert(512 + (24 + kManyStages * kTile) * sizeof(uint4) <= kManyHeader, "header too small");
+    uint4* s_ones = reinterpret_cast<uint4*>(smem_dyn + 512);       // [8] bf16 rows of three ones
+    uint4* s_stats = s_ones + 8;                                    // [2][kManyStages][128] three bf16 terms of half of -lse / scale, of half of -Delta, of the slot's rows
+    static_assert(512 + (8 + 2 * kManyStages * kTile) * sizeof(uint4) <= kManyHeader, "header too small");
     unsigned char* sK = smem_dyn + kManyHeader;                     // K of two items
     unsigned char* sV = sK + 2 * kTileBytes;
     unsigned char* sQ = sV + kTileBytes;                            // slots of (Q tile, dO tile)
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
         }
         tma_prefetch_desc(&map_acc);
     }
-    if (tid < 24) s_ones[tid] = tid < 8 ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : tid < 16 ? make_uint4(0u, 0x3f800000u, 0x3f803f80u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+    if (tid < 8) s_ones[tid] = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -281,7 +283,8 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
         const uint64_t d_q = umma_desc_sw128(smem_u32(sQ) + (warp == 0 ? 0 : kTileBytes), 16, 1024);                 // operand of the first product
         const uint64_t m_q = umma_desc_sw128(smem_u32(sQ) + (warp == 0 ? kTileBytes : 0), kTileBytes, 1024);         // of the second
         const uint32_t c_kv = tmem + (warp == 0 ? kColK : kColV), c_acc = tmem + (warp == 0 ? kColDv : kColDk), c_team = tmem + kColTeam + warp * 64;
-        const uint64_t d_ones = umma_desc_plain(smem_u32(s_ones + 8 * warp), (2 - warp) * 128, 0), d_stats = umma_desc_plain(smem_u32(s_stats), 0, 128);
+        // A k-step is two rows of eight: both are the same one, whence the halves.
+        const uint64_t d_ones = umma_desc_plain(smem_u32(s_ones), 0, 0), d_stats = umma_desc_plain(smem_u32(s_stats + warp * kManyStages * kTile), 0, 128);
         uint64_t* bar_first = warp == 0 ? bar_s : bar_dp;
         uint64_t* bar_handed = warp == 0 ? bar_p : bar_ds;
         uint64_t* bar_done = warp == 0 ? bar_dv_done : bar_dk_done;
@@ -431,7 +434,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             }
             __syncwarp();
         };
-        const float inv_scale = 1.f / P.scale;
+        const float half_inv = 0.5f / P.scale;
         uint32_t st = 0, ph = 0;
         publish(0);
         Item next = item_at(0);
@@ -469,9 +472,10 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     uint32_t l[3], d[3];
-                    split3(-st_lse[e] * inv_scale, l[0], l[1], l[2]);
-                    split3(-st_delta[e], d[0], d[1], d[2]);
-                    s_stats[st * kTile + e * 32 + lane] = make_uint4(l[0] | l[1] << 16, l[2] | d[0] << 16, d[1] | d[2] << 16, 0u);
+                    split3(-st_lse[e] * half_inv, l[0], l[1], l[2]);
+                    split3(-0.5f * st_delta[e], d[0], d[1], d[2]);
+                    s_stats[st * kTile + e * 32 + lane] = make_uint4(l[0] | l[1] << 16, l[2], 0u, 0u);
+                    s_stats[(kManyStages + st) * kTile + e * 32 + lane] = make_uint4(d[0] | d[1] << 16, d[2], 0u, 0u);
                 }
                 fence_proxy_async_smem();
                 warp_arrive(bar_q_full + st);

@@ -165,6 +165,26 @@ def test_attention_probabilities_are_rounded_against_the_first_keys(B, N, H, D, 
     assert float((got - want).norm() / want.norm()) <= 3.6e-4
 
 
+@pytest.mark.parametrize("where", ["v", "d_o"])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+@pytest.mark.parametrize("N,D,Ns", [(256, 64, None), (257, 64, None), (700, 32, None), (300, 64, 200), (1030, 32, 129), (2049, 64, 300)])
+def test_attention_one_element_that_is_not_finite(N, D, Ns, value, where):
+    """An infinity or NaN in one element of V or dO: the gradients that are finite by the chain rule are so (dV of an element of V, every other column of dV of one of dO, the
+    other head), whichever kernel serves the call, and within the tolerance."""
+    dev, _ = bf16_tokens(1, N, 2, D, 1.0, seed=N)
+    sel = None if Ns is None else pick(N, Ns, seed=N)
+    dev["q k v d_o".split().index(where)][0, int(sel[5]) if sel is not None and where == "v" else 5, 1, 7] = value
+    o, _, dq, dk, dv, status, _ = run_attention(dev, 1, N, 2, D, sel)
+    assert status == vd.OK
+    ref = [t.double().cpu().numpy() for t in dev]
+    wo, _ = oracle.attn_fwd(ref[0], ref[1], ref[2], sel)
+    wq, wk, wv = oracle.attn_bwd(ref[0], ref[1], ref[2], ref[3][:, :Ns or N], sel)
+    for got, want, name in ((o, wo, "o"), (dq, wq, "dq"), (dk, wk, "dk"), (dv, wv, "dv")):
+        finite = np.isfinite(want)
+        assert finite.any() and np.array_equal(np.isfinite(got), finite), name
+        assert_attn_close(got[finite], want[finite], name)
+
+
 def test_attention_identity_selection_equals_all_token_path():
     B, N, H, D = 1, 200, 2, 64
     dev, _ = bf16_tokens(B, N, H, D, 1.0, seed=3)
