@@ -186,12 +186,13 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
     uint64_t* bar_panel = bars + 26;                // [2] dS^T in shared memory
     uint64_t* bar_kv = bars + 28;                   // [2] K, V of an item in tensor memory
     uint64_t* bar_item = bars + 30;                 // [8] entry of the item list is written
+    uint64_t* bar_left = bars + 39;                 // [3] what an issuing warp whose wait gave up has issued is done
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
     struct alignas(16) Item { int jt, h, b, n_sel; };               // n_sel < 0 ends the list
-    Item* s_item = reinterpret_cast<Item*>(smem_dyn + 320);         // [8]
+    Item* s_item = reinterpret_cast<Item*>(smem_dyn + 384);         // [8]
     uint4* s_ones = reinterpret_cast<uint4*>(smem_dyn + 512);       // [8] bf16 rows of three ones
     uint4* s_stats = s_ones + 8;                                    // [2][kManyStages][128] three bf16 terms of half of -lse / scale, of half of -Delta, of the slot's rows
-    static_assert(512 + (8 + 2 * kManyStages * kTile) * sizeof(uint4) <= kManyHeader, "header too small");
+    static_assert(42 * 8 <= 512 - 8 * sizeof(Item) && 512 + (8 + 2 * kManyStages * kTile) * sizeof(uint4) <= kManyHeader, "header too small");
     unsigned char* sK = smem_dyn + kManyHeader;                     // K of two items
     unsigned char* sV = sK + 2 * kTileBytes;
     unsigned char* sQ = sV + kTileBytes;                            // slots of (Q tile, dO tile)
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
         mbar_init(bar_dk_free, 4);
         mbar_init(bar_gfree, 8);
         for (int i = 0; i < 8; ++i) mbar_init(bar_item + i, 1);
+        for (int w = 0; w < 3; ++w) mbar_init(bar_left + w, 1);
         mbar_fence_init();
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_do);
@@ -255,10 +257,16 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
         n_t = (kept + kTile - 1) / kTile;
         n_items = n_t * P.H * P.B;                             // (short instances skip some)
     };
-    auto item_at = [&](uint32_t i) {                           // n_sel -1 for an item that did not come
-        ok &= warp_wait_relaxed(bar_item + (i & 7), (i >> 3) & 1);
+    auto item_wait = [&](uint32_t i) { ok &= warp_wait_relaxed(bar_item + (i & 7), (i >> 3) & 1); };
+    auto item_read = [&](uint32_t i) {
         const int4 x = *reinterpret_cast<const int4*>(s_item + (i & 7));
-        return Item{x.x, x.y, x.z, ok ? x.w : -1};
+        return Item{x.x, x.y, x.z, x.w};
+    };
+    auto item_at = [&](uint32_t i) {                           // n_sel -1 for an item that did not come
+        item_wait(i);
+        Item it = item_read(i);
+        if (!ok) it.n_sel = -1;
+        return it;
     };
     auto warp_arrive = [&](uint64_t* bar) {                    // all lanes are done
         __syncwarp();
@@ -461,7 +469,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             stats_load(0);
 #pragma unroll 1
             for (int x = 0; x < n_q; ++x) {
-                ok = warp_wait_relaxed(bar_q_free + st, ph ^ 1);
+                ok &= warp_wait_relaxed(bar_q_free + st, ph ^ 1);
                 if (!ok) break;
                 if (lane == 0) {                         // the tiles first: the products wait for them a step ahead of anything the statistics are for
                     mbar_expect_tx(bar_q_full + st, 2 * kTileBytes);
@@ -508,12 +516,15 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             copy_32_picked((g == 0 ? sK + (i & 1) * kTileBytes : sV) + (warp & 3) * 32 * kRowBytes, (g == 0 ? P.k : P.v) + it.b * P.sB + it.h * P.sH, P.sN, pick, P.D);
             cp_async_arrive(g == 0 ? bar_k_full + (i & 1) : bar_v_full);
         };
-        if (kRows) load_rows(0, item_at(0));
+        // Nothing bounds a named barrier.  A warp whose wait gave up goes on to the last barrier of its query tile, where all four learn of it, and all leave there: no
+        // other exit but the end of the list, which all see, since each waits for the entry of the next item ahead of that barrier.
+        load_rows(0, item_at(0));
+        ok = group_sync_and(id, ok);
         uint32_t t = 0;
 #pragma unroll 1
-        for (uint32_t i = 0;; ++i) {
-            const Item it = item_at(i);
-            if (it.n_sel < 0) { ok = group_sync_and(id, ok); break; }
+        for (uint32_t i = 0; ok; ++i) {
+            const Item it = item_read(i);
+            if (it.n_sel < 0) break;
             const int n_q = (it.n_sel + kTile - 1) / kTile;
             // dV or dK of the item's keys: a warp's 32 rows through its part of the panel, eight lanes a row
             auto rows_out = [&](uint32_t col, uint64_t* done, uint64_t* freed, float mul, __nv_bfloat16* dst) {
@@ -552,8 +563,9 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             };
             // The next item's rows ahead of anything that waits for this one's products: those of its last query tile come behind them.
             if (kRows) load_rows(i + 1, item_at(i + 1));
+            int x = 0;
 #pragma unroll 1
-            for (int x = 0; x < n_q && ok; ++x, ++t) {
+            do {
                 if (x + 1 == n_q) {                      // complete ahead of the item's last dQ, and about when it is
                     if (g == 0) rows_out(kColDv, bar_dv_done, bar_dv_free, 1.f, P.dv);
                     else rows_out(kColDk, bar_dk_done, bar_dk_free, P.scale, P.dk);
@@ -574,13 +586,14 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
                 } else {
                     warp_arrive(bar_gfree);
                 }
+                if (!kRows && x == 0) item_wait(i + 1);  // (behind the hand-off that the next dQ waits for)
                 ok = group_sync_and(id, ok);             // the panel is complete
                 if (owner && columns) {
                     tma_reduce_add_4d(&map_acc, panel, g * 32, it.h, x * kTile, it.b);
                     bulk_commit_group();
                 }
-            }
-            if (!ok) break;
+                ++t;
+            } while (++x < n_q && ok);
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         if (owner) bulk_wait_group0();                   // the last reductions of dQ have landed
@@ -637,7 +650,13 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             }
         }
     }
-    if (!ok) set_status(P.status, VARDROP_ERR_TIMEOUT);
+    if (!ok) {
+        set_status(P.status, VARDROP_ERR_TIMEOUT);
+        if (warp < 3) {                                  // what it has issued is done before tensor memory is given back
+            tc_commit_w(bar_left + warp);
+            warp_wait(bar_left + warp, 0);
+        }
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kManyTmemCols);

@@ -103,6 +103,119 @@ def test_peers_shared_memory_is_reached_behind_a_cluster_barrier():
     assert set(seen) == {"select_cluster_kernel", "hash_dft_kernel"}
 
 
+# What the branch of bwd_many_kernel that takes results out needs around it to run on the host, a thread a warp: waits that succeed but for one, and a named
+# barrier that says when not all four come.
+HOST_WARPGROUP = r"""
+#include <chrono>
+#include <condition_variable>
+#include <cstdint>
+#include <mutex>
+#include <thread>
+struct uint4 { uint32_t x, y, z, w; };
+struct float4 { float x, y, z, w; };
+typedef uint16_t __nv_bfloat16;
+struct CUtensorMap {};
+struct Item { int jt, h, b, n_sel; };
+struct Params { __nv_bfloat16 *k, *v, *dk, *dv; const int32_t *sel_idx, *n_sel; long long sB, sN, sH; int B, N, H, D, S; float scale; } P;
+const int kTile = 128, kRowBytes = 128, kTileBytes = 16384;
+const uint32_t kColDq = 0, kColDv = 0, kColDk = 0;
+alignas(16) unsigned char buf_smem[8 * 16384];
+unsigned char *sK = buf_smem, *sV = buf_smem + 2 * kTileBytes, *sOut = buf_smem + 4 * kTileBytes;
+CUtensorMap map_acc;
+const Item items[5] = {{0, 0, 0, 300}, {1, 0, 0, 100}, {0, 1, 0, 200}, {0, 0, 0, -1}, {0, 0, 0, -1}};
+std::mutex m;
+std::condition_variable cv;
+int arrived, gone, phase, waits[4], fail_warp, fail_at;
+bool all_ok, result, hung;
+thread_local int me;
+bool group_sync_and(int, bool ok) {
+    std::unique_lock<std::mutex> l(m);
+    all_ok = (arrived ? all_ok : true) && ok;
+    const int p = phase;
+    if (++arrived == 4) { arrived = 0; ++phase; result = all_ok; cv.notify_all(); return result; }
+    cv.notify_all();
+    cv.wait(l, [&] { return phase != p || hung || arrived + gone == 4; });      // the last says that no more will come
+    if (phase == p) { hung = true; cv.notify_all(); return false; }
+    return result;
+}
+bool warp_wait_relaxed(uint64_t*, uint32_t) { return !(me == fail_warp && waits[me]++ == fail_at); }
+template <class T> T __ldg(const T* p) { return *p; }
+uint32_t pack2(float, float) { return 0; }
+uint4 make_uint4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) { return {a, b, c, d}; }
+float4 make_float4(float a, float b, float c, float d) { return {a, b, c, d}; }
+template <class... A> void nothing(A&&...) {}
+#define bulk_wait_group_read0 nothing
+#define bulk_wait_group0 nothing
+#define bulk_commit_group nothing
+#define tma_reduce_add_4d nothing
+#define copy_32_picked nothing
+#define cp_async_arrive nothing
+#define tc_fence_after nothing
+#define tc_fence_before nothing
+#define tmem_ld32(at, v) for (float& e : v) e = 0.f
+#define tmem_ld_wait nothing
+#define fence_proxy_async_smem nothing
+template <bool kRows> void role(int warp, bool& left_ok) {
+    const int lane = 0, tid = warp * 32;
+    uint32_t tmem = 0;
+    bool ok = true;
+    uint64_t bars[64];
+    uint64_t *bar_k_free = bars, *bar_v_free = bars, *bar_k_full = bars, *bar_v_full = bars, *bar_dv_done = bars, *bar_dv_free = bars, *bar_dk_done = bars, *bar_dk_free = bars,
+             *bar_g = bars, *bar_gfree = bars;
+    auto begin = [] {};
+    auto item_wait = [&](uint32_t) { ok &= warp_wait_relaxed(bars, 0); };
+    auto item_read = [&](uint32_t i) { return items[i]; };
+    auto item_at = [&](uint32_t i) { item_wait(i); Item it = item_read(i); if (!ok) it.n_sel = -1; return it; };
+    auto warp_arrive = [](uint64_t*) {};
+    me = warp & 3;
+BODY
+    left_ok = ok;
+    std::lock_guard<std::mutex> l(m);
+    ++gone;
+    cv.notify_all();
+}
+// number of waits of the warp; -1: a barrier that not all four reach, -2: a warp that leaves without having learnt of the wait that gave up
+extern "C" int run(int rows, int group, int failing, int at) {
+    static __nv_bfloat16 data[512 * 2 * 64];
+    static int32_t sel[512];
+    P = Params{data, data, data, data, sel, nullptr, 512 * 128, 128, 64, 1, 512, 2, 64, 1, 1.f};
+    arrived = gone = phase = 0; hung = false; fail_warp = failing; fail_at = at;
+    for (int& w : waits) w = 0;
+    bool ok[4];
+    std::thread t[4];
+    for (int w = 0; w < 4; ++w) t[w] = std::thread([=, &ok] { rows ? role<true>(4 + 4 * group + w, ok[w]) : role<false>(4 + 4 * group + w, ok[w]); });
+    for (auto& x : t) x.join();
+    if (hung) return -1;
+    const bool gave_up = waits[failing] > at;
+    for (bool o : ok) if (o == gave_up) return -2;
+    return waits[failing];
+}
+"""
+
+
+def test_warps_that_share_a_named_barrier_leave_together(tmp_path):
+    """Nothing bounds a named barrier.  The warps that take results out in the many-tile backward share one: whichever wait of whichever warp gives up, all four learn of
+    it and leave behind the same barrier.  The text of their branch, run on the host with every wait failing in turn."""
+    body = next(text for fn, name, text in kernel_bodies() if name == "bwd_many_kernel")
+    start = body.index("{", body.index("else if (warp < 12)")) + 1
+    depth, end = 1, start
+    while depth:
+        depth += {"{": 1, "}": -1}.get(body[end], 0)
+        end += 1
+    text = re.sub(r"asm volatile[^\n]*", "", body[start:end - 1])
+    assert "setmaxnreg" not in text and text.count("group_sync_and") >= 2
+    (tmp_path / "role.cpp").write_text(HOST_WARPGROUP.replace("BODY", text))
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-w", "-shared", "-fPIC", "-pthread", "-o", str(tmp_path / "role.so"), str(tmp_path / "role.cpp")])
+    lib = C.CDLL(str(tmp_path / "role.so"))
+    for rows in (0, 1):
+        for group in (0, 1):
+            for warp in range(4):
+                waits = lib.run(rows, group, warp, 1 << 30)
+                assert waits >= 3 + 6 + 3, "items, query tiles, finished items"
+                got = [lib.run(rows, group, warp, at) for at in range(waits)]
+                assert min(got) > 0, (rows, group, warp, got)
+
+
 @pytest.fixture(scope="module")
 def plan_lib(tmp_path_factory):
     """The host-side plan of the transform, which is plain C++."""
