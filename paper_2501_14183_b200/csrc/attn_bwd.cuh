@@ -44,6 +44,7 @@ struct BwdParams {
     long long sB, sN, sH;   // element strides of q, k, v
     int B, N, Ncap, H, D, S;
     float scale, scale_log2;
+    float half_inv_scale;   // many tiles: 0.5 / scale
 };
 
 inline BwdParams bwd_params(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* d_o, const int32_t* sel_idx, const int32_t* n_sel,

@@ -442,7 +442,6 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             }
             __syncwarp();
         };
-        const float half_inv = 0.5f / P.scale;
         uint32_t st = 0, ph = 0;
         publish(0);
         Item next = item_at(0);
@@ -480,7 +479,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     uint32_t l[3], d[3];
-                    split3(-st_lse[e] * half_inv, l[0], l[1], l[2]);
+                    split3(-st_lse[e] * P.half_inv_scale, l[0], l[1], l[2]);
                     split3(-0.5f * st_delta[e], d[0], d[1], d[2]);
                     s_stats[st * kTile + e * 32 + lane] = make_uint4(l[0] | l[1] << 16, l[2], 0u, 0u);
                     s_stats[(kManyStages + st) * kTile + e * 32 + lane] = make_uint4(d[0] | d[1] << 16, d[2], 0u, 0u);
@@ -754,7 +753,12 @@ int attn_bwd_many_launch(const void* q, const void* k, const void* v, const void
     const AttnWs w = attn_layout(c);
     const QkvLayout L = qkv_layout(c);
     char* base = static_cast<char*>(ws);
-    const BwdParams P = bwd_params(q, k, v, o, lse, d_o, sel_idx, n_sel, inv_idx, c, dq, dk, dv, ws);
+    BwdParams P = bwd_params(q, k, v, o, lse, d_o, sel_idx, n_sel, inv_idx, c, dq, dk, dv, ws);
+    // -lse / scale has to be finite: in the exponents a scale counts as 2^-120 at least, against which any score below 2^90 is nothing (lse is the logarithm of the
+    // kept count then).  dQ and dK get the scale as it is.
+    const float least = fmaxf(P.scale, 7.5231638e-37f);
+    P.scale_log2 = least * 1.4426950408889634f;
+    P.half_inv_scale = 0.5f / least;
     const int gx = max(1, 8 * sm_count() / c.B);                   // of prep and convert: about eight CTAs per SM in total
     {
         PrepParams R{};

@@ -11,11 +11,11 @@ from util import assert_attn_close, bf16_tokens
 pytestmark = pytest.mark.gpu
 
 
-def run_attention(dev, B, N, H, D, sel, poison=True):
+def run_attention(dev, B, N, H, D, sel, poison=True, scale=0.0):
     """Runs forward and backward through the C ABI.  `sel` is None (all tokens) or a sorted int array.
     Returns o[B,Ns,H,D], lse[B,H,Ns], dq, dk, dv (numpy, float64) and the device status."""
     q, k, v, d_full = dev
-    cfg = vd.AttnCfg(B, N, H, D, 0.0)
+    cfg = vd.AttnCfg(B, N, H, D, scale)
     ws = vd.alloc_ws(vd.vardrop_attn_workspace_bytes(cfg))
     if poison:
         ws.view(torch.int16).fill_(0x7FC1)        # bf16 NaN pattern everywhere in the scratch
@@ -163,6 +163,22 @@ def test_attention_probabilities_are_rounded_against_the_first_keys(B, N, H, D, 
     p = torch.exp2(s - s[..., :64].amax(dim=-1, keepdim=True))
     want = (p.float().to(torch.bfloat16).double() @ v / p.sum(dim=-1, keepdim=True)).transpose(1, 2).float().to(torch.bfloat16).double()
     assert float((got - want).norm() / want.norm()) <= 3.6e-4
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -100, 2.0 ** -126, 1e-40, 0.3, 2.0])
+@pytest.mark.parametrize("N,D,Ns", [(256, 64, None), (257, 64, None), (300, 32, 200), (1030, 32, 129), (2049, 64, 300)])
+def test_attention_of_any_scale(N, D, Ns, scale):
+    """Scales of the caller's own, down to the smallest floats, whose quotients of a row's log-sum-exp overflow: every key counts the same then.  The bound: as for large tokens."""
+    dev, ref = bf16_tokens(1, N, 2, D, 0.5, seed=N)
+    sel = None if Ns is None else pick(N, Ns, seed=N)
+    o, lse, dq, dk, dv, status, _ = run_attention(dev, 1, N, 2, D, sel, scale=scale)
+    assert status == vd.OK
+    wo, wl = oracle.attn_fwd(ref[0], ref[1], ref[2], sel, scale=scale)
+    wq, wk, wv = oracle.attn_bwd(ref[0], ref[1], ref[2], ref[3][:, :Ns or N], sel, scale=scale)
+    for got, want, name in ((o, wo, "o"), (lse, wl, "lse"), (dq, wq, "dq"), (dk, wk, "dk"), (dv, wv, "dv")):
+        bound = 2e-2 * float(np.abs(want).max()) + 1e-37
+        err = float(np.abs(got - want).max())
+        assert np.all(np.isfinite(got)) and err <= bound, f"{name}: max abs error {err:.3e} > {bound:.3e}"
 
 
 @pytest.mark.parametrize("where", ["v", "d_o"])
