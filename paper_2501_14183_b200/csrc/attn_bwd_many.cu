@@ -8,6 +8,7 @@
 //
 // Each row of dq / dk / dv is written exactly once.
 #include "attn_bwd.cuh"
+#include "attn_zero_rows.h"
 
 namespace vardrop {
 
@@ -693,13 +694,10 @@ __global__ void __launch_bounds__(256) bwd_convert_kernel(const ConvertParams P)
         const int kept = largest_kept(P.n_sel, P.S, P.N), n_t = (kept + kTile - 1) / kTile, n_long = n_t * P.H * P.B % P.main_grid;
         const int ctas = static_cast<int>(gridDim.x * gridDim.y), cta = static_cast<int>(blockIdx.y * gridDim.x + blockIdx.x);
         const int n_early = n_long ? min(ctas, 8 * (P.main_grid - n_long)) : 0;
-        const float share = static_cast<float>(rows) / ctas;
-        const float more = min(2700.f * 25.f / 8.f * n_t / (48.f * row_chunks) * P.N / max(1, P.N - kept), share * (ctas - n_early) / max(1, n_early));
-        const float late = share - more * n_early / ctas;
-        auto first_row = [&](int c) { return c >= ctas ? rows : min(rows, static_cast<int>(c * late + min(c, n_early) * more)); };
-        const int end = first_row(cta + 1);
+        const RowShares shares = row_shares(rows, ctas, n_early, 2700.f * 25.f / 8.f * n_t / (48.f * row_chunks) * P.N / max(1, P.N - kept));
+        const int end = first_row(shares, cta + 1);
 #pragma unroll 1
-        for (int at = first_row(cta) + static_cast<int>(threadIdx.x >> 5) * 8; at < end; at += 64) {
+        for (int at = first_row(shares, cta) + static_cast<int>(threadIdx.x >> 5) * 8; at < end; at += 64) {
             bool dropped = false;
             if (lane < 8 && at + lane < end) {
                 const int b = small_div(at + lane, P.N);

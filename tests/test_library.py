@@ -5,6 +5,7 @@ import os
 import re
 import subprocess
 
+import numpy as np
 import pytest
 
 from paper_2501_14183_b200 import binding as vd
@@ -214,6 +215,35 @@ def test_warps_that_share_a_named_barrier_leave_together(tmp_path):
                 assert waits >= 3 + 6 + 3, "items, query tiles, finished items"
                 got = [lib.run(rows, group, warp, at) for at in range(waits)]
                 assert min(got) > 0, (rows, group, warp, got)
+
+
+def test_shares_of_the_zero_rows_cover_every_row_once(tmp_path):
+    """Where a CTA ends, the next one begins, however the compiler fuses products and sums: the shares of one build give the same rows in the other.  All rows are
+    covered; an early CTA takes no fewer than a late one, and late ones keep their part of an even share."""
+    (tmp_path / "rows.cpp").write_text('#include "attn_zero_rows.h"\nusing namespace vardrop;\n'
+                                       'extern "C" void shares(int rows, int ctas, int early, float wanted, RowShares* s) { *s = row_shares(rows, ctas, early, wanted); }\n'
+                                       'extern "C" void first(const RowShares* s, int* at) { for (int c = 0; c <= s->ctas; ++c) at[c] = first_row(*s, c); }\n')
+
+    class Shares(C.Structure):
+        _fields_ = [("rows", C.c_int), ("ctas", C.c_int), ("n_early", C.c_int), ("late", C.c_longlong), ("more", C.c_longlong)]
+
+    libs = []
+    for flags in (["-ffp-contract=off"], ["-ffp-contract=fast", "-mfma"]):
+        so = tmp_path / f"rows{len(libs)}.so"
+        subprocess.check_call(["g++", "-std=c++17", "-O2", *flags, "-shared", "-fPIC", f"-I{ROOT}/paper_2501_14183_b200/csrc", "-o", str(so), str(tmp_path / "rows.cpp")])
+        libs.append(C.CDLL(str(so)))
+    for rows in (1, 2, 700, 1025, 8192 * 8, 5968 * 6, 2049 * 32, 32 * 65536, 2 ** 31 - 1):
+        for ctas in (1, 2, 148, 1184, 1176, 5000):
+            for early in {0, 1, ctas // 3, ctas - 1, ctas}:
+                for wanted in (0.1, 3.7, 33.3, 1e4, 1e12):
+                    s, at = Shares(), [(C.c_int * (ctas + 1))() for _ in libs]
+                    libs[0].shares(rows, ctas, early, C.c_float(wanted), C.byref(s))
+                    for lib, x in zip(libs, at):
+                        lib.first(C.byref(s), x)
+                    a, b = (np.ctypeslib.as_array(x) for x in at)
+                    assert np.array_equal(a, b) and a[0] == 0 and a[-1] == rows and (np.diff(a) >= 0).all(), (rows, ctas, early, wanted)
+                    assert s.more >= 0 and s.late * ctas >= rows * 1024 * (early / ctas if wanted > 1e3 else 0) * 0.99 - ctas, (rows, ctas, early, wanted)
+                    assert a[-1] - a[-2] <= rows / ctas + 2 + ctas / 1024 + rows * 1e-6, (rows, ctas, early, wanted)
 
 
 @pytest.fixture(scope="module")
