@@ -677,24 +677,25 @@ struct ConvertParams {
     float scale;
 };
 
-// What bounds it is memory: kept rows only (dropped ones were zeroed by the main kernel), 16-byte results, two in flight a thread.  1423 of 8192
-// kept, B = 8, H = 8: 12.6 us, 15.5 when it looked every variate up (events around the launch).
-// Before that, the zero rows of dq, dk, dv for every dropped variate, a warp a row, ahead of the wait for the main kernel: CTAs come in here as that
+// What bounds it is memory: the accumulator's kept rows in, 16-byte results, two in flight a thread.
+// Ahead of that, and of the wait for the main kernel, the zero rows of dq, dk, dv for every dropped variate, a warp a row: CTAs come in here as that
 // kernel's run out of items, and it writes no row of a dropped variate.  (What these rows hang on, the selection and whoever used the buffers before, is
 // done: the main kernel itself has waited for it before it let this one in.)  Beside the items, by a warp of the main kernel, they cost as much as the memory
 // takes for them: ordinary stores hold up the queue that every barrier of the SM goes through, bulk stores the copy engine (1423 of 8192 kept, B = 8, a
 // call: 175 us beside the items, 159 here).
-__global__ void __launch_bounds__(256) bwd_convert_kernel(const ConvertParams P) {
+constexpr int kConvertPerSm = 5;       // CTAs that an SM holds (48 registers a thread)
+__global__ void __launch_bounds__(256, kConvertPerSm) bwd_convert_kernel(const ConvertParams P) {
     if (P.inv_idx) {
         const int lane = threadIdx.x & 31, rows = P.B * P.N, row_chunks = P.H * (P.D / 8);
         const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-        // Eight CTAs fit an SM.  The first ones come in where the main kernel has an item less; they take as many rows more as an item is long (2700 cycles a
-        // query tile, 25 bytes written a cycle and SM), as long as the late ones keep the early ones' part of an even share (with the early ones taking all they
-        // have time for: 2400 of 8192 kept 522 -> 520 us forward and backward, but 300 of 3000, B = 2 32.7 -> 33.1, 102 of 2049, B = 32 66.0 -> 67.2).
+        // The first CTAs come in where the main kernel has an item less, as many as those SMs hold: they stay there until it is done, and the others come behind it.
+        // They take as many rows more as an item is long (2700 cycles a query tile, 25 bytes written a cycle and SM), as long as the late ones keep the early ones'
+        // part of an even share.  (By graphs, forward and backward, counted as eight an SM | five | six, with 40 registers | eight, with 32: 1423 of 8192 kept, B = 8
+        // 232.9 us | 227.5 | 227.8 | 231.6, 400 of 4000, B = 16 102.2 | 101.9 | 103.7 | 104.5, 300 of 3000, B = 8 47.4 | 46.2 | 46.6 | 47.8.)
         const int kept = largest_kept(P.n_sel, P.S, P.N), n_t = (kept + kTile - 1) / kTile, n_long = n_t * P.H * P.B % P.main_grid;
         const int ctas = static_cast<int>(gridDim.x * gridDim.y), cta = static_cast<int>(blockIdx.y * gridDim.x + blockIdx.x);
-        const int n_early = n_long ? min(ctas, 8 * (P.main_grid - n_long)) : 0;
-        const RowShares shares = row_shares(rows, ctas, n_early, 2700.f * 25.f / 8.f * n_t / (48.f * row_chunks) * P.N / max(1, P.N - kept));
+        const int n_early = n_long ? min(ctas, kConvertPerSm * (P.main_grid - n_long)) : 0;
+        const RowShares shares = row_shares(rows, ctas, n_early, 2700.f * 25.f / kConvertPerSm * n_t / (48.f * row_chunks) * P.N / max(1, P.N - kept));
         const int end = first_row(shares, cta + 1);
 #pragma unroll 1
         for (int at = first_row(shares, cta) + static_cast<int>(threadIdx.x >> 5) * 8; at < end; at += 64) {
