@@ -72,6 +72,19 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const PrepParams P) {
 // ---------------------------------------------------------------------------------------------------------
 // main
 // ---------------------------------------------------------------------------------------------------------
+struct ManyParams {
+    const __nv_bfloat16 *k, *v;       // read by the row copies of a selection (boxes go through the tensor maps)
+    const float* lse;                 // [B, H, N]
+    const float* delta;               // [B, H, Ncap]
+    __nv_bfloat16 *dk, *dv;           // [B, N, H, D]
+    const int32_t* sel_idx;           // [S, N]; NULL: identity
+    const int32_t* n_sel;             // [S]; NULL: N
+    int* status;
+    long long sB, sN, sH;             // element strides of k and v
+    int B, N, Ncap, H, D, S;
+    float scale, scale_log2, half_inv_scale;      // of dK; in the exponents, and 0.5 / scale there
+};
+
 constexpr int kManyThreads = 896;
 // Register split (setmaxnreg works on whole warpgroups): launched with 896 x 72 = 64512 registers; the first warpgroup keeps 56 a
 // thread, the two that take results out 64, the teams take 80: 128 x 56 + 256 x 64 + 512 x 80 = 64512.
@@ -164,7 +177,7 @@ constexpr uint32_t kColK = 0, kColV = 32, kColDv = 64, kColDk = 128, kColDq = 19
 template <bool kRows>
 __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                                                                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
-                                                                   const __grid_constant__ CUtensorMap map_acc, const BwdParams P) {
+                                                                   const __grid_constant__ CUtensorMap map_acc, const ManyParams P) {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];      // (every address below is a constant then: no registers)
     // Set-up first: it touches nothing another kernel produces, so it runs while the previous kernel of the stream is still finishing.
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_dyn);
@@ -752,7 +765,15 @@ int attn_bwd_many_launch(const void* q, const void* k, const void* v, const void
     const AttnWs w = attn_layout(c);
     const QkvLayout L = qkv_layout(c);
     char* base = static_cast<char*>(ws);
-    BwdParams P = bwd_params(q, k, v, o, lse, d_o, sel_idx, n_sel, inv_idx, c, dq, dk, dv, ws);
+    ManyParams P{};
+    P.k = static_cast<const __nv_bfloat16*>(k); P.v = static_cast<const __nv_bfloat16*>(v);
+    P.lse = lse; P.delta = reinterpret_cast<const float*>(base + w.delta);
+    P.dk = static_cast<__nv_bfloat16*>(dk); P.dv = static_cast<__nv_bfloat16*>(dv);
+    P.sel_idx = sel_idx; P.n_sel = sel_idx ? n_sel : nullptr;
+    P.status = reinterpret_cast<int*>(base);
+    P.sB = L.sB; P.sN = L.sN; P.sH = L.sH;
+    P.B = c.B; P.N = c.N; P.Ncap = w.Ncap; P.H = c.H; P.D = c.D; P.S = attn_sel_rows(c, sel_idx);
+    P.scale = c.sm_scale > 0.f ? c.sm_scale : 1.f / sqrtf(static_cast<float>(c.D));
     // -lse / scale has to be finite: in the exponents a scale counts as 2^-120 at least, against which any score below 2^90 is nothing (lse is the logarithm of the
     // kept count then).  dQ and dK get the scale as it is.
     const float least = fmaxf(P.scale, 7.5231638e-37f);
@@ -764,7 +785,7 @@ int attn_bwd_many_launch(const void* q, const void* k, const void* v, const void
         R.o = static_cast<const uint4*>(o); R.d_o = static_cast<const uint4*>(d_o);
         R.delta = reinterpret_cast<float*>(base + w.delta);
         R.dq_acc = attn_fwd_clears(c, sel_idx) ? nullptr : reinterpret_cast<float4*>(base + w.dq_acc);
-        R.q = P.q;
+        R.q = static_cast<const __nv_bfloat16*>(q);
         for (int i = 0; i < 2; ++i) R.staged[i] = reinterpret_cast<uint4*>(base + w.staged[i]);
         R.sel_idx = sel_idx;
         R.sB = L.sB; R.sN = L.sN; R.sH = L.sH;
@@ -807,7 +828,7 @@ int attn_bwd_many_launch(const void* q, const void* k, const void* v, const void
     F.dq = static_cast<uint4*>(dq);
     F.sel_idx = sel_idx;
     F.n_sel = P.n_sel;
-    F.inv_idx = P.inv_idx;
+    F.inv_idx = sel_idx ? inv_idx : nullptr;
     F.main_grid = grid;
     F.dk = static_cast<uint4*>(dk); F.dv = static_cast<uint4*>(dv);
     F.B = c.B; F.N = c.N; F.Ncap = w.Ncap; F.H = c.H; F.D = c.D; F.S = P.S; F.scale = P.scale;
