@@ -90,12 +90,13 @@ def test_attention_selected_at_path_boundaries(B, N, H, D, Ns):
 
 @pytest.mark.parametrize("B,N,H,D,Ns", [(1, 2048, 1, 64, 130), (2, 2049, 1, 64, 1), (1, 2049, 2, 32, 128), (1, 2049, 1, 64, 129), (1, 2300, 3, 64, 384), (1, 257, 2, 64, None), (1, 384, 2, 64, None),
                                         (1, 1024, 2, 64, 256), (1, 1025, 2, 64, 300), (16, 1025, 2, 32, 257), (32, 2048, 1, 32, 700),
-                                        (10, 600, 8, 32, None), (8, 2049, 8, 32, 600),
+                                        (10, 600, 8, 32, None), (8, 2049, 8, 32, 600), (64, 2049, 8, 32, 102), (32, 2049, 8, 64, 128),
                                         (2, 600, 2, 64, None), (2, 2049, 2, 64, 700), (3, 880, 3, 64, None), (24, 600, 8, 32, 300)])
 def test_attention_at_the_many_tile_boundary(B, N, H, D, Ns):
     """Both sides of the largest N whose selections count as few tiles (2048, or 1024 with few heads and
     instances; without a selection 256, in the forward pass 384): one kept row, full tiles, remainders; an odd number of key
-    tiles with several items a block, so that a team without a key tile in one item has one in the next, or in none of its block's items; blocks whose first item is the odd last
+    tiles with several items a block, so that a team without a key tile in one item has one in the next, or in none of its block's items; several items of one query tile a
+    block, where all of an item's hand-offs turn over at every step; blocks whose first item is the odd last
     tiles of two heads over five and more key tiles (the second of which starts a softmax later than the first)."""
     check_case(B, N, H, D, None if Ns is None else pick(N, Ns, seed=N + Ns), 1.0, seed=N + 3 * (Ns or 0))
 
@@ -222,11 +223,13 @@ def test_attention_forward_is_deterministic():
 
 
 @pytest.mark.parametrize("B,N,H,D,Ns", [(2, 300, 2, 64, 260), (2, 600, 2, 64, 300), (1, 700, 2, 64, None), (2, 321, 2, 64, 97), (1, 2100, 2, 64, 200),
-                                        (2, 2100, 2, 32, 400)])
+                                        (2, 2100, 2, 32, 400), (32, 2049, 8, 64, 102), (64, 2049, 8, 32, 128), (20, 2049, 8, 64, 250), (40, 2049, 8, 32, 256), (16, 600, 8, 64, None),
+                                        (16, 600, 8, 32, None)])
 def test_attention_backward_is_reproducible(B, N, H, D, Ns):
     """Few tiles, many tiles with a selection and of all tokens: every gradient is bit for bit the same from run to run while
     no (instance, head) pair has more than two key tiles' worth of additions per accumulator row (two fp32 addends commute);
-    with more tiles dq may differ in the last bits only.  Guards the shared-memory hand-offs inside the backward kernel."""
+    with more tiles dq may differ in the last bits only.  Guards the shared-memory hand-offs inside the backward kernels, and in the many-tile one the order of products that
+    it takes for given (scores over probabilities that the product issued before them reads): several items a block, of one, two and five key tiles, at both head sizes."""
     dev, _ = bf16_tokens(B, N, H, D, 1.0, seed=N + (Ns or 0))
     sel = None if Ns is None else pick(N, Ns, 3)
     runs = [run_attention(dev, B, N, H, D, sel, poison=False) for _ in range(3)]
@@ -300,7 +303,8 @@ def test_attention_per_instance_selections():
     (24, 260, 8, 32, [100 + (37 * i) % 160 for i in range(24)]),               # many of two and three: every CTA both kinds
     (3, 200, 1, 64, [129, 1, 128]), (2, 300, 2, 64, [130, 300]), (3, 300, 2, 64, [0, 128, 260]),
     # the many-tile kernels: nothing kept, one row, whole tiles, odd and even tile counts, more items than blocks
-    (5, 2100, 4, 64, [0, 1, 256, 300, 700]), (9, 1030, 3, 32, [5, 130, 257, 384, 640, 128, 900, 1, 129]), (16, 2060, 8, 32, [100 + 37 * i for i in range(16)])])
+    (5, 2100, 4, 64, [0, 1, 256, 300, 700]), (9, 1030, 3, 32, [5, 130, 257, 384, 640, 128, 900, 1, 129]), (16, 2060, 8, 32, [100 + 37 * i for i in range(16)]),
+    (64, 2049, 8, 32, [(128, 1, 100, 0, 127)[i % 5] for i in range(64)])])
 def test_attention_instances_of_one_and_of_several_tiles(B, N, H, D, counts):
     dev, ref = bf16_tokens(B, N, H, D, 1.0, seed=B + N)
     q, k, v, d_o = dev
