@@ -299,7 +299,7 @@ def kernel_work(w, n_sel, selected=True):
     kept = w.B * n_sel
     full = w.B * w.N
     grads = 3 * (full if selected else kept) * row                  # dq, dk, dv come back in the full layout
-    many = w.N > (2048 if selected else 256)                        # dq and the zero rows come from the convert kernel then, Delta from the prep kernel
+    many = w.N > ((1024 if w.B * w.H < 32 else 2048) if selected else 256)      # attn_many_tiles of csrc/attn_common.cuh: dq and the zero rows come from the convert kernel then, Delta from the prep kernel
     return {
         "hash_kernel": (w.B * w.N * w.L * 4 + w.N * (8 + 4 * w.k), None),
         "select_small_kernel": (w.N * (8 + 6 * 4), None),
