@@ -31,9 +31,10 @@ struct PrepParams {
 };
 
 // One thread per 16-byte chunk of a (token, head) row of 64; the 8 threads of a row reduce Delta by shuffles.  With a selection the rows
-// that the main kernel reads again for every pair of key tiles (Q, dO) are laid out here once, zeros up to the tile's end (rows of dO past the
-// kept ones may hold anything), so that it takes boxes: row copies by its two loader warps bound it at 1423 kept tokens (250 us against 170).
-// K and V it reads once, as rows, and under the end of the item before (laid out here too, a step of 8192 variates took 311.8 us instead of 304.6).
+// that the main kernel reads again for every key tile (Q, dO) are laid out here once, zeros up to the tile's end (rows of dO past the kept ones
+// may hold anything), so that it takes boxes.  K and V it reads once an item, as rows, under the products of the item before.  (Both measured with an earlier
+// main kernel, of two key tiles an item: Q and dO by row copies 250 us at 1423 kept of 8192 against 170, K and V laid out here too a step of 8192 variates 311.8 us
+// against 304.6.)
 __global__ void __launch_bounds__(256) bwd_prep_kernel(const PrepParams P) {
     chain_wait();
     chain_release();
@@ -157,19 +158,21 @@ __device__ __forceinline__ bool group_sync_and(int id, bool ok) {     // barrier
 //   warps 8-11   columns 32 to 63; dK of a finished item; V rows of a selection
 //   warps 12-19  team 0, warps 20-27  team 1: two threads a key row, 32 queries each.  A step: S^T to registers, P^T = exp2(S^T scale - lse) over it,
 //                dP^T to registers, dS^T = P^T o (dP^T - Delta) over it and to shared memory (for dQ, through the transposed view)
-// What bounds a step of 128 x 128 scores (2700 cycles): operands read by the tensor core from shared memory at 128 bytes a cycle, and the team's chain of
-// latencies; with every variate kept, B = 8, N = 8192, the power limit.
-//   - A operands come from tensor memory wherever they can (K and V copied there once an item, P^T, dS^T): a product of N = 64 then takes 32 cycles
-//     instead of 48, 1600 a step instead of 1920, and the shared-memory pipe 2200 instead of 2800.
+// What bounds a step of 128 x 128 scores (2700 cycles): the shared-memory pipe, 128 bytes a cycle, of which 1109 go to the tensor core's operands, 875 to the threads' own
+// accesses and 533 to the copy engine (2500 of 2800 under ncu, all of 1423 variates, B = 8); with every variate kept, B = 8, N = 8192, the power limit.
+//   - A operands come from tensor memory wherever they can (K and V copied there once an item, P^T, dS^T): a product of N = 64 then takes 32 cycles instead of 48
+//     and reads 2 KB instead of 6; 1600 cycles a step instead of 1920.
 //   - -lse / scale and -Delta of a query are three bf16 terms each (24 bits) of a fifth k-step of S^T and dP^T, against rows of ones: no thread reads them
 //     (64 broadcast loads a row and step), and without their registers nothing spills.  Each product has rows of its own and meets them with ones and with the
 //     zeros behind the terms only: a row of both, picked from by ones and zeros, takes a Delta that is not finite into S^T (0 times infinity), and so into every
-//     column of dV.  (6 KB more of shared memory; no difference in time that shows.)
-//   - The tensor core runs the products of one thread in order: S^T of the next query tile goes over P^T right behind the dV that reads it, dP^T over dS^T
-//     behind dK, so a team hands over three times a step and waits for neither.
+//     column of dV.  (6 KB more of shared memory; by events, 32 x 862 325.1 us -> 325.2, scale step 287.4 -> 287.8.)
+//   - S^T of the next query tile is issued over P^T right behind the dV that reads it, dP^T over dS^T behind dK, so a team hands over three times a step and waits for
+//     neither.  This takes for given that the products of one thread run in the order of their issue also where accumulators and shapes differ; the instruction set
+//     documents the order for the same accumulator and shape.  Held by gradients that are the same bit for bit from run to run, at both head sizes and with several
+//     items a CTA (test_attention_backward_is_reproducible).
 //   - At the end of an item the next K and V are copied in behind the last products that read the old ones; the teams never leave the steps.
-// Two 128-key tiles a CTA, a team each, with K and V from shared memory (before this), took 3500 cycles for as many scores: forward and backward, B = 8, H = 8,
-// 8192 variates 4810 -> 4560 us, 1423 of 8192 kept 258 -> 243 (by events), 700 of 8192 171 -> 120; B = 32, 862 variates 346 -> 321.
+// Two 128-key tiles a CTA, a team each, with K and V from shared memory (before this), took 3500 cycles for as many scores: forward and backward by graphs, H = 8, all of
+// 8192 variates, B = 8 4720 -> 4450 us, 1423 of 8192 kept 247.0 -> 227.5, 700 of 8192 158.5 -> 109.4; all of 862, B = 32 338.5 -> 294.
 // Tensor memory: K 32 | V 32 | dV 64 | dK 64 | dQ 64 | team 0: S^T, P^T 64, dP^T, dS^T 64 | team 1.
 constexpr uint32_t kColK = 0, kColV = 32, kColDv = 64, kColDk = 128, kColDq = 192, kColTeam = 256;
 
@@ -426,7 +429,7 @@ __global__ void __launch_bounds__(kManyThreads, 1) bwd_many_kernel(const __grid_
             }
         }
     } else {
-        // ------------------------------------------------------------ loads, items, zero rows ---------------------------
+        // ------------------------------------------------------------ loads, items --------------------------------------
         int k = blockIdx.x;                              // next item to publish, in grid steps
         auto publish = [&](uint32_t i) {
             Item it{0, 0, 0, -1};

@@ -43,6 +43,8 @@ __device__ __forceinline__ void set_status(int* status, int code) { atomicCAS(st
 // run their set-up (shared-memory tables, barriers, tensor-memory allocation) while the previous kernel of the
 // stream is still finishing.  chain_wait() returns once that kernel has completed and its writes are visible: nothing
 // that another kernel produces or reads is touched before it.  chain_release() lets the next kernel's CTAs in.
+// One exception: bwd_convert_kernel writes zero rows ahead of its wait.  The launch before it is always this library's main backward kernel, which writes no such
+// row and lets dependents in behind its own wait only, so whatever lies before the main kernel has completed.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
