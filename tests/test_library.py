@@ -228,7 +228,8 @@ def test_shares_of_the_zero_rows_cover_every_row_once(tmp_path):
         _fields_ = [("rows", C.c_int), ("ctas", C.c_int), ("n_early", C.c_int), ("late", C.c_longlong), ("more", C.c_longlong)]
 
     libs = []
-    for flags in (["-ffp-contract=off"], ["-ffp-contract=fast", "-mfma"]):
+    fma = ["-mfma"] if " fma " in open("/proc/cpuinfo").read() else []
+    for flags in (["-ffp-contract=off"], ["-ffp-contract=fast", *fma]):
         so = tmp_path / f"rows{len(libs)}.so"
         subprocess.check_call(["g++", "-std=c++17", "-O2", *flags, "-shared", "-fPIC", f"-I{ROOT}/paper_2501_14183_b200/csrc", "-o", str(so), str(tmp_path / "rows.cpp")])
         libs.append(C.CDLL(str(so)))
